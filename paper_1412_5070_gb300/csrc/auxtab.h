@@ -5,14 +5,36 @@
 // same way.
 #pragma once
 
+#include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <map>
+#include <thread>
 #include <vector>
 
 #include "aux.cuh"
 #include "termlist.h"
 
 namespace f12dev {
+
+// fn(i) for i < n on the host's cores (long double arithmetic is in software
+// on AArch64: the tables below took 3.6 s there on one core, and 0.28 s of
+// every f12int_set_factor).
+template <class Fn>
+inline void parallel_for(int n, Fn fn) {
+  const int nt = std::max(1, std::min({n, (int)std::thread::hardware_concurrency(), 16}));
+  std::atomic<int> next{0};
+  auto work = [&] {
+    for (int i = next++; i < n; i = next++) fn(i);
+  };
+  std::vector<std::thread> th;
+  try {
+    for (int t = 1; t < nt; ++t) th.emplace_back(work);
+  } catch (...) {   // no more threads: the ones there, and this one, do the work
+  }
+  work();
+  for (std::thread &t : th) t.join();
+}
 
 // Gauss-Hermite nodes and weights (weight e^{-t^2}) from the orthonormal
 // Hermite recurrence: sign changes on a fine grid, then Newton.
@@ -399,23 +421,21 @@ inline long double kummer_scaled(long double a, long double b, long double x) {
 inline void fill_kummer_table(std::vector<double> &tab) {
   tab.assign((size_t)(LAUX + 1) * MT_NA * MT_NX * MT_NT, 0.0);
   constexpr int NB = LAUX + MT_NT;   // b = 3/2 .. LAUX + MT_NT + 1/2
-  std::vector<long double> tb((size_t)NB);
-  for (int ia = 0; ia < MT_NA; ++ia) {
-    const long double a = 0.5L * (ia + 1);
-    for (int ix = 0; ix < MT_NX; ++ix) {
-      const long double x = (long double)ix * (long double)MT_DX;
-      for (int ib = 0; ib < NB; ++ib) tb[ib] = kummer_scaled(a, 1.5L + ib, x);
-      for (int l = 0; l <= LAUX; ++l) {
-        const long double b = 1.5L + l;
-        long double c = 1.0L;   // (-1)^m (b - a)_m / ((b)_m m!)
-        double *row = &tab[(((size_t)l * MT_NA + ia) * MT_NX + ix) * MT_NT];
-        for (int m = 0; m < MT_NT; ++m) {
-          row[m] = (double)(c * tb[l + m]);
-          c *= -(b - a + m) / ((b + m) * (m + 1));
-        }
+  parallel_for(MT_NA * MT_NX, [&](int i) {
+    const int ia = i / MT_NX, ix = i % MT_NX;
+    const long double a = 0.5L * (ia + 1), x = (long double)ix * (long double)MT_DX;
+    long double tb[NB];
+    for (int ib = 0; ib < NB; ++ib) tb[ib] = kummer_scaled(a, 1.5L + ib, x);
+    for (int l = 0; l <= LAUX; ++l) {
+      const long double b = 1.5L + l;
+      long double c = 1.0L;   // (-1)^m (b - a)_m / ((b)_m m!)
+      double *row = &tab[(((size_t)l * MT_NA + ia) * MT_NX + ix) * MT_NT];
+      for (int m = 0; m < MT_NT; ++m) {
+        row[m] = (double)(c * tb[l + m]);
+        c *= -(b - a + m) / ((b + m) * (m + 1));
       }
     }
-  }
+  });
 }
 
 // J_a(y) = int_0^inf t^a e^{y t - t^2} dt, a > -1, y >= 0, in long double from
@@ -455,7 +475,10 @@ inline void build_start_tables(ClassTables &ct) {
     const long double as = d.fp_minus1 ? 0.0L : (long double)d.alpha0;
     d.jrow = d.fp_minus1 ? 2 * JT_NK : JT_NK;
     d.jtab = (int)ct.jtab.size();
-    for (int i = 0; i < JT_NY; ++i) {
+    ct.jtab.resize(ct.jtab.size() + (size_t)JT_NY * (size_t)d.jrow);
+    double *rows = ct.jtab.data() + d.jtab;
+    parallel_for(JT_NY, [&](int i) {
+      double *row = rows + (size_t)i * (size_t)d.jrow;
       const long double y = (long double)i * (long double)JT_DY;
       long double J[JT_NK + 1];
       J[0] = jstart_host(as, y);
@@ -466,7 +489,7 @@ inline void build_start_tables(ClassTables &ct) {
       for (int k = 0; k < JT_NK; ++k) {
         if (k > 0) fk *= k;
         e[k] = J[k] / fk;
-        ct.jtab.push_back((double)e[k]);
+        *row++ = (double)e[k];
       }
       if (d.fp_minus1) {
         // t_m = y^m Gamma(m/2) / (2 m!): t_1 = y sqrt(pi)/2, t_{m+1} = t_m y g_m/(m+1)
@@ -482,10 +505,10 @@ inline void build_start_tables(ClassTables &ct) {
             if (m > 2.0L * y * y + 10 && t <= 1e-21L * T) break;
           }
         }
-        ct.jtab.push_back((double)T);
-        for (int k = 1; k < JT_NK; ++k) ct.jtab.push_back((double)(e[k - 1] / k));
+        *row++ = (double)T;
+        for (int k = 1; k < JT_NK; ++k) *row++ = (double)(e[k - 1] / k);
       }
-    }
+    });
   }
 }
 

@@ -28,6 +28,7 @@ struct EngineReq {
   int basis = 0;
   const f12int_ctx::BasisData *B = nullptr;   // stable: the deque never moves its elements
   uint32_t mask = 0;
+  bool grid = false;                  // every class from the auxiliary grid
   int precision = 0;                  // 1: FP32 recursion and contraction below the FP32 bound
   double thresh = 0.0;
   double *out = nullptr;
@@ -91,11 +92,12 @@ struct ClassLists {
   int64_t *offsets = nullptr;     // [qcap]
   int32_t *qslot = nullptr;       // [qcap]
   CTask *tasks = nullptr;         // [tcap], tier after tier
-  int64_t *counts = nullptr;      // n, npq, then (begin, end) of the tasks of each tier
+  int64_t *counts = nullptr;      // n, npq, npq before the thin quartets, then (begin, end) of the tasks of each tier
   PairView *views = nullptr;      // [scap]
   double **outs = nullptr;        // [scap]
 };
-constexpr int kCounts = 2 + 2 * kSlots;
+constexpr int kCounts = 3 + 2 * kSlots;
+constexpr int kTaskCounts = 3;           // first of the tiers' (begin, end)
 
 struct Engine {
   // limits
@@ -124,9 +126,11 @@ struct Engine {
   // graph
   cudaStream_t stream = nullptr;
   cudaStream_t branch[7] = {nullptr};   // capture streams of the class branches
-  cudaGraphExec_t exec = nullptr;
-  bool graph_dirty = true;
-  int items_blocks = 0, quad_blocks = 0, classify_blocks = 0, tier_blocks[kLaunches] = {0};
+  // one graph for batches evaluated from the auxiliary grid, one for batches
+  // evaluated family by family; a batch is all of one kind
+  cudaGraphExec_t exec[2] = {nullptr, nullptr};
+  bool graph_dirty[2] = {true, true};
+  int items_blocks = 0, quad_blocks = 0, classify_blocks = 0, grid_blocks = 0, tier_blocks[kLaunches] = {0};
   int thin_blocks = 0;           // persistent thin contraction launches
   double fp32_below = 1e-5;           // mixed requests: FP32 below this screening estimate
   // per-class schedule (f12int_batch_autotune): work target of a contraction
@@ -200,10 +204,10 @@ __global__ void k_zero_blocks(double *const *dst, const int64_t *len, const int6
 }
 
 // Capture the launch sequence of one batch (every class, every tier).
-static int engine_capture(f12int_ctx *ctx, Engine &E) {
-  if (E.exec) {
-    cudaGraphExecDestroy(E.exec);
-    E.exec = nullptr;
+static int engine_capture(f12int_ctx *ctx, Engine &E, bool grid) {
+  if (E.exec[grid]) {
+    cudaGraphExecDestroy(E.exec[grid]);
+    E.exec[grid] = nullptr;
   }
   for (int t = 0; t < kTiers; ++t)
     if (kTierCap[t] > 48 * 1024) {
@@ -225,9 +229,15 @@ static int engine_capture(f12int_ctx *ctx, Engine &E) {
       cudaStream_t bs = E.branch[cls];
       cudaStreamWaitEvent(bs, fork, 0);
       const int kcls = cls == 5 ? 3 : cls;
-      const int nf = ctx->tables.nfam[kcls];
+      // (a class without a grid has no quartets in a grid batch)
+      const GridView G = grid ? class_view(ctx, cls) : GridView{nullptr, nullptr, nullptr};
+      const int nf = G.direct() ? 1 : ctx->tables.nfam[kcls];
       const ClassLists &L = E.dev[cls];
       QuartetView QV{L.quartets, L.pq_off, 0, L.counts, L.qslot, L.views, L.outs};
+      if (G.direct()) {
+        k_direct_rows<true><<<E.grid_blocks, BLOCK_AUX, 0, bs>>>(G, none, QV, cls, 0, 0, E.keys[cls], E.part[cls],
+                                                               nullptr);
+      } else {
       cudaMemsetAsync(E.hist[cls], 0, sizeof(unsigned) * kNKeys, bs);
       k_items_classify<true><<<E.classify_blocks, BLOCK_AUX, 0, bs>>>(ctx->tables, none, QV, cls, 0, 0,
                                                                       E.keys[cls], E.hist[cls]);
@@ -241,15 +251,16 @@ static int engine_capture(f12int_ctx *ctx, Engine &E) {
         k_items_eval<true, true><<<E.quad_blocks, BLOCK_AUX, 0, bs>>>(ctx->tables, none, QV, cls, 0, 0,
                                                                        E.order[cls], E.keys[cls], E.part[cls],
                                                                        E.status, nullptr);
+      }
       for (int t = 0; t < kLaunches; ++t) {
         const int tt = t % kTiers;
         if (t < kTiers)
           k_contract<true, double><<<E.tier_blocks[t], 32 * kTierWarps[tt], kTierCap[tt], bs>>>(
-              none, QV, cls, nf, 0, L.tasks, 0, L.counts + 2 + 2 * t, E.keys[cls], E.part[cls], nullptr, L.offsets,
+              none, QV, cls, nf, 0, L.tasks, 0, L.counts + kTaskCounts + 2 * t, E.keys[cls], E.part[cls], nullptr, L.offsets,
               E.status, nullptr);
         else
           k_contract<true, float><<<E.tier_blocks[t], 32 * kTierWarps[tt], kTierCap[tt], bs>>>(
-              none, QV, cls, nf, 0, L.tasks, 0, L.counts + 2 + 2 * t, E.keys[cls], E.part[cls], nullptr, L.offsets,
+              none, QV, cls, nf, 0, L.tasks, 0, L.counts + kTaskCounts + 2 * t, E.keys[cls], E.part[cls], nullptr, L.offsets,
               E.status, nullptr);
       }
       // one persistent launch per thin (la, lb, lc, ld) of the class kind
@@ -257,7 +268,7 @@ static int engine_capture(f12int_ctx *ctx, Engine &E) {
         const int slot = thin_quartet(k, cls) ? thin_slot(k, cls == 5) : -1;
         if (slot < 0) continue;
         thin_kernel(k, cls == 5)<<<E.thin_blocks, 32 * kThinWarps, 0, bs>>>(
-            none, QV, nf, 0, L.tasks, 0, L.counts + 2 + 2 * (kThinSlot + slot), E.keys[cls], E.part[cls], nullptr,
+            none, QV, nf, 0, G, L.tasks, 0, L.counts + kTaskCounts + 2 * (kThinSlot + slot), E.keys[cls], E.part[cls], nullptr,
             L.offsets, nullptr);
       }
       cudaEventRecord(join[cls], bs);
@@ -265,13 +276,13 @@ static int engine_capture(f12int_ctx *ctx, Engine &E) {
     }
     e = cudaStreamEndCapture(cs, &g);
   }
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&E.exec, g, 0);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&E.exec[grid], g, 0);
   if (g) cudaGraphDestroy(g);
   cudaStreamDestroy(cs);
   cudaEventDestroy(fork);
   for (int c = 1; c <= 6; ++c) cudaEventDestroy(join[c]);
   if (e != cudaSuccess) return cuda_fail(e);
-  E.graph_dirty = false;
+  E.graph_dirty[grid] = false;
   return F12INT_OK;
 }
 
@@ -326,6 +337,8 @@ static int engine_init(f12int_ctx *ctx, Engine &E) {
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_items_eval<true, true>, BLOCK_AUX, 0));
   E.quad_blocks = nsm * std::max(per, 1);
   E.classify_blocks = nsm * 8;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_direct_rows<true>, BLOCK_AUX, 0));
+  E.grid_blocks = nsm * std::max(per, 1);
   for (int t = 0; t < kTiers; ++t) {
     if (kTierCap[t] > 48 * 1024) {
       CK(cudaFuncSetAttribute(k_contract<true, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTierCap[t]));
@@ -360,7 +373,7 @@ static void engine_finish_batch(Engine &E, int b) {
 }
 
 // Build the lists of one batch in staging buffer b and launch it.
-static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq *> &batch, int b) {
+static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq *> &batch, int b, bool grid) {
   struct Item {
     int64_t src;      // index into the flat per-class arrays below
     int tier, nsplit;
@@ -433,10 +446,11 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
     S.counts[1] = npq;
     int64_t i = 0;
     for (int t = 0; t < kSlots; ++t) {
-      S.counts[2 + 2 * t] = nt;
+      if (t == kThinSlot) S.counts[2] = S.pq_off[i];
+      S.counts[kTaskCounts + 2 * t] = nt;
       for (; i < n && items[i].tier == t; ++i)
         for (int sp = 0; sp < items[i].nsplit; ++sp) S.tasks[nt++] = CTask{(int32_t)i, (int16_t)sp, (int16_t)items[i].nsplit};
-      S.counts[3 + 2 * t] = nt;
+      S.counts[kTaskCounts + 1 + 2 * t] = nt;
     }
     // copy what this batch uses
     const ClassLists &D = E.dev[cls];
@@ -460,7 +474,7 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
     CK(cudaMemcpyAsync(E.zero_dst, E.zstage_dst[b], sizeof(double *) * nzero, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(E.zero_len, E.zstage_len[b], sizeof(int64_t) * nzero, cudaMemcpyHostToDevice, st));
   }
-  CK(cudaGraphLaunch(E.exec, st));
+  CK(cudaGraphLaunch(E.exec[grid], st));
   CK(cudaMemcpyAsync(E.stage_status[b], E.status, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
   CK(cudaMemsetAsync(E.status, 0, sizeof(unsigned), st));
   CK(cudaEventRecord(E.ev[b], st));
@@ -492,7 +506,7 @@ static void engine_worker(f12int_ctx *ctx, Engine *Ep) {
       for (int c = 1; c <= 6; ++c)
         if (nq[c] + R->quartets[c] > E.qcap || ni[c] + R->items[c] > E.icap || nt[c] + R->tasks[c] > E.tcap)
           fits = false;
-      if (!fits && !batch.empty()) break;
+      if (!batch.empty() && (!fits || R->grid != batch.front()->grid)) break;
       for (int c = 1; c <= 6; ++c) {
         nq[c] += R->quartets[c];
         ni[c] += R->items[c];
@@ -502,10 +516,11 @@ static void engine_worker(f12int_ctx *ctx, Engine *Ep) {
       E.pending.pop_front();
     }
     int rc = F12INT_OK;
-    if (E.graph_dirty) rc = engine_capture(ctx, E);
+    const bool grid = batch.front()->grid;
+    if (E.graph_dirty[grid]) rc = engine_capture(ctx, E, grid);
     for (EngineReq *R : batch) E.tickets[R->ticket].batch = b;
     lk.unlock();
-    if (rc == F12INT_OK) rc = engine_launch(ctx, E, batch, b);
+    if (rc == F12INT_OK) rc = engine_launch(ctx, E, batch, b, grid);
     lk.lock();
     for (EngineReq *R : batch) {
       if (rc == F12INT_OK) {
@@ -553,7 +568,8 @@ static void engine_shutdown(f12int_ctx *ctx) {
     if (E->branch[c]) cudaStreamDestroy(E->branch[c]);
   }
   ctx->used -= std::min(ctx->used, E->bytes);
-  if (E->exec) cudaGraphExecDestroy(E->exec);
+  for (cudaGraphExec_t x : E->exec)
+    if (x) cudaGraphExecDestroy(x);
   if (E->stream) cudaStreamDestroy(E->stream);
   for (EngineReq *R : E->pending) delete R;
   delete E;
@@ -577,7 +593,7 @@ static bool engine_idle(f12int_ctx *ctx) {
 static void engine_factor_changed(f12int_ctx *ctx) {
   if (ctx->engine) {
     std::lock_guard<std::mutex> lk(ctx->engine->mu);
-    ctx->engine->graph_dirty = true;
+    ctx->engine->graph_dirty[0] = ctx->engine->graph_dirty[1] = true;
   }
 }
 
@@ -641,6 +657,7 @@ int f12int_submit(f12int_ctx *ctx, int basis_id, const f12int_request *req, uint
   R->out = req->out_dev;
   R->q.assign(req->quartets, req->quartets + 4 * n);
   R->off.assign(req->offsets, req->offsets + (size_t)nclass * n);
+  R->grid = true;
   int64_t npq = 0;
   for (int64_t i = 0; i < n; ++i) {
     const int32_t *s = &R->q[4 * (size_t)i];
@@ -682,6 +699,7 @@ int f12int_submit(f12int_ctx *ctx, int basis_id, const f12int_request *req, uint
       delete R;
       return rc;
     }
+    if (R->grid && !grid_view(ctx, B, c).direct()) R->grid = false;
     R->quartets[c] = n;
     R->items[c] = npq * ctx->tables.nfam[c == 5 ? 3 : c];
   }
@@ -797,7 +815,7 @@ int f12int_batch_autotune(f12int_ctx *ctx, int basis_id, const int32_t *quartets
           std::lock_guard<std::mutex> lk(ctx->engine->mu);
           ctx->engine->task_target[c] = tg;
           ctx->engine->items_div[c] = dv;
-          ctx->engine->graph_dirty = true;
+          ctx->engine->graph_dirty[0] = ctx->engine->graph_dirty[1] = true;
         }
         double t1 = 0.0, t2 = 0.0;
         rc = run(c, &t1);   // first run after a change includes the graph capture
@@ -814,7 +832,7 @@ int f12int_batch_autotune(f12int_ctx *ctx, int basis_id, const int32_t *quartets
       std::lock_guard<std::mutex> lk(ctx->engine->mu);
       ctx->engine->task_target[c] = bt;
       ctx->engine->items_div[c] = bd;
-      ctx->engine->graph_dirty = true;
+      ctx->engine->graph_dirty[0] = ctx->engine->graph_dirty[1] = true;
     }
     if (report) {
       report[3 * (c - 1)] = bt;

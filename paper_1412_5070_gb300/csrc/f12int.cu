@@ -35,6 +35,7 @@
 #include "aux.cuh"
 #include "kernel_common.cuh"
 #include "auxtab.h"
+#include "grid.h"
 #include "termlist.h"
 
 using namespace f12dev;
@@ -59,41 +60,6 @@ __constant__ unsigned char c_cart[LSH + 3][28][3];  // shell l (<= 5) -> compone
 // device status word bits: 1 = an auxiliary series hit its length cap,
 // 4 = a quartet needs a radial order above LAUX
 
-
-// Growth of a kernel with distance, tabulated at this step (screening).
-constexpr double kGrowStep = 0.05, kGrowMax = 120.0;
-constexpr double kPrimScreen = 1e-26;
-
-
-// Primitive quartets whose Schwarz product is below kPrimScreen are skipped:
-// the skipped contributions stay below the absolute accuracy that elements
-// just above 1e-12 need for a relative error of 1e-10.  The diagonal
-// integrals behind qprim sample the kernel at short range; a kernel that
-// grows with r (Eq. rs12 with B > 0: I2, I3 like e^{Br}, k4 = f f' and
-// k6 = f_r f'_r like e^{2Br}) is larger at the separation R = |P - Q| of the
-// two charge distributions, whose overlap e^{-xi w^2} reaches out to R + w.
-// A candidate is weighed, as the shell screen weighs a shell quartet, by
-//   Gamma = max over w = 0, 0.5, .., 3 (units of 1/sqrt(xi)) of G(R + w) e^{-xi w^2}
-// (e^{-xi w^2} = e^{-k^2/4} at the k-th sample).
-__device__ __forceinline__ bool prim_negligible(const PairView &PV, int pab, int pcd) {
-  if (!PV.qprim) return false;
-  const double v = PV.qprim[pab] * PV.qprim[pcd];
-  if (v >= kPrimScreen) return false;
-  if (!PV.grow) return true;
-  const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
-               Z = pair_sep(PV.pp_P, pab, pcd, 2);
-  const double p = PV.pp_p[pab], q = PV.pp_p[pcd];
-  const double R = sqrt(X * X + Y * Y + Z * Z), hw = 0.5 * sqrt((p + q) / (p * q));
-  constexpr double kOverlap[7] = {1.0, 0.77880078307140487, 0.36787944117144233, 0.10539922456186433,
-                                  0.018315638888734179, 0.0019304541362277093, 0.00012340980408667956};
-  double gam = 0.0;
-#pragma unroll
-  for (int k = 0; k < 7; ++k) {
-    const int i = min(PV.ngrow - 1, (int)((R + k * hw) * (1.0 / kGrowStep)) + 1);
-    gam = fmax(gam, PV.grow[i] * kOverlap[k]);
-  }
-  return v * gam < kPrimScreen;
-}
 
 // ------------------------------------------------------------ pair builder --
 // E_0^{00} = exp(-(ab/p) X_AB^2)  (Eq. Erec0); upward in i and j with
@@ -377,12 +343,105 @@ __global__ void k_items_eval(Tables T, PairView PV, QuartetView QV, int cls, int
 
 
 
-// hat g_n at given (xi, D) points (no prefactor), for the aux-stage tests.
-__global__ void k_aux_points(Tables T, int cls, int64_t npts, const double *xi, const double *D, int nmax,
-                             double *out, unsigned int *status) {
+// Auxiliary functions of the general contraction's quartets from the grid (or
+// the Boys table): one thread per primitive quartet, hat g_n (n <= L) into its row, or its key set
+// to the skip key.  L is the same for whole stretches of the list, so a warp
+// nearly always takes one of the instances below.
+template <int L>
+__device__ __forceinline__ void direct_row(const GridView &G, double xi, double u, double2 *o) {
+  double h[L + 1];
+  aux_direct<L>(G, xi, u, h);
+  const double is = 1.0 / sqrt(xi);
+#pragma unroll
+  for (int l = 0; l <= (L | 3); l += 2)
+    o[l >> 1] = make_double2(l <= L ? is * h[l <= L ? l : 0] : 0.0, l + 1 <= L ? is * h[l + 1 <= L ? l + 1 : 0] : 0.0);
+}
+
+template <bool BATCH>
+__global__ void __launch_bounds__(BLOCK_AUX)
+k_direct_rows(GridView G, PairView PV0, QuartetView QV, int cls, int64_t pq0, int64_t npq, int *keys, double *part,
+            unsigned long long *fma_total) {
+  // in a batch count_dev[2] is the number of primitive quartets that the
+  // general contraction reads (the thin ones follow them in the list)
+  const int64_t n = BATCH ? QV.count_dev[2] : npq;
+  unsigned long long nfma = 0;
+  for (int64_t r0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & ~(int64_t)31; r0 < n;
+       r0 += (int64_t)gridDim.x * blockDim.x) {   // warp-uniform
+    const int lane = threadIdx.x & 31;
+    int64_t lo = lane == 0 ? find_quartet(QV.pq_off, qv_count(QV), pq0 + r0) : 0;
+    lo = __shfl_sync(0xffffffffu, lo, 0);
+    const int64_t r = r0 + lane, pq = pq0 + r;
+    if (r >= n) continue;
+    // every quartet holds at least one primitive quartet: the lane's lies within `lane` of the warp's first
+    int64_t hi = min(lo + lane, qv_count(QV) - 1);
+    while (lo < hi) {
+      const int64_t mid = (lo + hi + 1) >> 1;
+      if (QV.pq_off[mid] <= pq) lo = mid;
+      else hi = mid - 1;
+    }
+    const PairView &PV = qv_view<BATCH>(PV0, QV, lo);
+    const int32_t *s = QV.quartets + 4 * lo;
+    const int ns = PV.nshell;
+    const int ab = s[0] * ns + s[1], cd = s[2] * ns + s[3];
+    const int npcd = PV.pair_start[cd + 1] - PV.pair_start[cd];
+    const int k = (int)(pq - QV.pq_off[lo]);
+    const int pab = PV.pair_start[ab] + k / npcd, pcd = PV.pair_start[cd] + k % npcd;
+    if (prim_negligible(PV, pab, pcd)) {
+      keys[r] = SKIP_KEY;
+      continue;
+    }
+    keys[r] = 0;
+    const int L = PV.shell_l[s[0]] + PV.shell_l[s[1]] + PV.shell_l[s[2]] + PV.shell_l[s[3]] + (cls == 5 ? 2 : 0);
+    const double p = PV.pp_p[pab], q = PV.pp_p[pcd], xi = p * q / (p + q);
+    const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
+                 Z = pair_sep(PV.pp_P, pab, pcd, 2);
+    const double u = X * X + Y * Y + Z * Z;
+    double2 *o = reinterpret_cast<double2 *>(part + r * kPartPitch);
+    nfma += aux_direct_fmas(G.boys != nullptr, L);
+    switch (L) {
+      case 4: direct_row<4>(G, xi, u, o); break;
+      case 5: direct_row<5>(G, xi, u, o); break;
+      case 6: direct_row<6>(G, xi, u, o); break;
+      case 7: direct_row<7>(G, xi, u, o); break;
+      case 8: direct_row<8>(G, xi, u, o); break;
+      case 9: direct_row<9>(G, xi, u, o); break;
+      case 10: direct_row<10>(G, xi, u, o); break;
+      case 11: direct_row<11>(G, xi, u, o); break;
+      case 12: direct_row<12>(G, xi, u, o); break;
+      case 13: direct_row<13>(G, xi, u, o); break;
+      default: direct_row<14>(G, xi, u, o); break;
+    }
+  }
+  if (fma_total) {
+    for (int o = 16; o > 0; o >>= 1) nfma += __shfl_down_sync(0xffffffffu, nfma, o);
+    if ((threadIdx.x & 31) == 0 && nfma) atomicAdd(fma_total, nfma);
+  }
+}
+
+// hat g_n at given (xi, D) points (no prefactor), for the aux-stage tests:
+// from the grid where it holds the point, else family by family.
+__global__ void k_aux_points(Tables T, GridView G, const unsigned char *ok, int cls, int64_t npts, const double *xi,
+                             const double *D, int nmax, double *out, unsigned int *status) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= npts) return;
   double g[LAUX + 1];
+  if (G.boys) {
+    const double is = 1.0 / sqrt(xi[i]);
+    boys_eval<LAUX, false>(G.boys, xi[i], D[i] * D[i], nmax, g);
+    for (int n = 0; n <= nmax; ++n) out[i * (nmax + 1) + n] = is * g[n];
+    return;
+  }
+  if (G.cells) {
+    const GridPoint pt = grid_point(G.xt, xi[i], D[i] * D[i]);
+    if (pt.cell >= 0 && ok[pt.cell]) {
+      const double is = 1.0 / sqrt(xi[i]);
+      if (nmax <= 4) grid_eval<4, false>(G.cells, pt, nmax, g);
+      else if (nmax <= 8) grid_eval<8, false>(G.cells, pt, nmax, g);
+      else grid_eval<LAUX, false>(G.cells, pt, nmax, g);
+      for (int n = 0; n <= nmax; ++n) out[i * (nmax + 1) + n] = is * g[n];
+      return;
+    }
+  }
   int bad = aux_eval(T, cls == 5 ? 3 : cls, xi[i], D[i], nmax, g);
   if (bad) atomicOr(status, 1u);
   for (int n = 0; n <= nmax; ++n) out[i * (nmax + 1) + n] = g[n];
@@ -774,6 +833,7 @@ struct f12int_ctx {
   size_t jtab_bytes = 0;
   Tables tables{};
   size_t fam_bytes = 0, coef_bytes = 0;
+  std::shared_ptr<const f12grid::AuxGrid> grid;   // the factor's auxiliary grids (null: none)
   // basis
   struct BasisData {
     int nshell = 0;
@@ -790,6 +850,9 @@ struct f12int_ctx {
     std::vector<double> pair_bound[7];  // shell-pair bounds sqrt(max |(ab|k|ab)|) per class (lazily built)
     std::vector<double> pair_cen;       // [nshell^2][3] centre of the most diffuse primitive pair
     std::vector<double> pair_pmin;      // [nshell^2] its exponent sum
+    double exp_lo = 0.0, exp_hi = 0.0;  // range of the exponents: that of xi = pq/(p+q), p = a + b
+    double dmax = 0.0;                  // bound of the distances between primitive centres
+    bool grid_ok[7] = {false, false, false, false, false, false, false};   // the grid serves (basis, class)
   };
   std::deque<BasisData> bases;   // deque: growing it never moves existing entries
   // scratch of compute_class (grown on demand, bounded by the budget)
@@ -891,6 +954,30 @@ PairView pair_view(const f12int_ctx *ctx, const f12int_ctx::BasisData &B, int cl
   return v;
 }
 
+const double *g_boys = nullptr;   // the Kummer table's rows of a = 1 (upload_constants)
+static_assert(BY_LSTRIDE == MT_NA * MT_NX * MT_NT && BY_NT == MT_NT && BY_XMAX <= (MT_NX - 1) * MT_DX && MT_DX == 0.5,
+              "boys_eval reads the Kummer table");
+
+// How a class of a basis gets its auxiliary functions: I1 from the Boys
+// table, the others from the grid if it holds every (xi, D) of the basis,
+// else family by family.  A lowered series cap (a test aid) keeps to the
+// series.
+GridView class_view(const f12int_ctx *ctx, int cls) {
+  if (ctx->series_cap < KMAX) return GridView{nullptr, nullptr, nullptr};
+  if (cls == 1) return GridView{nullptr, nullptr, g_boys};
+  const int k = cls == 5 ? 3 : cls;
+  if (!ctx->grid || !ctx->grid->cells[k]) return GridView{nullptr, nullptr, nullptr};
+  return GridView{ctx->grid->cells[k], ctx->grid->xt, nullptr};
+}
+GridView grid_view(const f12int_ctx *ctx, const f12int_ctx::BasisData &B, int cls) {
+  return cls == 1 || B.grid_ok[cls] ? class_view(ctx, cls) : GridView{nullptr, nullptr, nullptr};
+}
+
+void mark_grid(const f12int_ctx *ctx, f12int_ctx::BasisData &B) {
+  for (int c = 2; c <= 6; ++c)
+    B.grid_ok[c] = ctx->grid && ctx->cls_ok[c] && f12grid::covers(*ctx->grid, c, B.exp_lo, B.exp_hi, B.dmax);
+}
+
 bool g_const_ready = false;
 std::mutex g_const_mu;
 
@@ -937,6 +1024,7 @@ int upload_constants() {
     CK(cudaMemcpy(dk, kt.data(), sizeof(double) * kt.size(), cudaMemcpyHostToDevice));
     const double *dkc = dk;
     CK(cudaMemcpyToSymbol(d_mtab, &dkc, sizeof(dkc)));
+    g_boys = dk + (size_t)1 * MT_NX * MT_NT;   // a = (1 + 1)/2
   }
   CK(cudaMemcpyToSymbol(c_tuv, tuv, sizeof(tuv)));
   CK(cudaMemcpyToSymbol(c_cart, cart, sizeof(cart)));
@@ -1343,6 +1431,13 @@ static int set_factor_lists(f12int_ctx *ctx, const f12::TermList &T1, const f12:
     if (rc != F12INT_OK) return rc;
     CK(cudaMemcpy(ctx->d_kgrow, all.data(), ctx->kgrow_bytes, cudaMemcpyHostToDevice));
   }
+  {
+    f12::TermList gk[7];
+    for (int c = 1; c <= 6; ++c) gk[c] = kt[c];
+    ctx->grid.reset();
+    ctx->grid = f12grid::acquire(ctx->device, gk, ctx->cls_ok, ctx->stream);
+    for (auto &b : ctx->bases) mark_grid(ctx, b);
+  }
   engine_factor_changed(ctx);
   ctx->factor_ready = true;
   return F12INT_OK;
@@ -1498,6 +1593,23 @@ int f12int_set_basis(f12int_ctx *ctx, int nshell, const double *centers, const i
     ctx->used -= std::min(ctx->used, B.bytes);
     return rc;
   }
+  B.exp_lo = *std::min_element(exps, exps + nptot);
+  B.exp_hi = *std::max_element(exps, exps + nptot);
+  {
+    // every primitive centre lies between two shells: the diagonal of the
+    // box of the shells bounds their distances
+    double d2 = 0.0;
+    for (int k = 0; k < 3; ++k) {
+      double lo = centers[k], hi = centers[k];
+      for (int i = 1; i < nshell; ++i) {
+        lo = std::min(lo, centers[3 * i + k]);
+        hi = std::max(hi, centers[3 * i + k]);
+      }
+      d2 += (hi - lo) * (hi - lo);
+    }
+    B.dmax = std::sqrt(d2);
+  }
+  mark_grid(ctx, B);
   ctx->bases.push_back(std::move(B));
   *basis_id = (int)ctx->bases.size() - 1;
   return F12INT_OK;
@@ -1625,15 +1737,39 @@ static const int kNKeys = MAXFAM * (LAUX + 1) * NZBIN + 1;
 // Queue the auxiliary stage (classify, scan, scatter, evaluate) and the
 // contraction for quartets [qa, qb) of the device list.
 static int launch_chunk(f12int_ctx *ctx, const f12int_ctx::BasisData &B, int cls, const int32_t *d_quartets,
-                        const int64_t *d_pqoff, int64_t n, int64_t qa, int64_t qb, int64_t pqa, int64_t pqb,
-                        size_t smem, double *out_dev, const int64_t *offsets_dev, cudaStream_t st,
+                        const int64_t *d_pqoff, const int64_t *h_pqoff, int64_t n, int64_t qa, int64_t qb,
+                        int64_t pqa, int64_t pqb, size_t smem, double *out_dev, const int64_t *offsets_dev, cudaStream_t st,
                         bool prim_screen = true) {
   PairView PV = pair_view(ctx, B, cls, B.prim_screen && prim_screen);
   QuartetView QV{d_quartets, d_pqoff, n, nullptr, nullptr, nullptr, nullptr};
   const int kcls = cls == 5 ? 3 : cls;
-  const int nf = ctx->tables.nfam[kcls];
-  const int64_t nitems = (pqb - pqa) * nf;
-  if (nitems > 0) {
+  const GridView G = grid_view(ctx, B, cls);
+  // the thin quartets are a suffix of the working order
+  int64_t qthin = qb;
+  while (qthin > qa && ctx->h_thin[qthin - 1] >= 0) --qthin;
+  // with the grid one row per primitive quartet of the general contraction
+  // (the thin kernel evaluates its own), else one item per family
+  const int nf = G.direct() ? 1 : ctx->tables.nfam[kcls];
+  const int64_t nitems = G.direct() ? h_pqoff[qthin] - pqa : (pqb - pqa) * nf;
+  if (nitems > 0 && G.direct()) {
+    int rc = ensure_buf(ctx, (void **)&ctx->d_keys, &ctx->keys_cap, sizeof(int) * nitems);
+    if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_part, &ctx->part_cap, sizeof(double) * nitems * kPartPitch);
+    if (rc != F12INT_OK) return rc;
+    std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
+    if (ctx->timing) {
+      ev = take_events(ctx);
+      cudaEventRecord(ev.first, st);
+    }
+    k_direct_rows<false><<<(unsigned)((nitems + BLOCK_AUX - 1) / BLOCK_AUX), BLOCK_AUX, 0, st>>>(
+        G, PV, QV, cls, pqa, nitems, ctx->d_keys, ctx->d_part, ctx->timing ? ctx->d_fma : nullptr);
+    if (ctx->timing) {
+      cudaEventRecord(ev.second, st);
+      ctx->ev_aux.push_back(ev);
+      ctx->aux_launches++;
+    }
+    ctx->launches++;
+    CK(cudaGetLastError());
+  } else if (nitems > 0) {
     int rc = ensure_buf(ctx, (void **)&ctx->d_keys, &ctx->keys_cap, sizeof(int) * nitems);
     if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_order, &ctx->order_cap, sizeof(unsigned) * nitems);
     if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_part, &ctx->part_cap, sizeof(double) * nitems * kPartPitch);
@@ -1679,9 +1815,6 @@ static int launch_chunk(f12int_ctx *ctx, const f12int_ctx::BasisData &B, int cls
     CK(cudaMemcpyAsync(ctx->d_tasks, tasks.data(), sizeof(CTask) * tasks.size(), cudaMemcpyHostToDevice, st));
   }
   int64_t t0 = 0;
-  // the thin quartets are a suffix of the working order
-  int64_t qthin = qb;
-  while (qthin > qa && ctx->h_thin[qthin - 1] >= 0) --qthin;
   for (int64_t ra = qa; ra < qthin;) {
     const int nw = ctx->h_nw[ra];
     const char f32 = ctx->h_fp32[ra];
@@ -1733,7 +1866,7 @@ static int launch_chunk(f12int_ctx *ctx, const f12int_ctx::BasisData &B, int cls
       cudaEventRecord(ev.first, st);
     }
     kern<<<(unsigned)((nt + kThinWarps - 1) / kThinWarps), 32 * kThinWarps, 0, st>>>(
-        PV, QV, nf, pqa, ctx->d_tasks + t0, nt, nullptr, ctx->d_keys, ctx->d_part, out_dev, offsets_dev,
+        PV, QV, nf, pqa, G, ctx->d_tasks + t0, nt, nullptr, ctx->d_keys, ctx->d_part, out_dev, offsets_dev,
         ctx->timing ? ctx->d_fma + 1 : nullptr);
     t0 += nt;
     if (ctx->timing) {
@@ -2039,10 +2172,12 @@ static int compute_class_impl(f12int_ctx *ctx, int basis_id, int cls, const int3
   plan_range.reset();
   ctx->plan_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_plan0).count();
   ctx->plan_calls++;
+  const bool gridded = grid_view(ctx, B, cls).direct();
   for (int64_t qa = 0; qa < n;) {
     int64_t qb = qa + 1;
-    while (qb < n && pqoff[qb + 1] - pqoff[qa] <= pq_chunk) ++qb;
-    rc = launch_chunk(ctx, B, cls, ctx->d_qperm, ctx->d_pqoff, n, qa, qb, pqoff[qa], pqoff[qb], smem, out_dev,
+    // (with the grid the thin quartets, last in the order, need no scratch)
+    while (qb < n && (pqoff[qb + 1] - pqoff[qa] <= pq_chunk || (gridded && ctx->h_thin[qb] >= 0))) ++qb;
+    rc = launch_chunk(ctx, B, cls, ctx->d_qperm, ctx->d_pqoff, pqoff.data(), n, qa, qb, pqoff[qa], pqoff[qb], smem, out_dev,
                       ctx->d_operm, st, prim_screen);
     if (rc != F12INT_OK) return rc;
     qa = qb;
@@ -2066,7 +2201,9 @@ int f12int_aux(f12int_ctx *ctx, int cls, int64_t npts, const double *xi_dev, con
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = pick_stream(ctx, cuda_stream);
   int64_t nb = (npts + BLOCK_AUX - 1) / BLOCK_AUX;
-  k_aux_points<<<(unsigned)nb, BLOCK_AUX, 0, st>>>(ctx->tables, cls, npts, xi_dev, D_dev, nmax, out_dev,
+  const GridView G = class_view(ctx, cls);
+  const unsigned char *ok = G.cells ? ctx->grid->ok[cls == 5 ? 3 : cls] : nullptr;
+  k_aux_points<<<(unsigned)nb, BLOCK_AUX, 0, st>>>(ctx->tables, G, ok, cls, npts, xi_dev, D_dev, nmax, out_dev,
                                                    ctx->d_status);
   ctx->launches++;
   CK(cudaGetLastError());
@@ -2342,15 +2479,24 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
   // every primitive quartet is evaluated
   PairView PV = pair_view(ctx, B, cls, B.prim_screen);
   QuartetView QV{d_q, d_pq, n, nullptr, nullptr, nullptr, nullptr};
+  const GridView G = grid_view(ctx, B, cls);
+  const int nfk = G.direct() ? 1 : nf;   // rows per primitive quartet
   int rc_launch = F12INT_OK;
   for (int64_t qa = 0; qa < n && rc_launch == F12INT_OK;) {
     int64_t qb = qa + 1;
     while (qb < n && pqoff[qb + 1] - pqoff[qa] <= pq_chunk) ++qb;
-    const int64_t pqa = pqoff[qa], nitems = (pqoff[qb] - pqa) * nf;
+    int64_t qthin = qb;   // thin quartets (no shared memory) are last
+    while (qthin > qa && hsm[qthin - 1] == 0) --qthin;
+    const int64_t pqa = pqoff[qa], nitems = G.direct() ? pqoff[qthin] - pqa : (pqoff[qb] - pqa) * nf;
     int *d_keys = (int *)items_base;
     unsigned *d_order = (unsigned *)(items_base + align256(sizeof(int) * (size_t)nitems));
     double *d_part = (double *)((unsigned char *)d_order + align256(sizeof(unsigned) * (size_t)nitems));
-    if (nitems > 0) {
+    if (nitems > 0 && G.direct()) {
+      k_direct_rows<false><<<(unsigned)((nitems + BLOCK_AUX - 1) / BLOCK_AUX), BLOCK_AUX, 0, st>>>(
+          G, PV, QV, cls, pqa, nitems, d_keys, d_part, nullptr);
+      ctx->launches++;
+      if (cudaGetLastError() != cudaSuccess) rc_launch = F12INT_ECUDA;
+    } else if (nitems > 0) {
       // the histogram must start at zero on every call: the array keeps the
       // previous call's contents
       if (cudaMemsetAsync(d_hist, 0, sizeof(unsigned) * kNKeys, st) != cudaSuccess) {
@@ -2390,7 +2536,7 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
           break;
         }
         kern<<<(unsigned)((nt + kThinWarps - 1) / kThinWarps), 32 * kThinWarps, 0, st>>>(
-            PV, QV, nf, pqa, d_tk + tfirst[ra], nt, nullptr, d_keys, d_part, out_dev, d_o, nullptr);
+            PV, QV, nfk, pqa, G, d_tk + tfirst[ra], nt, nullptr, d_keys, d_part, out_dev, d_o, nullptr);
         ctx->launches++;
         if (cudaGetLastError() != cudaSuccess) rc_launch = F12INT_ECUDA;
         ra = rb;
@@ -2404,7 +2550,7 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
         rc_launch = F12INT_ECUDA;
         break;
       }
-      k_contract<false, double><<<(unsigned)nt, 32 * nwr, smr, st>>>(PV, QV, cls, nf, pqa, d_tk + tfirst[ra], nt, nullptr,
+      k_contract<false, double><<<(unsigned)nt, 32 * nwr, smr, st>>>(PV, QV, cls, nfk, pqa, d_tk + tfirst[ra], nt, nullptr,
                                                                      d_keys, d_part, out_dev, d_o, ctx->d_status, nullptr);
       ctx->launches++;
       if (cudaGetLastError() != cudaSuccess) rc_launch = F12INT_ECUDA;

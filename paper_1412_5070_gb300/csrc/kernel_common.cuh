@@ -7,6 +7,8 @@
 
 #include <cstdint>
 
+#include "auxgrid.cuh"
+
 namespace f12k {
 
 constexpr int kLaux = 14;                          // highest radial order (I5 of f shells)
@@ -64,13 +66,67 @@ __device__ __forceinline__ double pair_sep(const double *ppP, int pab, int pcd, 
   return (ppP[6 * pcd + k] - ppP[6 * pab + k]) + (ppP[6 * pcd + 3 + k] - ppP[6 * pab + 3 + k]);
 }
 
+// Where a class's auxiliary functions come from, when not family by family:
+// the grid (auxgrid.cuh), or for I1 the table of the Boys function.
+struct GridView {
+  const double *cells;   // null: no grid
+  const double *xt;
+  const double *boys;    // null: not the Coulomb kernel
+  __host__ __device__ bool direct() const { return cells || boys; }
+};
+
+// sqrt(xi) hat g_l, l <= L
+template <int L>
+__device__ __forceinline__ void aux_direct(const GridView &G, double xi, double u, double *h) {
+  if (G.boys) f12dev::boys_eval<L, true>(G.boys, xi, u, L, h);
+  else f12dev::grid_eval<L, true>(G.cells, f12dev::grid_point(G.xt, xi, u), L, h);
+}
+__host__ __device__ constexpr int aux_direct_fmas(const bool boys, int L) {
+  return boys ? f12dev::BY_NT - 1 + L : f12dev::grid_fmas(L);
+}
+
+// Growth of a kernel with distance, tabulated at this step (screening).
+constexpr double kGrowStep = 0.05, kGrowMax = 120.0;
+constexpr double kPrimScreen = 1e-26;
+
+
+// Primitive quartets whose Schwarz product is below kPrimScreen are skipped:
+// the skipped contributions stay below the absolute accuracy that elements
+// just above 1e-12 need for a relative error of 1e-10.  The diagonal
+// integrals behind qprim sample the kernel at short range; a kernel that
+// grows with r (Eq. rs12 with B > 0: I2, I3 like e^{Br}, k4 = f f' and
+// k6 = f_r f'_r like e^{2Br}) is larger at the separation R = |P - Q| of the
+// two charge distributions, whose overlap e^{-xi w^2} reaches out to R + w.
+// A candidate is weighed, as the shell screen weighs a shell quartet, by
+//   Gamma = max over w = 0, 0.5, .., 3 (units of 1/sqrt(xi)) of G(R + w) e^{-xi w^2}
+// (e^{-xi w^2} = e^{-k^2/4} at the k-th sample).
+__device__ __forceinline__ bool prim_negligible(const PairView &PV, int pab, int pcd) {
+  if (!PV.qprim) return false;
+  const double v = PV.qprim[pab] * PV.qprim[pcd];
+  if (v >= kPrimScreen) return false;
+  if (!PV.grow) return true;
+  const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
+               Z = pair_sep(PV.pp_P, pab, pcd, 2);
+  const double p = PV.pp_p[pab], q = PV.pp_p[pcd];
+  const double R = sqrt(X * X + Y * Y + Z * Z), hw = 0.5 * sqrt((p + q) / (p * q));
+  constexpr double kOverlap[7] = {1.0, 0.77880078307140487, 0.36787944117144233, 0.10539922456186433,
+                                  0.018315638888734179, 0.0019304541362277093, 0.00012340980408667956};
+  double gam = 0.0;
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    const int i = min(PV.ngrow - 1, (int)((R + k * hw) * (1.0 / kGrowStep)) + 1);
+    gam = fmax(gam, PV.grow[i] * kOverlap[k]);
+  }
+  return v * gam < kPrimScreen;
+}
+
 // Thin contraction (thin_*.cu): quartets of total order L <= kThinL (I5:
 // L <= kThinL5), one warp per shell quartet, always in FP64 (on the mixed
 // path too: there it is faster than the FP32 general kernel).
 constexpr int kThinL = 3, kThinL5 = 2;
 constexpr int kThinWarps = 4;
-using ThinKernel = void (*)(PairView, QuartetView, int, int64_t, const CTask *, int64_t, const int64_t *, const int *,
-                            const double *, double *, const int64_t *, unsigned long long *);
+using ThinKernel = void (*)(PairView, QuartetView, int, int64_t, GridView, const CTask *, int64_t, const int64_t *,
+                            const int *, const double *, double *, const int64_t *, unsigned long long *);
 // The instance for class key (la << 6 | lb << 4 | lc << 2 | ld), or null.
 ThinKernel thin_kernel(int key, bool i5);
 // Index of a thin class key among the thin keys of its class kind (the batch

@@ -36,7 +36,7 @@ __host__ __device__ constexpr int cart_j(int l, int k) {   // y exponent
 // goes to o.
 template <int LA, int LB, int LC, int LD, bool I5>
 __device__ __forceinline__ void thin_quartet_body(const PairView &PV, const QuartetView &QV, int nf, int64_t pq0,
-                                                  int64_t q, const int *keys, const double *part, double *out_q,
+                                                  const GridView &G, int64_t q, const int *keys, const double *part, double *out_q,
                                                   unsigned long long *flops_total) {
   constexpr int EXT = I5 ? 2 : 0;
   constexpr int L = LA + LB + LC + LD + EXT;   // highest order of g_n and R
@@ -61,24 +61,32 @@ __device__ __forceinline__ void thin_quartet_body(const PairView &PV, const Quar
   for (int r = lane; r < np; r += 32) {
     const int iab = r / npcd, icd = r - iab * npcd;
     const int pab = ab0 + iab, pcd = cd0 + icd;
-    const int64_t pq = QV.pq_off[q] + r - pq0;
-    if (keys[pq * nf] == kSkipKey) continue;   // dropped by the primitive screen
-    ++nproc;
-    // g_n = sqrt(pi^5/(p+q))/(pq) * sum over families (fixed order)
     const double p = PV.pp_p[pab], qq = PV.pp_p[pcd];
-    const double pref = pi52 / (sqrt(p + qq) * p * qq);
-    double g[L + 1];
-#pragma unroll
-    for (int n = 0; n <= L; ++n) g[n] = 0.0;
-    for (int f = 0; f < nf; ++f) {
-      const double *pp = part + (pq * nf + f) * kPartPitch;
-#pragma unroll
-      for (int n = 0; n <= L; ++n) g[n] += pp[n];
-    }
-#pragma unroll
-    for (int n = 0; n <= L; ++n) g[n] *= pref;
     const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
                  Z = pair_sep(PV.pp_P, pab, pcd, 2);
+    double pref, g[L + 1];
+    if (G.direct()) {
+      if (prim_negligible(PV, pab, pcd)) continue;
+      // g_n = sqrt(pi^5/(p+q))/(pq) hat g_n = pi^{5/2} (pq)^{-3/2} sqrt(xi) hat g_n
+      const double pq_ = p * qq;
+      aux_direct<L>(G, pq_ / (p + qq), X * X + Y * Y + Z * Z, g);
+      pref = pi52 / (pq_ * sqrt(pq_));
+    } else {
+      const int64_t pq = QV.pq_off[q] + r - pq0;
+      if (keys[pq * nf] == kSkipKey) continue;   // dropped by the primitive screen
+      // g_n = sqrt(pi^5/(p+q))/(pq) * sum over families (fixed order)
+      pref = pi52 / (sqrt(p + qq) * p * qq);
+#pragma unroll
+      for (int n = 0; n <= L; ++n) g[n] = 0.0;
+      for (int f = 0; f < nf; ++f) {
+        const double *pp = part + (pq * nf + f) * kPartPitch;
+#pragma unroll
+        for (int n = 0; n <= L; ++n) g[n] += pp[n];
+      }
+    }
+    ++nproc;
+#pragma unroll
+    for (int n = 0; n <= L; ++n) g[n] *= pref;
     // Hermite recursion, levels n = L .. 0, in registers (every index is a
     // compile-time constant after unrolling)
     double R[NH], Rn[NH];
@@ -194,6 +202,8 @@ __device__ __forceinline__ void thin_quartet_body(const PairView &PV, const Quar
       const unsigned long long ket = 2ull * nh_count(LA + LB + EXT) * nh_count(LC + LD) * (NC * ND);
       const unsigned long long bra = 2ull * (NA * NB) * nh_count(LA + LB) * (NC * ND) * (I5 ? 4 : 1);
       atomicAdd(flops_total, (unsigned long long)tot * (r + ket + bra));
+      if (G.direct())   // the auxiliary stage's multiply-adds are the counter before
+        atomicAdd(flops_total - 1, (unsigned long long)tot * aux_direct_fmas(G.boys != nullptr, L));
     }
   }
 }
@@ -204,21 +214,21 @@ __device__ __forceinline__ void thin_quartet_body(const PairView &PV, const Quar
 // output array from its request's slot.
 template <int LA, int LB, int LC, int LD, bool I5>
 __global__ void __launch_bounds__(32 * kThinWarps)
-k_contract_thin(PairView PV, QuartetView QV, int nf, int64_t pq0, const CTask *tasks, int64_t ntask,
+k_contract_thin(PairView PV, QuartetView QV, int nf, int64_t pq0, GridView G, const CTask *tasks, int64_t ntask,
                 const int64_t *range, const int *keys, const double *part, double *out, const int64_t *offsets,
                 unsigned long long *flops_total) {
   const int64_t warp = (int64_t)blockIdx.x * kThinWarps + (threadIdx.x >> 5);
   if (!range) {
     if (warp >= ntask) return;   // warp-uniform
     const int64_t q = tasks[warp].q;
-    thin_quartet_body<LA, LB, LC, LD, I5>(PV, QV, nf, pq0, q, keys, part, out + offsets[q], flops_total);
+    thin_quartet_body<LA, LB, LC, LD, I5>(PV, QV, nf, pq0, G, q, keys, part, out + offsets[q], flops_total);
     return;
   }
   const int64_t t1 = range[1], stride = (int64_t)gridDim.x * kThinWarps;
   for (int64_t tk = range[0] + warp; tk < t1; tk += stride) {
     const int64_t q = tasks[tk].q;
     const int slot = QV.qslot[q];
-    thin_quartet_body<LA, LB, LC, LD, I5>(QV.slot_view[slot], QV, nf, pq0, q, keys, part,
+    thin_quartet_body<LA, LB, LC, LD, I5>(QV.slot_view[slot], QV, nf, pq0, G, q, keys, part,
                                           QV.slot_out[slot] + offsets[q], flops_total);
   }
 }
