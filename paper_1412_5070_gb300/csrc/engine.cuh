@@ -7,7 +7,8 @@
 // mix of (la, lb, lc, ld) -- into a batch, writes the batch's lists to pinned
 // staging memory, copies them to fixed device buffers and replays one
 // captured CUDA graph.  The graph holds, for every class, the four passes of
-// the auxiliary stage and one contraction launch per shared-memory tier, all
+// the auxiliary stage and one contraction launch per tier (threads and shared
+// memory of a block), all
 // persistent (grid-stride over counts read from device memory), so the same
 // graph serves every batch.  The six class pipelines are parallel branches
 // of the graph, each with its own work-item buffers.  Two staging buffers let the host build batch
@@ -16,9 +17,14 @@
 
 namespace {
 
-constexpr int kTiers = 5;                // shared-memory tiers per precision
-constexpr size_t kTierCap[kTiers] = {32 * 1024, 64 * 1024, 112 * 1024, 200 * 1024, 200 * 1024};
-constexpr int kTierWarps[kTiers] = {4, 4, 4, 4, 2};   // the last for quartets that need fewer warps
+// Default work of one contraction task of a batch, in flops, and the unit of
+// the schedules that f12int_batch_autotune tries.
+constexpr double kTaskFlops = 5e7;
+
+// contraction tiers: threads and shared memory of a block
+constexpr int kTiers = 6;                // per precision
+constexpr int kTierThreads[kTiers] = {32, 64, 96, 192, 256, 256};
+constexpr size_t kTierCap[kTiers] = {24 * 1024, 36 * 1024, 54 * 1024, 54 * 1024, 72 * 1024, 200 * 1024};
 constexpr int kLaunches = 2 * kTiers;     // FP64 tiers, then FP32 tiers (mixed requests)
 constexpr int kThinSlot = kLaunches;      // then the thin contraction (total order <= 3, I5 <= 2), one
 constexpr int kSlots = kLaunches + kThinKeys;   // launch per (la, lb, lc, ld)
@@ -45,42 +51,35 @@ struct TicketState {
   int batch = -1;                 // staging buffer of the batch that runs it
 };
 
-// Contraction plan of a quartet of nprimq primitive quartets in a batch:
-// ket ranges at 4 warps (the fewest that fit the largest tier, more while a
-// task would exceed kTaskFlops), the tier that holds them, and the work of
-// one task.
+// Contraction plan of a quartet in a batch: ket ranges (the fewest that fit,
+// more while a task would exceed `target` flops), the tier that holds them,
+// and the work of one task.
 struct BatchPlan {
   int tier, nsplit;
   double work;
 };
 
-static bool batch_plan(int la, int lb, int lc, int ld, int cls, int64_t nprimq, double target, BatchPlan *bp,
-                       bool fp32 = false) {
-  const int ncd = ncart(lc) * ncart(ld);
-  if (thin_quartet((la << 6) | (lb << 4) | (lc << 2) | ld, cls)) {   // one warp, FP64 (mixed requests too)
-    bp->tier = kThinSlot + thin_slot((la << 6) | (lb << 4) | (lc << 2) | ld, cls == 5);
+static bool batch_plan(int la, int lb, int lc, int ld, int cls, int64_t nprimq, int64_t npcd, double target,
+                       BatchPlan *bp, bool fp32 = false) {
+  const ContractShape s{la, lb, lc, ld, cls == 5 ? 2 : 0};
+  const int key = (la << 6) | (lb << 4) | (lc << 2) | ld;
+  if (thin_quartet(key, cls)) {   // one warp, FP64 (mixed requests too)
+    bp->tier = kThinSlot + thin_slot(key, cls == 5);
     bp->nsplit = 1;
-    bp->work = (double)nprimq * task_flops(la, lb, lc, ld, cls, ncd);
+    bp->work = (double)nprimq * task_fmas(s, npcd, s.ncd());
     return true;
   }
   const size_t esz = fp32 ? 4 : 8;
-  // 4-warp tiers first; the 2-warp tier only for what no 4-warp tier holds
-  for (int pass = 0; pass < 2; ++pass) {
-    const int nw = pass == 0 ? 4 : 2;
-    for (int ns = 1; ns <= ncd; ++ns) {
-      if (!valid_split(ncd, ns)) continue;
-      if (contract_smem(la, lb, lc, ld, cls, nw, ns, esz) > kTierCap[kTiers - 1]) continue;
-      const int nsw = work_split(la, lb, lc, ld, cls, nprimq, ns, target);
-      const size_t sm = contract_smem(la, lb, lc, ld, cls, nw, nsw, esz);
-      for (int t = 0; t < kTiers; ++t)
-        if (kTierWarps[t] == nw && sm <= kTierCap[t]) {
-          bp->tier = t + (fp32 ? kTiers : 0);
-          bp->nsplit = nsw;
-          bp->work = (double)nprimq * task_flops(la, lb, lc, ld, cls, (ncd + nsw - 1) / nsw);
-          return true;
-        }
+  const ContractPlan pl = contract_plan(la, lb, lc, ld, cls, nprimq, npcd, esz, 0.5 * target);
+  if (pl.smem == 0) return false;
+  const size_t least = contract_smem(s, 1, pl.nsplit, esz, 0);
+  for (int t = 0; t < kTiers; ++t)
+    if (kTierCap[t] >= least && (kTierThreads[t] >= pl.nthr || t == kTiers - 1)) {
+      bp->tier = t + (fp32 ? kTiers : 0);
+      bp->nsplit = pl.nsplit;
+      bp->work = (double)nprimq * task_fmas(s, npcd, (s.ncd() + pl.nsplit - 1) / pl.nsplit);
+      return true;
     }
-  }
   return false;
 }
 
@@ -89,6 +88,7 @@ static bool batch_plan(int la, int lb, int lc, int ld, int cls, int64_t nprimq, 
 struct ClassLists {
   int32_t *quartets = nullptr;    // [qcap][4]
   int64_t *pq_off = nullptr;      // [qcap + 1]
+  int64_t *row_off = nullptr;     // [qcap + 1] first double of a general quartet's Hermite rows
   int64_t *offsets = nullptr;     // [qcap]
   int32_t *qslot = nullptr;       // [qcap]
   CTask *tasks = nullptr;         // [tcap], tier after tier
@@ -98,6 +98,10 @@ struct ClassLists {
 };
 constexpr int kCounts = 3 + 2 * kSlots;
 constexpr int kTaskCounts = 3;           // first of the tiers' (begin, end)
+
+// Hermite rows that a class's buffer holds at least: one bra pair of 1000 ket
+// pairs at the highest order
+constexpr int64_t kRowsLeast = 684 * 1024;
 
 struct Engine {
   // limits
@@ -114,6 +118,8 @@ struct Engine {
   int *keys[7] = {nullptr};             // per class: item keys, key order, histogram, partials
   unsigned *order[7] = {nullptr}, *hist[7] = {nullptr};
   double *part[7] = {nullptr};
+  double *rows[2][7] = {};              // Hermite rows: per class by graph (the grid graph's in part)
+  int64_t rcap[2] = {0, 0};             // doubles of them
   unsigned *status = nullptr;
   size_t bytes = 0;
   // staging (pinned), two buffers
@@ -126,6 +132,7 @@ struct Engine {
   // graph
   cudaStream_t stream = nullptr;
   cudaStream_t branch[7] = {nullptr};   // capture streams of the class branches
+  cudaStream_t sub[7][3] = {};          // and of their parallel parts
   // one graph for batches evaluated from the auxiliary grid, one for batches
   // evaluated family by family; a batch is all of one kind
   cudaGraphExec_t exec[2] = {nullptr, nullptr};
@@ -166,6 +173,7 @@ static int stage_alloc(T **p, size_t n) {
 static int lists_alloc_dev(f12int_ctx *ctx, Engine &E, ClassLists &L) {
   int rc = engine_alloc(ctx, E, &L.quartets, 4 * (size_t)E.qcap);
   if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &L.pq_off, (size_t)E.qcap + 1);
+  if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &L.row_off, (size_t)E.qcap + 1);
   if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &L.offsets, (size_t)E.qcap);
   if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &L.qslot, (size_t)E.qcap);
   if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &L.tasks, (size_t)E.tcap);
@@ -178,6 +186,7 @@ static int lists_alloc_dev(f12int_ctx *ctx, Engine &E, ClassLists &L) {
 static int lists_alloc_host(Engine &E, ClassLists &L) {
   int rc = stage_alloc(&L.quartets, 4 * (size_t)E.qcap);
   if (rc == F12INT_OK) rc = stage_alloc(&L.pq_off, (size_t)E.qcap + 1);
+  if (rc == F12INT_OK) rc = stage_alloc(&L.row_off, (size_t)E.qcap + 1);
   if (rc == F12INT_OK) rc = stage_alloc(&L.offsets, (size_t)E.qcap);
   if (rc == F12INT_OK) rc = stage_alloc(&L.qslot, (size_t)E.qcap);
   if (rc == F12INT_OK) rc = stage_alloc(&L.tasks, (size_t)E.tcap);
@@ -188,7 +197,7 @@ static int lists_alloc_host(Engine &E, ClassLists &L) {
 }
 
 static void lists_free(ClassLists &L, bool host) {
-  void *ps[] = {L.quartets, L.pq_off, L.offsets, L.qslot, L.tasks, L.counts, L.views, L.outs};
+  void *ps[] = {L.quartets, L.pq_off, L.row_off, L.offsets, L.qslot, L.tasks, L.counts, L.views, L.outs};
   for (void *p : ps)
     if (p) host ? cudaFreeHost(p) : cudaFree(p);
   L = ClassLists{};
@@ -214,11 +223,34 @@ static int engine_capture(f12int_ctx *ctx, Engine &E, bool grid) {
       CK(cudaFuncSetAttribute(k_contract<true, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTierCap[t]));
       CK(cudaFuncSetAttribute(k_contract<true, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTierCap[t]));
     }
+  if (!grid && !E.rows[0][1]) {
+    // the family path's rows, at its first batch: 64 MB a class, or what the
+    // budget leaves (a batch that needs more runs in several passes)
+    int rc = F12INT_ENOMEM;
+    for (int64_t want : {std::min<int64_t>((int64_t)8 << 20, E.icap * 16 + kRowsLeast), kRowsLeast}) {
+      rc = F12INT_OK;
+      for (int c = 1; c <= 6 && rc == F12INT_OK; ++c) rc = engine_alloc(ctx, E, &E.rows[0][c], (size_t)want);
+      if (rc == F12INT_OK) {
+        E.rcap[0] = want;
+        break;
+      }
+      for (int c = 1; c <= 6; ++c)
+        if (E.rows[0][c]) {
+          dfree(ctx, E.rows[0][c], sizeof(double) * (size_t)want);
+          E.bytes -= sizeof(double) * (size_t)want;
+        }
+    }
+    if (rc != F12INT_OK) return rc;
+  }
   cudaStream_t cs = nullptr;
   CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-  cudaEvent_t fork = nullptr, join[7] = {nullptr};
+  cudaEvent_t fork = nullptr, join[7] = {nullptr}, mid[2][7] = {}, done[3][7] = {};
   CK(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
-  for (int c = 1; c <= 6; ++c) CK(cudaEventCreateWithFlags(&join[c], cudaEventDisableTiming));
+  for (int c = 1; c <= 6; ++c) {
+    CK(cudaEventCreateWithFlags(&join[c], cudaEventDisableTiming));
+    for (cudaEvent_t *e : {&mid[0][c], &mid[1][c], &done[0][c], &done[1][c], &done[2][c]})
+      CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+  }
   const PairView none{};
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
@@ -231,45 +263,72 @@ static int engine_capture(f12int_ctx *ctx, Engine &E, bool grid) {
       const int kcls = cls == 5 ? 3 : cls;
       // (a class without a grid has no quartets in a grid batch)
       const GridView G = grid ? class_view(ctx, cls) : GridView{nullptr, nullptr, nullptr};
+      if (grid && !G.direct()) {
+        cudaEventRecord(join[cls], bs);
+        cudaStreamWaitEvent(cs, join[cls], 0);
+        continue;
+      }
       const int nf = G.direct() ? 1 : ctx->tables.nfam[kcls];
+      if (nf <= 0) {   // a class the factor leaves out
+        cudaEventRecord(join[cls], bs);
+        cudaStreamWaitEvent(cs, join[cls], 0);
+        continue;
+      }
       const ClassLists &L = E.dev[cls];
       QuartetView QV{L.quartets, L.pq_off, 0, L.counts, L.qslot, L.views, L.outs};
+      const RowView rows{E.rows[grid][cls], L.row_off, 0, 0};
+      // parallel parts of the class: the branch itself and E.sub
+      cudaStream_t part[4] = {bs, E.sub[cls][0], E.sub[cls][1], E.sub[cls][2]};
+      auto spread = [&](cudaEvent_t ev) {
+        cudaEventRecord(ev, bs);
+        for (int i = 1; i < 4; ++i) cudaStreamWaitEvent(part[i], ev, 0);
+      };
+      auto thin = [&](int first, int count) {   // one persistent launch per thin (la, lb, lc, ld) of the class kind
+        int i = 0;
+        for (int k = 0; k < 256; ++k) {
+          const int slot = thin_quartet(k, cls) ? thin_slot(k, cls == 5) : -1;
+          if (slot < 0) continue;
+          thin_kernel(k, cls == 5)<<<E.thin_blocks, 32 * kThinWarps, 0, part[first + i++ % count]>>>(
+              none, QV, nf, 0, G, L.tasks, 0, L.counts + kTaskCounts + 2 * (kThinSlot + slot), E.keys[cls],
+              E.part[cls], nullptr, L.offsets, nullptr);
+        }
+      };
       if (G.direct()) {
-        k_direct_rows<true><<<E.grid_blocks, BLOCK_AUX, 0, bs>>>(G, none, QV, cls, 0, 0, E.keys[cls], E.part[cls],
-                                                               nullptr);
+        // the thin contraction needs no rows and runs beside them
+        spread(mid[0][cls]);
+        thin(2, 2);
+        k_hermite_rows<true, true><<<E.grid_blocks, BLOCK_AUX, 0, bs>>>(G, none, QV, cls, 1, 0, -1, E.keys[cls],
+                                                                        nullptr, rows, nullptr);
       } else {
-      cudaMemsetAsync(E.hist[cls], 0, sizeof(unsigned) * kNKeys, bs);
-      k_items_classify<true><<<E.classify_blocks, BLOCK_AUX, 0, bs>>>(ctx->tables, none, QV, cls, 0, 0,
-                                                                      E.keys[cls], E.hist[cls]);
-      k_items_scan<<<1, 1024, 0, bs>>>(E.hist[cls], kNKeys);
-      k_items_scatter<<<E.classify_blocks, BLOCK_AUX, 0, bs>>>(QV, nf, 0, E.keys[cls], E.hist[cls], 0,
-                                                               E.order[cls]);
-      k_items_eval<true><<<std::max(1, E.items_blocks / E.items_div[cls]), BLOCK_AUX, 0, bs>>>(
-          ctx->tables, none, QV, cls, 0, 0, E.order[cls], E.keys[cls],
-                                                               E.part[cls], E.status, nullptr);
-      if (ctx->cls_quad[cls])   // families evaluated by quadrature (b < 0, alpha0 < -1)
-        k_items_eval<true, true><<<E.quad_blocks, BLOCK_AUX, 0, bs>>>(ctx->tables, none, QV, cls, 0, 0,
-                                                                       E.order[cls], E.keys[cls], E.part[cls],
-                                                                       E.status, nullptr);
+        cudaMemsetAsync(E.hist[cls], 0, sizeof(unsigned) * kNKeys, bs);
+        k_items_classify<true><<<E.classify_blocks, BLOCK_AUX, 0, bs>>>(ctx->tables, none, QV, cls, 0, 0,
+                                                                        E.keys[cls], E.hist[cls]);
+        k_items_scan<<<1, 1024, 0, bs>>>(E.hist[cls], kNKeys);
+        k_items_scatter<<<E.classify_blocks, BLOCK_AUX, 0, bs>>>(QV, nf, 0, E.keys[cls], E.hist[cls], 0,
+                                                                 E.order[cls]);
+        k_items_eval<true><<<std::max(1, E.items_blocks / E.items_div[cls]), BLOCK_AUX, 0, bs>>>(
+            ctx->tables, none, QV, cls, 0, 0, E.order[cls], E.keys[cls], E.part[cls], E.status, nullptr);
+        if (ctx->cls_quad[cls])   // families evaluated by quadrature (b < 0, alpha0 < -1)
+          k_items_eval<true, true><<<E.quad_blocks, BLOCK_AUX, 0, bs>>>(ctx->tables, none, QV, cls, 0, 0,
+                                                                         E.order[cls], E.keys[cls], E.part[cls],
+                                                                         E.status, nullptr);
+        spread(mid[0][cls]);
+        thin(2, 2);
+        k_hermite_rows<true, false><<<E.grid_blocks, BLOCK_AUX, 0, bs>>>(G, none, QV, cls, nf, 0, -1, E.keys[cls],
+                                                                         E.part[cls], rows, nullptr);
       }
+      cudaEventRecord(mid[1][cls], bs);
+      cudaStreamWaitEvent(part[1], mid[1][cls], 0);
       for (int t = 0; t < kLaunches; ++t) {
         const int tt = t % kTiers;
-        if (t < kTiers)
-          k_contract<true, double><<<E.tier_blocks[t], 32 * kTierWarps[tt], kTierCap[tt], bs>>>(
-              none, QV, cls, nf, 0, L.tasks, 0, L.counts + kTaskCounts + 2 * t, E.keys[cls], E.part[cls], nullptr, L.offsets,
-              E.status, nullptr);
-        else
-          k_contract<true, float><<<E.tier_blocks[t], 32 * kTierWarps[tt], kTierCap[tt], bs>>>(
-              none, QV, cls, nf, 0, L.tasks, 0, L.counts + kTaskCounts + 2 * t, E.keys[cls], E.part[cls], nullptr, L.offsets,
-              E.status, nullptr);
+        const auto kern = t < kTiers ? k_contract<true, double> : k_contract<true, float>;
+        kern<<<E.tier_blocks[t], kTierThreads[tt], kTierCap[tt], part[t & 1]>>>(
+            none, QV, cls, nf, 0, L.tasks, 0, L.counts + kTaskCounts + 2 * t, E.keys[cls], rows, nullptr, L.offsets,
+            -1, -1, nullptr);
       }
-      // one persistent launch per thin (la, lb, lc, ld) of the class kind
-      for (int k = 0; k < 256; ++k) {
-        const int slot = thin_quartet(k, cls) ? thin_slot(k, cls == 5) : -1;
-        if (slot < 0) continue;
-        thin_kernel(k, cls == 5)<<<E.thin_blocks, 32 * kThinWarps, 0, bs>>>(
-            none, QV, nf, 0, G, L.tasks, 0, L.counts + kTaskCounts + 2 * (kThinSlot + slot), E.keys[cls], E.part[cls], nullptr,
-            L.offsets, nullptr);
+      for (int i = 1; i < 4; ++i) {
+        cudaEventRecord(done[i - 1][cls], part[i]);
+        cudaStreamWaitEvent(bs, done[i - 1][cls], 0);
       }
       cudaEventRecord(join[cls], bs);
       cudaStreamWaitEvent(cs, join[cls], 0);
@@ -280,7 +339,8 @@ static int engine_capture(f12int_ctx *ctx, Engine &E, bool grid) {
   if (g) cudaGraphDestroy(g);
   cudaStreamDestroy(cs);
   cudaEventDestroy(fork);
-  for (int c = 1; c <= 6; ++c) cudaEventDestroy(join[c]);
+  for (int c = 1; c <= 6; ++c)
+    for (cudaEvent_t e : {join[c], mid[0][c], mid[1][c], done[0][c], done[1][c], done[2][c]}) cudaEventDestroy(e);
   if (e != cudaSuccess) return cuda_fail(e);
   E.graph_dirty[grid] = false;
   return F12INT_OK;
@@ -309,10 +369,14 @@ static int engine_init(f12int_ctx *ctx, Engine &E) {
   for (int c = 1; c <= 6 && rc == F12INT_OK; ++c) {
     rc = engine_alloc(ctx, E, &E.keys[c], (size_t)E.icap);
     if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &E.order[c], (size_t)E.icap);
-    if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &E.part[c], (size_t)E.icap * kPartPitch);
+    E.rcap[1] = std::max<int64_t>(E.icap * kPartPitch, kRowsLeast);
+    if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &E.part[c], (size_t)E.rcap[1]);
+    E.rows[1][c] = E.part[c];
     if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &E.hist[c], (size_t)kNKeys);
     if (rc == F12INT_OK && cudaStreamCreateWithFlags(&E.branch[c], cudaStreamNonBlocking) != cudaSuccess)
       rc = F12INT_ECUDA;
+    for (cudaStream_t &t : E.sub[c])
+      if (rc == F12INT_OK && cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking) != cudaSuccess) rc = F12INT_ECUDA;
   }
   if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &E.status, 1);
   for (int b = 0; b < 2 && rc == F12INT_OK; ++b) {
@@ -337,18 +401,16 @@ static int engine_init(f12int_ctx *ctx, Engine &E) {
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_items_eval<true, true>, BLOCK_AUX, 0));
   E.quad_blocks = nsm * std::max(per, 1);
   E.classify_blocks = nsm * 8;
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_direct_rows<true>, BLOCK_AUX, 0));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_hermite_rows<true, true>, BLOCK_AUX, 0));
   E.grid_blocks = nsm * std::max(per, 1);
   for (int t = 0; t < kTiers; ++t) {
     if (kTierCap[t] > 48 * 1024) {
       CK(cudaFuncSetAttribute(k_contract<true, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTierCap[t]));
       CK(cudaFuncSetAttribute(k_contract<true, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTierCap[t]));
     }
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_contract<true, double>, 32 * kTierWarps[t],
-                                                     kTierCap[t]));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_contract<true, double>, kTierThreads[t], kTierCap[t]));
     E.tier_blocks[t] = nsm * std::max(per, 1);
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_contract<true, float>, 32 * kTierWarps[t],
-                                                     kTierCap[t]));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_contract<true, float>, kTierThreads[t], kTierCap[t]));
     E.tier_blocks[kTiers + t] = nsm * std::max(per, 1);
   }
   E.thin_blocks = nsm * 4;   // 16 warps per SM: the thin launches of a batch are mostly small
@@ -372,19 +434,67 @@ static void engine_finish_batch(Engine &E, int b) {
   E.inflight[b].clear();
 }
 
-// Build the lists of one batch in staging buffer b and launch it.
+// One general quartet whose Hermite rows exceed the class's buffer, alone in
+// the lists: a few of its bra primitive pairs at a time, by plain launches.
+static int engine_large(f12int_ctx *ctx, Engine &E, int cls, bool grid, int64_t npab, int64_t npq, int64_t rows_q,
+                        int tier) {
+  const ClassLists &L = E.dev[cls];
+  cudaStream_t st = E.stream;
+  const PairView none{};
+  QuartetView QV{L.quartets, L.pq_off, 0, L.counts, L.qslot, L.views, L.outs};
+  const GridView G = grid ? class_view(ctx, cls) : GridView{nullptr, nullptr, nullptr};
+  const int nf = G.direct() ? 1 : ctx->tables.nfam[cls == 5 ? 3 : cls];
+  if (!G.direct()) {
+    CK(cudaMemsetAsync(E.hist[cls], 0, sizeof(unsigned) * kNKeys, st));
+    k_items_classify<true><<<E.classify_blocks, BLOCK_AUX, 0, st>>>(ctx->tables, none, QV, cls, 0, 0, E.keys[cls],
+                                                                    E.hist[cls]);
+    k_items_scan<<<1, 1024, 0, st>>>(E.hist[cls], kNKeys);
+    k_items_scatter<<<E.classify_blocks, BLOCK_AUX, 0, st>>>(QV, nf, 0, E.keys[cls], E.hist[cls], 0, E.order[cls]);
+    k_items_eval<true><<<E.items_blocks, BLOCK_AUX, 0, st>>>(ctx->tables, none, QV, cls, 0, 0, E.order[cls],
+                                                             E.keys[cls], E.part[cls], E.status, nullptr);
+    if (ctx->cls_quad[cls])
+      k_items_eval<true, true><<<E.quad_blocks, BLOCK_AUX, 0, st>>>(ctx->tables, none, QV, cls, 0, 0, E.order[cls],
+                                                                     E.keys[cls], E.part[cls], E.status, nullptr);
+  }
+  const int64_t npcd = npq / npab, per = rows_q / npab, step = E.rcap[grid] / per;
+  if (step < 1) return F12INT_ENOMEM;
+  for (int64_t i0 = 0; i0 < npab; i0 += step) {
+    const int64_t i1 = std::min(npab, i0 + step), a = i0 * npcd, n = (i1 - i0) * npcd;
+    const RowView rows{E.rows[grid][cls], L.row_off, i0 * per, 0};
+    const unsigned nb = (unsigned)((n + BLOCK_AUX - 1) / BLOCK_AUX);
+    if (G.direct())
+      k_hermite_rows<true, true><<<nb, BLOCK_AUX, 0, st>>>(G, none, QV, cls, 1, a, n, E.keys[cls], nullptr, rows,
+                                                           nullptr);
+    else
+      k_hermite_rows<true, false><<<nb, BLOCK_AUX, 0, st>>>(G, none, QV, cls, nf, a, n, E.keys[cls] + a * nf,
+                                                            E.part[cls] + a * nf * kPartPitch, rows, nullptr);
+    const auto kern = tier < kTiers ? k_contract<true, double> : k_contract<true, float>;
+    kern<<<E.tier_blocks[tier], kTierThreads[tier % kTiers], kTierCap[tier % kTiers], st>>>(
+        none, QV, cls, nf, G.direct() ? a : 0, L.tasks, 0, L.counts + kTaskCounts + 2 * tier, E.keys[cls], rows,
+        nullptr, L.offsets, (int)i0, (int)i1, nullptr);
+  }
+  CK(cudaGetLastError());
+  return F12INT_OK;
+}
+
+// Build the lists of one batch in staging buffer b and launch it: one replay of
+// the graph, or several where the Hermite rows of the batch exceed a class's
+// buffer.
 static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq *> &batch, int b, bool grid) {
   struct Item {
-    int64_t src;      // index into the flat per-class arrays below
+    int32_t q[4];
+    int32_t req;
+    int64_t off;
+    int64_t npab, npcd, rows;
     int tier, nsplit;
     double work;      // per task
   };
   int64_t nzero = 0;
+  std::vector<Item> all[7];
   for (int cls = 1; cls <= 6; ++cls) {
-    ClassLists &S = E.stage[b][cls];
-    int64_t n = 0;
-    std::vector<Item> items;
+    std::vector<Item> &items = all[cls];
     // gather the class's quartets of every request
+    double total = 0.0;
     for (size_t r = 0; r < batch.size(); ++r) {
       const EngineReq &R = *batch[r];
       if (!(R.mask & (1u << (cls - 1)))) continue;
@@ -405,76 +515,134 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
           ++nzero;
           continue;
         }
-        BatchPlan bp{};
-        const int64_t np = (int64_t)B.nprim[s[0]] * B.nprim[s[1]] * B.nprim[s[2]] * B.nprim[s[3]];
-        const bool fp32 = mixed && est < E.fp32_below;
-        batch_plan(la, lb, lc, ld, cls, np, E.task_target[cls], &bp, fp32);   // checked at submit
-        for (int k = 0; k < 4; ++k) S.quartets[4 * n + k] = s[k];
-        S.offsets[n] = off;
-        S.qslot[n] = (int32_t)r;
-        items.push_back(Item{n, bp.tier, bp.nsplit, bp.work});
-        ++n;
+        Item it{};
+        for (int k = 0; k < 4; ++k) it.q[k] = s[k];
+        it.req = (int32_t)r;
+        it.off = off;
+        it.npab = (int64_t)B.nprim[s[0]] * B.nprim[s[1]];
+        it.npcd = (int64_t)B.nprim[s[2]] * B.nprim[s[3]];
+        it.tier = mixed && est < E.fp32_below ? 1 : 0;   // (the tier proper below)
+        const ContractShape sh{la, lb, lc, ld, cls == 5 ? 2 : 0};
+        if (!thin_quartet((la << 6) | (lb << 4) | (lc << 2) | ld, cls)) {
+          it.rows = it.npab * it.npcd * row_pitch(sh.L());
+          total += (double)(it.npab * it.npcd) * task_fmas(sh, it.npcd, sh.ncd());
+        }
+        items.push_back(it);
       }
-      S.views[r] = pair_view(ctx, B, cls, B.prim_screen);
-      S.outs[r] = R.out;
     }
+    // about a dozen tasks per SM where the batch has the work for it, within
+    // the task capacity (a block's result does not depend on the cut)
+    auto plan = [&](double target) {
+      int64_t nt = 0;
+      for (Item &it : items) {
+        const f12int_ctx::BasisData &B = *batch[(size_t)it.req]->B;
+        BatchPlan bp{};
+        const bool fp32 = it.tier >= kTiers ? it.tier < 2 * kTiers : false;
+        batch_plan(B.l[it.q[0]], B.l[it.q[1]], B.l[it.q[2]], B.l[it.q[3]], cls, it.npab * it.npcd, it.npcd, target,
+                   &bp, fp32);   // checked at submit
+        it.tier = bp.tier;
+        it.nsplit = bp.nsplit;
+        it.work = bp.work;
+        nt += bp.nsplit;
+      }
+      return nt;
+    };
+    for (Item &it : items) it.tier = it.tier ? kTiers : 0;
+    if (plan(std::min(E.task_target[cls], std::max(1e5, 2.0 * total / (152 * 12)))) > E.tcap)
+      plan(std::max(E.task_target[cls], kTaskFlops / 8));
     // working order: by tier, then decreasing work per task (the longest
-    // tasks start first); permute the lists
+    // tasks start first)
     std::stable_sort(items.begin(), items.end(), [](const Item &x, const Item &y) {
       if (x.tier != y.tier) return x.tier < y.tier;
       return x.work > y.work;
     });
-    std::vector<int32_t> q2((size_t)4 * n), sl2((size_t)n);
-    std::vector<int64_t> of2((size_t)n);
-    for (int64_t i = 0; i < n; ++i) {
-      const int64_t j = items[i].src;
-      for (int k = 0; k < 4; ++k) q2[4 * i + k] = S.quartets[4 * j + k];
-      of2[i] = S.offsets[j];
-      sl2[i] = S.qslot[j];
+  }
+  size_t at[7] = {0};
+  bool first = true;
+  for (;;) {
+    // a pass: of every class the next quartets whose rows fit
+    bool more = false;
+    int large = 0;   // class of a quartet larger than the buffer, alone in its pass
+    for (int cls = 1; cls <= 6 && !large; ++cls)
+      if (at[cls] < all[cls].size() && all[cls][at[cls]].rows > E.rcap[grid]) large = cls;
+    Item big{};
+    if (large) big = all[large][at[large]];
+    for (int cls = 1; cls <= 6; ++cls) {
+      ClassLists &S = E.stage[b][cls];
+      const std::vector<Item> &items = all[cls];
+      const size_t i0 = at[cls];
+      size_t i1 = i0;
+      int64_t rows = 0;
+      if (large) {
+        if (cls == large) i1 = i0 + 1;
+      } else {
+        while (i1 < items.size() && rows + items[i1].rows <= E.rcap[grid]) rows += items[i1++].rows;
+      }
+      at[cls] = i1;
+      more = more || i1 < items.size();
+      const int64_t n = (int64_t)(i1 - i0);
+      int64_t npq = 0, npq_gen = 0, nt = 0, row = 0, i = 0;
+      for (int t = 0; t < kSlots; ++t) {
+        if (t == kThinSlot) npq_gen = npq;
+        S.counts[kTaskCounts + 2 * t] = nt;
+        for (; i < n && items[i0 + (size_t)i].tier == t; ++i) {
+          const Item &it = items[i0 + (size_t)i];
+          for (int k = 0; k < 4; ++k) S.quartets[4 * i + k] = it.q[k];
+          S.offsets[i] = it.off;
+          S.qslot[i] = it.req;
+          S.pq_off[i] = npq;
+          S.row_off[i] = row;
+          npq += it.npab * it.npcd;
+          row += it.rows;
+          for (int sp = 0; sp < it.nsplit; ++sp) S.tasks[nt++] = CTask{(int32_t)i, (int16_t)sp, (int16_t)it.nsplit};
+        }
+        S.counts[kTaskCounts + 1 + 2 * t] = nt;
+      }
+      S.pq_off[n] = npq;
+      S.row_off[n] = row;
+      S.counts[0] = n;
+      S.counts[1] = npq;
+      S.counts[2] = npq_gen;
+      for (size_t r = 0; r < batch.size(); ++r) {
+        if (!(batch[r]->mask & (1u << (cls - 1)))) continue;
+        S.views[r] = pair_view(ctx, *batch[r]->B, cls, batch[r]->B->prim_screen);
+        S.outs[r] = batch[r]->out;
+      }
+      // copy what this pass uses
+      const ClassLists &D = E.dev[cls];
+      cudaStream_t st = E.stream;
+      const size_t ns = batch.size();
+      CK(cudaMemcpyAsync(D.counts, S.counts, sizeof(int64_t) * kCounts, cudaMemcpyHostToDevice, st));
+      if (n > 0) {
+        CK(cudaMemcpyAsync(D.quartets, S.quartets, sizeof(int32_t) * 4 * n, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(D.pq_off, S.pq_off, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(D.row_off, S.row_off, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(D.offsets, S.offsets, sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(D.qslot, S.qslot, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(D.tasks, S.tasks, sizeof(CTask) * nt, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(D.views, S.views, sizeof(PairView) * ns, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(D.outs, S.outs, sizeof(double *) * ns, cudaMemcpyHostToDevice, st));
+      }
     }
-    int64_t npq = 0, nt = 0;
-    for (int64_t i = 0; i < n; ++i) {
-      for (int k = 0; k < 4; ++k) S.quartets[4 * i + k] = q2[4 * i + k];
-      S.offsets[i] = of2[i];
-      S.qslot[i] = sl2[i];
-      const f12int_ctx::BasisData &B = *batch[sl2[i]]->B;
-      S.pq_off[i] = npq;
-      npq += (int64_t)B.nprim[q2[4 * i]] * B.nprim[q2[4 * i + 1]] * B.nprim[q2[4 * i + 2]] * B.nprim[q2[4 * i + 3]];
-    }
-    S.pq_off[n] = npq;
-    S.counts[0] = n;
-    S.counts[1] = npq;
-    int64_t i = 0;
-    for (int t = 0; t < kSlots; ++t) {
-      if (t == kThinSlot) S.counts[2] = S.pq_off[i];
-      S.counts[kTaskCounts + 2 * t] = nt;
-      for (; i < n && items[i].tier == t; ++i)
-        for (int sp = 0; sp < items[i].nsplit; ++sp) S.tasks[nt++] = CTask{(int32_t)i, (int16_t)sp, (int16_t)items[i].nsplit};
-      S.counts[kTaskCounts + 1 + 2 * t] = nt;
-    }
-    // copy what this batch uses
-    const ClassLists &D = E.dev[cls];
+    *E.zstage_count[b] = first ? nzero : 0;
     cudaStream_t st = E.stream;
-    const size_t ns = batch.size();
-    CK(cudaMemcpyAsync(D.counts, S.counts, sizeof(int64_t) * kCounts, cudaMemcpyHostToDevice, st));
-    if (n > 0) {
-      CK(cudaMemcpyAsync(D.quartets, S.quartets, sizeof(int32_t) * 4 * n, cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(D.pq_off, S.pq_off, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(D.offsets, S.offsets, sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(D.qslot, S.qslot, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(D.tasks, S.tasks, sizeof(CTask) * nt, cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(D.views, S.views, sizeof(PairView) * ns, cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(D.outs, S.outs, sizeof(double *) * ns, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(E.zero_count, E.zstage_count[b], sizeof(int64_t), cudaMemcpyHostToDevice, st));
+    if (first && nzero > 0) {
+      CK(cudaMemcpyAsync(E.zero_dst, E.zstage_dst[b], sizeof(double *) * nzero, cudaMemcpyHostToDevice, st));
+      CK(cudaMemcpyAsync(E.zero_len, E.zstage_len[b], sizeof(int64_t) * nzero, cudaMemcpyHostToDevice, st));
     }
+    if (large) {
+      const int rc = engine_large(ctx, E, large, grid, big.npab, big.npab * big.npcd, big.rows, big.tier);
+      if (rc != F12INT_OK) return rc;
+      if (first && nzero > 0) k_zero_blocks<<<4 * 152, 128, 0, st>>>(E.zero_dst, E.zero_len, E.zero_count);
+    } else {
+      CK(cudaGraphLaunch(E.exec[grid], st));
+    }
+    first = false;
+    if (!more) break;
+    CK(cudaStreamSynchronize(st));   // the next pass's lists take the staging buffer
   }
-  *E.zstage_count[b] = nzero;
   cudaStream_t st = E.stream;
-  CK(cudaMemcpyAsync(E.zero_count, E.zstage_count[b], sizeof(int64_t), cudaMemcpyHostToDevice, st));
-  if (nzero > 0) {
-    CK(cudaMemcpyAsync(E.zero_dst, E.zstage_dst[b], sizeof(double *) * nzero, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(E.zero_len, E.zstage_len[b], sizeof(int64_t) * nzero, cudaMemcpyHostToDevice, st));
-  }
-  CK(cudaGraphLaunch(E.exec[grid], st));
   CK(cudaMemcpyAsync(E.stage_status[b], E.status, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
   CK(cudaMemsetAsync(E.status, 0, sizeof(unsigned), st));
   CK(cudaEventRecord(E.ev[b], st));
@@ -562,10 +730,12 @@ static void engine_shutdown(f12int_ctx *ctx) {
   for (void *p : ds)
     if (p) cudaFree(p);
   for (int c = 1; c <= 6; ++c) {
-    void *cs[] = {E->keys[c], E->order[c], E->part[c], E->hist[c]};
+    void *cs[] = {E->keys[c], E->order[c], E->part[c], E->hist[c], E->rows[0][c]};
     for (void *p : cs)
       if (p) cudaFree(p);
     if (E->branch[c]) cudaStreamDestroy(E->branch[c]);
+    for (cudaStream_t t : E->sub[c])
+      if (t) cudaStreamDestroy(t);
   }
   ctx->used -= std::min(ctx->used, E->bytes);
   for (cudaGraphExec_t x : E->exec)
@@ -675,7 +845,8 @@ int f12int_submit(f12int_ctx *ctx, int basis_id, const f12int_request *req, uint
       const int32_t *s = &R->q[4 * (size_t)i];
       BatchPlan bp{};
       const int64_t np = (int64_t)B.nprim[s[0]] * B.nprim[s[1]] * B.nprim[s[2]] * B.nprim[s[3]];
-      if (!batch_plan(B.l[s[0]], B.l[s[1]], B.l[s[2]], B.l[s[3]], c, np, kTaskFlops / 8, &bp)) {
+      if (!batch_plan(B.l[s[0]], B.l[s[1]], B.l[s[2]], B.l[s[3]], c, np, (int64_t)B.nprim[s[2]] * B.nprim[s[3]],
+                      kTaskFlops / 8, &bp)) {
         delete R;
         return F12INT_EINVAL;
       }

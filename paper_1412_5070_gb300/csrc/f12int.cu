@@ -45,15 +45,8 @@ namespace {
 
 constexpr int LSH = 3;                 // highest shell angular momentum
 constexpr int NHMAX = 680;             // Hermite indices with t+u+v <= 14
-constexpr int BLOCK_CONTRACT = 128;
-// ket component order of a contraction task: 100 components at most (f f),
-// then the class starts (7 term counts at most for lc + ld <= 6)
-constexpr int KORD_CLS = 100;
-constexpr int KORD_SIZE = KORD_CLS + 16;
 constexpr int BLOCK_AUX = 64;
-
-__constant__ unsigned char c_tuv[NHMAX][3];   // Hermite index -> (t, u, v)
-__constant__ unsigned char c_cart[LSH + 3][28][3];  // shell l (<= 5) -> component exponents
+constexpr int NSIDE = 8;               // side streams of a call's contraction launches
 
 
 // ---------------------------------------------------------------------------
@@ -343,81 +336,6 @@ __global__ void k_items_eval(Tables T, PairView PV, QuartetView QV, int cls, int
 
 
 
-// Auxiliary functions of the general contraction's quartets from the grid (or
-// the Boys table): one thread per primitive quartet, hat g_n (n <= L) into its row, or its key set
-// to the skip key.  L is the same for whole stretches of the list, so a warp
-// nearly always takes one of the instances below.
-template <int L>
-__device__ __forceinline__ void direct_row(const GridView &G, double xi, double u, double2 *o) {
-  double h[L + 1];
-  aux_direct<L>(G, xi, u, h);
-  const double is = 1.0 / sqrt(xi);
-#pragma unroll
-  for (int l = 0; l <= (L | 3); l += 2)
-    o[l >> 1] = make_double2(l <= L ? is * h[l <= L ? l : 0] : 0.0, l + 1 <= L ? is * h[l + 1 <= L ? l + 1 : 0] : 0.0);
-}
-
-template <bool BATCH>
-__global__ void __launch_bounds__(BLOCK_AUX)
-k_direct_rows(GridView G, PairView PV0, QuartetView QV, int cls, int64_t pq0, int64_t npq, int *keys, double *part,
-            unsigned long long *fma_total) {
-  // in a batch count_dev[2] is the number of primitive quartets that the
-  // general contraction reads (the thin ones follow them in the list)
-  const int64_t n = BATCH ? QV.count_dev[2] : npq;
-  unsigned long long nfma = 0;
-  for (int64_t r0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & ~(int64_t)31; r0 < n;
-       r0 += (int64_t)gridDim.x * blockDim.x) {   // warp-uniform
-    const int lane = threadIdx.x & 31;
-    int64_t lo = lane == 0 ? find_quartet(QV.pq_off, qv_count(QV), pq0 + r0) : 0;
-    lo = __shfl_sync(0xffffffffu, lo, 0);
-    const int64_t r = r0 + lane, pq = pq0 + r;
-    if (r >= n) continue;
-    // every quartet holds at least one primitive quartet: the lane's lies within `lane` of the warp's first
-    int64_t hi = min(lo + lane, qv_count(QV) - 1);
-    while (lo < hi) {
-      const int64_t mid = (lo + hi + 1) >> 1;
-      if (QV.pq_off[mid] <= pq) lo = mid;
-      else hi = mid - 1;
-    }
-    const PairView &PV = qv_view<BATCH>(PV0, QV, lo);
-    const int32_t *s = QV.quartets + 4 * lo;
-    const int ns = PV.nshell;
-    const int ab = s[0] * ns + s[1], cd = s[2] * ns + s[3];
-    const int npcd = PV.pair_start[cd + 1] - PV.pair_start[cd];
-    const int k = (int)(pq - QV.pq_off[lo]);
-    const int pab = PV.pair_start[ab] + k / npcd, pcd = PV.pair_start[cd] + k % npcd;
-    if (prim_negligible(PV, pab, pcd)) {
-      keys[r] = SKIP_KEY;
-      continue;
-    }
-    keys[r] = 0;
-    const int L = PV.shell_l[s[0]] + PV.shell_l[s[1]] + PV.shell_l[s[2]] + PV.shell_l[s[3]] + (cls == 5 ? 2 : 0);
-    const double p = PV.pp_p[pab], q = PV.pp_p[pcd], xi = p * q / (p + q);
-    const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
-                 Z = pair_sep(PV.pp_P, pab, pcd, 2);
-    const double u = X * X + Y * Y + Z * Z;
-    double2 *o = reinterpret_cast<double2 *>(part + r * kPartPitch);
-    nfma += aux_direct_fmas(G.boys != nullptr, L);
-    switch (L) {
-      case 4: direct_row<4>(G, xi, u, o); break;
-      case 5: direct_row<5>(G, xi, u, o); break;
-      case 6: direct_row<6>(G, xi, u, o); break;
-      case 7: direct_row<7>(G, xi, u, o); break;
-      case 8: direct_row<8>(G, xi, u, o); break;
-      case 9: direct_row<9>(G, xi, u, o); break;
-      case 10: direct_row<10>(G, xi, u, o); break;
-      case 11: direct_row<11>(G, xi, u, o); break;
-      case 12: direct_row<12>(G, xi, u, o); break;
-      case 13: direct_row<13>(G, xi, u, o); break;
-      default: direct_row<14>(G, xi, u, o); break;
-    }
-  }
-  if (fma_total) {
-    for (int o = 16; o > 0; o >>= 1) nfma += __shfl_down_sync(0xffffffffu, nfma, o);
-    if ((threadIdx.x & 31) == 0 && nfma) atomicAdd(fma_total, nfma);
-  }
-}
-
 // hat g_n at given (xi, D) points (no prefactor), for the aux-stage tests:
 // from the grid where it holds the point, else family by family.
 __global__ void k_aux_points(Tables T, GridView G, const unsigned char *ok, int cls, int64_t npts, const double *xi,
@@ -447,368 +365,9 @@ __global__ void k_aux_points(Tables T, GridView G, const unsigned char *ok, int 
   for (int n = 0; n <= nmax; ++n) out[i * (nmax + 1) + n] = g[n];
 }
 
-// -------------------------------------------------------------- contract --
-// One block per shell quartet and range of ket components: a quartet whose
-// buffers would not fit in shared memory is split into NSPLIT blocks, each
-// owning a contiguous range of the c*d Cartesian components (every block
-// repeats the Hermite recursion, which is a small part of the work at the
-// angular momenta that need a split).  The NW warps of a block split the ket
-// primitive pairs.  Below, ncd is the number of ket components of the block.
-// Shared memory (doubles):
-//   per warp: R0, R1  two levels of the Hermite recursion        2 * nh(L)
-//             Rc      the last level (n = 0) in a cube [t][u][v] of
-//                     pitch L+1, so that the index of R_{t+t',u+u',v+v'}
-//                     is a bra part plus a ket part                  (L+1)^3
-//             W       ket-contracted integrals, bra order <= lab
-//                     (+2 for I5), summed over the warp's ket
-//                     primitive pairs                             nh(Lb) * ncd
-//             g       the radial derivatives g_n                  LAUX + 1
-//             E3cd    E^{cd}_{t'u'v'} = E_t' E_u' E_v' of the
-//                     current ket primitive pair, per component   ne3(lc, ld)
-//   block:    O       output accumulator                          nab * ncd
-//             ck, hb  (ints) cube offset of every ket Hermite product
-//                     and W offset hidx(t,u,v)*ncd of every bra one
-//             E3ab    E^{ab}_{tuv} of the current bra primitive
-//                     pair (times (a-b)/2p for I5), and for I5 the
-//                     three dE/dAB-weighted products              ne3(la, lb) (x4 for I5)
-// The per-warp W are summed in warp order, so results do not depend on
-// scheduling; the sum also applies the bra sign (-1)^{t+u+v} of Eq. ii.
-__host__ __device__ __forceinline__ size_t contract_warp_doubles(int nhL, int nhB, int ncd, int ne3cd, int L) {
-  return (size_t)2 * nhL + (size_t)(L + 1) * (L + 1) * (L + 1) + (size_t)nhB * ncd + (LAUX + 1) + (size_t)ne3cd;
-}
-
-// number of Hermite products over all component pairs of shells (l1, l2)
-__host__ __device__ inline int ne3_count(int l1, int l2) {
-  int n = 0;
-  for (int i = l1; i >= 0; --i)
-    for (int j = l1 - i; j >= 0; --j)
-      for (int i2 = l2; i2 >= 0; --i2)
-        for (int j2 = l2 - i2; j2 >= 0; --j2) n += (i + i2 + 1) * (j + j2 + 1) * (l1 - i - j + l2 - i2 - j2 + 1);
-  return n;
-}
-
-// largest number of Hermite products over the ranges of jc consecutive
-// component pairs (same lexicographic order as the kernel's)
-static inline int ne3_chunk_max(int l1, int l2, int jc) {
-  int best = 0, cur = 0, k = 0;
-  for (int i = l1; i >= 0; --i)
-    for (int j = l1 - i; j >= 0; --j)
-      for (int i2 = l2; i2 >= 0; --i2)
-        for (int j2 = l2 - i2; j2 >= 0; --j2) {
-          cur += (i + i2 + 1) * (j + j2 + 1) * (l1 - i - j + l2 - i2 - j2 + 1);
-          if (++k == jc) {
-            best = cur > best ? cur : best;
-            cur = k = 0;
-          }
-        }
-  return cur > best ? cur : best;
-}
-
-__device__ __forceinline__ double tfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float tfma(float a, float b, float c) { return fmaf(a, b, c); }
-
-// One contraction task (quartet and ket range) by the whole block.  T is the
-// type of the Hermite recursion, the E products and every accumulation
-// (double, or float on the mixed path); g_n are always summed in double.
-template <bool BATCH, class T>
-__device__ __forceinline__ void contract_task(const PairView &PV0, const QuartetView &QV, int cls, int nf,
-                                              int64_t pq0, const CTask task, const int *keys, const double *part,
-                                              double *out,
-                                              const int64_t *offsets, unsigned long long *flops_total,
-                                              T *smem, int *off_ab, int *off_cd, int *kord) {
-  const int64_t q = task.q;
-  const int split = task.split, nsplit = task.nsplit;
-  const PairView &PV = qv_view<BATCH>(PV0, QV, q);
-  const int32_t *s = QV.quartets + 4 * q;
-  const int ns = PV.nshell;
-  const int la = PV.shell_l[s[0]], lb = PV.shell_l[s[1]], lc = PV.shell_l[s[2]], ld = PV.shell_l[s[3]];
-  const int ext = cls == 5 ? 2 : 0;
-  const int lab = la + lb, lcd = lc + ld;
-  const int L = lab + lcd + ext;
-  const int Lb = lab + ext;
-  const int na = ncart(la), nb = ncart(lb), nc = ncart(lc), nd = ncart(ld);
-  const int ncd_all = nc * nd, nab = na * nb;
-  const int jc = (ncd_all + nsplit - 1) / nsplit, j0 = split * jc;
-  const int ncd = min(jc, ncd_all - j0);   // ket components of this block: j0 .. j0+ncd-1
-  if (ncd <= 0) return;                     // block-uniform
-  const int nhL = nh_count(L), nhB = nh_count(Lb);
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
-  if (tid == 0) {
-    int o = 0;
-    for (int j = 0; j < ncd; ++j) {
-      off_cd[j] = o;
-      const unsigned char *ec = c_cart[lc][(j0 + j) / nd], *ed = c_cart[ld][(j0 + j) % nd];
-      o += (ec[0] + ed[0] + 1) * (ec[1] + ed[1] + 1) * (ec[2] + ed[2] + 1);
-    }
-    off_cd[ncd] = o;
-    // ket components in order of increasing term count (the ket step's loop
-    // length), one class per count: kord[0..ncd) the components,
-    // kord[KORD_CLS + c] the first position of class c (ncd after the last).
-    // Lanes that take consecutive entries of the (class, bra index,
-    // component) order run loops of one length.
-    int nc_ = 0, pos = 0;
-    while (pos < ncd) {
-      int len = 1 << 30;
-      for (int j = 0; j < ncd; ++j) {
-        const int lj = off_cd[j + 1] - off_cd[j];
-        if (lj > (nc_ ? off_cd[kord[pos - 1] + 1] - off_cd[kord[pos - 1]] : 0) && lj < len) len = lj;
-      }
-      kord[KORD_CLS + nc_] = pos;
-      for (int j = 0; j < ncd; ++j)
-        if (off_cd[j + 1] - off_cd[j] == len) kord[pos++] = j;
-      ++nc_;
-    }
-    kord[KORD_CLS + nc_] = ncd;
-    o = 0;
-    for (int j = 0; j < nab; ++j) {
-      off_ab[j] = o;
-      const unsigned char *ea = c_cart[la][j / nb], *eb = c_cart[lb][j % nb];
-      o += (ea[0] + eb[0] + 1) * (ea[1] + eb[1] + 1) * (ea[2] + eb[2] + 1);
-    }
-    off_ab[nab] = o;
-  }
-  __syncthreads();
-  const int ne3cd = off_cd[ncd], ne3ab = off_ab[nab];
-  const size_t wsz = contract_warp_doubles(nhL, nhB, ncd, ne3cd, L);
-  const int P = L + 1;   // cube pitch of Rc
-  T *R0 = smem + warp * wsz;
-  T *R1 = R0 + nhL;
-  T *Rc = R1 + nhL;
-  T *W = Rc + (size_t)P * P * P;
-  T *gw = W + (size_t)nhB * ncd;
-  T *E3cd = gw + (LAUX + 1);
-  T *Oacc = smem + nw * wsz;
-  T *E3ab = Oacc + (size_t)nab * ncd;
-  T *E3fx = E3ab + ne3ab, *E3fy = E3fx + ne3ab, *E3fz = E3fy + ne3ab;
-  int *ck = reinterpret_cast<int *>(E3ab + (size_t)ne3ab * (cls == 5 ? 4 : 1));
-  int *hb = ck + ne3cd;
-  // index tables of this task (same for every primitive quartet)
-  for (int j = tid; j < ncd; j += nthr) {
-    const unsigned char *ec = c_cart[lc][(j0 + j) / nd], *ed = c_cart[ld][(j0 + j) % nd];
-    const int tx = ec[0] + ed[0], ty = ec[1] + ed[1], tz = ec[2] + ed[2];
-    int m = off_cd[j];
-    for (int t2 = 0; t2 <= tx; ++t2)
-      for (int u2 = 0; u2 <= ty; ++u2)
-        for (int v2 = 0; v2 <= tz; ++v2) ck[m++] = (t2 * P + u2) * P + v2;
-  }
-  for (int c = tid; c < nab; c += nthr) {
-    const unsigned char *ea = c_cart[la][c / nb], *eb = c_cart[lb][c % nb];
-    const int tx = ea[0] + eb[0], ty = ea[1] + eb[1], tz = ea[2] + eb[2];
-    int m = off_ab[c];
-    for (int t = 0; t <= tx; ++t)
-      for (int u = 0; u <= ty; ++u)
-        for (int v = 0; v <= tz; ++v) hb[m++] = hidx(t, u, v) * ncd;
-  }
-  __syncthreads();
-  const int ab = s[0] * ns + s[1], cd = s[2] * ns + s[3];
-  const int ab0 = PV.pair_start[ab], npab = PV.pair_start[ab + 1] - ab0;
-  const int cd0 = PV.pair_start[cd], npcd = PV.pair_start[cd + 1] - cd0;
-  const int ntab = lab + 1, ntcd = lcd + 1;
-  const int n1ab = (la + 1) * (lb + 1) * ntab;
-  const int n1cd = (lc + 1) * (ld + 1) * ntcd;
-  const double pi52 = 17.493418327624862846;  // pi^{5/2}
-
-  for (int i = tid; i < nab * ncd; i += nthr) Oacc[i] = 0.0;
-  unsigned long long nproc = 0;   // primitive quartets this warp processed
-
-  for (int iab = 0; iab < npab; ++iab) {
-    const int pab = ab0 + iab;
-    for (int i = lane; i < nhB * ncd; i += 32) W[i] = 0.0;
-    __syncwarp();
-    for (int icd = warp; icd < npcd; icd += nw) {
-      const int pcd = cd0 + icd;
-      const int64_t pq = QV.pq_off[q] + (int64_t)iab * npcd + icd - pq0;
-      if (keys[pq * nf] == SKIP_KEY) continue;   // dropped by the primitive screen; warp-uniform
-      ++nproc;
-      const T X = (T)pair_sep(PV.pp_P, pab, pcd, 0), Y = (T)pair_sep(PV.pp_P, pab, pcd, 1),
-                   Z = (T)pair_sep(PV.pp_P, pab, pcd, 2);
-      // g_n = sqrt(pi^5/(p+q))/(pq) * sum over families (fixed order)
-      if (lane <= L) {
-        const double p = PV.pp_p[pab], qq = PV.pp_p[pcd];
-        double acc = 0.0;
-        for (int fm = 0; fm < nf; ++fm) acc += part[(pq * nf + fm) * kPartPitch + lane];
-        gw[lane] = (T)(pi52 / (sqrt(p + qq) * p * qq) * acc);
-      }
-      // E^{cd}_{t'u'v'} products of this ket primitive pair
-      const double *Ecd = PV.epool + PV.pp_eoff[pcd];
-      for (int j = lane; j < ncd; j += 32) {
-        const unsigned char *ec = c_cart[lc][(j0 + j) / nd], *ed = c_cart[ld][(j0 + j) % nd];
-        const double *ex = Ecd + (ec[0] * (ld + 1) + ed[0]) * ntcd;
-        const double *ey = Ecd + n1cd + (ec[1] * (ld + 1) + ed[1]) * ntcd;
-        const double *ez = Ecd + 2 * n1cd + (ec[2] * (ld + 1) + ed[2]) * ntcd;
-        const int tx = ec[0] + ed[0], ty = ec[1] + ed[1], tz = ec[2] + ed[2];
-        T *e = E3cd + off_cd[j];
-        int m = 0;
-        for (int t2 = 0; t2 <= tx; ++t2)
-          for (int u2 = 0; u2 <= ty; ++u2) {
-            const double exy = ex[t2] * ey[u2];
-            for (int v2 = 0; v2 <= tz; ++v2) e[m++] = (T)(exy * ez[v2]);
-          }
-      }
-      __syncwarp();
-      // Hermite recursion from level n = L down to 0, ping-pong between R0/R1
-      T *cur = R0, *nxt = R1;
-      if (lane == 0) {
-        cur[0] = gw[L];
-        if (L == 0) Rc[0] = gw[0];
-      }
-      __syncwarp();
-      for (int n = L - 1; n >= 0; --n) {
-        const int cnt = nh_count(L - n);
-        for (int idx = lane; idx < cnt; idx += 32) {
-          const int t = c_tuv[idx][0], u = c_tuv[idx][1], v = c_tuv[idx][2];
-          T val;
-          if (idx == 0) {
-            val = gw[n];
-          } else if (t > 0) {
-            val = X * cur[hidx(t - 1, u, v)];
-            if (t > 1) val += (t - 1) * cur[hidx(t - 2, u, v)];
-          } else if (u > 0) {
-            val = Y * cur[hidx(t, u - 1, v)];
-            if (u > 1) val += (u - 1) * cur[hidx(t, u - 2, v)];
-          } else {
-            val = Z * cur[hidx(t, u, v - 1)];
-            if (v > 1) val += (v - 1) * cur[hidx(t, u, v - 2)];
-          }
-          if (n > 0) nxt[idx] = val;
-          else Rc[(t * P + u) * P + v] = val;   // the last level, in the cube
-        }
-        __syncwarp();
-        T *tmp = cur;
-        cur = nxt;
-        nxt = tmp;
-      }
-      // inner (ket) sum of Eq. ii:  W[tuv][cd] += sum E^{cd}_{t'u'v'} R_{t+t',u+u',v+v'},
-      // entries taken in (term-count class, bra index, component) order
-      for (int r = lane, c = 0; r < nhB * ncd; r += 32) {
-        while (r >= nhB * kord[KORD_CLS + c + 1]) ++c;
-        const int c0 = kord[KORD_CLS + c], n_c = kord[KORD_CLS + c + 1] - c0;
-        const int rr = r - nhB * c0;
-        const int bi = rr / n_c;
-        const int j = kord[c0 + rr - bi * n_c];
-        const int cb = (c_tuv[bi][0] * P + c_tuv[bi][1]) * P + c_tuv[bi][2];
-        const int m0 = off_cd[j], m1 = off_cd[j + 1];
-        T acc = 0;
-        for (int m = m0; m < m1; ++m) acc = tfma(E3cd[m], Rc[cb + ck[m]], acc);
-        W[bi * ncd + j] += acc;
-      }
-      __syncwarp();
-    }
-    __syncthreads();
-    // sum the warps' W into warp 0's buffer (fixed order), with the bra sign
-    const size_t woff = (size_t)2 * nhL + (size_t)P * P * P;   // W within a warp's region
-    T *W0 = smem + woff;
-    for (int i = tid; i < nhB * ncd; i += nthr) {
-      T acc = W0[i];
-      for (int w = 1; w < nw; ++w) acc += smem[w * wsz + woff + i];
-      const int bi = i / ncd;
-      W0[i] = ((c_tuv[bi][0] + c_tuv[bi][1] + c_tuv[bi][2]) & 1) ? -acc : acc;
-    }
-    // E^{ab}_{tuv} products of this bra primitive pair
-    const double *Eab = PV.epool + PV.pp_eoff[pab];
-    const double *Fab = Eab + 3 * n1ab;
-    const double a = PV.pp_ab[2 * pab], b = PV.pp_ab[2 * pab + 1];
-    const double c5 = (a - b) / (2.0 * (a + b));
-    for (int c = tid; c < nab; c += nthr) {
-      const unsigned char *ea = c_cart[la][c / nb], *eb = c_cart[lb][c % nb];
-      const int ox = (ea[0] * (lb + 1) + eb[0]) * ntab;
-      const int oy = n1ab + (ea[1] * (lb + 1) + eb[1]) * ntab;
-      const int oz = 2 * n1ab + (ea[2] * (lb + 1) + eb[2]) * ntab;
-      const int tx = ea[0] + eb[0], ty = ea[1] + eb[1], tz = ea[2] + eb[2];
-      const int o = off_ab[c];
-      int m = 0;
-      for (int t = 0; t <= tx; ++t)
-        for (int u = 0; u <= ty; ++u)
-          for (int v = 0; v <= tz; ++v, ++m) {
-            const double exy = Eab[ox + t] * Eab[oy + u];
-            if (cls != 5) {
-              E3ab[o + m] = (T)(exy * Eab[oz + v]);
-            } else {
-              E3ab[o + m] = (T)(c5 * exy * Eab[oz + v]);
-              E3fx[o + m] = (T)(Fab[ox + t] * Eab[oy + u] * Eab[oz + v]);
-              E3fy[o + m] = (T)(Eab[ox + t] * Fab[oy + u] * Eab[oz + v]);
-              E3fz[o + m] = (T)(exy * Fab[oz + v]);
-            }
-          }
-    }
-    __syncthreads();
-    // outer (bra) sum
-    for (int i = tid; i < nab * ncd; i += nthr) {
-      const int iabc = i / ncd, j = i - iabc * ncd;
-      const int ia = iabc / nb, ib = iabc - ia * nb;
-      const unsigned char *ea = c_cart[la][ia], *eb = c_cart[lb][ib];
-      const int tx = ea[0] + eb[0], ty = ea[1] + eb[1], tz = ea[2] + eb[2];
-      const int o = off_ab[iabc];
-      T acc = 0;
-      int m = 0;
-      for (int t = 0; t <= tx; ++t)
-        for (int u = 0; u <= ty; ++u)
-          for (int v = 0; v <= tz; ++v, ++m) {
-            if (cls != 5) {
-              acc = tfma(E3ab[o + m], W0[hb[o + m] + j], acc);
-            } else {
-              // Eq. I5byI3_ with the second coefficient -1 (see the derivation note
-              // below); W0 carries the bra sign, so the gradient term changes sign
-              const T lap = W0[hidx(t + 2, u, v) * ncd + j] + W0[hidx(t, u + 2, v) * ncd + j] +
-                                 W0[hidx(t, u, v + 2) * ncd + j];
-              acc = tfma(E3ab[o + m], lap, acc);
-              acc = tfma(E3fx[o + m], W0[hidx(t + 1, u, v) * ncd + j], acc);
-              acc = tfma(E3fy[o + m], W0[hidx(t, u + 1, v) * ncd + j], acc);
-              acc = tfma(E3fz[o + m], W0[hidx(t, u, v + 1) * ncd + j], acc);
-            }
-          }
-      Oacc[i] += acc;
-    }
-    __syncthreads();
-  }
-  double *o;
-  if constexpr (BATCH) o = QV.slot_out[QV.qslot[q]] + offsets[q];
-  else o = out + offsets[q];
-  for (int i = tid; i < nab * ncd; i += nthr) {
-    const int iabc = i / ncd;
-    o[(size_t)iabc * ncd_all + j0 + (i - iabc * ncd)] = (double)Oacc[i];
-  }
-  if (flops_total && lane == 0 && nproc) {
-    // algorithmic FP64 flops per primitive quartet: Hermite recursion 2 C(L+4,4)
-    // (counted once per quartet, not per split), ket step 2 nh(lab+ext) nh(lcd)
-    // ncd, bra step 2 nab nh(lab) ncd (x4 for I5)
-    const unsigned long long r = split == 0 ? 2ull * (L + 1) * (L + 2) * (L + 3) * (L + 4) / 24 : 0ull;
-    const unsigned long long ket = 2ull * nhB * nh_count(lcd) * ncd;
-    const unsigned long long bra = 2ull * nab * nh_count(lab) * ncd * (cls == 5 ? 4 : 1);
-    atomicAdd(flops_total, nproc * (r + ket + bra));
-  }
-}
-
-template <bool BATCH, class T>
-__global__ void __launch_bounds__(BLOCK_CONTRACT)
-k_contract(PairView PV0, QuartetView QV, int cls, int nf, int64_t pq0, const CTask *tasks, int64_t ntask,
-           const int64_t *ntask_dev, const int *keys, const double *part, double *out, const int64_t *offsets,
-           unsigned int *status, unsigned long long *flops_total) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T *smem = reinterpret_cast<T *>(smem_raw);
-  __shared__ int off_ab[101], off_cd[101], kord[KORD_SIZE];
-  if constexpr (BATCH) {
-    // ntask_dev = {first, end} of this launch's tasks
-    const int64_t te = ntask_dev[1];
-    for (int64_t tk = ntask_dev[0] + blockIdx.x; tk < te; tk += gridDim.x) {
-      __syncthreads();   // the previous task's shared-memory reads are done
-      contract_task<BATCH, T>(PV0, QV, cls, nf, pq0, tasks[tk], keys, part, out, offsets, flops_total, smem, off_ab,
-                              off_cd, kord);
-    }
-  } else {
-    if (blockIdx.x < ntask)
-      contract_task<BATCH, T>(PV0, QV, cls, nf, pq0, tasks[blockIdx.x], keys, part, out, offsets, flops_total, smem,
-                              off_ab, off_cd, kord);
-  }
-}
-// Derivation note for I5: with d/dA_x = (a/p) d/dP_x + d/dAB_x and
-// d/dB_x = (b/p) d/dP_x - d/dAB_x (E depends on AB only, R on P only),
-//   1/2 (lap_A - lap_B) = sum_x [ (a-b)/(2p) d^2/dP_x^2 + d/dP_x d/dAB_x ],
-// and d/dP_x = -d/dQ_x on R; hence the coefficient of the gradient term is
-// -(a+b)/p = -1.
-
 }  // namespace
+
+#include "contract.cuh"
 
 // ================================================================ host API ==
 
@@ -863,6 +422,13 @@ struct f12int_ctx {
   int32_t *d_qperm = nullptr;
   int64_t *d_operm = nullptr;
   CTask *d_tasks = nullptr;
+  double *d_rows = nullptr;      // Hermite rows of a chunk
+  int64_t *d_rowoff = nullptr;   // first double of every general quartet's rows
+  size_t rows_cap = 0, rowoff_cap = 0;
+  // the contraction launches of a call are independent of one another: they
+  // run on these streams, between two events on the call's
+  cudaStream_t side[NSIDE] = {nullptr};
+  cudaEvent_t fork = nullptr, join[NSIDE] = {nullptr};
   size_t pqoff_cap = 0, keys_cap = 0, order_cap = 0, hist_cap = 0, part_cap = 0, qperm_cap = 0, operm_cap = 0;
   size_t tasks_cap = 0;
   // optional per-kernel timing (events on the launching stream) and counters
@@ -871,11 +437,6 @@ struct f12int_ctx {
   double aux_ms = 0.0, contract_ms = 0.0;
   int64_t aux_launches = 0, contract_launches = 0;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_aux, ev_con, ev_pool;
-  std::vector<int> h_nw;       // warps per contraction block, per quartet in the working order
-  std::vector<int> h_split;    // ket-component ranges (blocks) per quartet, same order
-  std::vector<char> h_fp32;    // 1: Hermite recursion and contraction in FP32 (mixed path), same order
-  std::vector<size_t> h_smem;  // contraction shared memory, per quartet in the working order
-  std::vector<int16_t> h_thin; // class key of a quartet for k_contract_thin, -1: the general kernel; same order
   std::mutex mu;
   std::recursive_mutex bounds_mu;   // first-time primitive and shell-pair bounds
   bool cls_ok[7] = {false, false, false, false, false, false, false};   // classes the factor supports
@@ -984,28 +545,17 @@ std::mutex g_const_mu;
 int upload_constants() {
   std::lock_guard<std::mutex> lk(g_const_mu);
   if (g_const_ready) return F12INT_OK;
-  unsigned char tuv[NHMAX][3];
+  unsigned tuv[NHMAX];
   for (int s = 0; s <= 14; ++s)
     for (int t = s; t >= 0; --t)
       for (int v = 0; v <= s - t; ++v) {
-        int u = s - t - v;
-        int i = hidx(t, u, v);
-        tuv[i][0] = (unsigned char)t;
-        tuv[i][1] = (unsigned char)u;
-        tuv[i][2] = (unsigned char)v;
+        const int u = s - t - v;
+        tuv[hidx(t, u, v)] = (unsigned)(t | u << 4 | v << 8);
       }
-  unsigned char cart[LSH + 3][28][3];
-  std::memset(cart, 0, sizeof(cart));
-  for (int l = 0; l < LSH + 3; ++l) {
-    int k = 0;
-    for (int i = l; i >= 0; --i)
-      for (int j = l - i; j >= 0; --j) {
-        cart[l][k][0] = (unsigned char)i;
-        cart[l][k][1] = (unsigned char)j;
-        cart[l][k][2] = (unsigned char)(l - i - j);
-        ++k;
-      }
-  }
+  const HostPairTabs &pt = pair_tabs();
+  if (pt.term.size() > (size_t)PT_TERMS) return F12INT_ECUDA;
+  CK(cudaMemcpyToSymbol(d_pt, pt.pt, sizeof(pt.pt)));
+  CK(cudaMemcpyToSymbol(d_pt_term, pt.term.data(), sizeof(uint2) * pt.term.size()));
   static AuxConst ac;
   fill_aux_const(ac);
   CK(cudaMemcpyToSymbol(c_cratio, ac.cratio, sizeof(ac.cratio)));
@@ -1026,8 +576,7 @@ int upload_constants() {
     CK(cudaMemcpyToSymbol(d_mtab, &dkc, sizeof(dkc)));
     g_boys = dk + (size_t)1 * MT_NX * MT_NT;   // a = (1 + 1)/2
   }
-  CK(cudaMemcpyToSymbol(c_tuv, tuv, sizeof(tuv)));
-  CK(cudaMemcpyToSymbol(c_cart, cart, sizeof(cart)));
+  CK(cudaMemcpyToSymbol(d_htuv, tuv, sizeof(tuv)));
   CK(cudaMemcpyToSymbol(c_gh_x, ac.gh_x, sizeof(ac.gh_x)));
   CK(cudaMemcpyToSymbol(c_gh_w, ac.gh_w, sizeof(ac.gh_w)));
   CK(cudaMemcpyToSymbol(c_gl_x, ac.gl_x, sizeof(ac.gl_x)));
@@ -1096,6 +645,11 @@ int f12int_create(f12int_ctx **out, int device, size_t hbm_budget_bytes, void *c
   int rc = upload_constants();
   if (rc == F12INT_OK) rc = dalloc(ctx, &ctx->d_status, sizeof(unsigned int));
   if (rc == F12INT_OK && cudaMemset(ctx->d_status, 0, sizeof(unsigned int)) != cudaSuccess) rc = F12INT_ECUDA;
+  for (int i = 0; i < NSIDE && rc == F12INT_OK; ++i)
+    if (cudaStreamCreateWithFlags(&ctx->side[i], cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->join[i], cudaEventDisableTiming) != cudaSuccess)
+      rc = F12INT_ECUDA;
+  if (rc == F12INT_OK && cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) != cudaSuccess) rc = F12INT_ECUDA;
   if (rc != F12INT_OK) {
     f12int_destroy(ctx);
     return rc;
@@ -1137,6 +691,13 @@ int f12int_destroy(f12int_ctx *ctx) {
   cudaFree(ctx->d_qperm);
   cudaFree(ctx->d_operm);
   cudaFree(ctx->d_tasks);
+  cudaFree(ctx->d_rows);
+  cudaFree(ctx->d_rowoff);
+  for (int i = 0; i < NSIDE; ++i) {
+    if (ctx->side[i]) cudaStreamDestroy(ctx->side[i]);
+    if (ctx->join[i]) cudaEventDestroy(ctx->join[i]);
+  }
+  if (ctx->fork) cudaEventDestroy(ctx->fork);
   cudaFree(ctx->d_status);
   cudaFree(ctx->d_fma);
   for (auto &e : ctx->ev_pool) {
@@ -1629,79 +1190,6 @@ static int ensure_buf(f12int_ctx *ctx, void **p, size_t *cap, size_t bytes) {
   return rc;
 }
 
-// shared memory of a contraction block with nw warps and nsplit ket ranges
-// (esz: bytes per element, 8 for FP64, 4 for the FP32 path)
-static size_t contract_smem(int la, int lb, int lc, int ld, int cls, int nw, int nsplit, size_t esz = 8) {
-  int ext = cls == 5 ? 2 : 0;
-  int L = la + lb + lc + ld + ext;
-  int nhL = nh_count(L), nhB = nh_count(la + lb + ext);
-  int ncd = ncart(lc) * ncart(ld), nab = ncart(la) * ncart(lb);
-  int jc = (ncd + nsplit - 1) / nsplit;
-  size_t e3ab = (size_t)ne3_count(la, lb) * (cls == 5 ? 4 : 1);
-  const int ne3cd = ne3_chunk_max(lc, ld, jc), ne3ab = ne3_count(la, lb);
-  return esz * ((size_t)nw * contract_warp_doubles(nhL, nhB, jc, ne3cd, L) + (size_t)nab * jc + e3ab) +
-         sizeof(int) * ((size_t)ne3cd + ne3ab);
-}
-
-struct ContractPlan {
-  int nw, nsplit;
-  size_t smem;
-};
-
-// Algorithmic FP64 flops per primitive quartet of a task that owns jc ket
-// components: Hermite recursion (repeated by every task of a quartet), ket
-// and bra steps (x4 for I5).
-static double task_flops(int la, int lb, int lc, int ld, int cls, int jc) {
-  const int ext = cls == 5 ? 2 : 0;
-  const int L = la + lb + lc + ld + ext;
-  const double r = 2.0 * (L + 1) * (L + 2) * (L + 3) * (L + 4) / 24.0;
-  const double ket = 2.0 * nh_count(la + lb + ext) * nh_count(lc + ld) * jc;
-  const double bra = 2.0 * ncart(la) * ncart(lb) * nh_count(la + lb) * jc * (cls == 5 ? 4 : 1);
-  return r + ket + bra;
-}
-
-// Work one contraction block should carry at most: a quartet with more is
-// split into more ket ranges than its shared memory needs, so that its
-// primitive quartets do not keep one SM busy while the others idle.
-constexpr double kTaskFlops = 5e7;
-
-static bool valid_split(int ncd, int ns) {
-  const int jc = (ncd + ns - 1) / ns;
-  return (ncd + jc - 1) / jc == ns;   // no empty ranges
-}
-
-static int work_split(int la, int lb, int lc, int ld, int cls, int64_t nprimq, int ns_min,
-                      double target = kTaskFlops) {
-  const int ncd = ncart(lc) * ncart(ld);
-  for (int ns = ns_min; ns <= ncd; ++ns) {
-    if (!valid_split(ncd, ns)) continue;
-    if ((double)nprimq * task_flops(la, lb, lc, ld, cls, (ncd + ns - 1) / ns) <= target) return ns;
-  }
-  return ncd;
-}
-
-// Warps and ket ranges per contraction block for a quartet of nprimq
-// primitive quartets: 4 warps, else 2, on the whole ket; where neither fits
-// in 200 KB of shared memory, the fewest ket ranges that fit with 4 warps,
-// else 2, else 1; then more ranges while a block would exceed kTaskFlops.
-// smem = 0 when nothing fits.
-static ContractPlan contract_plan(int la, int lb, int lc, int ld, int cls, int64_t nprimq, size_t esz = 8) {
-  const size_t cap = 200 * 1024;
-  const int ncd = ncart(lc) * ncart(ld);
-  int nw = 0, ns = 1;
-  for (int w = BLOCK_CONTRACT / 32; w > 1 && !nw; w /= 2)
-    if (contract_smem(la, lb, lc, ld, cls, w, 1, esz) <= cap) nw = w;
-  for (int w = BLOCK_CONTRACT / 32; w >= 1 && !nw; w /= 2)
-    for (int k = 2; k <= ncd && !nw; ++k)
-      if (valid_split(ncd, k) && contract_smem(la, lb, lc, ld, cls, w, k, esz) <= cap) {
-        nw = w;
-        ns = k;
-      }
-  if (!nw) return ContractPlan{1, 1, 0};
-  ns = work_split(la, lb, lc, ld, cls, nprimq, ns);
-  return ContractPlan{nw, ns, contract_smem(la, lb, lc, ld, cls, nw, ns, esz)};
-}
-
 static std::pair<cudaEvent_t, cudaEvent_t> take_events(f12int_ctx *ctx) {
   if (!ctx->ev_pool.empty()) {
     auto e = ctx->ev_pool.back();
@@ -1732,154 +1220,419 @@ static void collect_events(f12int_ctx *ctx) {
 
 // items of the auxiliary stage per chunk (bounds the scratch memory)
 static const int64_t kItemChunk = (int64_t)32 << 20;
+// doubles of Hermite rows per chunk (1 GB)
+static const int64_t kRowChunk = (int64_t)128 << 20;
 static const int kNKeys = MAXFAM * (LAUX + 1) * NZBIN + 1;
 
-// Queue the auxiliary stage (classify, scan, scatter, evaluate) and the
-// contraction for quartets [qa, qb) of the device list.
-static int launch_chunk(f12int_ctx *ctx, const f12int_ctx::BasisData &B, int cls, const int32_t *d_quartets,
-                        const int64_t *d_pqoff, const int64_t *h_pqoff, int64_t n, int64_t qa, int64_t qb,
-                        int64_t pqa, int64_t pqb, size_t smem, double *out_dev, const int64_t *offsets_dev, cudaStream_t st,
-                        bool prim_screen = true) {
-  PairView PV = pair_view(ctx, B, cls, B.prim_screen && prim_screen);
-  QuartetView QV{d_quartets, d_pqoff, n, nullptr, nullptr, nullptr, nullptr};
-  const int kcls = cls == 5 ? 3 : cls;
-  const GridView G = grid_view(ctx, B, cls);
-  // the thin quartets are a suffix of the working order
-  int64_t qthin = qb;
-  while (qthin > qa && ctx->h_thin[qthin - 1] >= 0) --qthin;
-  // with the grid one row per primitive quartet of the general contraction
-  // (the thin kernel evaluates its own), else one item per family
-  const int nf = G.direct() ? 1 : ctx->tables.nfam[kcls];
-  const int64_t nitems = G.direct() ? h_pqoff[qthin] - pqa : (pqb - pqa) * nf;
-  if (nitems > 0 && G.direct()) {
-    int rc = ensure_buf(ctx, (void **)&ctx->d_keys, &ctx->keys_cap, sizeof(int) * nitems);
-    if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_part, &ctx->part_cap, sizeof(double) * nitems * kPartPitch);
-    if (rc != F12INT_OK) return rc;
-    std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
-    if (ctx->timing) {
-      ev = take_events(ctx);
-      cudaEventRecord(ev.first, st);
-    }
-    k_direct_rows<false><<<(unsigned)((nitems + BLOCK_AUX - 1) / BLOCK_AUX), BLOCK_AUX, 0, st>>>(
-        G, PV, QV, cls, pqa, nitems, ctx->d_keys, ctx->d_part, ctx->timing ? ctx->d_fma : nullptr);
-    if (ctx->timing) {
-      cudaEventRecord(ev.second, st);
-      ctx->ev_aux.push_back(ev);
-      ctx->aux_launches++;
-    }
-    ctx->launches++;
-    CK(cudaGetLastError());
-  } else if (nitems > 0) {
-    int rc = ensure_buf(ctx, (void **)&ctx->d_keys, &ctx->keys_cap, sizeof(int) * nitems);
-    if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_order, &ctx->order_cap, sizeof(unsigned) * nitems);
-    if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_part, &ctx->part_cap, sizeof(double) * nitems * kPartPitch);
-    if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_hist, &ctx->hist_cap, sizeof(unsigned) * kNKeys);
-    if (rc != F12INT_OK) return rc;
-    CK(cudaMemsetAsync(ctx->d_hist, 0, sizeof(unsigned) * kNKeys, st));
-    const unsigned nb = (unsigned)((nitems + BLOCK_AUX - 1) / BLOCK_AUX);
-    const unsigned nbq = (unsigned)((pqb - pqa + BLOCK_AUX - 1) / BLOCK_AUX);
-    k_items_classify<false><<<nbq, BLOCK_AUX, 0, st>>>(ctx->tables, PV, QV, cls, pqa, nitems, ctx->d_keys,
-                                                       ctx->d_hist);
-    k_items_scan<<<1, 1024, 0, st>>>(ctx->d_hist, kNKeys);
-    k_items_scatter<<<nb, BLOCK_AUX, 0, st>>>(QV, nf, pqa, ctx->d_keys, ctx->d_hist, nitems, ctx->d_order);
-    std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
-    if (ctx->timing) {
-      ev = take_events(ctx);
-      cudaEventRecord(ev.first, st);
-    }
-    k_items_eval<false><<<nb, BLOCK_AUX, 0, st>>>(ctx->tables, PV, QV, cls, pqa, nitems, ctx->d_order, ctx->d_keys,
-                                                  ctx->d_part, ctx->d_status, ctx->timing ? ctx->d_fma : nullptr);
-    if (ctx->cls_quad[cls]) {
-      k_items_eval<false, true><<<nb, BLOCK_AUX, 0, st>>>(ctx->tables, PV, QV, cls, pqa, nitems, ctx->d_order,
-                                                          ctx->d_keys, ctx->d_part, ctx->d_status,
-                                                          ctx->timing ? ctx->d_fma : nullptr);
-      ctx->launches++;
-    }
-    if (ctx->timing) {
-      cudaEventRecord(ev.second, st);
-      ctx->ev_aux.push_back(ev);
-      ctx->aux_launches++;
-    }
-    ctx->launches += 4;
-    CK(cudaGetLastError());
-  }
-  // contraction: quartets are ordered by decreasing shared-memory need; one
-  // launch per tier of warps and shared memory (powers of two), one block per
-  // (quartet, ket range) task
-  std::vector<CTask> tasks;
-  for (int64_t i = qa; i < qb; ++i)
-    for (int sp = 0; sp < ctx->h_split[i]; ++sp) tasks.push_back(CTask{(int32_t)i, (int16_t)sp, (int16_t)ctx->h_split[i]});
+}  // extern "C"
+
+// Work one contraction block should carry at most, in multiply-adds: a longer
+// one would keep an SM busy while the others idle at the end of a launch.
+constexpr double kTaskFmas = 2e6;
+
+// A planned list: quartets in the working order -- those of the general
+// contraction first, by launch group (precision, threads, shared memory within
+// a factor of two), then decreasing work per task (the longest blocks start
+// first), then the thin ones by class key -- and the launches over them.
+struct ListPlan {
+  struct Group {           // quartets [first, end) of one launch
+    int64_t first, end;
+    int nthr;
+    size_t smem;
+    bool fp32;
+    int thin;              // class key, or -1
+  };
+  std::vector<Group> groups;
+  int64_t n = 0, nthin = 0;            // quartets; first thin one
+  std::vector<int32_t> quartets;       // [4 n]
+  std::vector<int64_t> offsets;        // [n]
+  std::vector<int64_t> pqoff;          // [n + 1] first primitive quartet
+  std::vector<int64_t> rowoff;         // [nthin + 1] first double of the Hermite rows
+  std::vector<int> npab;               // [nthin] bra primitive pairs
+  std::vector<CTask> tasks;            // quartet by quartet
+  std::vector<int64_t> tfirst;         // [n + 1] first task
+};
+
+// Plans the list hq0 (ho0: output offsets).  fp32(s): the mixed path's choice
+// for quartet s; fewest: as few tasks as fit in shared memory.  Returns
+// F12INT_EINVAL for a shell index out of range.
+template <class Fp32>
+static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const int32_t *hq0, const int64_t *ho0,
+                     Fp32 fp32, ListPlan &P, bool fewest = false) {
+  // Every quartet with the same (primitive pairs of bra and ket, FP32 or not,
+  // class key) has the same plan: the distinct ones are planned once, ordered,
+  // and the quartets placed group by group in their list order (a counting
+  // sort: linear in n).
+  struct Kind {
+    int64_t key;
+    int la, lb, lc, ld, f32;
+    int64_t nab, ncd, count, first;
+    bool thin;
+    ContractPlan pl;
+    double work;
+    int tier;
+  };
+  std::vector<Kind> kinds;
+  std::vector<int32_t> kid((size_t)n);
+  const int ns = B.nshell;
+  double total = 0.0;   // multiply-adds of the general contraction
   {
-    int rc = ensure_buf(ctx, (void **)&ctx->d_tasks, &ctx->tasks_cap, sizeof(CTask) * tasks.size());
-    if (rc != F12INT_OK) return rc;
-    CK(cudaMemcpyAsync(ctx->d_tasks, tasks.data(), sizeof(CTask) * tasks.size(), cudaMemcpyHostToDevice, st));
+    std::vector<int64_t> slot_key(4096, -1);   // open-addressing map from a kind's key to its index
+    std::vector<int32_t> slot_val(4096, -1);
+    size_t mask = slot_key.size() - 1;
+    auto find = [&](const std::vector<int64_t> &keys, size_t m, int64_t key) {
+      size_t h = (size_t)((uint64_t)key * 0x9E3779B97F4A7C15ull >> 40) & m;
+      while (keys[h] != -1 && keys[h] != key) h = (h + 1) & m;
+      return h;
+    };
+    for (int64_t i = 0; i < n; ++i) {
+      const int32_t *s = hq0 + 4 * i;
+      for (int k = 0; k < 4; ++k)
+        if (s[k] < 0 || s[k] >= ns) return F12INT_EINVAL;
+      const int lk = (B.l[s[0]] << 6) | (B.l[s[1]] << 4) | (B.l[s[2]] << 2) | B.l[s[3]];
+      const int64_t nab = (int64_t)B.nprim[s[0]] * B.nprim[s[1]], ncd = (int64_t)B.nprim[s[2]] * B.nprim[s[3]];
+      const int f32 = thin_quartet(lk, cls) ? 0 : fp32(s);   // the thin kernel is FP64
+      const int64_t key = (((nab << 26) + ncd) << 9) | (f32 << 8) | lk;
+      size_t h = find(slot_key, mask, key);
+      if (slot_key[h] == -1) {
+        if (kinds.size() * 2 >= slot_key.size()) {   // grow and rehash
+          std::vector<int64_t> nk(slot_key.size() * 2, -1);
+          std::vector<int32_t> nv(slot_key.size() * 2, -1);
+          for (size_t t = 0; t < slot_key.size(); ++t)
+            if (slot_key[t] != -1) {
+              const size_t g = find(nk, nk.size() - 1, slot_key[t]);
+              nk[g] = slot_key[t];
+              nv[g] = slot_val[t];
+            }
+          slot_key.swap(nk);
+          slot_val.swap(nv);
+          mask = slot_key.size() - 1;
+          h = find(slot_key, mask, key);
+        }
+        Kind k{};
+        k.key = key;
+        k.la = lk >> 6;
+        k.lb = (lk >> 4) & 3;
+        k.lc = (lk >> 2) & 3;
+        k.ld = lk & 3;
+        k.f32 = f32;
+        k.nab = nab;
+        k.ncd = ncd;
+        k.thin = thin_quartet(lk, cls);
+        slot_key[h] = key;
+        slot_val[h] = (int32_t)kinds.size();
+        kinds.push_back(k);
+      }
+      kid[(size_t)i] = slot_val[h];
+      kinds[(size_t)slot_val[h]].count++;
+    }
   }
-  int64_t t0 = 0;
-  for (int64_t ra = qa; ra < qthin;) {
-    const int nw = ctx->h_nw[ra];
-    const char f32 = ctx->h_fp32[ra];
-    const size_t sm0 = ctx->h_smem[ra];
-    int64_t rb = ra + 1, nt = ctx->h_split[ra];
-    while (rb < qthin && ctx->h_nw[rb] == nw && ctx->h_fp32[rb] == f32 && 2 * ctx->h_smem[rb] > sm0)
-      nt += ctx->h_split[rb++];
-    std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
-    if (ctx->timing) {
-      ev = take_events(ctx);
-      cudaEventRecord(ev.first, st);
+  for (const Kind &k : kinds)
+    if (!k.thin) {
+      const ContractShape s{k.la, k.lb, k.lc, k.ld, cls == 5 ? 2 : 0};
+      total += (double)k.count * (double)(k.nab * k.ncd) * task_fmas(s, k.ncd, s.ncd());
     }
-    if (f32) {
-      if (sm0 > 48 * 1024)
-        CK(cudaFuncSetAttribute(k_contract<false, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm0));
-      k_contract<false, float><<<(unsigned)nt, 32 * nw, sm0, st>>>(
-          PV, QV, cls, nf, pqa, ctx->d_tasks + t0, nt, nullptr, ctx->d_keys, ctx->d_part, out_dev, offsets_dev,
-          ctx->d_status,
-          ctx->timing ? ctx->d_fma + 1 : nullptr);
-    } else {
-      if (sm0 > 48 * 1024)
-        CK(cudaFuncSetAttribute(k_contract<false, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm0));
-      k_contract<false, double><<<(unsigned)nt, 32 * nw, sm0, st>>>(
-          PV, QV, cls, nf, pqa, ctx->d_tasks + t0, nt, nullptr, ctx->d_keys, ctx->d_part, out_dev, offsets_dev,
-          ctx->d_status,
-          ctx->timing ? ctx->d_fma + 1 : nullptr);
+  // about a dozen tasks per SM where the list has the work for it (a block's
+  // result does not depend on how a quartet is cut into ranges)
+  const double target = fewest ? 1e300 : std::min(kTaskFmas, std::max(5e4, total / (152 * 12)));
+  for (Kind &k : kinds) {
+    k.pl = ContractPlan{32, 1, 0};
+    if (k.thin) {
+      k.work = (double)(k.nab * k.ncd);
+      continue;
     }
-    t0 += nt;
-    if (ctx->timing) {
-      cudaEventRecord(ev.second, st);
-      ctx->ev_con.push_back(ev);
-      ctx->contract_launches++;
-    }
-    ctx->launches++;
-    CK(cudaGetLastError());
-    ra = rb;
+    const ContractShape s{k.la, k.lb, k.lc, k.ld, cls == 5 ? 2 : 0};
+    k.pl = contract_plan(k.la, k.lb, k.lc, k.ld, cls, k.nab * k.ncd, k.ncd, k.f32 ? 4 : 8, target, fewest);
+    if (k.pl.smem == 0) return F12INT_EINVAL;
+    k.work = (double)(k.nab * k.ncd) * task_fmas(s, k.ncd, (s.ncd() + k.pl.nsplit - 1) / k.pl.nsplit);
+    k.tier = 0;
+    while (((size_t)8192 << k.tier) < k.pl.smem) ++k.tier;
   }
-  // thin quartets: one launch per (la, lb, lc, ld), one warp per quartet
-  for (int64_t ra = qthin; ra < qb;) {
-    const int key = ctx->h_thin[ra];
-    int64_t rb = ra + 1;
-    while (rb < qb && ctx->h_thin[rb] == key) ++rb;
-    const int64_t nt = rb - ra;   // one task each
-    const ThinKernel kern = thin_kernel(key, cls == 5);
-    if (!kern) return F12INT_EINVAL;
-    std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
-    if (ctx->timing) {
-      ev = take_events(ctx);
-      cudaEventRecord(ev.first, st);
-    }
-    kern<<<(unsigned)((nt + kThinWarps - 1) / kThinWarps), 32 * kThinWarps, 0, st>>>(
-        PV, QV, nf, pqa, G, ctx->d_tasks + t0, nt, nullptr, ctx->d_keys, ctx->d_part, out_dev, offsets_dev,
-        ctx->timing ? ctx->d_fma + 1 : nullptr);
-    t0 += nt;
-    if (ctx->timing) {
-      cudaEventRecord(ev.second, st);
-      ctx->ev_con.push_back(ev);
-      ctx->contract_launches++;
-    }
-    ctx->launches++;
-    CK(cudaGetLastError());
-    ra = rb;
+  std::vector<int32_t> order(kinds.size());
+  for (size_t g = 0; g < kinds.size(); ++g) order[g] = (int32_t)g;
+  std::sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+    const Kind &a = kinds[(size_t)x], &b = kinds[(size_t)y];
+    if (a.thin != b.thin) return b.thin;
+    const int ka = (int)(a.key & 0xFF), kb = (int)(b.key & 0xFF);
+    if (a.thin) return ka != kb ? ka < kb : (a.work != b.work ? a.work > b.work : a.key < b.key);
+    if (a.f32 != b.f32) return a.f32 < b.f32;
+    if (a.tier != b.tier) return a.tier > b.tier;
+    if (a.pl.nthr != b.pl.nthr) return a.pl.nthr > b.pl.nthr;
+    if (a.work != b.work) return a.work > b.work;
+    return a.key < b.key;
+  });
+  P = ListPlan{};
+  P.n = n;
+  int64_t run = 0;
+  for (size_t at = 0; at < order.size(); ++at) {
+    Kind &k = kinds[(size_t)order[at]];
+    const int thin = k.thin ? (int)(k.key & 0xFF) : -1;
+    if (P.groups.empty() || P.groups.back().thin != thin ||
+        (!k.thin && (P.groups.back().fp32 != (k.f32 != 0) || P.groups.back().nthr != k.pl.nthr ||
+                     kinds[(size_t)order[at - 1]].tier != k.tier)))
+      P.groups.push_back(ListPlan::Group{run, run, k.pl.nthr, 0, k.f32 != 0, thin});
+    ListPlan::Group &G = P.groups.back();
+    G.smem = std::max(G.smem, k.pl.smem);
+    k.first = run;
+    run += k.count;
+    G.end = run;
+    if (!k.thin) P.nthin = run;
   }
+  std::vector<int64_t> perm((size_t)n);
+  {
+    std::vector<int64_t> at(kinds.size());
+    for (size_t g = 0; g < kinds.size(); ++g) at[g] = kinds[g].first;
+    for (int64_t i = 0; i < n; ++i) perm[(size_t)at[(size_t)kid[(size_t)i]]++] = i;
+  }
+  P.quartets.resize((size_t)4 * n);
+  P.offsets.resize((size_t)n);
+  P.pqoff.resize((size_t)n + 1);
+  P.tfirst.resize((size_t)n + 1);
+  P.rowoff.resize((size_t)P.nthin + 1);
+  P.npab.resize((size_t)P.nthin);
+  P.tasks.reserve((size_t)n);
+  int64_t npq = 0, nrow = 0;
+  for (int64_t i = 0; i < n; ++i) {
+    const int64_t j = perm[(size_t)i];
+    const Kind &k = kinds[(size_t)kid[(size_t)j]];
+    for (int c = 0; c < 4; ++c) P.quartets[(size_t)(4 * i + c)] = hq0[4 * j + c];
+    P.offsets[(size_t)i] = ho0[j];
+    P.pqoff[(size_t)i] = npq;
+    npq += k.nab * k.ncd;
+    if (!k.thin) {
+      P.rowoff[(size_t)i] = nrow;
+      P.npab[(size_t)i] = (int)k.nab;
+      nrow += k.nab * k.ncd * row_pitch(k.la + k.lb + k.lc + k.ld + (cls == 5 ? 2 : 0));
+    }
+    P.tfirst[(size_t)i] = (int64_t)P.tasks.size();
+    for (int sp = 0; sp < k.pl.nsplit; ++sp) P.tasks.push_back(CTask{(int32_t)i, (int16_t)sp, (int16_t)k.pl.nsplit});
+  }
+  P.pqoff[(size_t)n] = npq;
+  P.rowoff[(size_t)P.nthin] = nrow;
+  P.tfirst[(size_t)n] = (int64_t)P.tasks.size();
   return F12INT_OK;
 }
+
+// Device arrays that a planned list runs with.
+struct ListBufs {
+  const int32_t *quartets;
+  const int64_t *offsets, *pqoff, *rowoff;
+  const CTask *tasks;
+  int *keys;
+  unsigned *order, *hist;
+  double *part, *rows;
+  int64_t keys_cap, part_cap, rows_cap;   // ints, doubles, doubles
+  int64_t part_thin;                      // doubles of D.part when no rows are in use
+  int pitch = 0;                          // > 0: every row takes so many doubles (rowoff unused)
+};
+
+// Queue the list's kernels on st: the thin contraction, and chunk by chunk of
+// the general one the auxiliary functions, the Hermite rows and the
+// contraction.  F12INT_ENOMEM when the buffers do not hold one
+// bra primitive pair of a general quartet, or one thin quartet.
+static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, const PairView &PV, const GridView &G,
+                       int cls, double *out_dev, cudaStream_t st, bool timing) {
+  const int nf = ctx->tables.nfam[cls == 5 ? 3 : cls];
+  QuartetView QV{D.quartets, D.pqoff, P.n, nullptr, nullptr, nullptr, nullptr};
+  const bool direct = G.direct();
+  unsigned long long *fma_aux = timing ? ctx->d_fma : nullptr, *fma_con = timing ? ctx->d_fma + 1 : nullptr;
+  std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
+  auto time_begin = [&] {
+    if (!timing) return;
+    ev = take_events(ctx);
+    cudaEventRecord(ev.first, st);
+  };
+  auto time_end = [&](bool aux) {
+    if (!timing) return;
+    cudaEventRecord(ev.second, st);
+    (aux ? ctx->ev_aux : ctx->ev_con).push_back(ev);
+    (aux ? ctx->aux_launches : ctx->contract_launches)++;
+  };
+  // the independent launches go round the side streams, between fork and join
+  int used = 0, next = 0;
+  auto fork = [&] {
+    used = next = 0;
+    return cudaEventRecord(ctx->fork, st) == cudaSuccess;
+  };
+  auto side = [&]() -> cudaStream_t {
+    const int i = next++ % NSIDE;
+    if (i >= used) {
+      cudaStreamWaitEvent(ctx->side[i], ctx->fork, 0);
+      used = i + 1;
+    }
+    return ctx->side[i];
+  };
+  auto join = [&] {
+    for (int i = 0; i < used; ++i) {
+      cudaEventRecord(ctx->join[i], ctx->side[i]);
+      cudaStreamWaitEvent(st, ctx->join[i], 0);
+    }
+  };
+  // items of the primitive quartets [pq0, pq1), family by family, into D.part
+  auto items = [&](int64_t pq0, int64_t pq1) -> int {
+    const int64_t nitems = (pq1 - pq0) * nf;
+    CK(cudaMemsetAsync(D.hist, 0, sizeof(unsigned) * kNKeys, st));
+    const unsigned nb = (unsigned)((nitems + BLOCK_AUX - 1) / BLOCK_AUX);
+    const unsigned nbq = (unsigned)((pq1 - pq0 + BLOCK_AUX - 1) / BLOCK_AUX);
+    k_items_classify<false><<<nbq, BLOCK_AUX, 0, st>>>(ctx->tables, PV, QV, cls, pq0, nitems, D.keys, D.hist);
+    k_items_scan<<<1, 1024, 0, st>>>(D.hist, kNKeys);
+    k_items_scatter<<<nb, BLOCK_AUX, 0, st>>>(QV, nf, pq0, D.keys, D.hist, nitems, D.order);
+    time_begin();
+    k_items_eval<false><<<nb, BLOCK_AUX, 0, st>>>(ctx->tables, PV, QV, cls, pq0, nitems, D.order, D.keys, D.part,
+                                                  ctx->d_status, fma_aux);
+    if (ctx->cls_quad[cls]) {
+      k_items_eval<false, true><<<nb, BLOCK_AUX, 0, st>>>(ctx->tables, PV, QV, cls, pq0, nitems, D.order, D.keys,
+                                                          D.part, ctx->d_status, fma_aux);
+      ctx->launches++;
+    }
+    time_end(true);
+    ctx->launches += 4;
+    CK(cudaGetLastError());
+    return F12INT_OK;
+  };
+  // thin quartets [qa, qb) of the list; pq0: the first primitive quartet of D.part
+  auto thin = [&](int64_t qa, int64_t qb, int64_t pq0) -> int {
+    for (const ListPlan::Group &g : P.groups) {
+      const int64_t a = std::max(qa, g.first), b = std::min(qb, g.end);
+      if (g.thin < 0 || a >= b) continue;
+      const ThinKernel kern = thin_kernel(g.thin, cls == 5);
+      if (!kern) return F12INT_EINVAL;
+      const int64_t nt = b - a;   // one task each
+      kern<<<(unsigned)((nt + kThinWarps - 1) / kThinWarps), 32 * kThinWarps, 0, side()>>>(
+          PV, QV, direct ? 1 : nf, pq0, G, D.tasks + P.tfirst[(size_t)a], nt, nullptr, D.keys, D.part, out_dev,
+          D.offsets, fma_con);
+      ctx->launches++;
+      CK(cudaGetLastError());
+    }
+    return F12INT_OK;
+  };
+  // general quartets [qa, qb), bra primitive pairs [i0, i1) (-1: all); row0: the
+  // first double of D.rows
+  auto general = [&](int64_t qa, int64_t qb, int64_t pq0, int64_t row0, int i0, int i1) -> int {
+    for (const ListPlan::Group &g : P.groups) {
+      const int64_t a = std::max(qa, g.first), b = std::min(qb, g.end);
+      if (g.thin >= 0 || a >= b) continue;
+      const int64_t t0 = P.tfirst[(size_t)a], nt = P.tfirst[(size_t)b] - t0;
+      const auto kern = g.fp32 ? k_contract<false, float> : k_contract<false, double>;
+      if (g.smem > 48 * 1024)
+        CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+      kern<<<(unsigned)nt, g.nthr, g.smem, side()>>>(PV, QV, cls, direct ? 1 : nf, pq0, D.tasks + t0, nt, nullptr,
+                                                     D.keys, RowView{D.rows, D.rowoff, row0, D.pitch}, out_dev,
+                                                     D.offsets, i0, i1, fma_con);
+      ctx->launches++;
+      CK(cudaGetLastError());
+    }
+    return F12INT_OK;
+  };
+  auto hermite = [&](int64_t pq0, int64_t pq1, int64_t row0, int64_t part0) -> int {
+    const unsigned nb = (unsigned)((pq1 - pq0 + BLOCK_AUX - 1) / BLOCK_AUX);
+    if (direct) {
+      time_begin();
+      k_hermite_rows<false, true><<<nb, BLOCK_AUX, 0, st>>>(G, PV, QV, cls, 1, pq0, pq1 - pq0, D.keys, nullptr,
+                                                            RowView{D.rows, D.rowoff, row0, D.pitch}, fma_aux);
+      time_end(true);
+    } else {
+      k_hermite_rows<false, false><<<nb, BLOCK_AUX, 0, st>>>(G, PV, QV, cls, nf, pq0, pq1 - pq0,
+                                                             D.keys + (pq0 - part0) * nf,
+                                                             D.part + (pq0 - part0) * nf * kPartPitch,
+                                                             RowView{D.rows, D.rowoff, row0, D.pitch}, nullptr);
+    }
+    ctx->launches++;
+    CK(cudaGetLastError());
+    return F12INT_OK;
+  };
+  int rc = F12INT_OK;
+  if (direct) {
+    // the thin contraction needs none of the rows: it runs beside them
+    if (P.nthin < P.n) {
+      if (!fork()) return F12INT_ECUDA;
+      time_begin();
+      rc = thin(P.nthin, P.n, 0);
+      if (P.nthin == 0 || timing) join();
+      time_end(false);
+      if (rc != F12INT_OK) return rc;
+    }
+  }
+  const int thin_used = used;   // side streams that still carry thin launches
+  // first double of the rows of primitive quartet pq (of quartet q) in the list's order
+  auto row_of = [&](int64_t q, int64_t pq) -> int64_t {
+    if (D.pitch) return pq * D.pitch;
+    const int64_t npq = P.pqoff[(size_t)q + 1] - P.pqoff[(size_t)q];
+    return npq ? P.rowoff[(size_t)q] + (P.rowoff[(size_t)q + 1] - P.rowoff[(size_t)q]) / npq * (pq - P.pqoff[(size_t)q])
+               : P.rowoff[(size_t)q];
+  };
+  auto row_end = [&](int64_t q) -> int64_t { return D.pitch ? P.pqoff[(size_t)q + 1] * D.pitch : P.rowoff[(size_t)q + 1]; };
+  const int64_t per_pq = (int64_t)std::max(nf, 1) * kPartPitch;
+  const int64_t fit = direct ? (int64_t)1 << 60 : D.part_cap / per_pq;          // primitive quartets whose items fit
+  int64_t part0 = 0, part1 = 0;   // family path: primitive quartets whose items are in D.part
+  for (int64_t qa = 0; qa < P.nthin && rc == F12INT_OK;) {
+    const int64_t pq0 = P.pqoff[(size_t)qa], npq = P.pqoff[(size_t)qa + 1] - pq0, row0 = row_of(qa, pq0);
+    const bool fits = row_end(qa) - row0 <= D.rows_cap && npq <= fit && (!direct || npq <= D.keys_cap);
+    if (fits) {
+      if (!direct && pq0 >= part1) {   // items of as many quartets as fit
+        int64_t qe = qa + 1;
+        while (qe < P.nthin && P.pqoff[(size_t)qe + 1] - pq0 <= fit) ++qe;
+        part0 = pq0;
+        part1 = P.pqoff[(size_t)qe];
+        rc = items(part0, part1);
+        if (rc != F12INT_OK) break;
+      }
+      int64_t qb = qa + 1;
+      while (qb < P.nthin && row_end(qb) - row0 <= D.rows_cap &&
+             (direct ? P.pqoff[(size_t)qb + 1] - pq0 <= D.keys_cap : P.pqoff[(size_t)qb + 1] <= part1))
+        ++qb;
+      rc = hermite(pq0, P.pqoff[(size_t)qb], row0, part0);
+      if (rc == F12INT_OK && !fork()) rc = F12INT_ECUDA;
+      if (rc != F12INT_OK) break;
+      time_begin();
+      rc = general(qa, qb, direct ? pq0 : part0, row0, -1, -1);
+      join();
+      time_end(false);
+      qa = qb;
+      continue;
+    }
+    // one quartet larger than the scratch: a few of its bra primitive pairs at a time
+    const int npab = P.npab[(size_t)qa];
+    const int64_t npcd = npq / npab, per = (row_end(qa) - row0) / npab;   // doubles of one bra pair's rows
+    int64_t step = std::min<int64_t>(D.rows_cap / per, fit / npcd);
+    if (direct) step = std::min<int64_t>(step, D.keys_cap / npcd);
+    if (step < 1) return F12INT_ENOMEM;
+    for (int64_t i0 = 0; i0 < npab && rc == F12INT_OK; i0 += step) {
+      const int64_t i1 = std::min<int64_t>(npab, i0 + step), a = pq0 + i0 * npcd, b = pq0 + i1 * npcd;
+      if (!direct) rc = items(a, b);
+      if (rc == F12INT_OK) rc = hermite(a, b, row0 + i0 * per, a);
+      if (rc == F12INT_OK && !fork()) rc = F12INT_ECUDA;
+      if (rc != F12INT_OK) break;
+      time_begin();
+      rc = general(qa, qa + 1, a, row0 + i0 * per, (int)i0, (int)i1);
+      join();
+      time_end(false);
+    }
+    part1 = 0;
+    ++qa;
+  }
+  for (int64_t qa = P.nthin; !direct && qa < P.n && rc == F12INT_OK;) {   // family path: the thin quartets
+    const int64_t pq0 = P.pqoff[(size_t)qa], most = D.part_thin / per_pq;
+    int64_t qb = qa + 1;
+    while (qb < P.n && P.pqoff[(size_t)qb + 1] - pq0 <= most) ++qb;
+    if (P.pqoff[(size_t)qb] - pq0 > most) return F12INT_ENOMEM;
+    rc = items(pq0, P.pqoff[(size_t)qb]);
+    if (rc == F12INT_OK && !fork()) rc = F12INT_ECUDA;
+    if (rc != F12INT_OK) break;
+    time_begin();
+    rc = thin(qa, qb, pq0);
+    join();
+    time_end(false);
+    qa = qb;
+  }
+  if (direct && P.nthin > 0 && P.nthin < P.n && !timing) {
+    used = std::max(used, thin_used);
+    join();
+  }
+  return rc;
+}
+
+extern "C" {
 
 // Primitive Schwarz factors Q_ab = sqrt(max |(ab|k|ab)|) of every primitive
 // pair of the basis for class cls (the I3 kernel for I5), from the diagonal
@@ -2028,159 +1781,81 @@ static int compute_class_impl(f12int_ctx *ctx, int basis_id, int cls, const int3
   NvtxRange call_range("f12int.compute_class");
   const auto t_plan0 = std::chrono::steady_clock::now();
   std::unique_ptr<NvtxRange> plan_range(new NvtxRange("f12int.plan"));
-  // quartet metadata: order by (la, lb, lc, ld), primitive-quartet offsets
   std::vector<int32_t> hq0((size_t)4 * n);
   std::vector<int64_t> ho0((size_t)n);
   CK(cudaMemcpyAsync(hq0.data(), quartets_dev, sizeof(int32_t) * 4 * n, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(ho0.data(), offsets_dev, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  const int ns = B.nshell;
-  std::vector<int> key0((size_t)n);
+  ListPlan P;
+  // mixed path: FP32 Hermite recursion and contraction below the bound
+  int rc = plan_list(B, cls, n, hq0.data(), ho0.data(), [&](const int32_t *s) {
+    return fp32_below > 0.0 && screen_estimate(ctx, B, cls, s[0], s[1], s[2], s[3]) < fp32_below ? 1 : 0;
+  }, P);
+  if (rc != F12INT_OK) return rc;
+  const GridView G = grid_view(ctx, B, cls);
+  const int64_t nf = std::max(1, ctx->tables.nfam[cls == 5 ? 3 : cls]);
+  const int64_t npq = P.pqoff[(size_t)n], npq_gen = P.pqoff[(size_t)P.nthin];
+  int64_t big_pq = 1, big_thin = 1, big_row = 1;   // largest quartet, thin quartet, bra pair's rows
   for (int64_t i = 0; i < n; ++i) {
-    const int32_t *s = &hq0[4 * i];
-    for (int k = 0; k < 4; ++k)
-      if (s[k] < 0 || s[k] >= ns) return F12INT_EINVAL;
-    key0[i] = (B.l[s[0]] << 6) | (B.l[s[1]] << 4) | (B.l[s[2]] << 2) | B.l[s[3]];
-  }
-  // Every quartet with the same (primitive quartets, FP32 or not, class key)
-  // has the same plan: the distinct ones ("plan groups") are planned once,
-  // ordered -- FP64 first, decreasing shared-memory need (a tier launches
-  // with the need of its first quartet, so no later one may need more),
-  // decreasing work per task (the longest blocks start first), class key --
-  // and the quartets are placed group by group in their list order (a
-  // counting sort: linear in n).
-  struct PlanGroup {
-    ContractPlan pl;
-    double work;
-    int64_t key;
-    int64_t count, first;
-    bool thin;   // contracted by k_contract_thin
-  };
-  std::vector<PlanGroup> groups;
-  std::vector<int32_t> gid((size_t)n);
-  {
-    // open-addressing map from the group key to its index
-    std::vector<int64_t> slot_key(4096, -1);
-    std::vector<int32_t> slot_val(4096, -1);
-    size_t mask = slot_key.size() - 1;
-    const std::vector<double> *pb = fp32_below > 0.0 ? &B.pair_bound[cls == 5 ? 3 : cls] : nullptr;
-    for (int64_t i = 0; i < n; ++i) {
-      const int k = key0[i];
-      const int32_t *s = &hq0[4 * i];
-      const int64_t np = (int64_t)B.nprim[s[0]] * B.nprim[s[1]] * B.nprim[s[2]] * B.nprim[s[3]];
-      // mixed path: FP32 Hermite recursion and contraction below the bound
-      const int f32 = (pb && screen_estimate(ctx, B, cls, s[0], s[1], s[2], s[3]) < fp32_below) ? 1 : 0;
-      const int64_t gk = (np << 9) | (f32 << 8) | k;
-      size_t h = (size_t)((uint64_t)gk * 0x9E3779B97F4A7C15ull >> 40) & mask;
-      while (slot_key[h] != -1 && slot_key[h] != gk) h = (h + 1) & mask;
-      if (slot_key[h] == -1) {
-        if (groups.size() * 2 >= slot_key.size()) {   // grow and rehash
-          std::vector<int64_t> nk(slot_key.size() * 2, -1);
-          std::vector<int32_t> nv(slot_key.size() * 2, -1);
-          const size_t nm = nk.size() - 1;
-          for (size_t t = 0; t < slot_key.size(); ++t)
-            if (slot_key[t] != -1) {
-              size_t g = (size_t)((uint64_t)slot_key[t] * 0x9E3779B97F4A7C15ull >> 40) & nm;
-              while (nk[g] != -1) g = (g + 1) & nm;
-              nk[g] = slot_key[t];
-              nv[g] = slot_val[t];
-            }
-          slot_key.swap(nk);
-          slot_val.swap(nv);
-          mask = nm;
-          h = (size_t)((uint64_t)gk * 0x9E3779B97F4A7C15ull >> 40) & mask;
-          while (slot_key[h] != -1 && slot_key[h] != gk) h = (h + 1) & mask;
-        }
-        const int la = (k >> 6) & 3, lb = (k >> 4) & 3, lc = (k >> 2) & 3, ld = k & 3;
-        PlanGroup g{};
-        g.pl = contract_plan(la, lb, lc, ld, cls, np, f32 ? 4 : 8);
-        if (g.pl.smem == 0) return F12INT_EINVAL;
-        g.thin = thin_quartet(k, cls);
-        if (g.thin) g.pl = ContractPlan{1, 1, 0};   // one warp of the thin kernel, no shared memory
-        const int ncd = ncart(lc) * ncart(ld);
-        g.work = (double)np * task_flops(la, lb, lc, ld, cls, (ncd + g.pl.nsplit - 1) / g.pl.nsplit);
-        g.key = gk;
-        slot_key[h] = gk;
-        slot_val[h] = (int32_t)groups.size();
-        groups.push_back(g);
-      }
-      const int32_t g = slot_val[h];
-      gid[i] = g;
-      groups[g].count++;
+    const int64_t k = P.pqoff[(size_t)i + 1] - P.pqoff[(size_t)i];
+    if (i < P.nthin) {
+      big_pq = std::max(big_pq, k);
+      big_row = std::max(big_row, (P.rowoff[(size_t)i + 1] - P.rowoff[(size_t)i]) / P.npab[(size_t)i]);
+    } else {
+      big_thin = std::max(big_thin, k);
     }
   }
-  {
-    std::vector<int32_t> order(groups.size());
-    for (size_t g = 0; g < groups.size(); ++g) order[g] = (int32_t)g;
-    std::sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
-      const PlanGroup &A = groups[x], &Bg = groups[y];
-      if (A.thin != Bg.thin) return Bg.thin;   // the thin quartets last, by class key
-      if (A.thin) return (A.key & 0xFF) < (Bg.key & 0xFF) || ((A.key & 0xFF) == (Bg.key & 0xFF) && A.key < Bg.key);
-      const int fa = (int)((A.key >> 8) & 1), fb = (int)((Bg.key >> 8) & 1);
-      if (fa != fb) return fa < fb;
-      if (A.pl.smem != Bg.pl.smem) return A.pl.smem > Bg.pl.smem;
-      if (A.work != Bg.work) return A.work > Bg.work;
-      return (A.key & 0xFF) < (Bg.key & 0xFF) || ((A.key & 0xFF) == (Bg.key & 0xFF) && A.key < Bg.key);
-    });
-    int64_t run = 0;
-    for (int32_t g : order) {
-      groups[g].first = run;
-      run += groups[g].count;
-    }
-  }
-  std::vector<int64_t> perm((size_t)n);
-  for (int64_t i = 0; i < n; ++i) perm[groups[gid[i]].first++] = i;
-  std::vector<int32_t> hq((size_t)4 * n);
-  std::vector<int64_t> ho((size_t)n);
-  ctx->h_nw.resize((size_t)n);
-  ctx->h_split.resize((size_t)n);
-  ctx->h_smem.resize((size_t)n);
-  ctx->h_fp32.resize((size_t)n);
-  ctx->h_thin.resize((size_t)n);
-  for (int64_t i = 0; i < n; ++i) {
-    const int64_t j = perm[i];
-    for (int k = 0; k < 4; ++k) hq[4 * i + k] = hq0[4 * j + k];
-    ho[i] = ho0[j];
-    const PlanGroup &g = groups[gid[j]];
-    ctx->h_nw[i] = g.pl.nw;
-    ctx->h_split[i] = g.pl.nsplit;
-    ctx->h_smem[i] = g.pl.smem;
-    ctx->h_fp32[i] = (char)(g.thin ? 0 : (g.key >> 8) & 1);   // the thin kernel is FP64
-    ctx->h_thin[i] = g.thin ? (int16_t)(g.key & 0xFF) : (int16_t)-1;
-  }
-  std::vector<int64_t> pqoff((size_t)n + 1);
-  int64_t npq = 0;
-  size_t smem = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    const int32_t *s = &hq[4 * i];
-    pqoff[i] = npq;
-    npq += (int64_t)B.nprim[s[0]] * B.nprim[s[1]] * B.nprim[s[2]] * B.nprim[s[3]];
-    smem = std::max(smem, ctx->h_smem[i]);
-  }
-  pqoff[n] = npq;
-  if (smem > 227 * 1024) return F12INT_EINVAL;
-  int rc = ensure_buf(ctx, (void **)&ctx->d_pqoff, &ctx->pqoff_cap, sizeof(int64_t) * ((size_t)n + 1));
+  rc = ensure_buf(ctx, (void **)&ctx->d_pqoff, &ctx->pqoff_cap, sizeof(int64_t) * ((size_t)n + 1));
   if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_qperm, &ctx->qperm_cap, sizeof(int32_t) * 4 * n);
   if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_operm, &ctx->operm_cap, sizeof(int64_t) * n);
+  if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_rowoff, &ctx->rowoff_cap, sizeof(int64_t) * P.rowoff.size());
+  if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_tasks, &ctx->tasks_cap, sizeof(CTask) * P.tasks.size());
   if (rc != F12INT_OK) return rc;
-  CK(cudaMemcpyAsync(ctx->d_pqoff, pqoff.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(ctx->d_qperm, hq.data(), sizeof(int32_t) * 4 * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(ctx->d_operm, ho.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-  const int kcls = cls == 5 ? 3 : cls;
-  const int64_t nf = ctx->tables.nfam[kcls];
-  const int64_t pq_chunk = std::max<int64_t>(1, kItemChunk / std::max<int64_t>(nf, 1));
+  ListBufs D{ctx->d_qperm, ctx->d_operm, ctx->d_pqoff, ctx->d_rowoff, ctx->d_tasks};
+  // scratch of one chunk: Hermite rows to kRowChunk doubles, on the family path
+  // also the items; under a budget no more than an item per family would take
+  const int64_t all_rows = P.rowoff[(size_t)P.nthin];
+  if (G.direct()) {
+    int64_t want = std::min(all_rows, kRowChunk);
+    if (ctx->budget) want = std::min(want, npq * nf * 17);
+    D.rows_cap = std::max(want, all_rows ? big_row : 0);
+    D.keys_cap = std::min(npq_gen, std::max(D.rows_cap / 36 + 1, big_pq));
+  } else {
+    D.part_cap = std::min(npq, std::max(std::max(big_pq, big_thin), kItemChunk / nf)) * nf * kPartPitch;
+    D.part_thin = D.part_cap;
+    D.keys_cap = D.part_cap / kPartPitch;
+    D.rows_cap = std::max(std::min(all_rows, kRowChunk / 4), all_rows ? big_row : 0);
+    rc = ensure_buf(ctx, (void **)&ctx->d_order, &ctx->order_cap, sizeof(unsigned) * (size_t)D.keys_cap);
+    if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_part, &ctx->part_cap, sizeof(double) * (size_t)D.part_cap);
+    if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_hist, &ctx->hist_cap, sizeof(unsigned) * kNKeys);
+  }
+  if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_keys, &ctx->keys_cap, sizeof(int) * (size_t)D.keys_cap);
+  if (rc == F12INT_OK) {
+    rc = ensure_buf(ctx, (void **)&ctx->d_rows, &ctx->rows_cap, sizeof(double) * (size_t)D.rows_cap);
+    while (rc == F12INT_ENOMEM && !G.direct() && D.rows_cap > big_row) {   // the family path's rows take what is left
+      D.rows_cap = std::max(big_row, D.rows_cap / 4);
+      rc = ensure_buf(ctx, (void **)&ctx->d_rows, &ctx->rows_cap, sizeof(double) * (size_t)D.rows_cap);
+    }
+  }
+  if (rc != F12INT_OK) return rc;
+  D.keys = ctx->d_keys;
+  D.order = ctx->d_order;
+  D.hist = ctx->d_hist;
+  D.part = ctx->d_part;
+  D.rows = ctx->d_rows;
+  CK(cudaMemcpyAsync(ctx->d_pqoff, P.pqoff.data(), sizeof(int64_t) * P.pqoff.size(), cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(ctx->d_qperm, P.quartets.data(), sizeof(int32_t) * 4 * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(ctx->d_operm, P.offsets.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(ctx->d_rowoff, P.rowoff.data(), sizeof(int64_t) * P.rowoff.size(), cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(ctx->d_tasks, P.tasks.data(), sizeof(CTask) * P.tasks.size(), cudaMemcpyHostToDevice, st));
   plan_range.reset();
   ctx->plan_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_plan0).count();
   ctx->plan_calls++;
-  const bool gridded = grid_view(ctx, B, cls).direct();
-  for (int64_t qa = 0; qa < n;) {
-    int64_t qb = qa + 1;
-    // (with the grid the thin quartets, last in the order, need no scratch)
-    while (qb < n && (pqoff[qb + 1] - pqoff[qa] <= pq_chunk || (gridded && ctx->h_thin[qb] >= 0))) ++qb;
-    rc = launch_chunk(ctx, B, cls, ctx->d_qperm, ctx->d_pqoff, pqoff.data(), n, qa, qb, pqoff[qa], pqoff[qb], smem, out_dev,
-                      ctx->d_operm, st, prim_screen);
-    if (rc != F12INT_OK) return rc;
-    qa = qb;
+  rc = launch_list(ctx, P, D, pair_view(ctx, B, cls, B.prim_screen && prim_screen), G, cls, out_dev, st, ctx->timing);
+  if (rc != F12INT_OK) {
+    cudaStreamSynchronize(st);   // the queued copies read this call's vectors
+    for (cudaStream_t t : ctx->side) cudaStreamSynchronize(t);
+    return rc;
   }
   // keep the host buffer alive until the copy has been consumed
   CK(cudaStreamSynchronize(st));
@@ -2402,165 +2077,86 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
   CK(cudaMemcpyAsync(hq0.data(), quartets_dev, sizeof(int32_t) * 4 * n, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(ho0.data(), offsets_dev, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  const int ns = B.nshell;
-  std::vector<size_t> sm0((size_t)n);
-  std::vector<int> nw0((size_t)n), sp0((size_t)n), key0((size_t)n);
-  for (int64_t i = 0; i < n; ++i) {
-    const int32_t *s = &hq0[4 * i];
-    for (int k = 0; k < 4; ++k)
-      if (s[k] < 0 || s[k] >= ns) return F12INT_EINVAL;
-    key0[i] = (B.l[s[0]] << 6) | (B.l[s[1]] << 4) | (B.l[s[2]] << 2) | B.l[s[3]];
-    const ContractPlan pl = contract_plan(B.l[s[0]], B.l[s[1]], B.l[s[2]], B.l[s[3]], cls,
-                                          (int64_t)B.nprim[s[0]] * B.nprim[s[1]] * B.nprim[s[2]] * B.nprim[s[3]]);
-    if (pl.smem == 0 || pl.smem > 227 * 1024) return F12INT_EINVAL;
-    nw0[i] = pl.nw;
-    sp0[i] = pl.nsplit;
-    sm0[i] = pl.smem;
-    if (thin_quartet(key0[i], cls)) {   // k_contract_thin: sorted last (no shared memory), by key
-      nw0[i] = 1;
-      sp0[i] = 1;
-      sm0[i] = 0;
-    }
-  }
-  std::vector<int64_t> perm((size_t)n);
-  for (int64_t i = 0; i < n; ++i) perm[i] = i;
-  std::stable_sort(perm.begin(), perm.end(), [&](int64_t x, int64_t y) {
-    if (sm0[x] != sm0[y]) return sm0[x] > sm0[y];
-    return key0[x] < key0[y];
-  });
-  std::vector<int32_t> hq((size_t)4 * n);
-  std::vector<int64_t> ho((size_t)n), pqoff((size_t)n + 1);
-  std::vector<int> hnw((size_t)n), hsp((size_t)n);
-  std::vector<size_t> hsm((size_t)n);
-  int64_t npq = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    for (int k = 0; k < 4; ++k) hq[4 * i + k] = hq0[4 * perm[i] + k];
-    ho[i] = ho0[perm[i]];
-    hnw[i] = nw0[perm[i]];
-    hsp[i] = sp0[perm[i]];
-    hsm[i] = sm0[perm[i]];
-    const int32_t *s = &hq[4 * i];
-    pqoff[i] = npq;
-    npq += (int64_t)B.nprim[s[0]] * B.nprim[s[1]] * B.nprim[s[2]] * B.nprim[s[3]];
-  }
-  pqoff[n] = npq;
-  // contraction tasks (one per quartet and ket range), then the work items
-  std::vector<CTask> tasks;
-  for (int64_t i = 0; i < n; ++i)
-    for (int sp = 0; sp < hsp[i]; ++sp) tasks.push_back(CTask{(int32_t)i, (int16_t)sp, (int16_t)hsp[i]});
-  std::vector<int64_t> tfirst((size_t)n + 1, 0);
-  for (int64_t i = 0; i < n; ++i) tfirst[i + 1] = tfirst[i] + hsp[i];
+  ListPlan P;
+  auto fp64 = [](const int32_t *) { return 0; };
+  rc = plan_list(B, cls, n, hq0.data(), ho0.data(), fp64, P);
+  if (rc != F12INT_OK) return rc;
   // layout of the array: quartets, offsets and primitive offsets in the
   // working order, the key histogram and the task list (all sized exactly
-  // now), then the work items of one chunk.  Every size check happens here,
+  // now), then the scratch of one chunk.  Every size check happens here,
   // before anything is queued, so that an F12INT_EINVAL leaves the array and
   // the output untouched.
+  auto fixed_bytes = [&] {
+    return align256(sizeof(int32_t) * 4 * (size_t)n) + align256(sizeof(int64_t) * (size_t)n) +
+           align256(sizeof(int64_t) * ((size_t)n + 1)) + align256(sizeof(unsigned) * kNKeys) +
+           align256(sizeof(CTask) * P.tasks.size());
+  };
+  // one chunk at least: the items of every quartet on its own, and the rows of
+  // one of its bra primitive pairs
+  const int64_t nf = std::max(1, ctx->tables.nfam[cls == 5 ? 3 : cls]);
+  const GridView G = grid_view(ctx, B, cls);
+  int64_t big_pq = 1, pitch = 4, big_cd = 1;
+  for (int64_t i = 0; i < n; ++i) {
+    const int64_t k = P.pqoff[(size_t)i + 1] - P.pqoff[(size_t)i];
+    big_pq = std::max(big_pq, k);
+    if (i < P.nthin && k > 0) {
+      big_cd = std::max(big_cd, k / P.npab[(size_t)i]);
+      pitch = std::max(pitch, (P.rowoff[(size_t)i + 1] - P.rowoff[(size_t)i]) / k);
+    }
+  }
+  auto room = [&]() -> int64_t {   // bytes of the chunk's scratch, negative when the list does not fit
+    return (int64_t)F12INT_STATIC_SCRATCH_BYTES - (int64_t)fixed_bytes() - 4 * 256;
+  };
+  auto enough = [&] {
+    const int64_t r = room();
+    return r >= big_pq * nf * (int64_t)item_bytes && r >= big_cd * (nf * (int64_t)item_bytes + pitch * 8 + 64);
+  };
+  if (!enough()) {   // fewer and longer tasks leave more of the array
+    rc = plan_list(B, cls, n, hq0.data(), ho0.data(), fp64, P, /*fewest=*/true);
+    if (rc != F12INT_OK) return rc;
+    if (!enough()) return F12INT_EINVAL;
+  }
   int32_t *d_q = (int32_t *)base;
   int64_t *d_o = (int64_t *)(base + align256(sizeof(int32_t) * 4 * (size_t)n));
   int64_t *d_pq = (int64_t *)((unsigned char *)d_o + align256(sizeof(int64_t) * (size_t)n));
   unsigned *d_hist = (unsigned *)((unsigned char *)d_pq + align256(sizeof(int64_t) * ((size_t)n + 1)));
   CTask *d_tk = (CTask *)((unsigned char *)d_hist + align256(sizeof(unsigned) * kNKeys));
-  unsigned char *items_base = (unsigned char *)d_tk + align256(sizeof(CTask) * tasks.size());
-  const size_t used_fixed = (size_t)(items_base - base);
-  if (used_fixed + 3 * 256 + item_bytes > F12INT_STATIC_SCRATCH_BYTES) return F12INT_EINVAL;
-  const int64_t max_items = (int64_t)((F12INT_STATIC_SCRATCH_BYTES - used_fixed - 3 * 256) / item_bytes);
-  const int kcls = cls == 5 ? 3 : cls;
-  const int nf = ctx->tables.nfam[kcls];
-  const int64_t pq_chunk = std::max<int64_t>(1, max_items / std::max(nf, 1));
-  for (int64_t i = 0; i < n; ++i)
-    if (pqoff[i + 1] - pqoff[i] > pq_chunk) return F12INT_EINVAL;   // one quartet larger than the scratch
-  CK(cudaMemcpyAsync(d_tk, tasks.data(), sizeof(CTask) * tasks.size(), cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(d_q, hq.data(), sizeof(int32_t) * 4 * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(d_o, ho.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(d_pq, pqoff.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
-
+  unsigned char *scratch = (unsigned char *)d_tk + align256(sizeof(CTask) * P.tasks.size());
+  ListBufs D{d_q, d_o, d_pq, nullptr, d_tk};
+  D.pitch = (int)pitch;
+  D.hist = d_hist;
+  D.keys = (int *)scratch;
+  const int64_t r = room();
+  if (G.direct()) {
+    const int64_t rows = r / (int64_t)(sizeof(int) + sizeof(double) * (size_t)pitch);   // primitive quartets
+    D.keys_cap = rows;
+    D.rows = (double *)(scratch + align256(sizeof(int) * (size_t)rows));
+    D.rows_cap = rows * pitch;
+  } else {
+    // items over the whole of it for the thin quartets; the general ones leave
+    // its end to the rows (a quarter, or one bra pair's)
+    const int64_t items = r / (int64_t)item_bytes;
+    D.keys_cap = items;
+    D.order = (unsigned *)(scratch + align256(sizeof(int) * (size_t)items));
+    D.part = (double *)((unsigned char *)D.order + align256(sizeof(unsigned) * (size_t)items));
+    D.part_thin = items * kPartPitch;
+    D.rows_cap = std::max(items * kPartPitch / 4, big_cd * pitch) & ~(int64_t)3;
+    D.part_cap = (D.part_thin - D.rows_cap) & ~(int64_t)15;
+    D.rows = D.part + D.part_cap;
+  }
+  CK(cudaMemcpyAsync(d_tk, P.tasks.data(), sizeof(CTask) * P.tasks.size(), cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(d_q, P.quartets.data(), sizeof(int32_t) * 4 * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(d_o, P.offsets.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(d_pq, P.pqoff.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
   // the primitive screen of f12int_compute_class when its table for this
   // (basis, class) exists already (building it would allocate); without it
   // every primitive quartet is evaluated
-  PairView PV = pair_view(ctx, B, cls, B.prim_screen);
-  QuartetView QV{d_q, d_pq, n, nullptr, nullptr, nullptr, nullptr};
-  const GridView G = grid_view(ctx, B, cls);
-  const int nfk = G.direct() ? 1 : nf;   // rows per primitive quartet
-  int rc_launch = F12INT_OK;
-  for (int64_t qa = 0; qa < n && rc_launch == F12INT_OK;) {
-    int64_t qb = qa + 1;
-    while (qb < n && pqoff[qb + 1] - pqoff[qa] <= pq_chunk) ++qb;
-    int64_t qthin = qb;   // thin quartets (no shared memory) are last
-    while (qthin > qa && hsm[qthin - 1] == 0) --qthin;
-    const int64_t pqa = pqoff[qa], nitems = G.direct() ? pqoff[qthin] - pqa : (pqoff[qb] - pqa) * nf;
-    int *d_keys = (int *)items_base;
-    unsigned *d_order = (unsigned *)(items_base + align256(sizeof(int) * (size_t)nitems));
-    double *d_part = (double *)((unsigned char *)d_order + align256(sizeof(unsigned) * (size_t)nitems));
-    if (nitems > 0 && G.direct()) {
-      k_direct_rows<false><<<(unsigned)((nitems + BLOCK_AUX - 1) / BLOCK_AUX), BLOCK_AUX, 0, st>>>(
-          G, PV, QV, cls, pqa, nitems, d_keys, d_part, nullptr);
-      ctx->launches++;
-      if (cudaGetLastError() != cudaSuccess) rc_launch = F12INT_ECUDA;
-    } else if (nitems > 0) {
-      // the histogram must start at zero on every call: the array keeps the
-      // previous call's contents
-      if (cudaMemsetAsync(d_hist, 0, sizeof(unsigned) * kNKeys, st) != cudaSuccess) {
-        rc_launch = F12INT_ECUDA;
-        break;
-      }
-      const unsigned nb = (unsigned)((nitems + BLOCK_AUX - 1) / BLOCK_AUX);
-      const unsigned nbq = (unsigned)((pqoff[qb] - pqa + BLOCK_AUX - 1) / BLOCK_AUX);
-      k_items_classify<false><<<nbq, BLOCK_AUX, 0, st>>>(ctx->tables, PV, QV, cls, pqa, nitems, d_keys, d_hist);
-      k_items_scan<<<1, 1024, 0, st>>>(d_hist, kNKeys);
-      k_items_scatter<<<nb, BLOCK_AUX, 0, st>>>(QV, nf, pqa, d_keys, d_hist, nitems, d_order);
-      k_items_eval<false><<<nb, BLOCK_AUX, 0, st>>>(ctx->tables, PV, QV, cls, pqa, nitems, d_order, d_keys, d_part,
-                                                    ctx->d_status, nullptr);
-      ctx->launches += 4;
-      if (ctx->cls_quad[cls]) {
-        k_items_eval<false, true><<<nb, BLOCK_AUX, 0, st>>>(ctx->tables, PV, QV, cls, pqa, nitems, d_order, d_keys,
-                                                            d_part, ctx->d_status, nullptr);
-        ctx->launches++;
-      }
-      if (cudaGetLastError() != cudaSuccess) rc_launch = F12INT_ECUDA;
-    }
-    for (int64_t ra = qa; ra < qb && rc_launch == F12INT_OK;) {
-      const int nwr = hnw[ra];
-      const size_t smr = hsm[ra];
-      int64_t rb = ra + 1;
-      if (smr == 0) {   // thin quartets: one launch per class key
-        const int key = (B.l[hq[4 * ra]] << 6) | (B.l[hq[4 * ra + 1]] << 4) | (B.l[hq[4 * ra + 2]] << 2) |
-                        B.l[hq[4 * ra + 3]];
-        auto key_of = [&](int64_t i) {
-          return (B.l[hq[4 * i]] << 6) | (B.l[hq[4 * i + 1]] << 4) | (B.l[hq[4 * i + 2]] << 2) | B.l[hq[4 * i + 3]];
-        };
-        while (rb < qb && hsm[rb] == 0 && key_of(rb) == key) ++rb;
-        const int64_t nt = tfirst[rb] - tfirst[ra];
-        const ThinKernel kern = thin_kernel(key, cls == 5);
-        if (!kern) {
-          rc_launch = F12INT_EINVAL;
-          break;
-        }
-        kern<<<(unsigned)((nt + kThinWarps - 1) / kThinWarps), 32 * kThinWarps, 0, st>>>(
-            PV, QV, nfk, pqa, G, d_tk + tfirst[ra], nt, nullptr, d_keys, d_part, out_dev, d_o, nullptr);
-        ctx->launches++;
-        if (cudaGetLastError() != cudaSuccess) rc_launch = F12INT_ECUDA;
-        ra = rb;
-        continue;
-      }
-      while (rb < qb && hnw[rb] == nwr && 2 * hsm[rb] > smr) ++rb;
-      const int64_t nt = tfirst[rb] - tfirst[ra];
-      if (smr > 48 * 1024 &&
-          cudaFuncSetAttribute(k_contract<false, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr) !=
-              cudaSuccess) {
-        rc_launch = F12INT_ECUDA;
-        break;
-      }
-      k_contract<false, double><<<(unsigned)nt, 32 * nwr, smr, st>>>(PV, QV, cls, nfk, pqa, d_tk + tfirst[ra], nt, nullptr,
-                                                                     d_keys, d_part, out_dev, d_o, ctx->d_status, nullptr);
-      ctx->launches++;
-      if (cudaGetLastError() != cudaSuccess) rc_launch = F12INT_ECUDA;
-      ra = rb;
-    }
-    qa = qb;
-  }
+  const int rc_launch = launch_list(ctx, P, D, pair_view(ctx, B, cls, B.prim_screen), G, cls, out_dev, st, false);
   // the host vectors above stay alive until the queued copies are consumed,
   // and on an error nothing of this call is still running when it returns
   cudaError_t e = cudaStreamSynchronize(st);
+  if (rc_launch != F12INT_OK)
+    for (cudaStream_t t : ctx->side) cudaStreamSynchronize(t);
   if (rc_launch != F12INT_OK) return rc_launch;
   if (e != cudaSuccess) return cuda_fail(e);
   return F12INT_OK;
