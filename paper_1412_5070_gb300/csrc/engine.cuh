@@ -56,28 +56,32 @@ struct TicketState {
 // and the work of one task.
 struct BatchPlan {
   int tier, nsplit;
+  bool swap;        // listed as (cd|ab), the bra inner
   double work;
 };
 
-static bool batch_plan(int la, int lb, int lc, int ld, int cls, int64_t nprimq, int64_t npcd, double target,
+static bool batch_plan(int la, int lb, int lc, int ld, int cls, int64_t npab, int64_t npcd, double target,
                        BatchPlan *bp, bool fp32 = false) {
-  const ContractShape s{la, lb, lc, ld, cls == 5 ? 2 : 0};
   const int key = (la << 6) | (lb << 4) | (lc << 2) | ld;
+  bp->swap = false;
   if (thin_quartet(key, cls)) {   // one warp, FP64 (mixed requests too)
     bp->tier = kThinSlot + thin_slot(key, cls == 5);
     bp->nsplit = 1;
-    bp->work = (double)nprimq * task_fmas(s, npcd, s.ncd());
+    bp->work = (double)(npab * npcd);
     return true;
   }
+  bp->swap = bra_inner(la, lb, lc, ld, cls, npab, npcd);
+  const ContractShape s = contract_shape(la, lb, lc, ld, cls, bp->swap);
+  const int64_t nprimq = npab * npcd, nin = bp->swap ? npab : npcd;
   const size_t esz = fp32 ? 4 : 8;
-  const ContractPlan pl = contract_plan(la, lb, lc, ld, cls, nprimq, npcd, esz, 0.5 * target);
+  const ContractPlan pl = contract_plan(s, nprimq, nin, esz, 0.5 * target);
   if (pl.smem == 0) return false;
   const size_t least = contract_smem(s, 1, pl.nsplit, esz, 0);
   for (int t = 0; t < kTiers; ++t)
     if (kTierCap[t] >= least && (kTierThreads[t] >= pl.nthr || t == kTiers - 1)) {
       bp->tier = t + (fp32 ? kTiers : 0);
       bp->nsplit = pl.nsplit;
-      bp->work = (double)nprimq * task_fmas(s, npcd, (s.ncd() + pl.nsplit - 1) / pl.nsplit);
+      bp->work = (double)nprimq * task_fmas(s, nin, (s.ncd() + pl.nsplit - 1) / pl.nsplit);
       return true;
     }
   return false;
@@ -487,6 +491,7 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
     int64_t off;
     int64_t npab, npcd, rows;
     int tier, nsplit;
+    bool swap;
     double work;      // per task
   };
   int64_t nzero = 0;
@@ -522,10 +527,11 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
         it.npab = (int64_t)B.nprim[s[0]] * B.nprim[s[1]];
         it.npcd = (int64_t)B.nprim[s[2]] * B.nprim[s[3]];
         it.tier = mixed && est < E.fp32_below ? 1 : 0;   // (the tier proper below)
-        const ContractShape sh{la, lb, lc, ld, cls == 5 ? 2 : 0};
         if (!thin_quartet((la << 6) | (lb << 4) | (lc << 2) | ld, cls)) {
+          it.swap = bra_inner(la, lb, lc, ld, cls, it.npab, it.npcd);
+          const ContractShape sh = contract_shape(la, lb, lc, ld, cls, it.swap);
           it.rows = it.npab * it.npcd * row_pitch(sh.L());
-          total += (double)(it.npab * it.npcd) * task_fmas(sh, it.npcd, sh.ncd());
+          total += (double)(it.npab * it.npcd) * task_fmas(sh, it.swap ? it.npab : it.npcd, sh.ncd());
         }
         items.push_back(it);
       }
@@ -538,8 +544,8 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
         const f12int_ctx::BasisData &B = *batch[(size_t)it.req]->B;
         BatchPlan bp{};
         const bool fp32 = it.tier >= kTiers ? it.tier < 2 * kTiers : false;
-        batch_plan(B.l[it.q[0]], B.l[it.q[1]], B.l[it.q[2]], B.l[it.q[3]], cls, it.npab * it.npcd, it.npcd, target,
-                   &bp, fp32);   // checked at submit
+        batch_plan(B.l[it.q[0]], B.l[it.q[1]], B.l[it.q[2]], B.l[it.q[3]], cls, it.npab, it.npcd, target, &bp,
+                   fp32);   // checked at submit
         it.tier = bp.tier;
         it.nsplit = bp.nsplit;
         it.work = bp.work;
@@ -587,14 +593,15 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
         S.counts[kTaskCounts + 2 * t] = nt;
         for (; i < n && items[i0 + (size_t)i].tier == t; ++i) {
           const Item &it = items[i0 + (size_t)i];
-          for (int k = 0; k < 4; ++k) S.quartets[4 * i + k] = it.q[k];
+          for (int k = 0; k < 4; ++k) S.quartets[4 * i + k] = it.q[it.swap ? k ^ 2 : k];
           S.offsets[i] = it.off;
           S.qslot[i] = it.req;
           S.pq_off[i] = npq;
           S.row_off[i] = row;
           npq += it.npab * it.npcd;
           row += it.rows;
-          for (int sp = 0; sp < it.nsplit; ++sp) S.tasks[nt++] = CTask{(int32_t)i, (int16_t)sp, (int16_t)it.nsplit};
+          const int16_t mark = (int16_t)(it.swap ? -it.nsplit : it.nsplit);
+          for (int sp = 0; sp < it.nsplit; ++sp) S.tasks[nt++] = CTask{(int32_t)i, (int16_t)sp, mark};
         }
         S.counts[kTaskCounts + 1 + 2 * t] = nt;
       }
@@ -632,7 +639,7 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
       CK(cudaMemcpyAsync(E.zero_len, E.zstage_len[b], sizeof(int64_t) * nzero, cudaMemcpyHostToDevice, st));
     }
     if (large) {
-      const int rc = engine_large(ctx, E, large, grid, big.npab, big.npab * big.npcd, big.rows, big.tier);
+      const int rc = engine_large(ctx, E, large, grid, big.swap ? big.npcd : big.npab, big.npab * big.npcd, big.rows, big.tier);
       if (rc != F12INT_OK) return rc;
       if (first && nzero > 0) k_zero_blocks<<<4 * 152, 128, 0, st>>>(E.zero_dst, E.zero_len, E.zero_count);
     } else {
@@ -844,9 +851,8 @@ int f12int_submit(f12int_ctx *ctx, int basis_id, const f12int_request *req, uint
     for (int64_t i = 0; i < n; ++i) {
       const int32_t *s = &R->q[4 * (size_t)i];
       BatchPlan bp{};
-      const int64_t np = (int64_t)B.nprim[s[0]] * B.nprim[s[1]] * B.nprim[s[2]] * B.nprim[s[3]];
-      if (!batch_plan(B.l[s[0]], B.l[s[1]], B.l[s[2]], B.l[s[3]], c, np, (int64_t)B.nprim[s[2]] * B.nprim[s[3]],
-                      kTaskFlops / 8, &bp)) {
+      if (!batch_plan(B.l[s[0]], B.l[s[1]], B.l[s[2]], B.l[s[3]], c, (int64_t)B.nprim[s[0]] * B.nprim[s[1]],
+                      (int64_t)B.nprim[s[2]] * B.nprim[s[3]], kTaskFlops / 8, &bp)) {
         delete R;
         return F12INT_EINVAL;
       }

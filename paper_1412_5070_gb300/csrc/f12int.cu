@@ -1248,7 +1248,7 @@ struct ListPlan {
   std::vector<int64_t> offsets;        // [n]
   std::vector<int64_t> pqoff;          // [n + 1] first primitive quartet
   std::vector<int64_t> rowoff;         // [nthin + 1] first double of the Hermite rows
-  std::vector<int> npab;               // [nthin] bra primitive pairs
+  std::vector<int> npab;               // [nthin] outer primitive pairs
   std::vector<CTask> tasks;            // quartet by quartet
   std::vector<int64_t> tfirst;         // [n + 1] first task
 };
@@ -1267,7 +1267,8 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
     int64_t key;
     int la, lb, lc, ld, f32;
     int64_t nab, ncd, count, first;
-    bool thin;
+    bool thin, swap;   // swap: listed as (cd|ab), the bra inner
+    ContractShape shape;
     ContractPlan pl;
     double work;
     int tier;
@@ -1319,6 +1320,9 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
         k.nab = nab;
         k.ncd = ncd;
         k.thin = thin_quartet(lk, cls);
+        k.swap = !k.thin && bra_inner(k.la, k.lb, k.lc, k.ld, cls, nab, ncd);
+        k.shape = contract_shape(k.la, k.lb, k.lc, k.ld, cls, k.swap);
+        if (k.swap) std::swap(k.nab, k.ncd);   // outer, inner
         slot_key[h] = key;
         slot_val[h] = (int32_t)kinds.size();
         kinds.push_back(k);
@@ -1328,10 +1332,7 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
     }
   }
   for (const Kind &k : kinds)
-    if (!k.thin) {
-      const ContractShape s{k.la, k.lb, k.lc, k.ld, cls == 5 ? 2 : 0};
-      total += (double)k.count * (double)(k.nab * k.ncd) * task_fmas(s, k.ncd, s.ncd());
-    }
+    if (!k.thin) total += (double)k.count * (double)(k.nab * k.ncd) * task_fmas(k.shape, k.ncd, k.shape.ncd());
   // about a dozen tasks per SM where the list has the work for it (a block's
   // result does not depend on how a quartet is cut into ranges)
   const double target = fewest ? 1e300 : std::min(kTaskFmas, std::max(5e4, total / (152 * 12)));
@@ -1341,10 +1342,9 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
       k.work = (double)(k.nab * k.ncd);
       continue;
     }
-    const ContractShape s{k.la, k.lb, k.lc, k.ld, cls == 5 ? 2 : 0};
-    k.pl = contract_plan(k.la, k.lb, k.lc, k.ld, cls, k.nab * k.ncd, k.ncd, k.f32 ? 4 : 8, target, fewest);
+    k.pl = contract_plan(k.shape, k.nab * k.ncd, k.ncd, k.f32 ? 4 : 8, target, fewest);
     if (k.pl.smem == 0) return F12INT_EINVAL;
-    k.work = (double)(k.nab * k.ncd) * task_fmas(s, k.ncd, (s.ncd() + k.pl.nsplit - 1) / k.pl.nsplit);
+    k.work = (double)(k.nab * k.ncd) * task_fmas(k.shape, k.ncd, (k.shape.ncd() + k.pl.nsplit - 1) / k.pl.nsplit);
     k.tier = 0;
     while (((size_t)8192 << k.tier) < k.pl.smem) ++k.tier;
   }
@@ -1395,7 +1395,7 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
   for (int64_t i = 0; i < n; ++i) {
     const int64_t j = perm[(size_t)i];
     const Kind &k = kinds[(size_t)kid[(size_t)j]];
-    for (int c = 0; c < 4; ++c) P.quartets[(size_t)(4 * i + c)] = hq0[4 * j + c];
+    for (int c = 0; c < 4; ++c) P.quartets[(size_t)(4 * i + c)] = hq0[4 * j + (k.swap ? c ^ 2 : c)];
     P.offsets[(size_t)i] = ho0[j];
     P.pqoff[(size_t)i] = npq;
     npq += k.nab * k.ncd;
@@ -1405,7 +1405,8 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
       nrow += k.nab * k.ncd * row_pitch(k.la + k.lb + k.lc + k.ld + (cls == 5 ? 2 : 0));
     }
     P.tfirst[(size_t)i] = (int64_t)P.tasks.size();
-    for (int sp = 0; sp < k.pl.nsplit; ++sp) P.tasks.push_back(CTask{(int32_t)i, (int16_t)sp, (int16_t)k.pl.nsplit});
+    const int16_t mark = (int16_t)(k.swap ? -k.pl.nsplit : k.pl.nsplit);
+    for (int sp = 0; sp < k.pl.nsplit; ++sp) P.tasks.push_back(CTask{(int32_t)i, (int16_t)sp, mark});
   }
   P.pqoff[(size_t)n] = npq;
   P.rowoff[(size_t)P.nthin] = nrow;

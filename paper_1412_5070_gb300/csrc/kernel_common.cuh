@@ -46,8 +46,8 @@ struct QuartetView {
 };
 
 
-// One block of contraction work: quartet q (index into the list), ket range
-// split of nsplit.
+// One block of contraction work: quartet q (index into the list), range split
+// of |nsplit| (nsplit < 0: the quartet is listed with its pairs swapped).
 struct CTask {
   int32_t q;
   int16_t split, nsplit;
