@@ -74,9 +74,19 @@ constexpr double GR_TB = 480.0;           // region B: xi u >= GR_TB (T' >= GR_T
 // e^{bD}: 13 terms hold 3e-13 to |b| D of about 40, and full precision to 25.
 F12_HD constexpr int grid_terms(int L) { return L <= 8 ? 13 : 14; }
 
+// Coefficients of row L + k that a point of highest order L reads: the k-th
+// Taylor term is smaller by some 0.1^k, and so is what its last coefficients
+// add (with 15 - k the errors against the oracle stay those of all 12; 13 - k
+// costs an order at L = 8).  Takes 52 of 143 multiply-adds off the rows past L.
+F12_HD constexpr int grid_coefs(int L, int k) {
+  return k <= 3 || L > 8 ? GR_NC : (k >= 11 ? 4 : 15 - k);
+}
+
 // multiply-adds of one point
 F12_HD constexpr int grid_fmas(int L) {
-  return (L + grid_terms(L) + 1) * (GR_NC - 1) + (L + 1) * (grid_terms(L) + 1);
+  int n = (L + 1) * (GR_NC - 1) + (L + 1) * (grid_terms(L) + 1);
+  for (int k = 1; k <= grid_terms(L); ++k) n += grid_coefs(L, k) - 1;
+  return n;
 }
 
 F12_HD inline int grid_hi(double x) {
@@ -414,13 +424,15 @@ F12_DEV inline void grid_eval(const double *cells, const GridPoint &pt, int L, d
   for (int m = LMAX + NMAX; m >= 0; --m) {
     if (!FIXED && m > L + N) continue;
     const double *row = cell + m * GR_NC;
+    const int nc = FIXED && m > LMAX ? grid_coefs(LMAX, m - LMAX) : GR_NC;
     double c[GR_NC];
     grid_load4(row, c);
-    grid_load4(row + 4, c + 4);
-    grid_load4(row + 8, c + 8);
-    double r = c[GR_NC - 1];
+    if (nc > 4) grid_load4(row + 4, c + 4);
+    if (nc > 8) grid_load4(row + 8, c + 8);
+    double r = 0.0;
 #pragma unroll
-    for (int i = GR_NC - 2; i >= 0; --i) r = fma(r, pt.a, c[i]);
+    for (int i = GR_NC - 1; i >= 0; --i)
+      if (i < nc) r = i == nc - 1 ? c[i] : fma(r, pt.a, c[i]);
 #pragma unroll
     for (int l = 0; l <= LMAX; ++l)
       if (m - l >= 0 && m - l <= NMAX && (FIXED || (l <= L && m - l <= N))) h[l] = fma(r, w[m - l], h[l]);
