@@ -17,8 +17,10 @@
 // Two regions:
 //   A  xi in [2^GR_XLO, 2^GR_XHI), eight cells per octave (sixteen in the
 //      lowest, where a kernel that grows like e^{br} makes the functions grow
-//      like e^{b^2/(4 xi)}), c the geometric mean of a cell's ends, local coordinate (xi - c)/(xi + c) scaled to
-//      [-1, 1]; T' = c u < GR_TMAX: cells of width 1/4 below 8, then sixteen
+//      like e^{b^2/(4 xi)}), c the geometric mean of a cell's ends, local
+//      coordinate y(c/xi - 1) scaled to [-1, 1], y(d) = d - d^2/2 + d^3/4 (three
+//      terms of 2 (c - xi)/(c + xi), on which the singularities, xi = 0 and the
+//      negative axis, lie farthest from the cell); T' = c u < GR_TMAX: cells of width 1/4 below 8, then sixteen
 //      per octave;
 //   B  T' >= GR_TMAX (distant charge distributions): sixteen cells per octave
 //      of u in [2^GR_ULO, 2^GR_UHI), local coordinate 1/xi scaled to [-1, 1].
@@ -110,9 +112,18 @@ F12_HD inline double hi_double(int hi) {
 #endif
 }
 
-// Cell of xi, or -1.
-F12_HD inline int grid_xindex(double xi) {
-  const int h = grid_hi(xi);
+// product rounded on its own (the builder's u_c is that product)
+F12_HD inline double mul_rn(double a, double b) {
+#ifdef __CUDA_ARCH__
+  return __dmul_rn(a, b);
+#else
+  volatile double p = a * b;
+  return p;
+#endif
+}
+
+// Cell of xi, or -1, from the high word of the double.
+F12_HD inline int grid_xindex(int h) {
   if (h < (1023 + GR_XLO) << 20 || h >= (1023 + GR_XHI) << 20) return -1;
   return h < (1023 + GR_XLO + GR_XFINE) << 20 ? (h >> 16) - (1023 + GR_XLO) * 16
                                              : (h >> 17) - (1023 + GR_XLO - GR_XFINE) * 8;
@@ -125,9 +136,10 @@ struct GridPoint {
   double hd;      // (u - u_c)/2
 };
 
-// c and 1/max|z| of a cell of xi (z = (xi - c)/(xi + c) at its upper end);
-// GR_XT values per cell in the table that grid_point reads: c, 1/max|z|, 1/c, 0
+// GR_XT values per cell of xi in the table that grid_point reads: c, 1/c and the
+// scale of y
 constexpr int GR_XT = 4;
+F12_HD inline double grid_y(double d) { return fma(fma(d, 0.25, -0.5) * d, d, d); }
 F12_HD inline void grid_xends(int ix, double *lo, double *hi) {
   if (ix < 16 * GR_XFINE) {
     *lo = hi_double(((1023 + GR_XLO) * 16 + ix) << 16);
@@ -137,11 +149,20 @@ F12_HD inline void grid_xends(int ix, double *lo, double *hi) {
     *hi = hi_double(((1023 + GR_XLO - GR_XFINE) * 8 + ix + 1) << 17);
   }
 }
-F12_HD inline void grid_xcell(int ix, double *c, double *iz) {
+F12_HD inline void grid_xcell(int ix, double *r) {
   double lo, hi;
   grid_xends(ix, &lo, &hi);
-  *c = sqrt(lo * hi);
-  *iz = (hi + *c) / (hi - *c);
+  r[0] = sqrt(lo * hi);
+  r[1] = 1.0 / r[0];
+  r[2] = 1.0 / fmax(fabs(grid_y(r[0] / lo - 1.0)), fabs(grid_y(r[0] / hi - 1.0)));
+  r[3] = 0.0;
+}
+// xi at local coordinate a of a cell (r: its GR_XT values), by Newton's method
+F12_HD inline double grid_xi(const double *r, double a) {
+  const double y = a / r[2];
+  double d = y / (1.0 - 0.5 * y);
+  for (int i = 0; i < 4; ++i) d -= (grid_y(d) - y) / (1.0 - d + 0.75 * d * d);
+  return r[0] / (1.0 + d);
 }
 F12_HD inline int grid_octave(int ix) { return ix < 16 * GR_XFINE ? ix >> 4 : (ix >> 3) - GR_XFINE; }
 // ends of a cell of T' (or of u: the same subdivision of an octave)
@@ -159,25 +180,41 @@ F12_HD inline void grid_ucell(int iu, double *lo, double *hi) {
   *hi = hi_double(((1023 + GR_ULO) * 16 + iu + 1) << 16);
 }
 
-// Local coordinates of (xi, u); xt: GR_XT values per cell of xi.
-F12_DEV inline GridPoint grid_point(const double *xt, double xi, double u) {
+// Local coordinates of (xi, u) with v = 1/xi; xt: GR_XT values per cell of xi.
+// The cell of xi comes from a single-precision reciprocal (a cell's polynomials
+// hold a little past its ends), the cell and its middle of T' from the bits of
+// the double, so that a point costs no FP64 division.
+F12_DEV inline GridPoint grid_point(const double *xt, double v, double u) {
   GridPoint g;
-  const int ix = grid_xindex(xi);
+  const float xf = 1.0f / (float)v;
+  int b;
+#ifdef __CUDA_ARCH__
+  b = __float_as_int(xf);
+#else
+  std::memcpy(&b, &xf, sizeof b);
+#endif
+  const int ix = grid_xindex((b >> 3) + ((1023 - 127) << 20));   // the bits as those of a double's high word
   if (ix < 0) {
     g.cell = -1;
     return g;
   }
-  const double c = xt[GR_XT * ix];
-  const double T = c * u;
-  if (T < GR_TMAX) {
+  const double *r = xt + GR_XT * ix;
+  const double T = r[0] * u;
+  const int hT = grid_hi(T);
+  if (hT < (1023 + GR_TEXP) << 20) {   // T < GR_TMAX
+    double mid;
     int it;
-    double lo, hi;
-    if (T < 8.0) it = (int)(4.0 * T);
-    else it = GR_TLIN + (grid_hi(T) >> 16) - (1023 + 3) * 16;
-    grid_tcell(it, &lo, &hi);
+    if (hT < (1023 + 3) << 20) {       // T < 8: the cells of [8, 16) in T + 8
+      const int h8 = grid_hi(T + 8.0);
+      it = (h8 >> 15) - (1023 + 3) * 32;
+      mid = hi_double((h8 & ~0x7FFF) | 0x4000) - 8.0;
+    } else {
+      it = GR_TLIN + (hT >> 16) - (1023 + 3) * 16;
+      mid = hi_double((hT & ~0xFFFF) | 0x8000);
+    }
     g.cell = ix * GR_NT + it;
-    g.a = (xi - c) / (xi + c) * xt[GR_XT * ix + 1];
-    g.hd = 0.5 * (u - 0.5 * (lo + hi) * xt[GR_XT * ix + 2]);
+    g.a = grid_y(fma(r[0], v, -1.0)) * r[2];
+    g.hd = 0.5 * (u - mul_rn(mid, r[1]));
   } else {
     const int iu = (grid_hi(u) >> 16) - (1023 + GR_ULO) * 16;
     if (iu < 0 || iu >= GR_NU) {
@@ -187,7 +224,7 @@ F12_DEV inline GridPoint grid_point(const double *xt, double xi, double u) {
     double lo, hi;
     grid_ucell(iu, &lo, &hi);
     g.cell = GR_NX * GR_NT + iu;
-    g.a = 2.0 * GR_TB / (hi * xi) - 1.0;
+    g.a = 2.0 * GR_TB / hi * v - 1.0;
     g.hd = 0.5 * (u - 0.5 * (lo + hi));
   }
   return g;
@@ -355,16 +392,16 @@ constexpr double GR_BW = 0.25;
 
 // ------------------------------------------------------------ evaluation --
 // The Coulomb kernel (I1): sqrt(xi) hat g_l = 2 sqrt(xi) (-2 xi)^l F_l(x), F_l the
-// Boys function and x = xi u.  tab is the table of e^{-x} M(1, l + 3/2, x) =
+// Boys function and x = xi u, xi = 1/v.  tab is the table of e^{-x} M(1, l + 3/2, x) =
 // (2l + 1) F_l(x) (aux.cuh: Taylor rows on a grid of x), read for the highest
 // order; the others follow by F_{l-1} = (2 x F_l + e^{-x})/(2l - 1), every term
 // positive.  Past the table e^{-x} is below double precision of F_l.
 constexpr int BY_LSTRIDE = 40 * 201 * 14, BY_NT = 14;   // between orders, per row
 constexpr double BY_XMAX = 100.0;
 template <int LMAX, bool FIXED>
-F12_DEV inline void boys_eval(const double *tab, double xi, double u, int L_, double *h) {
+F12_DEV inline void boys_eval(const double *tab, double v, double u, int L_, double *h) {
   const int L = FIXED ? LMAX : L_;
-  const double x = xi * u;
+  const double xi = 1.0 / v, x = xi * u;
   if (x < BY_XMAX) {
     const double r = rint(2.0 * x), d = x - 0.5 * r;
     const double *row = tab + (size_t)L * BY_LSTRIDE + (int)r * BY_NT;

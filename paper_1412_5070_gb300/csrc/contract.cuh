@@ -187,12 +187,10 @@ __device__ __noinline__ void hermite_row_any(int L, const double *g, double X, d
 }
 
 template <int L>
-__device__ __forceinline__ void direct_row(const GridView &G, double pref, double xi, double X, double Y, double Z,
-                                           double *out) {
+__device__ __forceinline__ void direct_row(const GridView &G, const PairView &PV, int pab, int pcd, double X, double Y,
+                                           double Z, double *out) {
   double g[L + 1];
-  aux_direct<L>(G, xi, X * X + Y * Y + Z * Z, g);
-#pragma unroll
-  for (int l = 0; l <= L; ++l) g[l] *= pref;
+  aux_direct<L>(G, PV, pab, pcd, X * X + Y * Y + Z * Z, g);
   if constexpr (L <= 6) hermite_row<L>(g, X, Y, Z, out);
   else hermite_row_any(L, g, X, Y, Z, out);
 }
@@ -243,29 +241,27 @@ k_hermite_rows(GridView G, PairView PV0, QuartetView QV, int cls, int nf, int64_
       continue;
     }
     const int L = PV.shell_l[s[0]] + PV.shell_l[s[1]] + PV.shell_l[s[2]] + PV.shell_l[s[3]] + (cls == 5 ? 2 : 0);
-    const double p = PV.pp_p[pab], q = PV.pp_p[pcd];
     const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
                  Z = pair_sep(PV.pp_P, pab, pcd, 2);
     double *o = rows.quartet(QV, lo) + (int64_t)k * rows.stride(row_pitch(L));
     if constexpr (DIRECT) {
-      // g_n = pi^{5/2}/(sqrt(p+q) pq) hat g_n = pi^{5/2} (pq)^{-3/2} sqrt(xi) hat g_n
-      const double pq_ = p * q, xi = pq_ / (p + q), pref = pi52 / (pq_ * sqrt(pq_));
       nfma += aux_direct_fmas(G.boys != nullptr, L);
       switch (L) {
-        case 4: direct_row<4>(G, pref, xi, X, Y, Z, o); break;
-        case 5: direct_row<5>(G, pref, xi, X, Y, Z, o); break;
-        case 6: direct_row<6>(G, pref, xi, X, Y, Z, o); break;
-        case 7: direct_row<7>(G, pref, xi, X, Y, Z, o); break;
-        case 8: direct_row<8>(G, pref, xi, X, Y, Z, o); break;
-        case 9: direct_row<9>(G, pref, xi, X, Y, Z, o); break;
-        case 10: direct_row<10>(G, pref, xi, X, Y, Z, o); break;
-        case 11: direct_row<11>(G, pref, xi, X, Y, Z, o); break;
-        case 12: direct_row<12>(G, pref, xi, X, Y, Z, o); break;
-        case 13: direct_row<13>(G, pref, xi, X, Y, Z, o); break;
-        default: direct_row<14>(G, pref, xi, X, Y, Z, o); break;
+        case 4: direct_row<4>(G, PV, pab, pcd, X, Y, Z, o); break;
+        case 5: direct_row<5>(G, PV, pab, pcd, X, Y, Z, o); break;
+        case 6: direct_row<6>(G, PV, pab, pcd, X, Y, Z, o); break;
+        case 7: direct_row<7>(G, PV, pab, pcd, X, Y, Z, o); break;
+        case 8: direct_row<8>(G, PV, pab, pcd, X, Y, Z, o); break;
+        case 9: direct_row<9>(G, PV, pab, pcd, X, Y, Z, o); break;
+        case 10: direct_row<10>(G, PV, pab, pcd, X, Y, Z, o); break;
+        case 11: direct_row<11>(G, PV, pab, pcd, X, Y, Z, o); break;
+        case 12: direct_row<12>(G, PV, pab, pcd, X, Y, Z, o); break;
+        case 13: direct_row<13>(G, PV, pab, pcd, X, Y, Z, o); break;
+        default: direct_row<14>(G, PV, pab, pcd, X, Y, Z, o); break;
       }
     } else {
       double g[LAUX + 1];
+      const double p = PV.pp_p[pab], q = PV.pp_p[pcd];
       const double pref = pi52 / (sqrt(p + q) * p * q);
       for (int l = 0; l <= L; ++l) {
         double acc = 0.0;
@@ -400,7 +396,7 @@ __device__ __forceinline__ void contract_task(const PairView &PV0, const Quartet
   const int kE = ncdt * S.inner4();   // products of one staged pair
   // the four products of a term for the pair with I5's operator
   auto products5 = [&](const double *E, const double *Fp, int pair, unsigned w, T *e, int stride) {
-    const double a = PV.pp_ab[2 * pair], b = PV.pp_ab[2 * pair + 1];
+    const double a = PV.pp_ab[4 * pair], b = PV.pp_ab[4 * pair + 1];
     const double c5 = (a - b) / (2.0 * (a + b));
     const double ex = E[w & 1023], ey = E[w >> 10 & 1023], ez = E[w >> 20];
     e[0] = (T)(c5 * ex * ey * ez);

@@ -72,14 +72,14 @@ __global__ void __launch_bounds__(NODES *ITB) k_rows_a(Build B) {
   __shared__ double sx[TILE], sw[TILE];
   const int ix = blockIdx.x, oct = grid_octave(ix);
   const int n = threadIdx.x % NODES, it0 = blockIdx.y * ITB, it = it0 + threadIdx.x / NODES;
-  const double c = B.xt[GR_XT * ix], iz = B.xt[GR_XT * ix + 1], ic = B.xt[GR_XT * ix + 2];
+  const double c = B.xt[GR_XT * ix], ic = B.xt[GR_XT * ix + 1];
   const bool live = it < GR_NT;
   const int cell = ix * GR_NT + it;
   double lo = 0.0, hi = 0.0;
   if (live) grid_tcell(it, &lo, &hi);
   const double a = n < GR_NC ? B.node[n] : check_a(cell);
-  const double z = a / iz, xi = c * (1.0 + z) / (1.0 - z);
-  double u = 0.5 * (lo + hi) * ic;
+  const double xi = grid_xi(B.xt + GR_XT * ix, a);
+  double u = mul_rn(0.5 * (lo + hi), ic);
   if (n == GR_NC) u += check_s(cell) * (hi - lo) * ic;
   const double D = sqrt(u);
   const int nrow = B.ncls * GR_ROWS;
@@ -87,7 +87,8 @@ __global__ void __launch_bounds__(NODES *ITB) k_rows_a(Build B) {
   for (int k = 0; k < nrow; ++k) acc[k] = 0.0;
   // panels that reach the window of any node of the block: past it e^{-xi (x-D)^2}
   // times the growth of j_m (below D) and of F_m (above) is below double precision
-  const double clo = c * (1.0 - 1.0 / iz) / (1.0 + 1.0 / iz);   // smallest xi of the cell
+  double clo, chi;   // ends of the cell of xi
+  grid_xends(ix, &clo, &chi);
   double tl, th, dummy;
   grid_tcell(it0, &tl, &dummy);
   grid_tcell(min(it0 + ITB, GR_NT) - 1, &dummy, &th);
@@ -217,7 +218,7 @@ __global__ void k_check(Build B) {
   double lo, hi, hd, a = check_a(cell);
   if (cell < GR_NX * GR_NT) {
     grid_tcell(cell % GR_NT, &lo, &hi);
-    hd = 0.5 * check_s(cell) * (hi - lo) * B.xt[GR_XT * (cell / GR_NT) + 2];
+    hd = 0.5 * check_s(cell) * (hi - lo) * B.xt[GR_XT * (cell / GR_NT) + 1];
   } else {
     grid_ucell(cell - GR_NX * GR_NT, &lo, &hi);
     hd = 0.5 * check_s(cell) * (hi - lo);
@@ -355,11 +356,7 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
     bx[(size_t)j] = std::cos(th);
     bw[(size_t)j] = ((j & 1) ? -1.0 : 1.0) * std::sin(th);
   }
-  for (int i = 0; i < GR_NX; ++i) {
-    double *r = &xt[(size_t)GR_XT * (size_t)i];
-    grid_xcell(i, r, r + 1);
-    r[2] = 1.0 / r[0];
-  }
+  for (int i = 0; i < GR_NX; ++i) grid_xcell(i, &xt[(size_t)GR_XT * (size_t)i]);
 
   std::shared_ptr<AuxGrid> g = std::make_shared<AuxGrid>();
   g->device = device;
@@ -421,14 +418,16 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
 bool covers(const AuxGrid &g, int cls, double xi_lo, double xi_hi, double dmax) {
   const int c = cls == 5 ? 3 : cls;
   if (!g.cells[c]) return false;
-  // a little room for the rounding of the exponents' sums and distances
-  const double lo = xi_lo * (1.0 - 1e-9), hi = xi_hi * (1.0 + 1e-9), u = dmax * dmax * (1.0 + 1e-9) + 1e-9;
-  const int x0 = grid_xindex(lo), x1 = grid_xindex(hi);
+  // a little room for the rounding of the exponents' sums and distances, and
+  // for grid_point's single-precision cell of xi
+  const double lo = xi_lo * (1.0 - 1e-6), hi = xi_hi * (1.0 + 1e-6), u = dmax * dmax * (1.0 + 1e-9) + 1e-9;
+  const int x0 = grid_xindex(grid_hi(lo)), x1 = grid_xindex(grid_hi(hi));
   if (!(lo > 0.0) || x0 < 0 || x1 < x0) return false;
   const std::vector<unsigned char> &ok = g.ok_host[c];
   for (int ix = x0; ix <= x1; ++ix) {
-    double cc, iz;
-    grid_xcell(ix, &cc, &iz);
+    double r[GR_XT];
+    grid_xcell(ix, r);
+    const double cc = r[0];
     for (int it = 0; it < GR_NT; ++it) {
       double tl, th;
       grid_tcell(it, &tl, &th);
@@ -437,8 +436,9 @@ bool covers(const AuxGrid &g, int cls, double xi_lo, double xi_hi, double dmax) 
     }
   }
   // region B, from the smallest u that reaches it at the largest xi
-  double cc, iz;
-  grid_xcell(x1, &cc, &iz);
+  double r[GR_XT];
+  grid_xcell(x1, r);
+  const double cc = r[0];
   if (cc * u >= GR_TMAX) {
     if (u >= std::ldexp(1.0, GR_UHI)) return false;
     for (int iu = 0; iu < GR_NU; ++iu) {

@@ -19,7 +19,7 @@ struct AuxGrid {
   double *cells[7] = {nullptr};         // device
   unsigned char *ok[7] = {nullptr};     // device, per cell
   std::vector<unsigned char> ok_host[7];
-  double *xt = nullptr;                 // device: centre and scale of every cell of xi
+  double *xt = nullptr;                 // device: grid_point's values of every cell of xi
   size_t bytes = 0;
   AuxGrid() = default;
   AuxGrid(const AuxGrid &) = delete;

@@ -20,7 +20,7 @@ struct PairView {
   const int *pair_start;     // [nshell*nshell + 1] first primitive pair of shell pair (i,j)
   const double *pp_p;        // exponent sum p
   const double *pp_P;        // [6*npp] centre P as heavy centre H (3) + offset P - H (3)
-  const double *pp_ab;       // [2*npp] exponents a, b
+  const double *pp_ab;       // [4*npp] exponents a, b, 1/p, pi^{5/4} p^{-3/2}
   const int64_t *pp_eoff;    // offset into epool of this primitive pair's tables
   const double *epool;       // E (3 dims) then F (3 dims), each (la+1)(lb+1)(la+lb+1)
   const int *shell_l;
@@ -75,11 +75,20 @@ struct GridView {
   __host__ __device__ bool direct() const { return cells || boys; }
 };
 
-// sqrt(xi) hat g_l, l <= L
+// g_n, n <= L, of a primitive quartet, u = |P - Q|^2: with
+//   g_n = pi^{5/2}/(sqrt(p+q) pq) hat g_n = pi^{5/2} (pq)^{-3/2} [sqrt(xi) hat g_n]
+// and 1/xi = 1/p + 1/q both factors come from the pairs' tables without a
+// division or a square root (some 60 FP64 instructions, a tenth of a thin
+// primitive quartet's).
 template <int L>
-__device__ __forceinline__ void aux_direct(const GridView &G, double xi, double u, double *h) {
-  if (G.boys) f12dev::boys_eval<L, true>(G.boys, xi, u, L, h);
-  else f12dev::grid_eval<L, true>(G.cells, f12dev::grid_point(G.xt, xi, u), L, h);
+__device__ __forceinline__ void aux_direct(const GridView &G, const PairView &PV, int pab, int pcd, double u,
+                                           double *g) {
+  const double v = PV.pp_ab[4 * pab + 2] + PV.pp_ab[4 * pcd + 2];
+  if (G.boys) f12dev::boys_eval<L, true>(G.boys, v, u, L, g);
+  else f12dev::grid_eval<L, true>(G.cells, f12dev::grid_point(G.xt, v, u), L, g);
+  const double pref = PV.pp_ab[4 * pab + 3] * PV.pp_ab[4 * pcd + 3];
+#pragma unroll
+  for (int l = 0; l <= L; ++l) g[l] *= pref;
 }
 __host__ __device__ constexpr int aux_direct_fmas(const bool boys, int L) {
   return boys ? f12dev::BY_NT - 1 + L : f12dev::grid_fmas(L);

@@ -61,21 +61,18 @@ __device__ __forceinline__ void thin_quartet_body(const PairView &PV, const Quar
   for (int r = lane; r < np; r += 32) {
     const int iab = r / npcd, icd = r - iab * npcd;
     const int pab = ab0 + iab, pcd = cd0 + icd;
-    const double p = PV.pp_p[pab], qq = PV.pp_p[pcd];
     const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
                  Z = pair_sep(PV.pp_P, pab, pcd, 2);
-    double pref, g[L + 1];
+    double g[L + 1];
     if (G.direct()) {
       if (prim_negligible(PV, pab, pcd)) continue;
-      // g_n = sqrt(pi^5/(p+q))/(pq) hat g_n = pi^{5/2} (pq)^{-3/2} sqrt(xi) hat g_n
-      const double pq_ = p * qq;
-      aux_direct<L>(G, pq_ / (p + qq), X * X + Y * Y + Z * Z, g);
-      pref = pi52 / (pq_ * sqrt(pq_));
+      aux_direct<L>(G, PV, pab, pcd, X * X + Y * Y + Z * Z, g);
     } else {
       const int64_t pq = QV.pq_off[q] + r - pq0;
       if (keys[pq * nf] == kSkipKey) continue;   // dropped by the primitive screen
       // g_n = sqrt(pi^5/(p+q))/(pq) * sum over families (fixed order)
-      pref = pi52 / (sqrt(p + qq) * p * qq);
+      const double p = PV.pp_p[pab], qq = PV.pp_p[pcd];
+      const double pref = pi52 / (sqrt(p + qq) * p * qq);
 #pragma unroll
       for (int n = 0; n <= L; ++n) g[n] = 0.0;
       for (int f = 0; f < nf; ++f) {
@@ -83,10 +80,10 @@ __device__ __forceinline__ void thin_quartet_body(const PairView &PV, const Quar
 #pragma unroll
         for (int n = 0; n <= L; ++n) g[n] += pp[n];
       }
+#pragma unroll
+      for (int n = 0; n <= L; ++n) g[n] *= pref;
     }
     ++nproc;
-#pragma unroll
-    for (int n = 0; n <= L; ++n) g[n] *= pref;
     // Hermite recursion, levels n = L .. 0, in registers (every index is a
     // compile-time constant after unrolling)
     double R[NH], Rn[NH];
@@ -115,7 +112,7 @@ __device__ __forceinline__ void thin_quartet_body(const PairView &PV, const Quar
     const double *Fab = Eab + 3 * N1AB;   // dE/dAB (I5)
     double c5 = 0.0;
     if constexpr (I5) {
-      const double a = PV.pp_ab[2 * pab], b = PV.pp_ab[2 * pab + 1];
+      const double a = PV.pp_ab[4 * pab], b = PV.pp_ab[4 * pab + 1];
       c5 = (a - b) / (2.0 * (a + b));
     }
 #pragma unroll
