@@ -74,8 +74,10 @@ __global__ void k_build_pairs(int npp, const int *pp_shell_a, const int *pp_shel
   double da = coefs[pp_prim_a[i]], db = coefs[pp_prim_b[i]];
   double p = a + b;
   pp_p[i] = p;
-  pp_ab[2 * i] = a;
-  pp_ab[2 * i + 1] = b;
+  pp_ab[4 * i] = a;
+  pp_ab[4 * i + 1] = b;
+  pp_ab[4 * i + 2] = 1.0 / p;
+  pp_ab[4 * i + 3] = 4.1825133983795991 / (p * sqrt(p));   // pi^{5/4} p^{-3/2}
   const int nt = la + lb + 1;
   const int n1 = (la + 1) * (lb + 1) * nt;
   double *E = epool + pp_eoff[i];
@@ -345,12 +347,12 @@ __global__ void k_aux_points(Tables T, GridView G, const unsigned char *ok, int 
   double g[LAUX + 1];
   if (G.boys) {
     const double is = 1.0 / sqrt(xi[i]);
-    boys_eval<LAUX, false>(G.boys, xi[i], D[i] * D[i], nmax, g);
+    boys_eval<LAUX, false>(G.boys, 1.0 / xi[i], D[i] * D[i], nmax, g);
     for (int n = 0; n <= nmax; ++n) out[i * (nmax + 1) + n] = is * g[n];
     return;
   }
   if (G.cells) {
-    const GridPoint pt = grid_point(G.xt, xi[i], D[i] * D[i]);
+    const GridPoint pt = grid_point(G.xt, 1.0 / xi[i], D[i] * D[i]);
     if (pt.cell >= 0 && ok[pt.cell]) {
       const double is = 1.0 / sqrt(xi[i]);
       if (nmax <= 4) grid_eval<4, false>(G.cells, pt, nmax, g);
@@ -1100,7 +1102,7 @@ int f12int_set_basis(f12int_ctx *ctx, int nshell, const double *centers, const i
   A(&B.d_pair_start, sizeof(int) * B.pair_start.size());
   A(&B.d_pp_p, sizeof(double) * npp);
   A(&B.d_pp_P, sizeof(double) * 6 * npp);
-  A(&B.d_pp_ab, sizeof(double) * 2 * npp);
+  A(&B.d_pp_ab, sizeof(double) * 4 * npp);
   A(&B.d_pp_eoff, sizeof(int64_t) * npp);
   A(&B.d_epool, sizeof(double) * std::max<int64_t>(epos, 1));
   B.bytes = bytes;
