@@ -22,7 +22,12 @@ namespace f12dev {
 // every f12int_set_factor).
 template <class Fn>
 inline void parallel_for(int n, Fn fn) {
-  const int nt = std::max(1, std::min({n, (int)std::thread::hardware_concurrency(), 16}));
+  static const int cores = std::max(1, std::min((int)std::thread::hardware_concurrency(), 16));   // (a slow query)
+  const int nt = std::max(1, std::min(n, cores));
+  if (nt == 1) {
+    for (int i = 0; i < n; ++i) fn(i);
+    return;
+  }
   std::atomic<int> next{0};
   auto work = [&] {
     for (int i = next++; i < n; i = next++) fn(i);

@@ -22,6 +22,8 @@
 #include <cstdio>
 #include <cstring>
 #include <deque>
+#include <cstdlib>
+#include <map>
 #include <memory>
 #include <mutex>
 #include <new>
@@ -377,6 +379,54 @@ namespace {
 struct Engine;   // batched requests (engine.cuh)
 }
 
+// Where the arrays of a planned list lie, on the device and in its host staging.
+struct ListLayout {
+  size_t offsets, pqoff, rowoff, tasks, bytes;   // (the quartets are first)
+  ListLayout(int64_t n, int64_t nthin, int64_t ntask) {
+    offsets = (16 * (size_t)n + 15) & ~(size_t)15;
+    pqoff = offsets + 8 * (size_t)n;
+    rowoff = pqoff + 8 * ((size_t)n + 1);
+    tasks = rowoff + 8 * ((size_t)nthin + 1);
+    bytes = tasks + sizeof(CTask) * (size_t)ntask;
+  }
+};
+
+// Host staging of a call's list: page-locked from kPinLeast to kPinMost bytes
+// (copies run at the link's rate and need no intermediate copy: with the cores
+// of plan_kinds 3.6 ms off a call of 200,000 quartets), plain memory below (the
+// driver takes a small copy from plain memory 14 us sooner per call) and past
+// that.  Grown on demand, given back with the context.
+struct HostStage {
+  static constexpr size_t kPinLeast = (size_t)256 << 10, kPinMost = (size_t)64 << 20;
+  unsigned char *p = nullptr;
+  size_t cap = 0;
+  bool pinned = false;
+  bool reserve(size_t bytes, size_t keep = 0) {   // the first `keep` bytes stay
+    if (bytes <= cap) return true;
+    const size_t want = std::max(bytes + bytes / 4, (size_t)1 << 16);
+    unsigned char *q = nullptr;
+    bool pin = want >= kPinLeast && want <= kPinMost && cudaHostAlloc((void **)&q, want, cudaHostAllocDefault) == cudaSuccess;
+    if (!pin) {
+      cudaGetLastError();
+      q = (unsigned char *)std::malloc(want);
+    }
+    if (!q) return false;
+    if (keep) std::memcpy(q, p, keep);
+    release();
+    p = q;
+    cap = want;
+    pinned = pin;
+    return true;
+  }
+  void release() {
+    if (pinned) cudaFreeHost(p);
+    else std::free(p);
+    p = nullptr;
+    cap = 0;
+    pinned = false;
+  }
+};
+
 struct f12int_ctx {
   int device = 0;
   size_t budget = 0;
@@ -404,6 +454,7 @@ struct f12int_ctx {
     double *d_pp_p = nullptr, *d_pp_P = nullptr, *d_pp_ab = nullptr, *d_epool = nullptr;
     int64_t *d_pp_eoff = nullptr;
     std::vector<int> l, nprim, pair_start;
+    std::vector<int> type, type_l, type_nprim;   // per shell: its type, (l, primitives); per type
     std::vector<double> centers, exps, coefs;
     size_t bytes = 0;
     bool prim_screen = true;            // false for the internal per-primitive basis
@@ -417,22 +468,18 @@ struct f12int_ctx {
   };
   std::deque<BasisData> bases;   // deque: growing it never moves existing entries
   // scratch of compute_class (grown on demand, bounded by the budget)
-  int64_t *d_pqoff = nullptr;
+  unsigned char *d_list = nullptr;   // a planned list (ListLayout)
+  HostStage stage;                   // its staging on the host
   int *d_keys = nullptr;
   unsigned *d_order = nullptr, *d_hist = nullptr;
   double *d_part = nullptr;
-  int32_t *d_qperm = nullptr;
-  int64_t *d_operm = nullptr;
-  CTask *d_tasks = nullptr;
   double *d_rows = nullptr;      // Hermite rows of a chunk
-  int64_t *d_rowoff = nullptr;   // first double of every general quartet's rows
-  size_t rows_cap = 0, rowoff_cap = 0;
+  size_t rows_cap = 0;
   // the contraction launches of a call are independent of one another: they
   // run on these streams, between two events on the call's
   cudaStream_t side[NSIDE] = {nullptr};
   cudaEvent_t fork = nullptr, join[NSIDE] = {nullptr};
-  size_t pqoff_cap = 0, keys_cap = 0, order_cap = 0, hist_cap = 0, part_cap = 0, qperm_cap = 0, operm_cap = 0;
-  size_t tasks_cap = 0;
+  size_t list_cap = 0, keys_cap = 0, order_cap = 0, hist_cap = 0, part_cap = 0;
   // optional per-kernel timing (events on the launching stream) and counters
   bool timing = false;
   unsigned long long *d_fma = nullptr;
@@ -685,16 +732,12 @@ int f12int_destroy(f12int_ctx *ctx) {
   cudaFree(ctx->d_grp);
   cudaFree(ctx->d_jtab);
   cudaFree(ctx->d_kgrow);
-  cudaFree(ctx->d_pqoff);
+  cudaFree(ctx->d_list);
   cudaFree(ctx->d_keys);
   cudaFree(ctx->d_order);
   cudaFree(ctx->d_hist);
   cudaFree(ctx->d_part);
-  cudaFree(ctx->d_qperm);
-  cudaFree(ctx->d_operm);
-  cudaFree(ctx->d_tasks);
   cudaFree(ctx->d_rows);
-  cudaFree(ctx->d_rowoff);
   for (int i = 0; i < NSIDE; ++i) {
     if (ctx->side[i]) cudaStreamDestroy(ctx->side[i]);
     if (ctx->join[i]) cudaEventDestroy(ctx->join[i]);
@@ -702,6 +745,7 @@ int f12int_destroy(f12int_ctx *ctx) {
   if (ctx->fork) cudaEventDestroy(ctx->fork);
   cudaFree(ctx->d_status);
   cudaFree(ctx->d_fma);
+  ctx->stage.release();
   for (auto &e : ctx->ev_pool) {
     cudaEventDestroy(e.first);
     cudaEventDestroy(e.second);
@@ -1053,6 +1097,17 @@ int f12int_set_basis(f12int_ctx *ctx, int nshell, const double *centers, const i
     poff[i] = o;
     o += nprim[i];
   }
+  {
+    std::map<std::pair<int, int>, int> types;
+    for (int i = 0; i < nshell; ++i) {
+      const auto it = types.emplace(std::make_pair(l[i], nprim[i]), (int)types.size());
+      if (it.second) {
+        B.type_l.push_back(l[i]);
+        B.type_nprim.push_back(nprim[i]);
+      }
+      B.type.push_back(it.first->second);
+    }
+  }
   // primitive pairs of every ordered shell pair (i, j), i outer
   std::vector<int> sa, sb, pa, pb;
   std::vector<int64_t> eoff;
@@ -1246,25 +1301,47 @@ struct ListPlan {
   };
   std::vector<Group> groups;
   int64_t n = 0, nthin = 0;            // quartets; first thin one
-  std::vector<int32_t> quartets;       // [4 n]
-  std::vector<int64_t> offsets;        // [n]
-  std::vector<int64_t> pqoff;          // [n + 1] first primitive quartet
-  std::vector<int64_t> rowoff;         // [nthin + 1] first double of the Hermite rows
-  std::vector<int> npab;               // [nthin] outer primitive pairs
-  std::vector<CTask> tasks;            // quartet by quartet
-  std::vector<int64_t> tfirst;         // [n + 1] first task
+  // runs of quartets of one kind, in the working order
+  struct Run {
+    int64_t first, count, npq, npab, pitch;   // primitive quartets, outer pairs and row doubles of one quartet
+    int64_t pq0, row0, task0;                 // of the first
+    int nsplit;
+    bool swap, thin;
+  };
+  std::vector<Run> runs, kind_run;            // (kind_run: by the index in kid)
+  int64_t ntask = 0, npq = 0, nrow = 0;       // totals
+  int64_t big_pq = 1, big_row = 1;            // largest quartet, largest bra pair's rows
+  std::vector<int32_t> kid;                   // kind of every quartet of the list
+  std::vector<std::vector<int64_t>> at;       // per part of the list and kind: where its quartets go
+  // filled by plan_fill
+  int32_t *quartets = nullptr;                // [4 n]
+  int64_t *offsets = nullptr, *pqoff = nullptr, *rowoff = nullptr;   // [n], [n + 1], [nthin + 1] (may be null)
+  CTask *tasks = nullptr;                     // [ntask], quartet by quartet
+  const Run &run_of(int64_t q) const {
+    size_t lo = 0, hi = runs.size() - 1;
+    while (lo < hi) {
+      const size_t mid = (lo + hi + 1) / 2;
+      if (runs[mid].first <= q) lo = mid;
+      else hi = mid - 1;
+    }
+    return runs[lo];
+  }
+  int64_t tfirst(int64_t q) const {
+    if (q >= n) return ntask;
+    const Run &r = run_of(q);
+    return r.task0 + (q - r.first) * r.nsplit;
+  }
 };
 
-// Plans the list hq0 (ho0: output offsets).  fp32(s): the mixed path's choice
-// for quartet s; fewest: as few tasks as fit in shared memory.  Returns
-// F12INT_EINVAL for a shell index out of range.
+// Plans the list hq0.  fp32(s): the mixed path's choice for quartet s; fewest:
+// as few tasks as fit in shared memory.  Returns F12INT_EINVAL for a shell index
+// out of range.  Every quartet of the same kind (types of the four shells, FP32
+// or not) has the same plan: the kinds are planned once, ordered, and the
+// quartets placed run by run in their list order (a counting sort, its passes
+// over the list on several cores when it is long).
 template <class Fp32>
-static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const int32_t *hq0, const int64_t *ho0,
-                     Fp32 fp32, ListPlan &P, bool fewest = false) {
-  // Every quartet with the same (primitive pairs of bra and ket, FP32 or not,
-  // class key) has the same plan: the distinct ones are planned once, ordered,
-  // and the quartets placed group by group in their list order (a counting
-  // sort: linear in n).
+static int plan_kinds(const f12int_ctx::BasisData &B, int cls, int64_t n, const int32_t *hq0, Fp32 fp32, ListPlan &P,
+                      bool fewest = false) {
   struct Kind {
     int64_t key;
     int la, lb, lc, ld, f32;
@@ -1276,11 +1353,78 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
     int tier;
   };
   std::vector<Kind> kinds;
-  std::vector<int32_t> kid((size_t)n);
+  P = ListPlan{};
+  P.n = n;
   const int ns = B.nshell;
+  const int64_t T = (int64_t)B.type_l.size();
   double total = 0.0;   // multiply-adds of the general contraction
-  {
-    std::vector<int64_t> slot_key(4096, -1);   // open-addressing map from a kind's key to its index
+  auto make_kind = [&](int64_t code) {
+    Kind k{};
+    k.key = code;
+    k.f32 = (int)(code & 1);
+    int64_t c = code >> 1;
+    int t[4];
+    for (int i = 3; i >= 0; --i) {
+      t[i] = (int)(c % T);
+      c /= T;
+    }
+    k.la = B.type_l[(size_t)t[0]];
+    k.lb = B.type_l[(size_t)t[1]];
+    k.lc = B.type_l[(size_t)t[2]];
+    k.ld = B.type_l[(size_t)t[3]];
+    k.nab = (int64_t)B.type_nprim[(size_t)t[0]] * B.type_nprim[(size_t)t[1]];
+    k.ncd = (int64_t)B.type_nprim[(size_t)t[2]] * B.type_nprim[(size_t)t[3]];
+    k.thin = thin_quartet(k.la << 6 | k.lb << 4 | k.lc << 2 | k.ld, cls);
+    k.swap = !k.thin && bra_inner(k.la, k.lb, k.lc, k.ld, cls, k.nab, k.ncd);
+    k.shape = contract_shape(k.la, k.lb, k.lc, k.ld, cls, k.swap);
+    if (k.swap) std::swap(k.nab, k.ncd);   // outer, inner
+    kinds.push_back(k);
+  };
+  // code of a quartet, -1 for a shell out of range
+  auto code_of = [&](const int32_t *s) -> int64_t {
+    for (int k = 0; k < 4; ++k)
+      if (s[k] < 0 || s[k] >= ns) return -1;
+    const int *t = B.type.data();
+    const int64_t c = ((t[s[0]] * T + t[s[1]]) * T + t[s[2]]) * T + t[s[3]];
+    const bool thin = thin_quartet(B.l[s[0]] << 6 | B.l[s[1]] << 4 | B.l[s[2]] << 2 | B.l[s[3]], cls);
+    return 2 * c + (thin ? 0 : fp32(s));   // (the thin kernel is FP64)
+  };
+  P.kid.resize((size_t)n);
+  const int parts = n >= 65536 ? 8 : 1;
+  auto part_begin = [&](int t) { return n * t / parts; };
+  const double ncode = 2.0 * (double)T * (double)T * (double)T * (double)T;
+  if (ncode <= std::max(4096.0, 4.0 * (double)n)) {
+    std::vector<unsigned char> seen((size_t)ncode, 0);
+    std::atomic<bool> bad{false};
+    parallel_for(parts, [&](int t) {
+      for (int64_t i = part_begin(t); i < part_begin(t + 1); ++i) {
+        const int64_t c = code_of(hq0 + 4 * i);
+        if (c < 0) {
+          bad = true;
+          return;
+        }
+        P.kid[(size_t)i] = (int32_t)c;
+        if (!__atomic_load_n(&seen[(size_t)c], __ATOMIC_RELAXED)) __atomic_store_n(&seen[(size_t)c], 1, __ATOMIC_RELAXED);
+      }
+    });
+    if (bad) return F12INT_EINVAL;
+    std::vector<int32_t> map((size_t)ncode, -1);
+    for (size_t c = 0; c < seen.size(); ++c)
+      if (seen[c]) {
+        map[c] = (int32_t)kinds.size();
+        make_kind((int64_t)c);
+      }
+    P.at.assign((size_t)parts, std::vector<int64_t>(kinds.size(), 0));
+    parallel_for(parts, [&](int t) {
+      std::vector<int64_t> &cnt = P.at[(size_t)t];
+      for (int64_t i = part_begin(t); i < part_begin(t + 1); ++i) {
+        int32_t &k = P.kid[(size_t)i];
+        k = map[(size_t)k];
+        ++cnt[(size_t)k];
+      }
+    });
+  } else {   // a short list of many types of shells: open-addressing map from code to kind
+    std::vector<int64_t> slot_key(4096, -1);
     std::vector<int32_t> slot_val(4096, -1);
     size_t mask = slot_key.size() - 1;
     auto find = [&](const std::vector<int64_t> &keys, size_t m, int64_t key) {
@@ -1289,13 +1433,8 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
       return h;
     };
     for (int64_t i = 0; i < n; ++i) {
-      const int32_t *s = hq0 + 4 * i;
-      for (int k = 0; k < 4; ++k)
-        if (s[k] < 0 || s[k] >= ns) return F12INT_EINVAL;
-      const int lk = (B.l[s[0]] << 6) | (B.l[s[1]] << 4) | (B.l[s[2]] << 2) | B.l[s[3]];
-      const int64_t nab = (int64_t)B.nprim[s[0]] * B.nprim[s[1]], ncd = (int64_t)B.nprim[s[2]] * B.nprim[s[3]];
-      const int f32 = thin_quartet(lk, cls) ? 0 : fp32(s);   // the thin kernel is FP64
-      const int64_t key = (((nab << 26) + ncd) << 9) | (f32 << 8) | lk;
+      const int64_t key = code_of(hq0 + 4 * i);
+      if (key < 0) return F12INT_EINVAL;
       size_t h = find(slot_key, mask, key);
       if (slot_key[h] == -1) {
         if (kinds.size() * 2 >= slot_key.size()) {   // grow and rehash
@@ -1312,27 +1451,19 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
           mask = slot_key.size() - 1;
           h = find(slot_key, mask, key);
         }
-        Kind k{};
-        k.key = key;
-        k.la = lk >> 6;
-        k.lb = (lk >> 4) & 3;
-        k.lc = (lk >> 2) & 3;
-        k.ld = lk & 3;
-        k.f32 = f32;
-        k.nab = nab;
-        k.ncd = ncd;
-        k.thin = thin_quartet(lk, cls);
-        k.swap = !k.thin && bra_inner(k.la, k.lb, k.lc, k.ld, cls, nab, ncd);
-        k.shape = contract_shape(k.la, k.lb, k.lc, k.ld, cls, k.swap);
-        if (k.swap) std::swap(k.nab, k.ncd);   // outer, inner
         slot_key[h] = key;
         slot_val[h] = (int32_t)kinds.size();
-        kinds.push_back(k);
+        make_kind(key);
       }
-      kid[(size_t)i] = slot_val[h];
-      kinds[(size_t)slot_val[h]].count++;
+      P.kid[(size_t)i] = slot_val[h];
     }
+    P.at.assign((size_t)parts, std::vector<int64_t>(kinds.size(), 0));
+    parallel_for(parts, [&](int t) {
+      for (int64_t i = part_begin(t); i < part_begin(t + 1); ++i) ++P.at[(size_t)t][(size_t)P.kid[(size_t)i]];
+    });
   }
+  for (size_t k = 0; k < kinds.size(); ++k)
+    for (const auto &c : P.at) kinds[k].count += c[k];
   for (const Kind &k : kinds)
     if (!k.thin) total += (double)k.count * (double)(k.nab * k.ncd) * task_fmas(k.shape, k.ncd, k.shape.ncd());
   // about a dozen tasks per SM where the list has the work for it (a block's
@@ -1355,7 +1486,7 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
   std::sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
     const Kind &a = kinds[(size_t)x], &b = kinds[(size_t)y];
     if (a.thin != b.thin) return b.thin;
-    const int ka = (int)(a.key & 0xFF), kb = (int)(b.key & 0xFF);
+    const int ka = a.la << 6 | a.lb << 4 | a.lc << 2 | a.ld, kb = b.la << 6 | b.lb << 4 | b.lc << 2 | b.ld;
     if (a.thin) return ka != kb ? ka < kb : (a.work != b.work ? a.work > b.work : a.key < b.key);
     if (a.f32 != b.f32) return a.f32 < b.f32;
     if (a.tier != b.tier) return a.tier > b.tier;
@@ -1363,12 +1494,11 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
     if (a.work != b.work) return a.work > b.work;
     return a.key < b.key;
   });
-  P = ListPlan{};
-  P.n = n;
   int64_t run = 0;
+  std::vector<int32_t> place(kinds.size());   // kind -> run
   for (size_t at = 0; at < order.size(); ++at) {
     Kind &k = kinds[(size_t)order[at]];
-    const int thin = k.thin ? (int)(k.key & 0xFF) : -1;
+    const int thin = k.thin ? k.la << 6 | k.lb << 4 | k.lc << 2 | k.ld : -1;
     if (P.groups.empty() || P.groups.back().thin != thin ||
         (!k.thin && (P.groups.back().fp32 != (k.f32 != 0) || P.groups.back().nthr != k.pl.nthr ||
                      kinds[(size_t)order[at - 1]].tier != k.tier)))
@@ -1376,44 +1506,74 @@ static int plan_list(const f12int_ctx::BasisData &B, int cls, int64_t n, const i
     ListPlan::Group &G = P.groups.back();
     G.smem = std::max(G.smem, k.pl.smem);
     k.first = run;
+    ListPlan::Run r{};
+    r.first = run;
+    r.count = k.count;
+    r.npq = k.nab * k.ncd;
+    r.npab = k.nab;
+    r.pitch = k.thin ? 0 : r.npq * row_pitch(k.shape.L());
+    r.pq0 = P.npq;
+    r.row0 = P.nrow;
+    r.task0 = P.ntask;
+    r.nsplit = k.pl.nsplit;
+    r.swap = k.swap;
+    r.thin = k.thin;
+    place[(size_t)order[at]] = (int32_t)P.runs.size();
+    P.runs.push_back(r);
     run += k.count;
+    P.npq += k.count * r.npq;
+    P.nrow += k.count * r.pitch;
+    P.ntask += k.count * r.nsplit;
+    P.big_pq = std::max(P.big_pq, r.npq);
+    if (!k.thin) P.big_row = std::max(P.big_row, r.pitch / r.npab);
     G.end = run;
     if (!k.thin) P.nthin = run;
   }
-  std::vector<int64_t> perm((size_t)n);
-  {
-    std::vector<int64_t> at(kinds.size());
-    for (size_t g = 0; g < kinds.size(); ++g) at[g] = kinds[g].first;
-    for (int64_t i = 0; i < n; ++i) perm[(size_t)at[(size_t)kid[(size_t)i]]++] = i;
-  }
-  P.quartets.resize((size_t)4 * n);
-  P.offsets.resize((size_t)n);
-  P.pqoff.resize((size_t)n + 1);
-  P.tfirst.resize((size_t)n + 1);
-  P.rowoff.resize((size_t)P.nthin + 1);
-  P.npab.resize((size_t)P.nthin);
-  P.tasks.reserve((size_t)n);
-  int64_t npq = 0, nrow = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    const int64_t j = perm[(size_t)i];
-    const Kind &k = kinds[(size_t)kid[(size_t)j]];
-    for (int c = 0; c < 4; ++c) P.quartets[(size_t)(4 * i + c)] = hq0[4 * j + (k.swap ? c ^ 2 : c)];
-    P.offsets[(size_t)i] = ho0[j];
-    P.pqoff[(size_t)i] = npq;
-    npq += k.nab * k.ncd;
-    if (!k.thin) {
-      P.rowoff[(size_t)i] = nrow;
-      P.npab[(size_t)i] = (int)k.nab;
-      nrow += k.nab * k.ncd * row_pitch(k.la + k.lb + k.lc + k.ld + (cls == 5 ? 2 : 0));
+  // where each part of the list puts its quartets of a kind
+  for (size_t k = 0; k < kinds.size(); ++k) {
+    int64_t pos = kinds[k].first;
+    for (auto &c : P.at) {
+      const int64_t cnt = c[k];
+      c[k] = pos;
+      pos += cnt;
     }
-    P.tfirst[(size_t)i] = (int64_t)P.tasks.size();
-    const int16_t mark = (int16_t)(k.swap ? -k.pl.nsplit : k.pl.nsplit);
-    for (int sp = 0; sp < k.pl.nsplit; ++sp) P.tasks.push_back(CTask{(int32_t)i, (int16_t)sp, mark});
   }
-  P.pqoff[(size_t)n] = npq;
-  P.rowoff[(size_t)P.nthin] = nrow;
-  P.tfirst[(size_t)n] = (int64_t)P.tasks.size();
+  // (the arrays stay by kind: runs of a kind are found through place)
+  {
+    std::vector<ListPlan::Run> by_kind(P.runs.size());
+    for (size_t k = 0; k < kinds.size(); ++k) by_kind[k] = P.runs[(size_t)place[k]];
+    P.kind_run.swap(by_kind);
+  }
   return F12INT_OK;
+}
+
+// Writes the planned list into the caller's arrays.
+static void plan_fill(ListPlan &P, const int32_t *hq0, const int64_t *ho0, int32_t *quartets, int64_t *offsets,
+                      int64_t *pqoff, int64_t *rowoff, CTask *tasks) {
+  P.quartets = quartets;
+  P.offsets = offsets;
+  P.pqoff = pqoff;
+  P.rowoff = rowoff;
+  P.tasks = tasks;
+  const int parts = (int)P.at.size();
+  parallel_for(parts, [&](int t) {
+    std::vector<int64_t> &at = P.at[(size_t)t];
+    for (int64_t i = P.n * t / parts; i < P.n * (t + 1) / parts; ++i) {
+      const size_t k = (size_t)P.kid[(size_t)i];
+      const ListPlan::Run &r = P.kind_run[k];
+      const int64_t q = at[k]++, in = q - r.first;
+      const int flip = r.swap ? 2 : 0;
+      for (int c = 0; c < 4; ++c) quartets[4 * q + c] = hq0[4 * i + (c ^ flip)];
+      offsets[q] = ho0[i];
+      pqoff[q] = r.pq0 + in * r.npq;
+      if (rowoff && !r.thin) rowoff[q] = r.row0 + in * r.pitch;
+      CTask *tk = tasks + r.task0 + in * r.nsplit;
+      const int16_t mark = (int16_t)(r.swap ? -r.nsplit : r.nsplit);
+      for (int sp = 0; sp < r.nsplit; ++sp) tk[sp] = CTask{(int32_t)q, (int16_t)sp, mark};
+    }
+  });
+  pqoff[P.n] = P.npq;
+  if (rowoff) rowoff[P.nthin] = P.nrow;
 }
 
 // Device arrays that a planned list runs with.
@@ -1502,7 +1662,7 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
       if (!kern) return F12INT_EINVAL;
       const int64_t nt = b - a;   // one task each
       kern<<<(unsigned)((nt + kThinWarps - 1) / kThinWarps), 32 * kThinWarps, 0, side()>>>(
-          PV, QV, direct ? 1 : nf, pq0, G, D.tasks + P.tfirst[(size_t)a], nt, nullptr, D.keys, D.part, out_dev,
+          PV, QV, direct ? 1 : nf, pq0, G, D.tasks + P.tfirst(a), nt, nullptr, D.keys, D.part, out_dev,
           D.offsets, fma_con);
       ctx->launches++;
       CK(cudaGetLastError());
@@ -1515,7 +1675,7 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
     for (const ListPlan::Group &g : P.groups) {
       const int64_t a = std::max(qa, g.first), b = std::min(qb, g.end);
       if (g.thin >= 0 || a >= b) continue;
-      const int64_t t0 = P.tfirst[(size_t)a], nt = P.tfirst[(size_t)b] - t0;
+      const int64_t t0 = P.tfirst(a), nt = P.tfirst(b) - t0;
       const auto kern = g.fp32 ? k_contract<false, float> : k_contract<false, double>;
       if (g.smem > 48 * 1024)
         CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
@@ -1557,34 +1717,29 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
     }
   }
   const int thin_used = used;   // side streams that still carry thin launches
-  // first double of the rows of primitive quartet pq (of quartet q) in the list's order
-  auto row_of = [&](int64_t q, int64_t pq) -> int64_t {
-    if (D.pitch) return pq * D.pitch;
-    const int64_t npq = P.pqoff[(size_t)q + 1] - P.pqoff[(size_t)q];
-    return npq ? P.rowoff[(size_t)q] + (P.rowoff[(size_t)q + 1] - P.rowoff[(size_t)q]) / npq * (pq - P.pqoff[(size_t)q])
-               : P.rowoff[(size_t)q];
-  };
-  auto row_end = [&](int64_t q) -> int64_t { return D.pitch ? P.pqoff[(size_t)q + 1] * D.pitch : P.rowoff[(size_t)q + 1]; };
+  // first double of the rows of quartet q, and their end, in the list's order
+  auto row_of = [&](int64_t q) -> int64_t { return D.pitch ? P.pqoff[q] * D.pitch : P.rowoff[q]; };
+  auto row_end = [&](int64_t q) -> int64_t { return D.pitch ? P.pqoff[q + 1] * D.pitch : P.rowoff[q + 1]; };
   const int64_t per_pq = (int64_t)std::max(nf, 1) * kPartPitch;
   const int64_t fit = direct ? (int64_t)1 << 60 : D.part_cap / per_pq;          // primitive quartets whose items fit
   int64_t part0 = 0, part1 = 0;   // family path: primitive quartets whose items are in D.part
   for (int64_t qa = 0; qa < P.nthin && rc == F12INT_OK;) {
-    const int64_t pq0 = P.pqoff[(size_t)qa], npq = P.pqoff[(size_t)qa + 1] - pq0, row0 = row_of(qa, pq0);
+    const int64_t pq0 = P.pqoff[qa], npq = P.pqoff[qa + 1] - pq0, row0 = row_of(qa);
     const bool fits = row_end(qa) - row0 <= D.rows_cap && npq <= fit && (!direct || npq <= D.keys_cap);
     if (fits) {
       if (!direct && pq0 >= part1) {   // items of as many quartets as fit
         int64_t qe = qa + 1;
-        while (qe < P.nthin && P.pqoff[(size_t)qe + 1] - pq0 <= fit) ++qe;
+        while (qe < P.nthin && P.pqoff[qe + 1] - pq0 <= fit) ++qe;
         part0 = pq0;
-        part1 = P.pqoff[(size_t)qe];
+        part1 = P.pqoff[qe];
         rc = items(part0, part1);
         if (rc != F12INT_OK) break;
       }
       int64_t qb = qa + 1;
       while (qb < P.nthin && row_end(qb) - row0 <= D.rows_cap &&
-             (direct ? P.pqoff[(size_t)qb + 1] - pq0 <= D.keys_cap : P.pqoff[(size_t)qb + 1] <= part1))
+             (direct ? P.pqoff[qb + 1] - pq0 <= D.keys_cap : P.pqoff[qb + 1] <= part1))
         ++qb;
-      rc = hermite(pq0, P.pqoff[(size_t)qb], row0, part0);
+      rc = hermite(pq0, P.pqoff[qb], row0, part0);
       if (rc == F12INT_OK && !fork()) rc = F12INT_ECUDA;
       if (rc != F12INT_OK) break;
       time_begin();
@@ -1595,13 +1750,13 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
       continue;
     }
     // one quartet larger than the scratch: a few of its bra primitive pairs at a time
-    const int npab = P.npab[(size_t)qa];
+    const int64_t npab = P.run_of(qa).npab;
     const int64_t npcd = npq / npab, per = (row_end(qa) - row0) / npab;   // doubles of one bra pair's rows
     int64_t step = std::min<int64_t>(D.rows_cap / per, fit / npcd);
     if (direct) step = std::min<int64_t>(step, D.keys_cap / npcd);
     if (step < 1) return F12INT_ENOMEM;
     for (int64_t i0 = 0; i0 < npab && rc == F12INT_OK; i0 += step) {
-      const int64_t i1 = std::min<int64_t>(npab, i0 + step), a = pq0 + i0 * npcd, b = pq0 + i1 * npcd;
+      const int64_t i1 = std::min(npab, i0 + step), a = pq0 + i0 * npcd, b = pq0 + i1 * npcd;
       if (!direct) rc = items(a, b);
       if (rc == F12INT_OK) rc = hermite(a, b, row0 + i0 * per, a);
       if (rc == F12INT_OK && !fork()) rc = F12INT_ECUDA;
@@ -1615,11 +1770,11 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
     ++qa;
   }
   for (int64_t qa = P.nthin; !direct && qa < P.n && rc == F12INT_OK;) {   // family path: the thin quartets
-    const int64_t pq0 = P.pqoff[(size_t)qa], most = D.part_thin / per_pq;
+    const int64_t pq0 = P.pqoff[qa], most = D.part_thin / per_pq;
     int64_t qb = qa + 1;
-    while (qb < P.n && P.pqoff[(size_t)qb + 1] - pq0 <= most) ++qb;
-    if (P.pqoff[(size_t)qb] - pq0 > most) return F12INT_ENOMEM;
-    rc = items(pq0, P.pqoff[(size_t)qb]);
+    while (qb < P.n && P.pqoff[qb + 1] - pq0 <= most) ++qb;
+    if (P.pqoff[qb] - pq0 > most) return F12INT_ENOMEM;
+    rc = items(pq0, P.pqoff[qb]);
     if (rc == F12INT_OK && !fork()) rc = F12INT_ECUDA;
     if (rc != F12INT_OK) break;
     time_begin();
@@ -1784,47 +1939,42 @@ static int compute_class_impl(f12int_ctx *ctx, int basis_id, int cls, const int3
   NvtxRange call_range("f12int.compute_class");
   const auto t_plan0 = std::chrono::steady_clock::now();
   std::unique_ptr<NvtxRange> plan_range(new NvtxRange("f12int.plan"));
-  std::vector<int32_t> hq0((size_t)4 * n);
-  std::vector<int64_t> ho0((size_t)n);
-  CK(cudaMemcpyAsync(hq0.data(), quartets_dev, sizeof(int32_t) * 4 * n, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(ho0.data(), offsets_dev, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, st));
+  // host staging: the list as given, then as planned (one copy each way)
+  HostStage &hs = ctx->stage;
+  if (!hs.reserve(24 * (size_t)n)) return F12INT_ENOMEM;
+  CK(cudaMemcpyAsync(hs.p, quartets_dev, sizeof(int32_t) * 4 * n, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(hs.p + 16 * n, offsets_dev, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   ListPlan P;
   // mixed path: FP32 Hermite recursion and contraction below the bound
-  int rc = plan_list(B, cls, n, hq0.data(), ho0.data(), [&](const int32_t *s) {
+  int rc = plan_kinds(B, cls, n, (const int32_t *)hs.p, [&](const int32_t *s) {
     return fp32_below > 0.0 && screen_estimate(ctx, B, cls, s[0], s[1], s[2], s[3]) < fp32_below ? 1 : 0;
   }, P);
   if (rc != F12INT_OK) return rc;
+  const ListLayout at(n, P.nthin, P.ntask);
+  if (!hs.reserve(24 * (size_t)n + at.bytes, 24 * (size_t)n)) return F12INT_ENOMEM;
+  unsigned char *list = hs.p + 24 * (size_t)n;
+  plan_fill(P, (const int32_t *)hs.p, (const int64_t *)(hs.p + 16 * n), (int32_t *)list, (int64_t *)(list + at.offsets),
+            (int64_t *)(list + at.pqoff), (int64_t *)(list + at.rowoff), (CTask *)(list + at.tasks));
   const GridView G = grid_view(ctx, B, cls);
   const int64_t nf = std::max(1, ctx->tables.nfam[cls == 5 ? 3 : cls]);
-  const int64_t npq = P.pqoff[(size_t)n], npq_gen = P.pqoff[(size_t)P.nthin];
-  int64_t big_pq = 1, big_thin = 1, big_row = 1;   // largest quartet, thin quartet, bra pair's rows
-  for (int64_t i = 0; i < n; ++i) {
-    const int64_t k = P.pqoff[(size_t)i + 1] - P.pqoff[(size_t)i];
-    if (i < P.nthin) {
-      big_pq = std::max(big_pq, k);
-      big_row = std::max(big_row, (P.rowoff[(size_t)i + 1] - P.rowoff[(size_t)i]) / P.npab[(size_t)i]);
-    } else {
-      big_thin = std::max(big_thin, k);
-    }
-  }
-  rc = ensure_buf(ctx, (void **)&ctx->d_pqoff, &ctx->pqoff_cap, sizeof(int64_t) * ((size_t)n + 1));
-  if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_qperm, &ctx->qperm_cap, sizeof(int32_t) * 4 * n);
-  if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_operm, &ctx->operm_cap, sizeof(int64_t) * n);
-  if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_rowoff, &ctx->rowoff_cap, sizeof(int64_t) * P.rowoff.size());
-  if (rc == F12INT_OK) rc = ensure_buf(ctx, (void **)&ctx->d_tasks, &ctx->tasks_cap, sizeof(CTask) * P.tasks.size());
+  const int64_t npq = P.npq, npq_gen = P.pqoff[P.nthin];
+  const int64_t big_pq = P.big_pq, big_row = P.big_row;   // largest quartet, bra pair's rows
+  rc = ensure_buf(ctx, (void **)&ctx->d_list, &ctx->list_cap, at.bytes);
   if (rc != F12INT_OK) return rc;
-  ListBufs D{ctx->d_qperm, ctx->d_operm, ctx->d_pqoff, ctx->d_rowoff, ctx->d_tasks};
+  ListBufs D{(const int32_t *)ctx->d_list, (const int64_t *)(ctx->d_list + at.offsets),
+             (const int64_t *)(ctx->d_list + at.pqoff), (const int64_t *)(ctx->d_list + at.rowoff),
+             (const CTask *)(ctx->d_list + at.tasks)};
   // scratch of one chunk: Hermite rows to kRowChunk doubles, on the family path
   // also the items; under a budget no more than an item per family would take
-  const int64_t all_rows = P.rowoff[(size_t)P.nthin];
+  const int64_t all_rows = P.nrow;
   if (G.direct()) {
     int64_t want = std::min(all_rows, kRowChunk);
     if (ctx->budget) want = std::min(want, npq * nf * 17);
     D.rows_cap = std::max(want, all_rows ? big_row : 0);
     D.keys_cap = std::min(npq_gen, std::max(D.rows_cap / 36 + 1, big_pq));
   } else {
-    D.part_cap = std::min(npq, std::max(std::max(big_pq, big_thin), kItemChunk / nf)) * nf * kPartPitch;
+    D.part_cap = std::min(npq, std::max(big_pq, kItemChunk / nf)) * nf * kPartPitch;
     D.part_thin = D.part_cap;
     D.keys_cap = D.part_cap / kPartPitch;
     D.rows_cap = std::max(std::min(all_rows, kRowChunk / 4), all_rows ? big_row : 0);
@@ -1846,17 +1996,13 @@ static int compute_class_impl(f12int_ctx *ctx, int basis_id, int cls, const int3
   D.hist = ctx->d_hist;
   D.part = ctx->d_part;
   D.rows = ctx->d_rows;
-  CK(cudaMemcpyAsync(ctx->d_pqoff, P.pqoff.data(), sizeof(int64_t) * P.pqoff.size(), cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(ctx->d_qperm, P.quartets.data(), sizeof(int32_t) * 4 * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(ctx->d_operm, P.offsets.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(ctx->d_rowoff, P.rowoff.data(), sizeof(int64_t) * P.rowoff.size(), cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(ctx->d_tasks, P.tasks.data(), sizeof(CTask) * P.tasks.size(), cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(ctx->d_list, list, at.bytes, cudaMemcpyHostToDevice, st));
   plan_range.reset();
   ctx->plan_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_plan0).count();
   ctx->plan_calls++;
   rc = launch_list(ctx, P, D, pair_view(ctx, B, cls, B.prim_screen && prim_screen), G, cls, out_dev, st, ctx->timing);
   if (rc != F12INT_OK) {
-    cudaStreamSynchronize(st);   // the queued copies read this call's vectors
+    cudaStreamSynchronize(st);   // the queued copies read the staging buffer
     for (cudaStream_t t : ctx->side) cudaStreamSynchronize(t);
     return rc;
   }
@@ -2075,14 +2221,14 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
 
   const f12int_ctx::BasisData &B = ctx->bases[basis_id];
   cudaStream_t st = pick_stream(ctx, cuda_stream);
-  std::vector<int32_t> hq0((size_t)4 * n);
-  std::vector<int64_t> ho0((size_t)n);
-  CK(cudaMemcpyAsync(hq0.data(), quartets_dev, sizeof(int32_t) * 4 * n, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(ho0.data(), offsets_dev, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, st));
+  HostStage &hs = ctx->stage;
+  if (!hs.reserve(24 * (size_t)n)) return F12INT_ENOMEM;
+  CK(cudaMemcpyAsync(hs.p, quartets_dev, sizeof(int32_t) * 4 * n, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(hs.p + 16 * n, offsets_dev, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   ListPlan P;
   auto fp64 = [](const int32_t *) { return 0; };
-  rc = plan_list(B, cls, n, hq0.data(), ho0.data(), fp64, P);
+  rc = plan_kinds(B, cls, n, (const int32_t *)hs.p, fp64, P);
   if (rc != F12INT_OK) return rc;
   // layout of the array: quartets, offsets and primitive offsets in the
   // working order, the key histogram and the task list (all sized exactly
@@ -2092,21 +2238,19 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
   auto fixed_bytes = [&] {
     return align256(sizeof(int32_t) * 4 * (size_t)n) + align256(sizeof(int64_t) * (size_t)n) +
            align256(sizeof(int64_t) * ((size_t)n + 1)) + align256(sizeof(unsigned) * kNKeys) +
-           align256(sizeof(CTask) * P.tasks.size());
+           align256(sizeof(CTask) * (size_t)P.ntask);
   };
   // one chunk at least: the items of every quartet on its own, and the rows of
   // one of its bra primitive pairs
   const int64_t nf = std::max(1, ctx->tables.nfam[cls == 5 ? 3 : cls]);
   const GridView G = grid_view(ctx, B, cls);
-  int64_t big_pq = 1, pitch = 4, big_cd = 1;
-  for (int64_t i = 0; i < n; ++i) {
-    const int64_t k = P.pqoff[(size_t)i + 1] - P.pqoff[(size_t)i];
-    big_pq = std::max(big_pq, k);
-    if (i < P.nthin && k > 0) {
-      big_cd = std::max(big_cd, k / P.npab[(size_t)i]);
-      pitch = std::max(pitch, (P.rowoff[(size_t)i + 1] - P.rowoff[(size_t)i]) / k);
+  int64_t pitch = 4, big_cd = 1;
+  const int64_t big_pq = P.big_pq;
+  for (const ListPlan::Run &r : P.runs)
+    if (!r.thin) {
+      big_cd = std::max(big_cd, r.npq / r.npab);
+      pitch = std::max(pitch, r.pitch / r.npq);
     }
-  }
   auto room = [&]() -> int64_t {   // bytes of the chunk's scratch, negative when the list does not fit
     return (int64_t)F12INT_STATIC_SCRATCH_BYTES - (int64_t)fixed_bytes() - 4 * 256;
   };
@@ -2115,16 +2259,21 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
     return r >= big_pq * nf * (int64_t)item_bytes && r >= big_cd * (nf * (int64_t)item_bytes + pitch * 8 + 64);
   };
   if (!enough()) {   // fewer and longer tasks leave more of the array
-    rc = plan_list(B, cls, n, hq0.data(), ho0.data(), fp64, P, /*fewest=*/true);
+    rc = plan_kinds(B, cls, n, (const int32_t *)hs.p, fp64, P, /*fewest=*/true);
     if (rc != F12INT_OK) return rc;
     if (!enough()) return F12INT_EINVAL;
   }
+  const ListLayout at(n, 0, P.ntask);   // (no row offsets: every row at one pitch)
+  if (!hs.reserve(24 * (size_t)n + at.bytes, 24 * (size_t)n)) return F12INT_ENOMEM;
+  unsigned char *list = hs.p + 24 * (size_t)n;
+  plan_fill(P, (const int32_t *)hs.p, (const int64_t *)(hs.p + 16 * n), (int32_t *)list, (int64_t *)(list + at.offsets),
+            (int64_t *)(list + at.pqoff), nullptr, (CTask *)(list + at.tasks));
   int32_t *d_q = (int32_t *)base;
   int64_t *d_o = (int64_t *)(base + align256(sizeof(int32_t) * 4 * (size_t)n));
   int64_t *d_pq = (int64_t *)((unsigned char *)d_o + align256(sizeof(int64_t) * (size_t)n));
   unsigned *d_hist = (unsigned *)((unsigned char *)d_pq + align256(sizeof(int64_t) * ((size_t)n + 1)));
   CTask *d_tk = (CTask *)((unsigned char *)d_hist + align256(sizeof(unsigned) * kNKeys));
-  unsigned char *scratch = (unsigned char *)d_tk + align256(sizeof(CTask) * P.tasks.size());
+  unsigned char *scratch = (unsigned char *)d_tk + align256(sizeof(CTask) * (size_t)P.ntask);
   ListBufs D{d_q, d_o, d_pq, nullptr, d_tk};
   D.pitch = (int)pitch;
   D.hist = d_hist;
@@ -2147,16 +2296,16 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
     D.part_cap = (D.part_thin - D.rows_cap) & ~(int64_t)15;
     D.rows = D.part + D.part_cap;
   }
-  CK(cudaMemcpyAsync(d_tk, P.tasks.data(), sizeof(CTask) * P.tasks.size(), cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(d_q, P.quartets.data(), sizeof(int32_t) * 4 * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(d_o, P.offsets.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(d_pq, P.pqoff.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(d_tk, P.tasks, sizeof(CTask) * (size_t)P.ntask, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(d_q, P.quartets, sizeof(int32_t) * 4 * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(d_o, P.offsets, sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(d_pq, P.pqoff, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
   // the primitive screen of f12int_compute_class when its table for this
   // (basis, class) exists already (building it would allocate); without it
   // every primitive quartet is evaluated
   const int rc_launch = launch_list(ctx, P, D, pair_view(ctx, B, cls, B.prim_screen), G, cls, out_dev, st, false);
-  // the host vectors above stay alive until the queued copies are consumed,
-  // and on an error nothing of this call is still running when it returns
+  // the staging buffer is free again once the queued copies are consumed, and
+  // on an error nothing of this call is still running when it returns
   cudaError_t e = cudaStreamSynchronize(st);
   if (rc_launch != F12INT_OK)
     for (cudaStream_t t : ctx->side) cudaStreamSynchronize(t);
