@@ -563,10 +563,18 @@ static double task_fmas(const ContractShape &s, int64_t npcd, int jc) {
 
 // Whether (ab|cd), with npab and npcd primitive pairs, is cheaper with the bra
 // inner (listed as (cd|ab)): on the 12-atom s/p/d workload this takes 28% off
-// the multiply-adds of the contraction, on f shells up to 44%.
+// the multiply-adds of the contraction, on f shells up to 44%.  Entries count
+// by whole warps (a sum of ten entries costs as much as one of 32).
 static bool bra_inner(int la, int lb, int lc, int ld, int cls, int64_t npab, int64_t npcd) {
   const ContractShape k{la, lb, lc, ld, cls == 5 ? 2 : 0, false}, b{lc, ld, la, lb, cls == 5 ? 2 : 0, cls == 5};
-  return task_fmas(b, npab, b.ncd()) < task_fmas(k, npcd, k.ncd());
+  auto cost = [](const ContractShape &s, int64_t nin) {
+    const int e = s.nhB() * s.ncd(), o = s.nab() * s.ncd();
+    const double pe = (double)((e + 31) / 32 * 32) / e, po = (double)((o + 31) / 32 * 32) / o;
+    const PairTab &K = pair_tabs().pt[s.lc * 4 + s.ld], &B = pair_tabs().pt[s.la * 4 + s.lb];
+    return pe * s.nhB() * K.nterm * (s.inner4() == 4 ? 6 : 1) +
+           po * s.ncd() * B.nterm * (s.outer4() == 4 ? 6 : 1) / (double)nin;
+  };
+  return cost(b, npab) < cost(k, npcd);
 }
 static ContractShape contract_shape(int la, int lb, int lc, int ld, int cls, bool swap) {
   return swap ? ContractShape{lc, ld, la, lb, cls == 5 ? 2 : 0, cls == 5}
@@ -590,9 +598,12 @@ static size_t contract_smem(const ContractShape &s, int64_t npcd, int nsplit, si
   return (fixed + k * per + 15) & ~(size_t)15;
 }
 
-// Soft limit of a block's shared memory (four blocks an SM), and what it may
-// take when even one staged pair does not fit that.
-constexpr size_t kSmemSoft = 54 * 1024, kSmemSplit = 72 * 1024, kSmemMax = 200 * 1024;
+// Soft limit of a block's shared memory, 16 warps an SM: four blocks of 128
+// threads, in proportion for fewer (blocks of one warp that staged 54 KB left
+// the FP64 pipe idle 80% of the time); and what a block may take when even one
+// staged pair does not fit that.
+static size_t smem_soft(int nthr) { return (size_t)54 * 1024 * (size_t)std::min(nthr, 128) / 128; }
+constexpr size_t kSmemSplit = 72 * 1024, kSmemMax = 200 * 1024;
 
 // Fewest ranges with which a block fits `cap`; 0: none.
 static int fit_split(const ContractShape &s, size_t esz, size_t cap) {
@@ -629,7 +640,7 @@ static ContractPlan contract_plan(const ContractShape &s, int64_t nprimq, int64_
     }
     if (t >= e) break;
   }
-  return ContractPlan{nthr, ns, contract_smem(s, npcd, ns, esz, kSmemSoft)};
+  return ContractPlan{nthr, ns, contract_smem(s, npcd, ns, esz, smem_soft(nthr))};
 }
 
 }  // namespace

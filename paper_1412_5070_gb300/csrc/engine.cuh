@@ -24,7 +24,7 @@ constexpr double kTaskFlops = 5e7;
 // contraction tiers: threads and shared memory of a block
 constexpr int kTiers = 6;                // per precision
 constexpr int kTierThreads[kTiers] = {32, 64, 96, 192, 256, 256};
-constexpr size_t kTierCap[kTiers] = {24 * 1024, 36 * 1024, 54 * 1024, 54 * 1024, 72 * 1024, 200 * 1024};
+constexpr size_t kTierCap[kTiers] = {14 * 1024, 28 * 1024, 42 * 1024, 54 * 1024, 72 * 1024, 200 * 1024};
 constexpr int kLaunches = 2 * kTiers;     // FP64 tiers, then FP32 tiers (mixed requests)
 constexpr int kThinSlot = kLaunches;      // then the thin contraction (total order <= 3, I5 <= 2), one
 constexpr int kSlots = kLaunches + kThinKeys;   // launch per (la, lb, lc, ld)
