@@ -451,10 +451,11 @@ F12_DEV inline void grid_eval(const double *cells, const GridPoint &pt, int L, d
   constexpr int NMAX = grid_terms(LMAX);
   const int N = FIXED ? NMAX : grid_terms(L);
   const double *cell = cells + (size_t)(pt.cell < 0 ? 0 : pt.cell) * GR_CELL;
-  double w[NMAX + 1];
-  w[0] = 1.0;
+  // rows, highest first, into the orders' Horner sums
+  //   h_l = H_l + t_1 (H_{l+1} + t_2 (H_{l+2} + ..)),  t_k = hd/k
+  double t[NMAX + 1];
 #pragma unroll
-  for (int k = 1; k <= NMAX; ++k) w[k] = w[k - 1] * (pt.hd * (1.0 / k));
+  for (int k = 1; k <= NMAX; ++k) t[k] = pt.hd * (1.0 / k);
 #pragma unroll
   for (int l = 0; l <= LMAX; ++l) h[l] = 0.0;
 #pragma unroll
@@ -471,8 +472,11 @@ F12_DEV inline void grid_eval(const double *cells, const GridPoint &pt, int L, d
     for (int i = GR_NC - 1; i >= 0; --i)
       if (i < nc) r = i == nc - 1 ? c[i] : fma(r, pt.a, c[i]);
 #pragma unroll
-    for (int l = 0; l <= LMAX; ++l)
-      if (m - l >= 0 && m - l <= NMAX && (FIXED || (l <= L && m - l <= N))) h[l] = fma(r, w[m - l], h[l]);
+    for (int l = 0; l <= LMAX; ++l) {
+      const int k = m - l;   // the row's term of order l
+      if (k < 0 || k > NMAX || (!FIXED && (l > L || k > N))) continue;
+      h[l] = k == (FIXED ? NMAX : N) ? r : fma(h[l], t[k + 1 <= NMAX ? k + 1 : NMAX], r);
+    }
   }
 }
 

@@ -231,8 +231,10 @@ k_hermite_rows(GridView G, PairView PV0, QuartetView QV, int cls, int nf, int64_
     const int npcd = PV.pair_start[cd + 1] - PV.pair_start[cd];
     const int k = (int)(pq - QV.pq_off[lo]);
     const int pab = PV.pair_start[ab] + k / npcd, pcd = PV.pair_start[cd] + k % npcd;
+    const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
+                 Z = pair_sep(PV.pp_P, pab, pcd, 2);
     if constexpr (DIRECT) {
-      if (prim_negligible(PV, pab, pcd)) {
+      if (prim_negligible(PV, pab, pcd, X * X + Y * Y + Z * Z)) {
         keys[r] = SKIP_KEY;
         continue;
       }
@@ -241,8 +243,6 @@ k_hermite_rows(GridView G, PairView PV0, QuartetView QV, int cls, int nf, int64_
       continue;
     }
     const int L = PV.shell_l[s[0]] + PV.shell_l[s[1]] + PV.shell_l[s[2]] + PV.shell_l[s[3]] + (cls == 5 ? 2 : 0);
-    const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
-                 Z = pair_sep(PV.pp_P, pab, pcd, 2);
     double *o = rows.quartet(QV, lo) + (int64_t)k * rows.stride(row_pitch(L));
     if constexpr (DIRECT) {
       nfma += aux_direct_fmas(G.boys != nullptr, L);

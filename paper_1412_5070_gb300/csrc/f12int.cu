@@ -169,7 +169,7 @@ __device__ __forceinline__ int64_t find_quartet(const int64_t *off, int64_t n, i
 
 // Work items of the auxiliary stage: item = (primitive quartet of the chunk) * nf + family.
 struct ItemGeom {
-  double xi, D;
+  double xi, D, u;
   int L;
   int iab, icd;
   const PairView *pv;
@@ -193,7 +193,8 @@ __device__ __forceinline__ ItemGeom item_geometry(const PairView &PV0, const Qua
   g.L = PV.shell_l[s[0]] + PV.shell_l[s[1]] + PV.shell_l[s[2]] + PV.shell_l[s[3]] + (cls == 5 ? 2 : 0);
   double p = PV.pp_p[iab], qq = PV.pp_p[icd];
   double X = pair_sep(PV.pp_P, iab, icd, 0), Y = pair_sep(PV.pp_P, iab, icd, 1), Z = pair_sep(PV.pp_P, iab, icd, 2);
-  g.D = sqrt(X * X + Y * Y + Z * Z);
+  g.u = X * X + Y * Y + Z * Z;
+  g.D = sqrt(g.u);
   g.xi = p * qq / (p + qq);
   return g;
 }
@@ -227,7 +228,7 @@ __global__ void k_items_classify(Tables T, PairView PV, QuartetView QV, int cls,
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < npq;
        r += (int64_t)gridDim.x * blockDim.x) {
     ItemGeom g = item_geometry<BATCH>(PV, QV, cls, pq0 + r);
-    const bool skip = prim_negligible(*g.pv, g.iab, g.icd);
+    const bool skip = prim_negligible(*g.pv, g.iab, g.icd, g.u);
     for (int f = 0; f < nf; ++f) {
       const FamDev &F = T.fam[T.fam0[kcls] + f];
       const int key = skip ? SKIP_KEY : item_key(f, min(g.L, LAUX), item_bin(F, g.xi, g.D, g.L));
@@ -495,7 +496,7 @@ struct f12int_ctx {
   std::vector<double> kgrow[7];
   // the same tables on the device for the primitive screen ([7][kgrow_n]);
   // grows[cls]: the kernel of cls grows (G > 1 somewhere)
-  double *d_kgrow = nullptr;
+  float *d_kgrow = nullptr;
   size_t kgrow_bytes = 0;
   int kgrow_n = 0;
   bool grows[7] = {false, false, false, false, false, false, false};
@@ -1025,15 +1026,17 @@ static int set_factor_lists(f12int_ctx *ctx, const f12::TermList &T1, const f12:
     dfree(ctx, ctx->d_kgrow, ctx->kgrow_bytes);
     ctx->d_kgrow = nullptr;
     ctx->kgrow_n = (int)ctx->kgrow[1].size();
-    std::vector<double> all((size_t)7 * ctx->kgrow_n, 1.0);
+    std::vector<float> all((size_t)7 * ctx->kgrow_n, 1.0f);
     for (int c = 1; c <= 6; ++c) {
       ctx->grows[c] = false;
       for (int i = 0; i < ctx->kgrow_n; ++i) {
-        all[(size_t)c * ctx->kgrow_n + i] = ctx->kgrow[c][i];
+        // (rounded up; past single precision's range nothing is negligible)
+        const double g = ctx->kgrow[c][i] * (1.0 + 1e-6);
+        all[(size_t)c * ctx->kgrow_n + i] = g < 3e38 ? (float)g : INFINITY;
         ctx->grows[c] = ctx->grows[c] || ctx->kgrow[c][i] > 1.0;
       }
     }
-    ctx->kgrow_bytes = sizeof(double) * all.size();
+    ctx->kgrow_bytes = sizeof(float) * all.size();
     rc = dalloc(ctx, &ctx->d_kgrow, ctx->kgrow_bytes);
     if (rc != F12INT_OK) return rc;
     CK(cudaMemcpy(ctx->d_kgrow, all.data(), ctx->kgrow_bytes, cudaMemcpyHostToDevice));

@@ -26,7 +26,7 @@ struct PairView {
   const int *shell_l;
   int nshell;
   const double *qprim;       // [npp] primitive Schwarz factors of the class, or null
-  const double *grow;        // [ngrow] growth G(i kGrowStep) of the class's kernel, or null (no growth)
+  const float *grow;         // [ngrow] growth G(i kGrowStep) of the class's kernel, or null (no growth)
   int ngrow;
 };
 
@@ -109,24 +109,25 @@ constexpr double kPrimScreen = 1e-26;
 // A candidate is weighed, as the shell screen weighs a shell quartet, by
 //   Gamma = max over w = 0, 0.5, .., 3 (units of 1/sqrt(xi)) of G(R + w) e^{-xi w^2}
 // (e^{-xi w^2} = e^{-k^2/4} at the k-th sample).
-__device__ __forceinline__ bool prim_negligible(const PairView &PV, int pab, int pcd) {
+// The weighing is in single precision (an index into G's table of 0.05 bohr
+// steps and its largest value): in FP64 its square roots and division, taken by
+// the whole warp whenever one lane has a candidate, were a third of the thin
+// contraction's FP64 instructions.
+__device__ __forceinline__ bool prim_negligible(const PairView &PV, int pab, int pcd, double u) {
   if (!PV.qprim) return false;
   const double v = PV.qprim[pab] * PV.qprim[pcd];
   if (v >= kPrimScreen) return false;
   if (!PV.grow) return true;
-  const double X = pair_sep(PV.pp_P, pab, pcd, 0), Y = pair_sep(PV.pp_P, pab, pcd, 1),
-               Z = pair_sep(PV.pp_P, pab, pcd, 2);
-  const double p = PV.pp_p[pab], q = PV.pp_p[pcd];
-  const double R = sqrt(X * X + Y * Y + Z * Z), hw = 0.5 * sqrt((p + q) / (p * q));
-  constexpr double kOverlap[7] = {1.0, 0.77880078307140487, 0.36787944117144233, 0.10539922456186433,
-                                  0.018315638888734179, 0.0019304541362277093, 0.00012340980408667956};
-  double gam = 0.0;
+  const float R = sqrtf((float)u), hw = 0.5f * sqrtf((float)(PV.pp_ab[4 * pab + 2] + PV.pp_ab[4 * pcd + 2]));
+  constexpr float kOverlap[7] = {1.0f, 0.77880078307140487f, 0.36787944117144233f, 0.10539922456186433f,
+                                 0.018315638888734179f, 0.0019304541362277093f, 0.00012340980408667956f};
+  float gam = 0.0f;
 #pragma unroll
   for (int k = 0; k < 7; ++k) {
-    const int i = min(PV.ngrow - 1, (int)((R + k * hw) * (1.0 / kGrowStep)) + 1);
-    gam = fmax(gam, PV.grow[i] * kOverlap[k]);
+    const int i = min(PV.ngrow - 1, (int)((R + k * hw) * (float)(1.0 / kGrowStep)) + 1);
+    gam = fmaxf(gam, PV.grow[i] * kOverlap[k]);
   }
-  return v * gam < kPrimScreen;
+  return v * (double)gam < kPrimScreen;
 }
 
 // Thin contraction (thin_*.cu): quartets of total order L <= kThinL (I5:

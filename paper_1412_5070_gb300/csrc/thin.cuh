@@ -65,8 +65,9 @@ __device__ __forceinline__ void thin_quartet_body(const PairView &PV, const Quar
                  Z = pair_sep(PV.pp_P, pab, pcd, 2);
     double g[L + 1];
     if (G.direct()) {
-      if (prim_negligible(PV, pab, pcd)) continue;
-      aux_direct<L>(G, PV, pab, pcd, X * X + Y * Y + Z * Z, g);
+      const double u = X * X + Y * Y + Z * Z;
+      if (prim_negligible(PV, pab, pcd, u)) continue;
+      aux_direct<L>(G, PV, pab, pcd, u, g);
     } else {
       const int64_t pq = QV.pq_off[q] + r - pq0;
       if (keys[pq * nf] == kSkipKey) continue;   // dropped by the primitive screen
