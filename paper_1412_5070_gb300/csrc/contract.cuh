@@ -329,6 +329,29 @@ constexpr int KC_MAX = 16;   // staged inner primitive pairs at most
 __device__ __forceinline__ double tfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float tfma(float a, float b, float c) { return fmaf(a, b, c); }
 
+// The rows of the kept primitive quartets of a group, spread over their cubes:
+// asynchronous copies, so that the whole group's are in flight at once and the
+// products below are formed meanwhile (one load at a time, a block of one warp
+// waited about 20,000 cycles for 16 rows).
+__device__ __forceinline__ void stage_rows(double *cube, const double *rk, unsigned mask, int nk, int nhL, int pitch,
+                                           int P3, const int *cpos, int tid, int nthr) {
+  for (int i = tid; i < nhL; i += nthr) {
+    const unsigned to = (unsigned)__cvta_generic_to_shared(cube + cpos[i]);
+    for (int k = 0; k < nk; ++k)
+      if (mask >> k & 1)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to + 8u * (unsigned)(k * P3)),
+                     "l"(rk + (int64_t)k * pitch + i)
+                     : "memory");
+  }
+}
+__device__ __forceinline__ void stage_rows(float *cube, const double *rk, unsigned mask, int nk, int nhL, int pitch,
+                                           int P3, const int *cpos, int tid, int nthr) {
+  for (int i = tid; i < nhL; i += nthr)
+    for (int k = 0; k < nk; ++k)
+      if (mask >> k & 1) cube[k * P3 + cpos[i]] = (float)rk[(int64_t)k * pitch + i];
+}
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // One contraction task (quartet and range of inner components) by the whole
 // block; smem_bytes of shared memory.  nsplit < 0: the quartet is listed with
 // the bra inner.  iab0, iab1: outer primitive pairs of this launch (a quartet
@@ -354,7 +377,7 @@ __device__ __forceinline__ void contract_task(const PairView &PV0, const Quartet
   if (ncd <= 0) return;                     // block-uniform
   const int m0 = TK.off[j0], ncdt = TK.off[j0 + ncd] - m0, nabt = TB.nterm;
   const int nhL = nh_count(L), pitch = rows.stride(row_pitch(L)), P = L + 1, P3 = P * P * P;
-  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31;   // (whole warps)
   const int ab = s[0] * ns + s[1], cd = s[2] * ns + s[3];
   const int ab0 = PV.pair_start[ab], npab = PV.pair_start[ab + 1] - ab0;
   const int cd0 = PV.pair_start[cd], npcd = PV.pair_start[cd + 1] - cd0;
@@ -415,24 +438,21 @@ __device__ __forceinline__ void contract_task(const PairView &PV0, const Quartet
     for (int k0 = 0; k0 < npcd; k0 += kc) {
       const int nk = min(kc, npcd - k0);
       const int64_t pqk = pqq + (int64_t)iab * npcd + k0;
-      unsigned mask = 0;   // primitive quartets the screen kept
-      for (int k = 0; k < nk; ++k) mask |= (keys[(pqk + k) * kstride] != SKIP_KEY ? 1u : 0u) << k;
+      // primitive quartets the screen kept
+      const unsigned mask = __ballot_sync(0xffffffffu, lane < nk && keys[(pqk + min(lane, nk - 1)) * kstride] != SKIP_KEY);
       nproc += __popc(mask);
       const bool first = k0 == 0;
       const double *rk = rq + ((int64_t)iab * npcd + k0) * pitch;
       if (mask) {
-        for (int k = 0; k < nk; ++k) {
-          if (mask >> k & 1)
-            for (int i = tid; i < nhL; i += nthr) cube[k * P3 + cpos[i]] = (T)rk[(int64_t)k * pitch + i];
-          if (!have) {
+        stage_rows(cube, rk, mask, nk, nhL, pitch, P3, cpos, tid, nthr);
+        if (!have)
+          for (int x = tid; x < nk * ncdt; x += nthr) {
+            const int k = x / ncdt, m = x - k * ncdt;
             const double *E = PV.epool + PV.pp_eoff[cd0 + k0 + k];
-            for (int m = tid; m < ncdt; m += nthr) {
-              const unsigned w = d_pt_term[TK.first + m0 + m].y;
-              if (!S.op_inner) E3cd[k * kE + m] = (T)(E[w & 1023] * E[w >> 10 & 1023] * E[w >> 20]);
-              else products5(E, E + 3 * n1cd, cd0 + k0 + k, w, E3cd + k * kE + m, ncdt);
-            }
+            const unsigned w = d_pt_term[TK.first + m0 + m].y;
+            if (!S.op_inner) E3cd[k * kE + m] = (T)(E[w & 1023] * E[w >> 10 & 1023] * E[w >> 20]);
+            else products5(E, E + 3 * n1cd, cd0 + k0 + k, w, E3cd + k * kE + m, ncdt);
           }
-        }
         have = npcd <= kc;
       }
       if (first) {
@@ -444,6 +464,7 @@ __device__ __forceinline__ void contract_task(const PairView &PV0, const Quartet
           else products5(E, E + 3 * n1ab, pab, w, E3ab + m, nabt);
         }
       }
+      stage_wait();
       __syncthreads();
       // inner sum of Eq. ii: entry (bi, j) = sum over the staged pairs of
       // E_{t'u'v'} R_{t+t',u+u',v+v'}; consecutive threads take consecutive
