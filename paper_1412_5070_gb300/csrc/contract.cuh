@@ -585,7 +585,10 @@ static double task_fmas(const ContractShape &s, int64_t npcd, int jc) {
 // Whether (ab|cd), with npab and npcd primitive pairs, is cheaper with the bra
 // inner (listed as (cd|ab)): on the 12-atom s/p/d workload this takes 28% off
 // the multiply-adds of the contraction, on f shells up to 44%.  Entries count
-// by whole warps (a sum of ten entries costs as much as one of 32).
+// by whole warps (a sum of ten entries costs as much as one of 32).  Past 256
+// primitive pairs the smaller side is the inner one: the rows of one outer pair
+// are the least that a launch takes, and stay below 1.4 MB at the highest order
+// (so that no call is refused for them that its work items fit).
 static bool bra_inner(int la, int lb, int lc, int ld, int cls, int64_t npab, int64_t npcd) {
   const ContractShape k{la, lb, lc, ld, cls == 5 ? 2 : 0, false}, b{lc, ld, la, lb, cls == 5 ? 2 : 0, cls == 5};
   auto cost = [](const ContractShape &s, int64_t nin) {
@@ -595,6 +598,7 @@ static bool bra_inner(int la, int lb, int lc, int ld, int cls, int64_t npab, int
     return pe * s.nhB() * K.nterm * (s.inner4() == 4 ? 6 : 1) +
            po * s.ncd() * B.nterm * (s.outer4() == 4 ? 6 : 1) / (double)nin;
   };
+  if (std::max(npab, npcd) > 256 && npab != npcd) return npab < npcd;
   return cost(b, npab) < cost(k, npcd);
 }
 static ContractShape contract_shape(int la, int lb, int lc, int ld, int cls, bool swap) {
