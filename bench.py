@@ -426,10 +426,9 @@ def run_ours(args):
     con_ach = kst["contract_flops"] / (kst["contract_ms"] / 1e3) / 1e12 if kst["contract_ms"] > 0 else 0.0
     dom = "aux" if kst["aux_ms"] >= kst["contract_ms"] else "contract"
     ach = aux_ach if dom == "aux" else con_ach
-    traffic = aux_traffic_per_launch(nprimq, kst["aux_launches"] / args.steps) if dom == "aux" else None
-    kernels = {"k_items_eval": {"ms": kst["aux_ms"] / args.steps, "launches": kst["aux_launches"] // args.steps,
-                                "achieved_tflops": aux_ach, "flops": kst["aux_flops"] / args.steps,
-                                "share": kst["aux_ms"] / max(kst["aux_ms"] + kst["contract_ms"], 1e-9)},
+    kernels = {"k_hermite_rows": {"ms": kst["aux_ms"] / args.steps, "launches": kst["aux_launches"] // args.steps,
+                                   "achieved_tflops": aux_ach, "flops": kst["aux_flops"] / args.steps,
+                                   "share": kst["aux_ms"] / max(kst["aux_ms"] + kst["contract_ms"], 1e-9)},
                "k_contract": {"ms": kst["contract_ms"] / args.steps,
                               "launches": kst["contract_launches"] // args.steps,
                               "achieved_tflops": con_ach, "flops": kst["contract_flops"] / args.steps,
@@ -444,14 +443,12 @@ def run_ours(args):
             "setup_s": {"set_basis": t_basis, "screen_all_classes": t_screen},
             "gpu_launches": int(n_launch),
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h)},
-            "roofline": {"bound": "alu", "kernel": "k_items_eval" if dom == "aux" else "k_contract",
+            "roofline": {"bound": "alu", "kernel": "k_hermite_rows" if dom == "aux" else "k_contract",
                          "achieved": ach, "peak": peak64, "unit": "TFLOP/s",
-                         "frac": ach / peak64, "traffic": traffic,
-                         "traffic_note": "DRAM bytes per launch, scaled from an ncu capture of the 1% slices "
-                                         "(bytes per primitive quartet and class); mostly local memory of "
-                                         "the series (window and coefficient vector per thread)",
-                         "note": "FP64 pipe; achieved = counted FP64 flops of the kernel (series and quadrature "
-                                 "multiply-adds for k_items_eval, the algorithmic count for k_contract) / its "
+                         "frac": ach / peak64, "traffic": None,
+                         "traffic_note": "not captured for these kernels",
+                         "note": "FP64 pipe; achieved = FP64 flops of the kernel's launches (multiply-adds of the "
+                                 "auxiliary functions, the Hermite recursion and the products summed) / their "
                                  "event-timed launch durations; peak = FP64 FMA rate measured in this run "
                                  "(f12int_measure_peak), of measured"},
             "peaks_tflops": peaks,

@@ -68,7 +68,9 @@ typedef struct {
 } f12int_term;
 
 /* Create a context on CUDA device `device`.  hbm_budget_bytes caps the
- * device memory the context allocates (0 = no cap).  cuda_stream is the
+ * device memory the context allocates (0 = no cap; the grids of auxiliary
+ * functions, up to 280 MB per factor pair and shared by every context of the
+ * device that uses it, are not counted).  cuda_stream is the
  * default stream for the context (NULL = the legacy default stream).
  * On success *ctx receives a new context the caller must f12int_destroy. */
 int f12int_create(f12int_ctx **ctx, int device, size_t hbm_budget_bytes, void *cuda_stream);
@@ -213,8 +215,9 @@ int f12int_compute_class(f12int_ctx *ctx, int basis_id, int cls, const int32_t *
  * blocks are small in absolute terms: the error is bounded by about 1e-7
  * times the magnitude of the terms an element sums, not relative to the
  * element.  The first call of a (basis, class) computes its shell-pair
- * bounds.  Errors as for f12int_compute_class; F12INT_EINVAL for a negative
- * or NaN fp32_below. */
+ * bounds.  (The Hermite integrals are formed in FP64 and rounded once to FP32
+ * for the contraction.)  Errors as for f12int_compute_class; F12INT_EINVAL for
+ * a negative or NaN fp32_below. */
 int f12int_compute_class_mixed(f12int_ctx *ctx, int basis_id, int cls, const int32_t *quartets_dev,
                                int64_t n, double *out_dev, const int64_t *offsets_dev, double fp32_below,
                                void *cuda_stream);
@@ -314,7 +317,8 @@ int f12int_poll(f12int_ctx *ctx, uint64_t ticket, int64_t timeout_us, int *done)
 
 /* Capacity of one batch, per class: max_quartets shell quartets and
  * max_items auxiliary work items (primitive quartets times the kernel's term
- * families); each class has its own item buffers (136 bytes per item).
+ * families); each class has its own item buffers (136 bytes per item, which
+ * also hold the Hermite rows; a batch whose rows exceed them runs in passes).
  * Default 2^19 quartets; the default item capacity is set from free device
  * memory when the engine starts (the six classes' item buffers take at most
  * a quarter of it, 2^26 items per class at most).  Only before the first
@@ -325,7 +329,8 @@ int f12int_batch_limits(f12int_ctx *ctx, int64_t max_quartets, int64_t max_items
  * class_mask, run the n sample quartets (host [n][4] shell indices of the
  * basis) alone through the batch path under each candidate -- the work
  * target of one contraction task (6.25e6, 1.5e7, 5e7, 2e8 flops) times the
- * grid of the persistent auxiliary-stage launch (full or half residency) --
+ * grid of the persistent launch over work items (full or half residency; it
+ * matters for bases that the grid of auxiliary functions does not cover) --
  * and keep the fastest.  report (may be NULL) receives, per class c,
  * report[3(c-1)] the chosen target, [3(c-1)+1] the grid divisor and
  * [3(c-1)+2] the best time in seconds.  Needs an idle engine (no request
@@ -355,12 +360,15 @@ int64_t f12int_launch_count(const f12int_ctx *ctx);
 int f12int_set_timing(f12int_ctx *ctx, int on);
 
 /* Totals since the last reset, written to stats[0..5]:
- *   [0] milliseconds in auxiliary-evaluation launches, [1] their number,
- *   [2] milliseconds in contraction launches, [3] their number,
- *   [4] FP64 flops of the auxiliary stage's core multiply-adds (2 per FMA),
- *   [5] algorithmic FP64 flops of the Hermite recursion and contraction of
- *       the primitive quartets processed (2 C(L+4,4) + 2 nh(lab) nh(lcd) Ncd
- *       + 2 Nab nh(lab) Ncd per primitive quartet; bra step x4 and L+2 for I5).
+ *   [0] milliseconds in auxiliary-evaluation launches (with the Hermite
+ *       recursion, which they form in the same kernel), [1] their number,
+ *   [2] milliseconds in contraction launches (the thin ones form their own
+ *       auxiliary functions), [3] their number,
+ *   [4] FP64 flops of the auxiliary-evaluation launches: 2 per multiply-add of
+ *       g_n, and 2 C(L+4,4) per Hermite recursion,
+ *   [5] FP64 flops of the contraction launches: 2 per Hermite product summed
+ *       (10 where I5's operator is applied; products that are zero by
+ *       structure are not summed), and the g_n and recursion of the thin ones.
  * reset != 0 clears them.  Synchronises the context's stream. */
 int f12int_kernel_stats(f12int_ctx *ctx, int reset, double *stats);
 

@@ -245,7 +245,7 @@ k_hermite_rows(GridView G, PairView PV0, QuartetView QV, int cls, int nf, int64_
     const int L = PV.shell_l[s[0]] + PV.shell_l[s[1]] + PV.shell_l[s[2]] + PV.shell_l[s[3]] + (cls == 5 ? 2 : 0);
     double *o = rows.quartet(QV, lo) + (int64_t)k * rows.stride(row_pitch(L));
     if constexpr (DIRECT) {
-      nfma += aux_direct_fmas(G.boys != nullptr, L);
+      nfma += aux_direct_fmas(G.boys != nullptr, L) + (L + 1) * (L + 2) * (L + 3) * (L + 4) / 24;
       switch (L) {
         case 4: direct_row<4>(G, PV, pab, pcd, X, Y, Z, o); break;
         case 5: direct_row<5>(G, PV, pab, pcd, X, Y, Z, o); break;
@@ -524,16 +524,12 @@ __device__ __forceinline__ void contract_task(const PairView &PV0, const Quartet
   }
   for (int i = tid; i < nab * ncd; i += nthr) o[place(i)] = (double)O[i];
   if (flops_total && tid == 0 && nproc) {
-    // algorithmic FP64 flops per primitive quartet, with the ket inner: Hermite
-    // recursion 2 C(L+4,4) (counted once per quartet, not per split), ket step
-    // 2 nh(lab+ext) nh(lcd) ncd, bra step 2 nab nh(lab) ncd (x4 for I5), shared
-    // out over the ranges
-    const int lbra = swapped ? S.lc + S.ld : S.lab(), lket = swapped ? S.lab() : S.lc + S.ld;
-    const int nbra = swapped ? ncd_all : nab, nket = swapped ? nab : ncd_all;
-    const unsigned long long r = task.split == 0 ? 2ull * (L + 1) * (L + 2) * (L + 3) * (L + 4) / 24 : 0ull;
-    const unsigned long long ket = 2ull * nh_count(lbra + S.ext) * nh_count(lket) * nket * ncd / ncd_all;
-    const unsigned long long bra = 2ull * nbra * nh_count(lbra) * nket * (S.ext ? 4 : 1) * ncd / ncd_all;
-    atomicAdd(flops_total, nproc * (r + ket + bra));
+    // two flops per product summed, ten (four multiply-adds, two additions) with
+    // I5's operator; kept primitive quartets for the inner sum, outer pairs for
+    // the outer one
+    const unsigned long long in = (S.inner4() == 4 ? 10ull : 2ull) * nhB * ncdt;
+    const unsigned long long on = (S.outer4() == 4 ? 10ull : 2ull) * nabt * ncd;
+    atomicAdd(flops_total, nproc * in + (unsigned long long)(i1 - i0) * on);
   }
 }
 

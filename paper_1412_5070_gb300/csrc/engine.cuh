@@ -6,12 +6,17 @@
 // basis.  A worker thread merges the pending requests -- of any bases and any
 // mix of (la, lb, lc, ld) -- into a batch, writes the batch's lists to pinned
 // staging memory, copies them to fixed device buffers and replays one
-// captured CUDA graph.  The graph holds, for every class, the four passes of
-// the auxiliary stage and one contraction launch per tier (threads and shared
-// memory of a block), all
-// persistent (grid-stride over counts read from device memory), so the same
-// graph serves every batch.  The six class pipelines are parallel branches
-// of the graph, each with its own work-item buffers.  Two staging buffers let the host build batch
+// captured CUDA graph: one for bases inside the factor's grid of auxiliary
+// functions, one for those that go family by family (a batch holds requests of
+// one sort).  A graph holds, for every class, the Hermite rows of the general
+// quartets (behind the four passes over the work items in the second graph),
+// one contraction launch per tier (threads and shared memory of a block) and
+// one per key of the thin kernel, all persistent (grid-stride over counts read
+// from device memory), so the same graph serves every batch.  The six class
+// pipelines are parallel branches of the graph, each with its own buffers, and
+// the contraction launches of a class go over four streams.  A batch whose rows
+// exceed a class's buffer is replayed in passes; a single quartet that does is
+// launched by itself.  Two staging buffers let the host build batch
 // k+1 while batch k runs.  The method is that of f12int_compute_class; only
 // the scheduling differs.
 
@@ -224,8 +229,8 @@ static int engine_capture(f12int_ctx *ctx, Engine &E, bool grid) {
   }
   for (int t = 0; t < kTiers; ++t)
     if (kTierCap[t] > 48 * 1024) {
-      CK(cudaFuncSetAttribute(k_contract<true, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTierCap[t]));
-      CK(cudaFuncSetAttribute(k_contract<true, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTierCap[t]));
+      CK(cudaFuncSetAttribute(k_contract<true, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+      CK(cudaFuncSetAttribute(k_contract<true, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     }
   if (!grid && !E.rows[0][1]) {
     // the family path's rows, at its first batch: 64 MB a class, or what the
@@ -409,8 +414,8 @@ static int engine_init(f12int_ctx *ctx, Engine &E) {
   E.grid_blocks = nsm * std::max(per, 1);
   for (int t = 0; t < kTiers; ++t) {
     if (kTierCap[t] > 48 * 1024) {
-      CK(cudaFuncSetAttribute(k_contract<true, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTierCap[t]));
-      CK(cudaFuncSetAttribute(k_contract<true, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTierCap[t]));
+      CK(cudaFuncSetAttribute(k_contract<true, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+      CK(cudaFuncSetAttribute(k_contract<true, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     }
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_contract<true, double>, kTierThreads[t], kTierCap[t]));
     E.tier_blocks[t] = nsm * std::max(per, 1);

@@ -5,13 +5,18 @@
 //      E_t^{ij} (Eq. AB, Eqs. Erec0-Erect) with their AB derivatives
 //      F_t^{ij} = dE_t^{ij}/dAB_x for I5, one thread per primitive pair,
 //      resident in device memory for the life of the basis;
-//   2. auxiliary functions g_n = D_Q^n B_i per primitive quartet (aux.cuh);
+//   2. auxiliary functions g_n = D_Q^n B_i per primitive quartet: a point of the
+//      factor's grid (auxgrid.cuh; the Boys table for I1), inside the kernels of
+//      stage 3; the points of a basis that the grid does not hold go family by
+//      family through the work items of aux.cuh;
 //   3. the Hermite integrals R_tuv = d^t/dQx^t d^u/dQy^u d^v/dQz^v B_i
 //      (Eq. ri) by the Cartesian recursion for a radial function
 //        R^(n)_{t+1,u,v} = t R^(n+1)_{t-1,u,v} + X_QP R^(n+1)_{t,u,v},
-//      which holds because d/dQx D_Q^n B = X_QP D_Q^{n+1} B;
-//   4. the contraction of Eq. ii (inner ket sum, then bra sum) and for I5 the
-//      combination of Eq. I5byI3_, accumulated over primitive quartets.
+//      which holds because d/dQx D_Q^n B = X_QP D_Q^{n+1} B: one thread per
+//      primitive quartet (contract.cuh; in the registers of thin.cuh at low order);
+//   4. the contraction of Eq. ii (inner ket sum, then bra sum, or the mirror
+//      image where that is cheaper) and for I5 the combination of Eq. I5byI3_,
+//      accumulated over primitive quartets.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1681,7 +1686,7 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
       const int64_t t0 = P.tfirst(a), nt = P.tfirst(b) - t0;
       const auto kern = g.fp32 ? k_contract<false, float> : k_contract<false, double>;
       if (g.smem > 48 * 1024)
-        CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+        CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));   // (one value for every thread)
       kern<<<(unsigned)nt, g.nthr, g.smem, side()>>>(PV, QV, cls, direct ? 1 : nf, pq0, D.tasks + t0, nt, nullptr,
                                                      D.keys, RowView{D.rows, D.rowoff, row0, D.pitch}, out_dev,
                                                      D.offsets, i0, i1, fma_con);

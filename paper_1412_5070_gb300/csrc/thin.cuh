@@ -32,6 +32,17 @@ __host__ __device__ constexpr int cart_j(int l, int k) {   // y exponent
   return 0;
 }
 
+// Hermite products E_t E_u E_v of every component pair of two shells.
+__host__ __device__ constexpr int pair_terms(int l1, int l2) {
+  int n = 0;
+  for (int a = 0; a < (l1 + 1) * (l1 + 2) / 2; ++a)
+    for (int b = 0; b < (l2 + 1) * (l2 + 2) / 2; ++b) {
+      const int x = cart_i(l1, a) + cart_i(l2, b), y = cart_j(l1, a) + cart_j(l2, b);
+      n += (x + 1) * (y + 1) * (l1 + l2 - x - y + 1);
+    }
+  return n;
+}
+
 // One shell quartet q (index into the list) by the calling warp; its block
 // goes to o.
 template <int LA, int LB, int LC, int LD, bool I5>
@@ -191,17 +202,17 @@ __device__ __forceinline__ void thin_quartet_body(const PairView &PV, const Quar
     for (int i = 0; i < NE; ++i) out_q[i] = O[i];
   }
   if (flops_total) {
-    // the same algorithmic count per primitive quartet as the general kernel
+    // flops per primitive quartet: g_n, the recursion, and two per product summed
+    // (ten with I5's operator)
     unsigned tot = nproc;
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
     if (lane == 0 && tot) {
       const unsigned long long r = 2ull * (L + 1) * (L + 2) * (L + 3) * (L + 4) / 24;
-      const unsigned long long ket = 2ull * nh_count(LA + LB + EXT) * nh_count(LC + LD) * (NC * ND);
-      const unsigned long long bra = 2ull * (NA * NB) * nh_count(LA + LB) * (NC * ND) * (I5 ? 4 : 1);
-      atomicAdd(flops_total, (unsigned long long)tot * (r + ket + bra));
-      if (G.direct())   // the auxiliary stage's multiply-adds are the counter before
-        atomicAdd(flops_total - 1, (unsigned long long)tot * aux_direct_fmas(G.boys != nullptr, L));
+      const unsigned long long ket = 2ull * nh_count(LA + LB + EXT) * pair_terms(LC, LD);
+      constexpr unsigned long long bra = (I5 ? 10ull : 2ull) * pair_terms(LA, LB) * (NC * ND);
+      const unsigned long long aux = G.direct() ? 2ull * aux_direct_fmas(G.boys != nullptr, L) : 0ull;
+      atomicAdd(flops_total, (unsigned long long)tot * (aux + r + ket + bra));
     }
   }
 }
