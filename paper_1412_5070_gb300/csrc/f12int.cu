@@ -1295,6 +1295,10 @@ static const int kNKeys = MAXFAM * (LAUX + 1) * NZBIN + 1;
 // one would keep an SM busy while the others idle at the end of a launch.
 constexpr double kTaskFmas = 2e6;
 
+// A block of this many cycles (0.5 ms) is long enough for the order of launches
+// to matter.
+constexpr double kPoleCycles = 1e6;
+
 // A planned list: quartets in the working order -- those of the general
 // contraction first, by launch group (precision, threads, shared memory within
 // a factor of two), then decreasing work per task (the longest blocks start
@@ -1306,6 +1310,7 @@ struct ListPlan {
     size_t smem;
     bool fp32;
     int thin;              // class key, or -1
+    double longest, warps; // estimated cycles of its longest block, and of all its warps together
   };
   std::vector<Group> groups;
   int64_t n = 0, nthin = 0;            // quartets; first thin one
@@ -1510,9 +1515,15 @@ static int plan_kinds(const f12int_ctx::BasisData &B, int cls, int64_t n, const 
     if (P.groups.empty() || P.groups.back().thin != thin ||
         (!k.thin && (P.groups.back().fp32 != (k.f32 != 0) || P.groups.back().nthr != k.pl.nthr ||
                      kinds[(size_t)order[at - 1]].tier != k.tier)))
-      P.groups.push_back(ListPlan::Group{run, run, k.pl.nthr, 0, k.f32 != 0, thin});
+      P.groups.push_back(ListPlan::Group{run, run, k.pl.nthr, 0, k.f32 != 0, thin, 0.0, 0.0});
     ListPlan::Group &G = P.groups.back();
     G.smem = std::max(G.smem, k.pl.smem);
+    // cycles of a block (a thin quartet's warp): a primitive quartet's staging or
+    // grid point, and the chain of a thread's multiply-adds
+    const double cycles = k.thin ? 650.0 * (double)(k.nab * k.ncd + 31)
+                                 : 300.0 * (double)(k.nab * k.ncd) + 150.0 * k.work / k.pl.nthr;
+    G.longest = std::max(G.longest, cycles);
+    G.warps += cycles * (double)(k.count * k.pl.nsplit) * (k.thin ? 1.0 : k.pl.nthr / 32.0);
     k.first = run;
     ListPlan::Run r{};
     r.first = run;
@@ -1619,25 +1630,50 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
     (aux ? ctx->ev_aux : ctx->ev_con).push_back(ev);
     (aux ? ctx->aux_launches : ctx->contract_launches)++;
   };
-  // the independent launches go round the side streams, between fork and join
-  int used = 0, next = 0;
+  // The independent launches go round the side streams between fork and join.
+  // Launches whose longest block takes a good part of the whole list's time
+  // (quartets of thousands of primitive quartets and few entries: a few blocks of
+  // milliseconds each) go first, and every launch then to the stream with the
+  // least before it: in the list's order, smallest blocks last, they had the GPU
+  // to themselves in the end (2000 mixed I4 quartets 20.4 ms, so 18.2; 3000 f-shell
+  // I2 quartets 3.18 and 3.04).  Lists without such launches keep their order
+  // (sorting every launch by its longest block: 17.6 and 3.24 ms).
+  double all_warps = 0.0;
+  for (const ListPlan::Group &g : P.groups) all_warps += g.warps;
+  const double pole = 0.25 * all_warps / (152 * 16);   // cycles, at 16 warps an SM
+  auto is_pole = [&](const ListPlan::Group &g) { return g.longest > std::max(pole, kPoleCycles); };
+  bool poles = false;
+  std::vector<int> launch_order;
+  for (int pass = 0; pass < 2; ++pass)
+    for (size_t i = 0; i < P.groups.size(); ++i)
+      if (is_pole(P.groups[i]) == (pass == 0)) {
+        launch_order.push_back((int)i);
+        poles = poles || pass == 0;
+      }
+  unsigned used = 0;            // side streams that carry launches since the last join
+  unsigned waits = 0;           // ... that wait for the last fork
+  double load[NSIDE] = {0.0};
   auto fork = [&] {
-    used = next = 0;
+    waits = 0;
+    if (!poles) std::fill(load, load + NSIDE, 0.0);
     return cudaEventRecord(ctx->fork, st) == cudaSuccess;
   };
-  auto side = [&]() -> cudaStream_t {
-    const int i = next++ % NSIDE;
-    if (i >= used) {
-      cudaStreamWaitEvent(ctx->side[i], ctx->fork, 0);
-      used = i + 1;
-    }
+  auto side = [&](const ListPlan::Group &g) -> cudaStream_t {
+    const int i = (int)(std::min_element(load, load + NSIDE) - load);
+    load[i] += poles ? std::max(g.longest, g.warps / (152 * 16)) : 1.0;
+    if (!(waits >> i & 1)) cudaStreamWaitEvent(ctx->side[i], ctx->fork, 0);
+    waits |= 1u << i;
+    used |= 1u << i;
     return ctx->side[i];
   };
   auto join = [&] {
-    for (int i = 0; i < used; ++i) {
-      cudaEventRecord(ctx->join[i], ctx->side[i]);
-      cudaStreamWaitEvent(st, ctx->join[i], 0);
-    }
+    for (int i = 0; i < NSIDE; ++i)
+      if (used >> i & 1) {
+        cudaEventRecord(ctx->join[i], ctx->side[i]);
+        cudaStreamWaitEvent(st, ctx->join[i], 0);
+      }
+    used = 0;
+    std::fill(load, load + NSIDE, 0.0);
   };
   // items of the primitive quartets [pq0, pq1), family by family, into D.part
   auto items = [&](int64_t pq0, int64_t pq1) -> int {
@@ -1663,13 +1699,14 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
   };
   // thin quartets [qa, qb) of the list; pq0: the first primitive quartet of D.part
   auto thin = [&](int64_t qa, int64_t qb, int64_t pq0) -> int {
-    for (const ListPlan::Group &g : P.groups) {
+    for (int gi : launch_order) {
+      const ListPlan::Group &g = P.groups[(size_t)gi];
       const int64_t a = std::max(qa, g.first), b = std::min(qb, g.end);
       if (g.thin < 0 || a >= b) continue;
       const ThinKernel kern = thin_kernel(g.thin, cls == 5);
       if (!kern) return F12INT_EINVAL;
       const int64_t nt = b - a;   // one task each
-      kern<<<(unsigned)((nt + kThinWarps - 1) / kThinWarps), 32 * kThinWarps, 0, side()>>>(
+      kern<<<(unsigned)((nt + kThinWarps - 1) / kThinWarps), 32 * kThinWarps, 0, side(g)>>>(
           PV, QV, direct ? 1 : nf, pq0, G, D.tasks + P.tfirst(a), nt, nullptr, D.keys, D.part, out_dev,
           D.offsets, fma_con);
       ctx->launches++;
@@ -1680,14 +1717,15 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
   // general quartets [qa, qb), bra primitive pairs [i0, i1) (-1: all); row0: the
   // first double of D.rows
   auto general = [&](int64_t qa, int64_t qb, int64_t pq0, int64_t row0, int i0, int i1) -> int {
-    for (const ListPlan::Group &g : P.groups) {
+    for (int gi : launch_order) {
+      const ListPlan::Group &g = P.groups[(size_t)gi];
       const int64_t a = std::max(qa, g.first), b = std::min(qb, g.end);
       if (g.thin >= 0 || a >= b) continue;
       const int64_t t0 = P.tfirst(a), nt = P.tfirst(b) - t0;
       const auto kern = g.fp32 ? k_contract<false, float> : k_contract<false, double>;
       if (g.smem > 48 * 1024)
         CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));   // (one value for every thread)
-      kern<<<(unsigned)nt, g.nthr, g.smem, side()>>>(PV, QV, cls, direct ? 1 : nf, pq0, D.tasks + t0, nt, nullptr,
+      kern<<<(unsigned)nt, g.nthr, g.smem, side(g)>>>(PV, QV, cls, direct ? 1 : nf, pq0, D.tasks + t0, nt, nullptr,
                                                      D.keys, RowView{D.rows, D.rowoff, row0, D.pitch}, out_dev,
                                                      D.offsets, i0, i1, fma_con);
       ctx->launches++;
@@ -1724,7 +1762,6 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
       if (rc != F12INT_OK) return rc;
     }
   }
-  const int thin_used = used;   // side streams that still carry thin launches
   // first double of the rows of quartet q, and their end, in the list's order
   auto row_of = [&](int64_t q) -> int64_t { return D.pitch ? P.pqoff[q] * D.pitch : P.rowoff[q]; };
   auto row_end = [&](int64_t q) -> int64_t { return D.pitch ? P.pqoff[q + 1] * D.pitch : P.rowoff[q + 1]; };
@@ -1791,10 +1828,7 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
     time_end(false);
     qa = qb;
   }
-  if (direct && P.nthin > 0 && P.nthin < P.n && !timing) {
-    used = std::max(used, thin_used);
-    join();
-  }
+  join();   // (an error's or a thin launch's that is still on a side stream)
   return rc;
 }
 
