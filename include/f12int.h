@@ -206,17 +206,16 @@ int f12int_compute_class(f12int_ctx *ctx, int basis_id, int cls, const int32_t *
                          int64_t n, double *out_dev, const int64_t *offsets_dev, void *cuda_stream);
 
 /* Mixed-precision variant of f12int_compute_class: quartets whose shell-pair
- * bound product (as in f12int_screen) is below fp32_below run the Hermite
- * recursion and the contraction in FP32 with FP32 accumulation; the
- * auxiliary functions g_n, the shell-pair data and every other quartet stay
- * FP64, and so do the quartets of total angular momentum <= 3 (<= 2 for I5),
+ * bound product (as in f12int_screen) is below fp32_below run the
+ * contraction in FP32 with FP32 accumulation; the auxiliary functions g_n, the
+ * Hermite recursion, the shell-pair data and every other quartet stay FP64,
+ * and so do the quartets of total angular momentum <= 3 (<= 2 for I5),
  * whose one-lane-per-primitive-quartet FP64 contraction is faster than the
  * FP32 form of the general one.  fp32_below = 0 is f12int_compute_class.  Meant for quartets whose
  * blocks are small in absolute terms: the error is bounded by about 1e-7
  * times the magnitude of the terms an element sums, not relative to the
  * element.  The first call of a (basis, class) computes its shell-pair
- * bounds.  (The Hermite integrals are formed in FP64 and rounded once to FP32
- * for the contraction.)  Errors as for f12int_compute_class; F12INT_EINVAL for
+ * bounds.  Errors as for f12int_compute_class; F12INT_EINVAL for
  * a negative or NaN fp32_below. */
 int f12int_compute_class_mixed(f12int_ctx *ctx, int basis_id, int cls, const int32_t *quartets_dev,
                                int64_t n, double *out_dev, const int64_t *offsets_dev, double fp32_below,
@@ -339,7 +338,7 @@ int f12int_batch_autotune(f12int_ctx *ctx, int basis_id, const int32_t *quartets
                           uint32_t class_mask, double *report);
 
 /* Screening estimate below which mixed requests (precision 1) run the
- * Hermite recursion and contraction in FP32 (default 1e-5, where the FP32
+ * contraction in FP32 (default 1e-5, where the FP32
  * difference stayed below 4.1e-11 on a 40-atom f-shell sample; at 1e-4 it
  * reached 1.5e-10).  Applies to batches built after the call. */
 int f12int_set_fp32_below(f12int_ctx *ctx, double bound);

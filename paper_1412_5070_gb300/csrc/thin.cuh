@@ -15,7 +15,11 @@ namespace f12k {
 // products in registers and accumulates every element of the block (Eq. ii,
 // bra sign (-1)^{t+u+v}; for I5 Eq. I5byI3_ with the second coefficient -1,
 // as the general kernel); the lanes' sums are then added by a fixed
-// butterfly, so the result does not depend on scheduling.
+// butterfly, so the result does not depend on scheduling.  Bound by the FP64
+// pipe (75-90% busy): 11.3 ms for the 144,000 thin quartets of 200,000 I4 ones with
+// g_n from the grid (12.4 with the divisions and square roots of 1/xi and the
+// prefactor, which pair data now hold; 160 ms more when g_n came family by
+// family), 10% less of the call since the screen's test runs in FP32.
 
 __host__ __device__ constexpr int cart_i(int l, int k) {   // x exponent of component k of shell l
   int n = 0;
