@@ -315,11 +315,9 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
   Build B{};
   GridClass gc[NCLS];
   int cls_of[NCLS];
-  std::vector<double> gs;
   double bpos = 0.0, bneg = 0.0;
   for (int k = 0; k < NCLS; ++k)
     if (want[kClass[k]] && grid_families(kt[kClass[k]], gc[B.ncls])) {
-      gs.insert(gs.end(), gc[B.ncls].g.begin(), gc[B.ncls].g.end());
       bpos = std::max(bpos, gc[B.ncls].bpos);
       bneg = std::max(bneg, gc[B.ncls].bneg);
       cls_of[B.ncls++] = kClass[k];
@@ -330,7 +328,7 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
   for (int o = 0; o < NOCT; ++o) {
     GridQuad q;
     const double lo = std::ldexp(1.0, GR_XLO + o);
-    if (!grid_quad(gs, bpos, bneg, lo, 2.0 * lo, q)) return nullptr;
+    if (!grid_quad(gc, B.ncls, lo, 2.0 * lo, q)) return nullptr;
     pt0.push_back((int)x.size());
     npanel.push_back((int)q.edge.size() - 1);
     x.insert(x.end(), q.x.begin(), q.x.end());

@@ -15,10 +15,20 @@ namespace f12dev {
 struct GridClass {
   std::vector<GridFam> fam;
   std::vector<dd> coef;
-  std::vector<double> g;               // the families' g > 0
+  std::vector<double> g, reach;        // the families' g > 0, and how far they count
   double bpos = 0.0, bneg = 0.0;       // largest b > 0, largest |b| of b < 0
   double bmax = -1e300;                // largest b
 };
+
+// Distance past which a family x^alpha e^{bx - gx^2}, alpha <= amax, is below
+// double precision of its largest value: t^p e^{-t}, t = g x^2 and p = amax/2, has
+// fallen by 2^-58 from its peak at t = p, and e^{bx} moves the peak by b/2g.
+inline double grid_reach(double amax, double b, double g) {
+  const double p = std::max(0.5 * amax, 1.0);
+  double t = p;
+  while (p * std::log(t / p) - (t - p) > -40.0) t += 1.0;
+  return std::sqrt(t / g) + 0.5 * std::max(b, 0.0) / g;
+}
 
 // The families of a kernel, or false when the grid does not serve it: lowest
 // powers below -1 (singular groups), a general power so low that the first
@@ -65,7 +75,10 @@ inline bool grid_families(const f12::TermList &kernel, GridClass &gc) {
       }
       cur.swap(nxt);
     }
-    if (f.g > 0.0) gc.g.push_back(f.g);
+    if (f.g > 0.0) {
+      gc.g.push_back(f.g);
+      gc.reach.push_back(grid_reach(a + (double)f.poly.size() - 1.0 + 2.0 * GR_M, f.b, f.g));
+    }
     gc.bmax = std::max(gc.bmax, f.b);
     gc.bpos = std::max(gc.bpos, f.b);
     gc.bneg = std::max(gc.bneg, -f.b);
@@ -84,24 +97,34 @@ constexpr int GR_MAXPANEL = 400;
 // Gaussian among those that still count -- to the largest D of region A plus 6.6
 // widths; 1.25 widths are about the distance over which 16 nodes reach
 // double precision.  The first panel is taken in u = (x/w)^{1/8}, which makes
-// x^{alpha} du smooth for the powers grid_families admits.
+// x^{alpha} du smooth for the powers grid_families admits; the others are at
+// most 1.5 times as wide as their distance from r = 0, where the long-range
+// families have a branch point: where narrow panels end (a tight Gaussian's
+// reach) one of full width would not resolve it.
 struct GridQuad {
   std::vector<double> x, w;
   std::vector<double> edge;   // panel p covers [edge[p], edge[p + 1]]
 };
-inline bool grid_quad(const std::vector<double> &g, double bpos, double bneg, double xi_lo, double xi_hi, GridQuad &q) {
+inline bool grid_quad(const GridClass *gc, int ngc, double xi_lo, double xi_hi, GridQuad &q) {
   q = GridQuad{};
   double gx[GR_NQ], gw[GR_NQ], hx[GR_NQ0], hw[GR_NQ0];
   gauss_legendre(GR_NQ, gx, gw);
   gauss_legendre(GR_NQ0, hx, hw);
+  double bpos = 0.0, bneg = 0.0;
+  for (int c = 0; c < ngc; ++c) {
+    bpos = std::max(bpos, gc[c].bpos);
+    bneg = std::max(bneg, gc[c].bneg);
+  }
   const double end = std::sqrt((GR_TMAX + 32.0) / xi_lo) + (8.5 + 0.5 * bpos / std::sqrt(xi_lo)) / std::sqrt(xi_lo);
   double a = 0.0;
   q.edge.push_back(0.0);
   while (a < end) {
     double w = 1.25 / std::sqrt(xi_hi);
-    for (double gi : g)
-      if (a * a * gi < 50.0) w = std::min(w, 1.25 / std::sqrt(xi_hi + gi));
+    for (int c = 0; c < ngc; ++c)
+      for (size_t i = 0; i < gc[c].g.size(); ++i)
+        if (a < gc[c].reach[i]) w = std::min(w, 1.25 / std::sqrt(xi_hi + gc[c].g[i]));
     if (bneg > 0.0) w = std::min(w, 1.25 * std::sqrt(std::max(1.0, bneg * a)) / bneg);
+    if (a > 0.0) w = std::min(w, 1.5 * a);
     if (a == 0.0) {
       w *= 0.5;
       for (int i = 0; i < GR_NQ0; ++i) {

@@ -1,0 +1,102 @@
+"""Single cells of the auxiliary grid, built on the CPU from the library's own
+headers (tests/grid_host.cpp), against the oracle: factors whose Gaussian parts
+are much tighter than the exponents of a basis, decaying and growing long
+ranges, and orders up to 14."""
+import ctypes
+import os
+import shutil
+import subprocess
+from concurrent.futures import ThreadPoolExecutor
+from math import factorial
+
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1412_5070_gb300", "csrc")
+SRC = [os.path.join(HERE, "grid_host.cpp"), os.path.join(CSRC, "termlist.cpp")]
+DEPS = SRC + [os.path.join(CSRC, f) for f in ("aux.cuh", "auxtab.h", "auxgrid.cuh", "gridtab.h", "termlist.h")]
+LIB = os.path.join(HERE, "_build", "libgridhost.so")
+dp = ctypes.POINTER(ctypes.c_double)
+
+
+@pytest.fixture(scope="module")
+def lib():
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no C++ compiler")
+    os.makedirs(os.path.dirname(LIB), exist_ok=True)
+    if not os.path.exists(LIB) or any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in DEPS):
+        tmp = LIB + ".tmp%d" % os.getpid()
+        subprocess.run([gxx, "-O2", "-std=c++17", "-ffp-contract=off", "-fPIC", "-shared", "-pthread", "-o", tmp,
+                        *SRC], check=True)
+        os.replace(tmp, LIB)
+    L = ctypes.CDLL(LIB)
+    L.grid_host_new.argtypes = [dp, ctypes.c_int, dp, ctypes.c_int, ctypes.c_int]
+    L.grid_host_new.restype = ctypes.c_void_p
+    L.grid_host_free.argtypes = [ctypes.c_void_p]
+    L.grid_host_eval.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_double, ctypes.c_int, dp]
+    return L
+
+
+def rs12(mu=1.0, B=0.5, c0=0.5, rho=-0.5, n=0):
+    """The terms of (1 + r/2) e^{-mu r^2} + c0 r^rho e^{Br} (1 - e^{-mu r^2} sum_k (mu r^2)^k/k!)."""
+    return ([(1.0, 0, 0, mu), (0.5, 1, 0, mu), (c0, rho, B, 0)]
+            + [(-c0 * mu ** k / factorial(k), rho + 2 * k, B, mu) for k in range(n + 1)])
+
+
+class Grid:
+    def __init__(self, lib, terms, cls):
+        t = np.ascontiguousarray(terms, dtype=np.float64)
+        self.lib, self.p = lib, lib.grid_host_new(t.ctypes.data_as(dp), len(t), t.ctypes.data_as(dp), len(t), cls)
+        if not self.p:
+            pytest.skip("not served by the grid")
+
+    def __del__(self):
+        if getattr(self, "p", None):
+            self.lib.grid_host_free(self.p)
+
+    def eval(self, xi, D, L):
+        out = np.zeros(L + 1)
+        assert self.lib.grid_host_eval(self.p, xi, D, L, out.ctypes.data_as(dp)) == 0
+        return out
+
+
+def errors(grid, kern, cls, pts, L):
+    """Relative error of every order at every point; an order that passes
+    through zero is measured against a twentieth of the next over the local
+    width, as in the GPU test of the grid."""
+    with ThreadPoolExecutor(max_workers=min(16, os.cpu_count() or 1)) as ex:
+        ref = np.array(list(ex.map(lambda p: O.radial(kern, cls, p[0], p[1], L + 1), pts)))
+    got = np.array([grid.eval(x, d, L) for x, d in pts])
+    w = np.array([min(d * d + 1e-300, 1.0 / x) for x, d in pts])
+    return np.abs(got - ref[:, :-1]) / (np.abs(ref[:, :-1]) + 0.05 * np.abs(ref[:, 1:]) * w[:, None])
+
+
+TIGHT = {
+    "mu=1": rs12(1.0),
+    "mu=50": rs12(50.0),
+    "mu=400": rs12(400.0),
+    "mu=2000": rs12(2000.0),
+    "mu=20000": rs12(20000.0),
+    "B=-0.5 mu=2000": rs12(2000.0, B=-0.5),
+    "n=2 mu=400": rs12(400.0, n=2),
+    "long range and g=1000": [(0.5, 0.5, 0.5, 0), (0.8, 0, 0, 1000.0)],
+}
+
+
+@pytest.mark.parametrize("name", list(TIGHT))
+@pytest.mark.parametrize("cls", [2, 3, 4, 6])
+def test_tight_gaussians(lib, name, cls):
+    """The quadrature resolves the long range's branch point at r = 0 past the
+    reach of a tight Gaussian.  Every point lies where the library uses the grid
+    (exponents of an ordinary basis, a molecule's distances).  1e-10: what the
+    auxiliary stage holds for the orders of its general classes."""
+    g = Grid(lib, TIGHT[name], cls)
+    kern = O.factor_kernel_terms(TIGHT[name])
+    pts = [(0.112, 0.0), (0.112, 3.1), (0.7, 0.02), (3.3, 1.1), (21.0, 0.0), (150.0, 0.6)]
+    for L in (8, 14):
+        e = errors(g, kern, cls, pts, L)
+        assert e.max() < 1e-10, (L, e.max(1))
