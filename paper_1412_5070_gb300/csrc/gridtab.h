@@ -105,11 +105,57 @@ struct GridQuad {
   std::vector<double> x, w;
   std::vector<double> edge;   // panel p covers [edge[p], edge[p + 1]]
 };
+// Gauss-Legendre nodes and weights as double-doubles (long double inside), and for a
+// rule of n nodes what rounding its nodes takes: with nodes t + d, exact again up
+// to degree n - 1 are the weights w + c d (the changes of the moments of P_k, k < n,
+// by the rule's own discrete orthogonality).  Without it the rounding of
+// x, up to x sqrt(xi) u of a width, put several u into the rows.
+struct GridRule {
+  std::vector<dd> t, w;
+  std::vector<double> c;   // [n][n]
+};
+inline GridRule grid_rule(int n, bool corrected) {
+  GridRule r;
+  std::vector<double> P((size_t)n * n), Q((size_t)n * n);   // P_k(t_i) (2k + 1)/2, P_k'(t_i)
+  for (int i = 0; i < n; ++i) {
+    long double t = -std::cos(M_PI * (i + 0.75) / (n + 0.5)), dp = 1.0L;
+    for (int it = 0; it < 8; ++it) {
+      long double p0 = 1.0L, p1 = t;
+      for (int k = 2; k <= n; ++k) {
+        const long double p2 = ((2 * k - 1) * t * p1 - (k - 1) * p0) / k;
+        p0 = p1;
+        p1 = p2;
+      }
+      dp = n * (t * p1 - p0) / (t * t - 1.0L);
+      if (it < 7) t -= p1 / dp;
+    }
+    const long double w = 2.0L / ((1.0L - t * t) * dp * dp);
+    r.t.push_back(dd{(double)t, (double)(t - (double)t)});
+    r.w.push_back(dd{(double)w, (double)(w - (double)w)});
+    double p0 = 1.0, p1 = (double)t, d0 = 0.0, d1 = 1.0;
+    for (int k = 0; k < n; ++k) {
+      P[(size_t)i * n + k] = (k + 0.5) * p0;
+      Q[(size_t)i * n + k] = d0;
+      const double p2 = ((2 * k + 3) * (double)t * p1 - (k + 1) * p0) / (k + 2), d2 = d0 + (2 * k + 3) * p1;
+      p0 = p1;
+      p1 = p2;
+      d0 = d1;
+      d1 = d2;
+    }
+  }
+  if (!corrected) return r;
+  r.c.assign((size_t)n * n, 0.0);
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j < n; ++j) {
+      double s = 0.0;
+      for (int k = 0; k < n; ++k) s += P[(size_t)i * n + k] * Q[(size_t)j * n + k];
+      r.c[(size_t)i * n + j] = -r.w[i].h * r.w[j].h * s;
+    }
+  return r;
+}
 inline bool grid_quad(const GridClass *gc, int ngc, double xi_lo, double xi_hi, GridQuad &q) {
   q = GridQuad{};
-  double gx[GR_NQ], gw[GR_NQ], hx[GR_NQ0], hw[GR_NQ0];
-  gauss_legendre(GR_NQ, gx, gw);
-  gauss_legendre(GR_NQ0, hx, hw);
+  static const GridRule rule = grid_rule(GR_NQ, true), rule0 = grid_rule(GR_NQ0, false);
   double bpos = 0.0, bneg = 0.0;
   for (int c = 0; c < ngc; ++c) {
     bpos = std::max(bpos, gc[c].bpos);
@@ -128,17 +174,29 @@ inline bool grid_quad(const GridClass *gc, int ngc, double xi_lo, double xi_hi, 
     if (a == 0.0) {
       w *= 0.5;
       for (int i = 0; i < GR_NQ0; ++i) {
-        const double u = 0.5 * (hx[i] + 1.0), u2 = u * u, u4 = u2 * u2;
+        const double u = 0.5 * (rule0.t[i].h + 1.0) + 0.5 * rule0.t[i].l, u2 = u * u, u4 = u2 * u2;
         q.x.push_back(w * u4 * u4);
-        q.w.push_back(0.5 * hw[i] * w * 8.0 * u4 * u2 * u);
+        q.w.push_back(0.5 * rule0.w[i].h * w * 8.0 * u4 * u2 * u);
       }
+      a = w;
     } else {
+      const double e = a + w;
+      dd h = dd_sum(e, -a);
+      h = dd{0.5 * h.h, 0.5 * h.l};
+      double d[GR_NQ];
       for (int i = 0; i < GR_NQ; ++i) {
-        q.x.push_back(a + 0.5 * w * (gx[i] + 1.0));
-        q.w.push_back(0.5 * w * gw[i]);
+        const dd x = dd_add(dd{a, 0.0}, dd_mul(h, dd_add(dd{1.0, 0.0}, rule.t[i])));
+        q.x.push_back(x.h);
+        d[i] = -x.l / h.h;
       }
+      for (int i = 0; i < GR_NQ; ++i) {
+        double c = rule.w[i].l;
+        for (int j = 0; j < GR_NQ; ++j) c += rule.c[(size_t)i * GR_NQ + j] * d[j];
+        const dd wi = dd_mul(h, dd_fast(rule.w[i].h, c));
+        q.w.push_back(wi.h);
+      }
+      a = e;
     }
-    a += w;
     q.edge.push_back(a);
     if (q.edge.size() > GR_MAXPANEL) return false;
   }

@@ -48,15 +48,16 @@ double rows_a(HostGrid &G, int cell, double xi, double D, double *V) {
     for (size_t i = 0; i < O.q.x.size(); ++i)
       grid_radial(G.gc.fam.data(), (int)G.gc.fam.size(), G.gc.coef.data(), O.q.x[i], GR_M, &O.F[i * GR_ROWS]);
   }
-  double acc[GR_ROWS] = {0.0}, jh[GR_ROWS];
+  long double acc[GR_ROWS] = {0.0L};   // (the builder's sums carry their rounding)
+  double jh[GR_ROWS];
   for (size_t i = 0; i < O.q.x.size(); ++i) {
     const double x = O.q.x[i], e = O.q.w[i] * std::exp(-xi * (x - D) * (x - D));
     if (e == 0.0) continue;
     grid_jhat(G.ztab.data(), 2.0 * xi * D * x, jh);
-    for (int m = 0; m <= GR_M; ++m) acc[m] = std::fma(e * jh[m], O.F[i * GR_ROWS + m], acc[m]);
+    for (int m = 0; m <= GR_M; ++m) acc[m] += (long double)(e * jh[m]) * O.F[i * GR_ROWS + m];
   }
   double f = 4.0 * xi * std::sqrt(xi);
-  for (int m = 0; m <= GR_M; ++m, f *= 2.0 * xi) V[m] = f * acc[m];
+  for (int m = 0; m <= GR_M; ++m, f *= 2.0 * xi) V[m] = f * (double)acc[m];
   return 0.0;
 }
 

@@ -100,3 +100,19 @@ def test_tight_gaussians(lib, name, cls):
     for L in (8, 14):
         e = errors(g, kern, cls, pts, L)
         assert e.max() < 1e-10, (L, e.max(1))
+
+
+def test_rounding_of_the_quadrature(lib):
+    """The cells carry the rounding of a few operations, not of the quadrature's
+    nodes and sums: 3 u root mean square for f over a molecule's exponents and
+    distances (nodes and weights as rounded doubles, summed one by one: 5 u).
+    The point itself, the cell's polynomials and its Taylor sum account for 1 to
+    2 u."""
+    g = Grid(lib, rs12(), 3)
+    kern = O.factor_kernel_terms(rs12())
+    rng = np.random.default_rng(3)
+    pts = [(float(np.exp(rng.uniform(np.log(0.06), np.log(6.0)))), float(rng.uniform(0.0, 7.0))) for _ in range(40)]
+    with ThreadPoolExecutor(max_workers=min(16, os.cpu_count() or 1)) as ex:
+        ref = np.array(list(ex.map(lambda p: O.radial(kern, 3, p[0], p[1], 0)[0], pts)))
+    e = np.array([g.eval(x, d, 0)[0] for x, d in pts]) / ref - 1.0
+    assert np.sqrt(np.mean(e * e)) < 3.0 * 2.0 ** -53
