@@ -389,10 +389,56 @@ F12_DEV inline void grid_jhat(const double *ztab, double z, double *jh) {
 // Region B: quadrature nodes, and the Chebyshev points of x/D in
 // [1 - GR_BW, 1 + GR_BW] from which F_m is interpolated (barycentric form); the
 // rule's outermost node lies within 5.4 widths, a width is at most
-// D/sqrt(GR_TB).
+// D/sqrt(GR_TB).  The check point's rule has more nodes and takes F_m itself.
 constexpr int GR_NH = 20;
+constexpr int GR_NHC = 32;
 constexpr int GR_NB = 36;
 constexpr double GR_BW = 0.25;
+
+// Exponent b of a kernel's lowest rows over the interpolated range (F at its two
+// ends, dx apart): F_m e^{-b(x - D)} is interpolated, which varies little whatever
+// mixture of decays the kernel has (with one of its families' b instead, a
+// kernel like e^{-8x} beside Gaussians lost seven digits).
+F12_HD inline double grid_slope(const double *lo, const double *hi, double dx) {
+  double a = 0.0, b = 0.0;
+  for (int m = 0; m < 3; ++m) {
+    const double l = fabs(lo[m]), h = fabs(hi[m]), s = l + h;
+    if (s > 0.0) {
+      a += l / s;
+      b += h / s;
+    }
+  }
+  return a > 0.0 && b > 0.0 ? log(b / a) / dx : 0.0;
+}
+
+// ---------------------------------------------------------- check points --
+// Every cell is checked at one point: of region A one of its four corners, of
+// region B an end of its u at its widest Gaussian (where the rule is at its
+// least; a = 1 itself is left a margin).  a: the coordinate of xi, s: of u in
+// units of the cell's width, from its middle.
+F12_HD inline void grid_check(int cell, double *a, double *s) {
+  *a = cell >= GR_NX * GR_NT ? 0.97 : (cell & 1) ? 1.0 : -1.0;
+  *s = (cell & 2) ? 0.5 : -0.5;
+}
+// ends of a cell in T' (region A) or u (B)
+F12_HD inline void grid_cellu(int cell, double *lo, double *hi) {
+  if (cell < GR_NX * GR_NT) grid_tcell(cell % GR_NT, lo, hi);
+  else grid_ucell(cell - GR_NX * GR_NT, lo, hi);
+}
+// the point itself: its xi and u
+F12_HD inline void grid_check_point(const double *xt, int cell, double *xi, double *u) {
+  double lo, hi, a, s;
+  grid_cellu(cell, &lo, &hi);
+  grid_check(cell, &a, &s);
+  if (cell < GR_NX * GR_NT) {
+    const double *r = xt + GR_XT * (cell / GR_NT);
+    *xi = grid_xi(r, a);
+    *u = mul_rn(0.5 * (lo + hi), r[1]) + s * (hi - lo) * r[1];
+  } else {
+    *xi = 2.0 * GR_TB / (hi * (a + 1.0));
+    *u = 0.5 * (lo + hi) + s * (hi - lo);
+  }
+}
 
 // ------------------------------------------------------------ evaluation --
 // The Coulomb kernel (I1): sqrt(xi) hat g_l = 2 sqrt(xi) (-2 xi)^l F_l(x), F_l the
@@ -482,6 +528,51 @@ F12_DEV inline void grid_eval(const double *cells, const GridPoint &pt, int L, d
       h[l] = k == (FIXED ? NMAX : N) ? r : fma(h[l], t[k + 1 <= NMAX ? k + 1 : NMAX], r);
     }
   }
+}
+
+// ------------------------------------------------------------ acceptance --
+// A cell is in order when every form in which the kernels take it (highest
+// orders 0 to 8, each with its shortened rows, and 14, whose rows those of 9 to 13
+// are) agrees at its check point with rows V[0..LMAX] from a quadrature of its
+// own, to GR_TOL of the sum of the terms' magnitudes (the scale of the result
+// where it passes through zero).
+constexpr double GR_TOL = 1e-12;
+constexpr int GR_LMAX = 14;
+template <int L>
+F12_DEV inline bool grid_form_ok(const double *cell, const GridPoint &pt, const double *V, const double *sc) {
+  double h[L + 1];
+  grid_eval<L, true>(cell, pt, L, h);
+  bool ok = true;
+  for (int l = 0; l <= L; ++l) ok = ok && fabs(h[l] - V[l]) <= GR_TOL * sc[l];   // false for NaN
+  return ok;
+}
+F12_DEV inline bool grid_cell_ok(const double *xt, int cell, const double *C, const double *V) {
+  double lo, hi, a, s;
+  grid_cellu(cell, &lo, &hi);
+  grid_check(cell, &a, &s);
+  GridPoint pt;
+  pt.cell = 0;
+  pt.a = a;
+  pt.hd = 0.5 * s * (hi - lo) * (cell < GR_NX * GR_NT ? xt[GR_XT * (cell / GR_NT) + 1] : 1.0);
+  constexpr int N = grid_terms(GR_LMAX);
+  double row[GR_LMAX + N + 1], sc[GR_LMAX + 1];
+  for (int m = 0; m <= GR_LMAX + N; ++m) {
+    double r = C[m * GR_NC + GR_NC - 1];
+    for (int i = GR_NC - 2; i >= 0; --i) r = fma(r, a, C[m * GR_NC + i]);
+    row[m] = fabs(r);
+  }
+  for (int l = 0; l <= GR_LMAX; ++l) {
+    double w = 1.0;
+    sc[l] = 0.0;
+    for (int k = 0; k <= N; ++k) {
+      sc[l] = fma(row[l + k], w, sc[l]);
+      w *= fabs(pt.hd) / (k + 1);
+    }
+  }
+  return grid_form_ok<0>(C, pt, V, sc) && grid_form_ok<1>(C, pt, V, sc) && grid_form_ok<2>(C, pt, V, sc) &&
+         grid_form_ok<3>(C, pt, V, sc) && grid_form_ok<4>(C, pt, V, sc) && grid_form_ok<5>(C, pt, V, sc) &&
+         grid_form_ok<6>(C, pt, V, sc) && grid_form_ok<7>(C, pt, V, sc) && grid_form_ok<8>(C, pt, V, sc) &&
+         grid_form_ok<14>(C, pt, V, sc);
 }
 
 }  // namespace f12dev

@@ -1,13 +1,15 @@
 // grid.cu -- the builder of the auxiliary grids (auxgrid.cuh) and their
 // sharing between contexts.
 //
-// Four kernels, once per factor: the summed kernel derivatives F_m at the
+// Five kernels, once per factor: the summed kernel derivatives F_m at the
 // quadrature points of every octave of xi (double-double, one thread per
 // point), the rows at the Chebyshev points of every cell (one thread per cell
 // and point, all classes at once, since e^{-z} j_m is theirs in common), the
-// same for the far region, and the polynomial coefficients with the check of
-// every cell at one of its corners.  Bound by the FP64 pipe; setting a
-// factor pair with four kernels takes 0.17 s with it.
+// same for the far region, the polynomial coefficients, and the check of every
+// cell at one point.  The rows of that point come from a quadrature of its own
+// (the first two kernels again, with narrower panels): against the cells' own
+// quadrature, what that does not resolve would pass.  Bound by the FP64 pipe;
+// setting a factor pair with four kernels takes 0.17 s with it.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -25,7 +27,7 @@ namespace {
 constexpr int NCLS = 4;
 constexpr int kClass[NCLS] = {2, 3, 4, 6};
 constexpr int NODES = GR_NC + 1;              // Chebyshev points and the check point
-constexpr int ITB = 16;                       // cells of T' per block of k_rows_a
+constexpr int ITB = 16, ITC = 32;             // cells of T' per block of k_rows_a, of its check
 constexpr int NOCT = GR_XHI - GR_XLO;
 constexpr int TILE = 16;                      // quadrature points staged at a time
 
@@ -33,7 +35,6 @@ struct ClassDev {
   const GridFam *fam;
   const dd *coef;
   int nfam;
-  double b;   // largest b of its families
 };
 
 struct Build {
@@ -42,52 +43,57 @@ struct Build {
   double *cells[NCLS];
   unsigned char *ok[NCLS];
   double *V;                 // [cell][node][class][row]
-  // quadrature points, octave after octave
-  const double *x, *w;
-  const double *F;           // [point][class][row]
-  double *Fw;
-  int npts;
-  const int *pt0;            // [NOCT + 1] first point of an octave
-  const double *edge;        // [NOCT][GR_MAXPANEL + 1]
-  const int *npanel;         // [NOCT]
   double bpos, bneg;
-  const double *xt, *ztab, *node, *ghx, *ghw, *bx, *bw;
+  const double *xt, *ztab, *node, *ghx, *ghw, *ghcx, *ghcw, *bx, *bw;
   const dd *conv;
 };
 
-// Check point of a cell: one of its four corners.
-__device__ __forceinline__ double check_a(int cell) { return (cell & 1) ? 1.0 : -1.0; }
-__device__ __forceinline__ double check_s(int cell) { return (cell & 2) ? 0.5 : -0.5; }   // in units of the cell's width
+// Quadrature points, octave after octave.
+struct Quad {
+  const double *x, *w;
+  double *F;                 // [point][class][row]
+  int npts, rows;            // rows: 0 .. rows - 1
+  const int *pt0;            // [NOCT + 1] first point of an octave
+  const double *edge;        // [NOCT][GR_MAXPANEL + 1]
+  const int *npanel;         // [NOCT]
+};
 
-__global__ void k_radial(Build B) {
+__global__ void k_radial(Build B, Quad Q) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
-  if (i >= B.npts) return;
-  grid_radial(B.cls[c].fam, B.cls[c].nfam, B.cls[c].coef, B.x[i], GR_M, B.Fw + ((size_t)i * B.ncls + c) * GR_ROWS);
+  if (i >= Q.npts) return;
+  grid_radial(B.cls[c].fam, B.cls[c].nfam, B.cls[c].coef, Q.x[i], Q.rows - 1, Q.F + ((size_t)i * B.ncls + c) * Q.rows);
 }
 
-// Region A.  A block takes one cell of xi and ITB cells of T'; a thread one
-// of their (cell, node) pairs.  Bound by the FP64 pipe (e^{-z} j_m and the
-// sums); F_m of a tile of points is staged in shared memory for all threads.  A
+// Region A.  A block takes one cell of xi and IT cells of T'; a thread one
+// of their (cell, node) pairs, or (CHECK) a cell's check point.  Bound by the
+// FP64 pipe (e^{-z} j_m and the sums); F_m of a tile of points is staged in shared
+// memory for all threads.  A
 // tile's sum is added to the total with its rounding kept: some 300 points count,
-// and added one by one they left 4 u of noise in every row.
-__global__ void __launch_bounds__(NODES *ITB) k_rows_a(Build B) {
-  __shared__ double sF[TILE * NCLS * GR_ROWS];
+// and added one by one they left 4 u of noise in every row.  A check takes the
+// rows of the orders that are served only.
+template <bool CHECK>
+__global__ void __launch_bounds__(CHECK ? ITC : GR_NC *ITB) k_rows_a(Build B, Quad Q) {
+  constexpr int NN = CHECK ? 1 : GR_NC, IT = CHECK ? ITC : ITB, R = CHECK ? GR_LMAX + 1 : GR_ROWS;
+  __shared__ double sF[TILE * NCLS * R];
   __shared__ double sx[TILE], sw[TILE];
   const int ix = blockIdx.x, oct = grid_octave(ix);
-  const int n = threadIdx.x % NODES, it0 = blockIdx.y * ITB, it = it0 + threadIdx.x / NODES;
+  const int n = CHECK ? GR_NC : threadIdx.x % NN, it0 = blockIdx.y * IT, it = it0 + threadIdx.x / NN;
   const double c = B.xt[GR_XT * ix], ic = B.xt[GR_XT * ix + 1];
   const bool live = it < GR_NT;
-  const int cell = ix * GR_NT + it;
-  double lo = 0.0, hi = 0.0;
-  if (live) grid_tcell(it, &lo, &hi);
-  const double a = n < GR_NC ? B.node[n] : check_a(cell);
-  const double xi = grid_xi(B.xt + GR_XT * ix, a);
-  double u = mul_rn(0.5 * (lo + hi), ic);
-  if (n == GR_NC) u += check_s(cell) * (hi - lo) * ic;
+  const int cell = ix * GR_NT + min(it, GR_NT - 1);
+  double xi, u;
+  if (CHECK) {
+    grid_check_point(B.xt, cell, &xi, &u);
+  } else {
+    double lo, hi;
+    grid_cellu(cell, &lo, &hi);
+    xi = grid_xi(B.xt + GR_XT * ix, B.node[n]);
+    u = mul_rn(0.5 * (lo + hi), ic);
+  }
   const double D = sqrt(u);
-  const int nrow = B.ncls * GR_ROWS;
-  double acc[NCLS * GR_ROWS];
-  dd tot[NCLS * GR_ROWS];
+  const int nrow = B.ncls * R;
+  double acc[NCLS * R];
+  dd tot[NCLS * R];
   for (int k = 0; k < nrow; ++k) {
     acc[k] = 0.0;
     tot[k] = dd{0.0, 0.0};
@@ -98,20 +104,20 @@ __global__ void __launch_bounds__(NODES *ITB) k_rows_a(Build B) {
   grid_xends(ix, &clo, &chi);
   double tl, th, dummy;
   grid_tcell(it0, &tl, &dummy);
-  grid_tcell(min(it0 + ITB, GR_NT) - 1, &dummy, &th);
+  grid_tcell(min(it0 + IT, GR_NT) - 1, &dummy, &th);
   const double wl = sqrt(tl / c) - 10.5 / sqrt(clo) - 0.5 * B.bneg / clo;
   const double wh = sqrt(th / c) + 8.5 / sqrt(clo) + 0.5 * B.bpos / clo;
-  const double *edge = B.edge + (size_t)oct * (GR_MAXPANEL + 1);
-  const int p0 = B.pt0[oct];
-  for (int p = 0; p < B.npanel[oct]; ++p) {
+  const double *edge = Q.edge + (size_t)oct * (GR_MAXPANEL + 1);
+  const int p0 = Q.pt0[oct];
+  for (int p = 0; p < Q.npanel[oct]; ++p) {
     if (edge[p + 1] < wl || edge[p] > wh) continue;
     const int i0 = p0 + (p == 0 ? 0 : GR_NQ0 + (p - 1) * GR_NQ), np = p == 0 ? GR_NQ0 : GR_NQ;
     for (int t0 = 0; t0 < np; t0 += TILE) {
       __syncthreads();
-      for (int k = threadIdx.x; k < TILE * nrow; k += blockDim.x) sF[k] = B.F[(size_t)(i0 + t0) * nrow + k];
+      for (int k = threadIdx.x; k < TILE * nrow; k += blockDim.x) sF[k] = Q.F[(size_t)(i0 + t0) * nrow + k];
       if (threadIdx.x < TILE) {
-        sx[threadIdx.x] = B.x[i0 + t0 + threadIdx.x];
-        sw[threadIdx.x] = B.w[i0 + t0 + threadIdx.x];
+        sx[threadIdx.x] = Q.x[i0 + t0 + threadIdx.x];
+        sw[threadIdx.x] = Q.w[i0 + t0 + threadIdx.x];
       }
       __syncthreads();
       if (!live) continue;
@@ -120,9 +126,9 @@ __global__ void __launch_bounds__(NODES *ITB) k_rows_a(Build B) {
         double jh[GR_ROWS];
         grid_jhat(B.ztab, 2.0 * xi * D * x, jh);
         const double *f = sF + i * nrow;
-        for (int m = 0; m <= GR_M; ++m) {
+        for (int m = 0; m < R; ++m) {
           const double v = e * jh[m];
-          for (int k = 0; k < B.ncls; ++k) acc[k * GR_ROWS + m] = fma(v, f[k * GR_ROWS + m], acc[k * GR_ROWS + m]);
+          for (int k = 0; k < B.ncls; ++k) acc[k * R + m] = fma(v, f[k * R + m], acc[k * R + m]);
         }
       }
       for (int k = 0; k < nrow; ++k) {
@@ -134,43 +140,57 @@ __global__ void __launch_bounds__(NODES *ITB) k_rows_a(Build B) {
   }
   if (!live) return;
   double f = 4.0 * xi * sqrt(xi);
-  double *V = B.V + ((size_t)cell * NODES + n) * nrow;
-  for (int m = 0; m <= GR_M; ++m) {
-    for (int k = 0; k < B.ncls; ++k) V[k * GR_ROWS + m] = f * (tot[k * GR_ROWS + m].h + tot[k * GR_ROWS + m].l);
+  double *V = B.V + ((size_t)cell * NODES + n) * B.ncls * GR_ROWS;
+  for (int m = 0; m < R; ++m) {
+    for (int k = 0; k < B.ncls; ++k) V[k * GR_ROWS + m] = f * (tot[k * R + m].h + tot[k * R + m].l);
     f *= 2.0 * xi;
   }
 }
 
 // Region B: one block per cell of u.  F_m is evaluated at the Chebyshev points
-// of x/D and interpolated at the quadrature nodes.
+// of x/D and interpolated at the quadrature nodes; at the nodes of the check
+// point's rule it is evaluated itself.
 __global__ void __launch_bounds__(128) k_rows_b(Build B) {
-  extern __shared__ double sB[];   // [GR_NB][ncls][row], then a row of rows per node
+  extern __shared__ double sB[];   // [GR_NB][ncls][row], [GR_NHC][ncls][row], then a row of rows per node
   const int iu = blockIdx.x, cell = GR_NX * GR_NT + iu, nrow = B.ncls * GR_ROWS;
-  double lo, hi;
+  double *sC = sB + GR_NB * nrow;
+  double lo, hi, cxi, cu;
   grid_ucell(iu, &lo, &hi);
-  // the check point has its own u, inside the interpolated range of x
-  const double D0 = sqrt(0.5 * (lo + hi));
-  for (int t = threadIdx.x; t < GR_NB * B.ncls; t += blockDim.x) {
+  grid_check_point(B.xt, cell, &cxi, &cu);
+  const double D0 = sqrt(0.5 * (lo + hi)), cD = sqrt(cu), cis = 1.0 / sqrt(cxi);
+  for (int t = threadIdx.x; t < (GR_NB + GR_NHC) * B.ncls; t += blockDim.x) {
     const int j = t / B.ncls, k = t % B.ncls;
-    const double x = D0 * (1.0 + (GR_BW + 0.02) * B.bx[j]);
-    double *F = sB + j * nrow + k * GR_ROWS;
-    grid_radial(B.cls[k].fam, B.cls[k].nfam, B.cls[k].coef, x, GR_M, F);
-    // interpolated without the growth of e^{bx}, which would cost the small values their digits
-    const double e = exp(-B.cls[k].b * (x - D0));
-    for (int m = 0; m <= GR_M; ++m) F[m] *= e;
+    const double x = j < GR_NB ? D0 * (1.0 + (GR_BW + 0.02) * B.bx[j]) : cD + B.ghcx[j - GR_NB] * cis;
+    grid_radial(B.cls[k].fam, B.cls[k].nfam, B.cls[k].coef, x, GR_M, sB + j * nrow + k * GR_ROWS);
   }
   __syncthreads();
-  double *acc = sB + GR_NB * nrow + threadIdx.x * (nrow + 1);
+  double b[NCLS];
+  const double xlo = D0 * (1.0 + (GR_BW + 0.02) * B.bx[GR_NB - 1]), xhi = D0 * (1.0 + (GR_BW + 0.02) * B.bx[0]);
+  for (int k = 0; k < B.ncls; ++k)
+    b[k] = grid_slope(sB + (GR_NB - 1) * nrow + k * GR_ROWS, sB + k * GR_ROWS, xhi - xlo);
+  __syncthreads();
+  for (int t = threadIdx.x; t < GR_NB * B.ncls; t += blockDim.x) {
+    const int j = t / B.ncls, k = t % B.ncls;
+    const double e = exp(-b[k] * D0 * (GR_BW + 0.02) * B.bx[j]);
+    for (int m = 0; m <= GR_M; ++m) sB[j * nrow + k * GR_ROWS + m] *= e;
+  }
+  __syncthreads();
   const int n = threadIdx.x;
   if (n >= NODES) return;
-  const double a = n < GR_NC ? B.node[n] : 0.97 * check_a(cell);   // (a = -1 is xi = infinity)
-  const double xi = 2.0 * GR_TB / (hi * (a + 1.0)), is = 1.0 / sqrt(xi);
-  const double D = n < GR_NC ? D0 : sqrt(0.5 * (lo + hi) + check_s(cell) * (hi - lo));
+  double *acc = sC + GR_NHC * nrow + n * (nrow + 1);
+  const bool check = n == GR_NC;
+  const double xi = check ? cxi : 2.0 * GR_TB / (hi * (B.node[n] + 1.0)), is = 1.0 / sqrt(xi);   // (a = -1 is xi = infinity)
+  const double D = check ? cD : D0;
   for (int k = 0; k < nrow; ++k) acc[k] = 0.0;
-  for (int i = 0; i < GR_NH; ++i) {
-    const double x = D + B.ghx[i] * is;
-    double jh[GR_ROWS], bw[GR_NB], den = 0.0;
+  for (int i = 0; i < (check ? GR_NHC : GR_NH); ++i) {
+    const double x = D + (check ? B.ghcx[i] : B.ghx[i]) * is;
+    double jh[GR_ROWS];
     grid_jhat(B.ztab, 2.0 * xi * D * x, jh);
+    if (check) {
+      for (int k = 0; k < nrow; ++k) acc[k] = fma(B.ghcw[i] * jh[k % GR_ROWS], sC[i * nrow + k], acc[k]);
+      continue;
+    }
+    double bw[GR_NB], den = 0.0;
     const double y = (x / D0 - 1.0) / (GR_BW + 0.02);
     int hit = -1;
     for (int j = 0; j < GR_NB; ++j) {
@@ -181,7 +201,7 @@ __global__ void __launch_bounds__(128) k_rows_b(Build B) {
     }
     for (int j = 0; j < GR_NB; ++j) bw[j] = hit < 0 ? bw[j] / den : (j == hit ? 1.0 : 0.0);
     for (int c = 0; c < B.ncls; ++c) {
-      const double e = B.ghw[i] * exp(B.cls[c].b * (x - D0));
+      const double e = B.ghw[i] * exp(b[c] * (x - D0));
       for (int m = 0; m <= GR_M; ++m) {
         const int k = c * GR_ROWS + m;
         double f = 0.0;
@@ -216,44 +236,17 @@ __global__ void k_fit(Build B) {
   }
 }
 
-// A cell is in order when orders 0..8 at its check point agree with the
-// quadrature to kCellTol of the sum of the terms' magnitudes (the scale of the
-// result where it passes through zero).
-constexpr double kCellTol = 3e-13;
 __global__ void k_check(Build B) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int cell = (int)(t / B.ncls), c = (int)(t % B.ncls);
   if (cell >= GR_CELLS) return;
   const int nrow = B.ncls * GR_ROWS;
-  const double *V = B.V + ((size_t)cell * NODES + GR_NC) * nrow + c * GR_ROWS;
-  const double *C = B.cells[c] + (size_t)cell * GR_CELL;
-  double lo, hi, hd, a = check_a(cell);
-  if (cell < GR_NX * GR_NT) {
-    grid_tcell(cell % GR_NT, &lo, &hi);
-    hd = 0.5 * check_s(cell) * (hi - lo) * B.xt[GR_XT * (cell / GR_NT) + 1];
-  } else {
-    grid_ucell(cell - GR_NX * GR_NT, &lo, &hi);
-    hd = 0.5 * check_s(cell) * (hi - lo);
-    a *= 0.97;
-  }
-  constexpr int L = 8, N = grid_terms(L);
-  double row[L + N + 1];
-  for (int m = 0; m <= L + N; ++m) {
-    double r = C[m * GR_NC + GR_NC - 1];
-    for (int i = GR_NC - 2; i >= 0; --i) r = fma(r, a, C[m * GR_NC + i]);
-    row[m] = r;
-  }
+  double lo, hi;
+  grid_cellu(cell, &lo, &hi);
   // region B: e^{bx} must vary little enough over a width for the rule's 20 nodes
-  bool ok = cell < GR_NX * GR_NT || fmax(B.bpos, B.bneg) * sqrt(hi / GR_TB) <= 3.0;
-  for (int l = 0; l <= L; ++l) {
-    double s = 0.0, sc = 0.0, w = 1.0;
-    for (int k = 0; k <= N; ++k) {
-      s = fma(row[l + k], w, s);
-      sc += fabs(row[l + k] * w);
-      w *= hd / (k + 1);
-    }
-    ok = ok && fabs(s - V[l]) <= kCellTol * sc;   // false for NaN
-  }
+  const bool flat = cell < GR_NX * GR_NT || fmax(B.bpos, B.bneg) * sqrt(hi / GR_TB) <= 3.0;
+  const bool ok = flat && grid_cell_ok(B.xt, cell, B.cells[c] + (size_t)cell * GR_CELL,
+                                       B.V + ((size_t)cell * NODES + GR_NC) * nrow + c * GR_ROWS);
   B.ok[c][cell] = ok ? 1 : 0;
 }
 
@@ -334,19 +327,24 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
       cls_of[B.ncls++] = kClass[k];
     }
   if (!B.ncls) return nullptr;
-  std::vector<double> x, w, edge((size_t)NOCT * (GR_MAXPANEL + 1), 0.0);
-  std::vector<int> pt0, npanel;
-  for (int o = 0; o < NOCT; ++o) {
-    GridQuad q;
-    const double lo = std::ldexp(1.0, GR_XLO + o);
-    if (!grid_quad(gc, B.ncls, lo, 2.0 * lo, q)) return nullptr;
-    pt0.push_back((int)x.size());
-    npanel.push_back((int)q.edge.size() - 1);
-    x.insert(x.end(), q.x.begin(), q.x.end());
-    w.insert(w.end(), q.w.begin(), q.w.end());
-    std::copy(q.edge.begin(), q.edge.end(), edge.begin() + (size_t)o * (GR_MAXPANEL + 1));
+  struct HostQuad {   // the cells' quadrature, the check's
+    std::vector<double> x, w, edge;
+    std::vector<int> pt0, npanel;
+  } hq[2];
+  for (int k = 0; k < 2; ++k) {
+    hq[k].edge.assign((size_t)NOCT * (GR_MAXPANEL + 1), 0.0);
+    for (int o = 0; o < NOCT; ++o) {
+      GridQuad q;
+      const double lo = std::ldexp(1.0, GR_XLO + o);
+      if (!grid_quad(gc, B.ncls, lo, 2.0 * lo, q, k ? GR_CHECK_SCALE : 1.0)) return nullptr;
+      hq[k].pt0.push_back((int)hq[k].x.size());
+      hq[k].npanel.push_back((int)q.edge.size() - 1);
+      hq[k].x.insert(hq[k].x.end(), q.x.begin(), q.x.end());
+      hq[k].w.insert(hq[k].w.end(), q.w.begin(), q.w.end());
+      std::copy(q.edge.begin(), q.edge.end(), hq[k].edge.begin() + (size_t)o * (GR_MAXPANEL + 1));
+    }
+    hq[k].pt0.push_back((int)hq[k].x.size());
   }
-  pt0.push_back((int)x.size());
   static const std::vector<double> ztab = [] {
     std::vector<double> t;
     grid_ztab(t);
@@ -358,9 +356,10 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
     grid_conversion(m);
     std::memcpy(conv.data(), m, sizeof(m));
   }
-  std::vector<double> node(GR_NC), ghx(GR_NH), ghw(GR_NH), bx(GR_NB), bw(GR_NB), xt((size_t)GR_XT * GR_NX, 0.0);
+  std::vector<double> node(GR_NC), ghx(GR_NH), ghw(GR_NH), ghcx(GR_NHC), ghcw(GR_NHC), bx(GR_NB), bw(GR_NB), xt((size_t)GR_XT * GR_NX, 0.0);
   grid_nodes(node.data());
   gauss_hermite(GR_NH, ghx.data(), ghw.data());
+  gauss_hermite(GR_NHC, ghcx.data(), ghcw.data());
   for (int j = 0; j < GR_NB; ++j) {   // Chebyshev points of the first kind and their barycentric weights
     const double th = M_PI * (j + 0.5) / GR_NB;
     bx[(size_t)j] = std::cos(th);
@@ -374,7 +373,7 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
   Temp tmp;
   bool good = true;
   for (int k = 0; k < B.ncls && good; ++k) {
-    B.cls[k] = ClassDev{tmp.up(gc[k].fam, good), tmp.up(gc[k].coef, good), (int)gc[k].fam.size(), gc[k].bmax};
+    B.cls[k] = ClassDev{tmp.up(gc[k].fam, good), tmp.up(gc[k].coef, good), (int)gc[k].fam.size()};
     const int c = cls_of[k];
     good = good && cudaMalloc((void **)&g->cells[c], sizeof(double) * (size_t)GR_CELLS * GR_CELL) == cudaSuccess &&
            cudaMalloc((void **)&g->ok[c], (size_t)GR_CELLS) == cudaSuccess;
@@ -385,12 +384,13 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
   good = good && cudaMalloc((void **)&g->xt, sizeof(double) * xt.size()) == cudaSuccess &&
          cudaMemcpy(g->xt, xt.data(), sizeof(double) * xt.size(), cudaMemcpyHostToDevice) == cudaSuccess;
   const int nrow = B.ncls * GR_ROWS;
-  B.npts = (int)x.size();
-  B.x = tmp.up(x, good);
-  B.w = tmp.up(w, good);
-  B.pt0 = tmp.up(pt0, good);
-  B.npanel = tmp.up(npanel, good);
-  B.edge = tmp.up(edge, good);
+  Quad Q[2];
+  for (int k = 0; k < 2; ++k) {
+    const int rows = k ? GR_LMAX + 1 : GR_ROWS;
+    Q[k] = Quad{tmp.up(hq[k].x, good), tmp.up(hq[k].w, good),
+                tmp.get<double>(hq[k].x.size() * (size_t)(B.ncls * rows), good), (int)hq[k].x.size(), rows,
+                tmp.up(hq[k].pt0, good), tmp.up(hq[k].edge, good), tmp.up(hq[k].npanel, good)};
+  }
   B.ztab = tmp.up(ztab, good);
   B.node = tmp.up(node, good);
   B.ghx = tmp.up(ghx, good);
@@ -398,8 +398,8 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
   B.bx = tmp.up(bx, good);
   B.bw = tmp.up(bw, good);
   B.conv = tmp.up(conv, good);
-  B.Fw = tmp.get<double>((size_t)B.npts * nrow, good);
-  B.F = B.Fw;
+  B.ghcx = tmp.up(ghcx, good);
+  B.ghcw = tmp.up(ghcw, good);
   B.V = tmp.get<double>((size_t)GR_CELLS * NODES * nrow, good);
   B.xt = g->xt;
   B.bpos = bpos;
@@ -408,9 +408,10 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
     cudaGetLastError();
     return nullptr;
   }
-  k_radial<<<dim3((unsigned)((B.npts + 63) / 64), (unsigned)B.ncls), 64, 0, st>>>(B);
-  k_rows_a<<<dim3(GR_NX, (GR_NT + ITB - 1) / ITB), NODES * ITB, 0, st>>>(B);
-  const size_t smb = sizeof(double) * ((size_t)GR_NB * nrow + (size_t)NODES * (nrow + 1));
+  for (const Quad &q : Q) k_radial<<<dim3((unsigned)((q.npts + 63) / 64), (unsigned)B.ncls), 64, 0, st>>>(B, q);
+  k_rows_a<false><<<dim3(GR_NX, (GR_NT + ITB - 1) / ITB), GR_NC * ITB, 0, st>>>(B, Q[0]);
+  k_rows_a<true><<<dim3(GR_NX, (GR_NT + ITC - 1) / ITC), ITC, 0, st>>>(B, Q[1]);
+  const size_t smb = sizeof(double) * ((size_t)(GR_NB + GR_NHC) * nrow + (size_t)NODES * (nrow + 1));
   cudaFuncSetAttribute(k_rows_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
   k_rows_b<<<GR_NU, 128, smb, st>>>(B);
   k_fit<<<(unsigned)(((int64_t)GR_CELLS * nrow + 127) / 128), 128, 0, st>>>(B);

@@ -17,7 +17,6 @@ struct GridClass {
   std::vector<dd> coef;
   std::vector<double> g, reach;        // the families' g > 0, and how far they count
   double bpos = 0.0, bneg = 0.0;       // largest b > 0, largest |b| of b < 0
-  double bmax = -1e300;                // largest b
 };
 
 // Distance past which a family x^alpha e^{bx - gx^2}, alpha <= amax, is below
@@ -79,7 +78,6 @@ inline bool grid_families(const f12::TermList &kernel, GridClass &gc) {
       gc.g.push_back(f.g);
       gc.reach.push_back(grid_reach(a + (double)f.poly.size() - 1.0 + 2.0 * GR_M, f.b, f.g));
     }
-    gc.bmax = std::max(gc.bmax, f.b);
     gc.bpos = std::max(gc.bpos, f.b);
     gc.bneg = std::max(gc.bneg, -f.b);
     reach = reach || f.g == 0.0;
@@ -100,7 +98,8 @@ constexpr int GR_MAXPANEL = 400;
 // x^{alpha} du smooth for the powers grid_families admits; the others are at
 // most 1.5 times as wide as their distance from r = 0, where the long-range
 // families have a branch point: where narrow panels end (a tight Gaussian's
-// reach) one of full width would not resolve it.
+// reach) one of full width would not resolve it.  scale < 1: every panel that
+// much narrower (0.8: a thousandth of the error or less), for the cells' check.
 struct GridQuad {
   std::vector<double> x, w;
   std::vector<double> edge;   // panel p covers [edge[p], edge[p + 1]]
@@ -153,7 +152,9 @@ inline GridRule grid_rule(int n, bool corrected) {
     }
   return r;
 }
-inline bool grid_quad(const GridClass *gc, int ngc, double xi_lo, double xi_hi, GridQuad &q) {
+constexpr double GR_CHECK_SCALE = 0.8;
+inline bool grid_quad(const GridClass *gc, int ngc, double xi_lo, double xi_hi, GridQuad &q,
+                      double scale = 1.0) {
   q = GridQuad{};
   static const GridRule rule = grid_rule(GR_NQ, true), rule0 = grid_rule(GR_NQ0, false);
   double bpos = 0.0, bneg = 0.0;
@@ -171,6 +172,7 @@ inline bool grid_quad(const GridClass *gc, int ngc, double xi_lo, double xi_hi, 
         if (a < gc[c].reach[i]) w = std::min(w, 1.25 / std::sqrt(xi_hi + gc[c].g[i]));
     if (bneg > 0.0) w = std::min(w, 1.25 * std::sqrt(std::max(1.0, bneg * a)) / bneg);
     if (a > 0.0) w = std::min(w, 1.5 * a);
+    w *= scale;
     if (a == 0.0) {
       w *= 0.5;
       for (int i = 0; i < GR_NQ0; ++i) {

@@ -1,7 +1,7 @@
 """Single cells of the auxiliary grid, built on the CPU from the library's own
 headers (tests/grid_host.cpp), against the oracle: factors whose Gaussian parts
 are much tighter than the exponents of a basis, decaying and growing long
-ranges, and orders up to 14."""
+ranges, orders up to 14, and what the library's check of a cell accepts."""
 import ctypes
 import os
 import shutil
@@ -37,6 +37,7 @@ def lib():
     L.grid_host_new.argtypes = [dp, ctypes.c_int, dp, ctypes.c_int, ctypes.c_int]
     L.grid_host_new.restype = ctypes.c_void_p
     L.grid_host_free.argtypes = [ctypes.c_void_p]
+    L.grid_host_ok.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_double]
     L.grid_host_eval.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_double, ctypes.c_int, dp]
     return L
 
@@ -58,21 +59,27 @@ class Grid:
         if getattr(self, "p", None):
             self.lib.grid_host_free(self.p)
 
+    def ok(self, xi, D):
+        return self.lib.grid_host_ok(self.p, xi, D)
+
     def eval(self, xi, D, L):
         out = np.zeros(L + 1)
         assert self.lib.grid_host_eval(self.p, xi, D, L, out.ctypes.data_as(dp)) == 0
         return out
 
 
-def errors(grid, kern, cls, pts, L):
+def reference(kern, cls, pts):
+    with ThreadPoolExecutor(max_workers=min(16, os.cpu_count() or 1)) as ex:
+        return np.array(list(ex.map(lambda p: O.radial(kern, cls, p[0], p[1], 15), pts)))
+
+
+def errors(grid, ref, pts, L):
     """Relative error of every order at every point; an order that passes
     through zero is measured against a twentieth of the next over the local
     width, as in the GPU test of the grid."""
-    with ThreadPoolExecutor(max_workers=min(16, os.cpu_count() or 1)) as ex:
-        ref = np.array(list(ex.map(lambda p: O.radial(kern, cls, p[0], p[1], L + 1), pts)))
     got = np.array([grid.eval(x, d, L) for x, d in pts])
     w = np.array([min(d * d + 1e-300, 1.0 / x) for x, d in pts])
-    return np.abs(got - ref[:, :-1]) / (np.abs(ref[:, :-1]) + 0.05 * np.abs(ref[:, 1:]) * w[:, None])
+    return np.abs(got - ref[:, :L + 1]) / (np.abs(ref[:, :L + 1]) + 0.05 * np.abs(ref[:, 1:L + 2]) * w[:, None])
 
 
 TIGHT = {
@@ -95,10 +102,10 @@ def test_tight_gaussians(lib, name, cls):
     (exponents of an ordinary basis, a molecule's distances).  1e-10: what the
     auxiliary stage holds for the orders of its general classes."""
     g = Grid(lib, TIGHT[name], cls)
-    kern = O.factor_kernel_terms(TIGHT[name])
     pts = [(0.112, 0.0), (0.112, 3.1), (0.7, 0.02), (3.3, 1.1), (21.0, 0.0), (150.0, 0.6)]
+    ref = reference(O.factor_kernel_terms(TIGHT[name]), cls, pts)
     for L in (8, 14):
-        e = errors(g, kern, cls, pts, L)
+        e = errors(g, ref, pts, L)
         assert e.max() < 1e-10, (L, e.max(1))
 
 
@@ -116,3 +123,42 @@ def test_rounding_of_the_quadrature(lib):
         ref = np.array(list(ex.map(lambda p: O.radial(kern, 3, p[0], p[1], 0)[0], pts)))
     e = np.array([g.eval(x, d, 0)[0] for x, d in pts]) / ref - 1.0
     assert np.sqrt(np.mean(e * e)) < 3.0 * 2.0 ** -53
+
+
+ACCEPT = {
+    "default": rs12(),
+    "B=2": rs12(B=2.0),
+    "B=-0.5": rs12(B=-0.5),
+    "B=-1.3": rs12(B=-1.3),
+    "B=-4": rs12(B=-4.0),
+    "mu=2000": rs12(2000.0),
+    "long range and g=1000": [(0.5, 0.5, 0.5, 0), (0.8, 0, 0, 1000.0)],
+}
+
+
+@pytest.mark.parametrize("name", list(ACCEPT))
+@pytest.mark.parametrize("cls", [2, 3, 4, 6])
+def test_accepted_cells(lib, name, cls):
+    """In both regions, out to where the exponents are diffuse and the kernels
+    have grown or decayed, a cell that the check accepts holds every form that
+    the kernels take to 1e-10 anywhere inside, not at the check's point alone
+    (the check asks 1e-12 of one corner).  Points with next to no refusals as
+    well, so that a check that refuses everything fails."""
+    g = Grid(lib, ACCEPT[name], cls)
+    pts = [(0.0088, 0.0), (0.0102, 2.2), (0.0213, 1.0), (0.05, 9.3), (0.105, 0.0), (0.12, 20.2), (0.47, 6.9), (2.2, 14.3),
+           (3.0, 0.7), (22.0, 9.1), (112.0, 3.1), (112.0, 7.9), (300.0, 1.9)]
+    good = [p for p in pts if g.ok(*p) == 1]
+    assert (0.47, 6.9) in good and (3.0, 0.7) in good and (112.0, 3.1) in good
+    ref = reference(O.factor_kernel_terms(ACCEPT[name]), cls, good)
+    for L in (0, 4, 8, 14):
+        e = errors(g, ref, good, L)
+        assert e.max() < 1e-10, (L, good[int(e.max(1).argmax())], e.max())
+
+
+def test_default_factor_stays_on_the_grid(lib):
+    """The default factor and its decaying form over the exponents and
+    distances of the repository's molecules: nothing is refused."""
+    for terms in (rs12(), rs12(B=-0.5)):
+        for cls in (3, 4, 6):
+            g = Grid(lib, terms, cls)
+            assert all(g.ok(xi, D) == 1 for xi in (0.02, 0.0305, 4.1, 500.0) for D in (0.0, 8.0, 20.0))
