@@ -50,11 +50,7 @@ struct EngineReq {
   int64_t tasks[7] = {0};         // contraction tasks per class (before screening)
 };
 
-struct TicketState {
-  bool done = false;
-  int rc = F12INT_OK;
-  int batch = -1;                 // staging buffer of the batch that runs it
-};
+using f12engine::TicketState;
 
 // Contraction plan of a quartet in a batch: ket ranges (the fewest that fit,
 // more while a task would exceed `target` flops), the tier that holds them,
@@ -763,12 +759,8 @@ static bool engine_idle(f12int_ctx *ctx) {
   Engine *E = ctx->engine;
   if (!E) return true;
   std::lock_guard<std::mutex> lk(E->mu);
-  for (const auto &kv : E->tickets)
-    if (!kv.second.done) {
-      const int b = kv.second.batch;
-      if (b < 0 || cudaEventQuery(E->ev[b]) != cudaSuccess) return false;
-    }
-  return E->pending.empty();
+  return E->pending.empty() &&
+         f12engine::tickets_idle(E->tickets, E->inflight, [&](int b) { return cudaEventQuery(E->ev[b]) == cudaSuccess; });
 }
 
 // The captured graph holds the factor's tables by value.

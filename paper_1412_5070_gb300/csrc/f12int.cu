@@ -44,6 +44,7 @@
 #include "auxtab.h"
 #include "grid.h"
 #include "termlist.h"
+#include "tickets.h"
 
 using namespace f12dev;
 using namespace f12k;

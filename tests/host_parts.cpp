@@ -1,0 +1,22 @@
+// host_parts.cpp -- CPU build of the library's host-side parts that need no
+// CUDA, for tests.  The library never loads this file's build.
+#include <cstdint>
+#include <unordered_map>
+#include <vector>
+
+#include "../paper_1412_5070_gb300/csrc/tickets.h"
+
+extern "C" {
+
+// One ticket: done or not, its staging buffer (-1: none yet), whether it is in
+// flight there, and what the buffer's event says.
+int host_tickets_idle(int done, int batch, int in_flight, int event_done) {
+  std::unordered_map<uint64_t, f12engine::TicketState> t;
+  t[7].done = done != 0;
+  t[7].batch = batch;
+  std::vector<uint64_t> f[2];
+  if (in_flight) f[batch].push_back(7);
+  return f12engine::tickets_idle(t, f, [&](int) { return event_done != 0; }) ? 1 : 0;
+}
+
+}  // extern "C"

@@ -1,0 +1,67 @@
+"""State of the batch engine and its context on the GPU: what is refused while a
+batch runs, what a small budget leaves usable, and calls after an error."""
+import time
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_1412_5070_gb300 import build as B
+from paper_1412_5070_gb300 import f12int as F
+from paper_1412_5070_gb300 import molecules as M
+
+from test_gpu_batch import layout, per_call, sample
+
+
+def make(budget=0):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    B.build()
+    return F.f12int_create(0, budget, None)
+
+
+def finish(ctx, t, limit_s=120.0):
+    t0 = time.time()
+    while not F.f12int_poll(ctx, t, 100_000):
+        assert time.time() - t0 < limit_s, "request did not finish"
+
+
+def test_settings_are_refused_between_the_passes_of_a_batch():
+    """A batch whose Hermite rows exceed the class's buffer runs in passes.  Until
+    the last one is launched and done, calls that change what it reads are
+    refused (the series cap here, set to what it is)."""
+    ctx = make()
+    try:
+        F.f12int_set_factor(ctx, M.P0)
+        F.f12int_batch_limits(ctx, 4096, 1 << 18)
+        basis = M.random_molecule(5, 4, 8.0, 1.8, (1, 1, 2, 2), (2, 3), (0.1, 60.0))
+        bid = F.f12int_set_basis(ctx, basis)
+        q = sample(basis, 3, 2000, 4)
+        q = q[np.argsort(-basis.l[q].sum(axis=1))][:400]
+        pq = np.prod(basis.nprim[q], axis=1)
+        q = q[np.cumsum(pq) * 5 < (1 << 18)]      # five families at most: one request
+        off, tot = layout(basis, q, (3,))
+        out = torch.zeros(tot, dtype=torch.float64, device="cuda")
+        finish(ctx, F.f12int_submit(ctx, bid, q, (3,), out, off))   # bounds, buffers, graph
+        refused = 0
+        for _ in range(5):
+            t = F.f12int_submit(ctx, bid, q, (3,), out, off)
+            done = False
+            while not done:
+                try:
+                    F.f12int_set_series_cap(ctx, 0)
+                    accepted = True
+                except F.F12IntError as e:
+                    assert e.status == F.EINVAL
+                    accepted = False
+                    refused += 1
+                done = F.f12int_poll(ctx, t, 0)
+                assert done or not accepted
+        assert refused > 0
+        ref = per_call(ctx, bid, 3, q, basis)
+        tol = 1e-13 * np.abs(ref) + 1e-15 * np.max(np.abs(ref))
+        assert np.all(np.abs(out.cpu().numpy() - ref) <= tol)
+    finally:
+        F.f12int_destroy(ctx)

@@ -1,0 +1,39 @@
+"""Host-side parts of the library that need no GPU, compiled from its headers
+(tests/host_parts.cpp)."""
+import ctypes
+import glob
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1412_5070_gb300", "csrc")
+SRC = os.path.join(HERE, "host_parts.cpp")
+LIB = os.path.join(HERE, "_build", "libhostparts.so")
+
+
+@pytest.fixture(scope="module")
+def lib():
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no C++ compiler")
+    os.makedirs(os.path.dirname(LIB), exist_ok=True)
+    deps = [SRC] + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
+    if not os.path.exists(LIB) or any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in deps):
+        tmp = LIB + ".tmp%d" % os.getpid()
+        subprocess.run([gxx, "-O1", "-std=c++17", "-fPIC", "-shared", "-pthread", "-o", tmp, SRC], check=True)
+        os.replace(tmp, LIB)
+    return ctypes.CDLL(LIB)
+
+
+def test_a_batch_is_running_until_its_last_launch(lib):
+    """A ticket whose batch is being launched is not in flight yet; its staging
+    buffer's event is an earlier batch's, complete or never recorded."""
+    idle = lib.host_tickets_idle
+    assert idle(0, -1, 0, 1) == 0                          # queued
+    assert idle(0, 0, 0, 1) == 0 and idle(0, 1, 0, 1) == 0  # between the passes of its batch
+    assert idle(0, 0, 1, 0) == 0                           # in flight
+    assert idle(0, 0, 1, 1) == 1                           # finished, not yet reported
+    assert idle(1, -1, 0, 1) == 1                          # done
