@@ -142,7 +142,7 @@ def test_accepted_cells(lib, name, cls):
     """In both regions, out to where the exponents are diffuse and the kernels
     have grown or decayed, a cell that the check accepts holds every form that
     the kernels take to 1e-10 anywhere inside, not at the check's point alone
-    (the check asks 1e-12 of one corner).  Points with next to no refusals as
+    (the check asks 1e-12 of one corner, 5e-11 of orders past 8).  Points with next to no refusals as
     well, so that a check that refuses everything fails."""
     g = Grid(lib, ACCEPT[name], cls)
     pts = [(0.0088, 0.0), (0.0102, 2.2), (0.0213, 1.0), (0.05, 9.3), (0.105, 0.0), (0.12, 20.2), (0.47, 6.9), (2.2, 14.3),
@@ -162,3 +162,5 @@ def test_default_factor_stays_on_the_grid(lib):
         for cls in (3, 4, 6):
             g = Grid(lib, terms, cls)
             assert all(g.ok(xi, D) == 1 for xi in (0.02, 0.0305, 4.1, 500.0) for D in (0.0, 8.0, 20.0))
+            # (high orders pass through zero here)
+            assert all(g.ok(xi, np.sqrt(T / xi)) == 1 for xi in (0.133, 0.266, 0.53) for T in (0.3, 0.4, 0.9))
