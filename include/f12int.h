@@ -317,7 +317,10 @@ int f12int_poll(f12int_ctx *ctx, uint64_t ticket, int64_t timeout_us, int *done)
 /* Capacity of one batch, per class: max_quartets shell quartets and
  * max_items auxiliary work items (primitive quartets times the kernel's term
  * families); each class has its own item buffers (136 bytes per item, which
- * also hold the Hermite rows; a batch whose rows exceed them runs in passes).
+ * also hold the Hermite rows; a batch whose rows exceed them runs in passes),
+ * and room for the rows of one outer primitive pair (1.4 MB, or 5.4 kB times
+ * the square root of max_items where that is more; where memory allows, up to
+ * 64 MB more for bases that the grid of auxiliary functions does not cover).
  * Default 2^19 quartets; the default item capacity is set from free device
  * memory when the engine starts (the six classes' item buffers take at most
  * a quarter of it, 2^26 items per class at most).  Only before the first

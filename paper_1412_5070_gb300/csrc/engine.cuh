@@ -104,10 +104,6 @@ struct ClassLists {
 constexpr int kCounts = 3 + 2 * kSlots;
 constexpr int kTaskCounts = 3;           // first of the tiers' (begin, end)
 
-// Hermite rows that a class's buffer holds at least: one bra pair of 1000 ket
-// pairs at the highest order
-constexpr int64_t kRowsLeast = 684 * 1024;
-
 struct Engine {
   // limits
   int64_t qcap = (int64_t)1 << 19;   // quartets per class per batch
@@ -123,7 +119,8 @@ struct Engine {
   int *keys[7] = {nullptr};             // per class: item keys, key order, histogram, partials
   unsigned *order[7] = {nullptr}, *hist[7] = {nullptr};
   double *part[7] = {nullptr};
-  double *rows[2][7] = {};              // Hermite rows: per class by graph (the grid graph's in part)
+  double *rows[2][7] = {};              // Hermite rows: per class by graph (the grid graph's are all of part)
+  bool rows_own = false;                // rows[0] are buffers of their own (else the ends of part)
   int64_t rcap[2] = {0, 0};             // doubles of them
   unsigned *status = nullptr;
   size_t bytes = 0;
@@ -228,25 +225,6 @@ static int engine_capture(f12int_ctx *ctx, Engine &E, bool grid) {
       CK(cudaFuncSetAttribute(k_contract<true, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
       CK(cudaFuncSetAttribute(k_contract<true, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     }
-  if (!grid && !E.rows[0][1]) {
-    // the family path's rows, at its first batch: 64 MB a class, or what the
-    // budget leaves (a batch that needs more runs in several passes)
-    int rc = F12INT_ENOMEM;
-    for (int64_t want : {std::min<int64_t>((int64_t)8 << 20, E.icap * 16 + kRowsLeast), kRowsLeast}) {
-      rc = F12INT_OK;
-      for (int c = 1; c <= 6 && rc == F12INT_OK; ++c) rc = engine_alloc(ctx, E, &E.rows[0][c], (size_t)want);
-      if (rc == F12INT_OK) {
-        E.rcap[0] = want;
-        break;
-      }
-      for (int c = 1; c <= 6; ++c)
-        if (E.rows[0][c]) {
-          dfree(ctx, E.rows[0][c], sizeof(double) * (size_t)want);
-          E.bytes -= sizeof(double) * (size_t)want;
-        }
-    }
-    if (rc != F12INT_OK) return rc;
-  }
   cudaStream_t cs = nullptr;
   CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   cudaEvent_t fork = nullptr, join[7] = {nullptr}, mid[2][7] = {}, done[3][7] = {};
@@ -351,6 +329,31 @@ static int engine_capture(f12int_ctx *ctx, Engine &E, bool grid) {
   return F12INT_OK;
 }
 
+// Hermite rows of the family path's batches (a batch with more of them runs in
+// several passes): 64 MB a class where that is little of the memory left, else
+// the ends of the item buffers.  Allocated with the other buffers, under the
+// context's lock: the worker allocates nothing, and a request that was
+// admitted is not refused later for want of memory.
+static void engine_family_rows(f12int_ctx *ctx, Engine &E) {
+  const int64_t least = f12engine::rows_least(E.icap);
+  size_t left = 0, total = 0;
+  if (cudaMemGetInfo(&left, &total) != cudaSuccess) left = 0;
+  if (ctx->budget) left = std::min(left, ctx->budget > ctx->used ? ctx->budget - ctx->used : (size_t)0);
+  const int64_t want = std::min({(int64_t)8 << 20, E.icap * kPartPitch + least, (int64_t)(left / (16 * 6 * sizeof(double)))});
+  int rc = want > least ? F12INT_OK : F12INT_ENOMEM;
+  for (int c = 1; c <= 6 && rc == F12INT_OK; ++c) rc = engine_alloc(ctx, E, &E.rows[0][c], (size_t)want);
+  E.rows_own = rc == F12INT_OK;
+  E.rcap[0] = E.rows_own ? want : least;
+  if (E.rows_own) return;
+  for (int c = 1; c <= 6; ++c) {
+    if (E.rows[0][c]) {
+      dfree(ctx, E.rows[0][c], sizeof(double) * (size_t)want);
+      E.bytes -= sizeof(double) * (size_t)want;
+    }
+    E.rows[0][c] = E.part[c] + E.icap * kPartPitch;
+  }
+}
+
 // Buffers, streams and launch shapes; called once, at the first submit.
 static int engine_init(f12int_ctx *ctx, Engine &E) {
   if (E.icap == 0) {
@@ -374,7 +377,9 @@ static int engine_init(f12int_ctx *ctx, Engine &E) {
   for (int c = 1; c <= 6 && rc == F12INT_OK; ++c) {
     rc = engine_alloc(ctx, E, &E.keys[c], (size_t)E.icap);
     if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &E.order[c], (size_t)E.icap);
-    E.rcap[1] = std::max<int64_t>(E.icap * kPartPitch, kRowsLeast);
+    // the items' partial rows and, past them, the Hermite rows that any request
+    // needs; a batch on the grid has no items, and takes all of it for its rows
+    E.rcap[1] = E.icap * kPartPitch + f12engine::rows_least(E.icap);
     if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &E.part[c], (size_t)E.rcap[1]);
     E.rows[1][c] = E.part[c];
     if (rc == F12INT_OK) rc = engine_alloc(ctx, E, &E.hist[c], (size_t)kNKeys);
@@ -397,6 +402,7 @@ static int engine_init(f12int_ctx *ctx, Engine &E) {
     rc = F12INT_ECUDA;
   if (rc == F12INT_OK && cudaMemset(E.status, 0, sizeof(unsigned)) != cudaSuccess) rc = F12INT_ECUDA;
   if (rc != F12INT_OK) return rc;
+  engine_family_rows(ctx, E);
   // persistent launch shapes: resident blocks per SM from registers and shared memory
   int nsm = 0;
   CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
@@ -738,7 +744,7 @@ static void engine_shutdown(f12int_ctx *ctx) {
   for (void *p : ds)
     if (p) cudaFree(p);
   for (int c = 1; c <= 6; ++c) {
-    void *cs[] = {E->keys[c], E->order[c], E->part[c], E->hist[c], E->rows[0][c]};
+    void *cs[] = {E->keys[c], E->order[c], E->part[c], E->hist[c], E->rows_own ? E->rows[0][c] : nullptr};
     for (void *p : cs)
       if (p) cudaFree(p);
     if (E->branch[c]) cudaStreamDestroy(E->branch[c]);

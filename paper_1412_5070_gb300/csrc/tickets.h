@@ -1,8 +1,10 @@
-// tickets.h -- which requests of the batch engine are queued, running or done.
-// Plain C++ (a test exercises it without a GPU).
+// tickets.h -- which requests of the batch engine are queued, running or done,
+// and the least buffers it runs them with.  Plain C++ (a test exercises it
+// without a GPU).
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <unordered_map>
 #include <vector>
@@ -30,6 +32,14 @@ bool tickets_idle(const std::unordered_map<uint64_t, TicketState> &tickets, cons
     if (std::find(f.begin(), f.end(), kv.first) == f.end() || !event_done(t.batch)) return false;
   }
   return true;
+}
+
+// Doubles of Hermite rows with which any admitted request can run, outer pair
+// by outer pair: a quartet of at most icap primitive quartets, whose inner side
+// is the smaller one past 256 pairs, at the 680 doubles of order 14.
+inline int64_t rows_least(int64_t icap) {
+  const int64_t inner = std::max<int64_t>(256, (int64_t)std::ceil(std::sqrt((double)icap)));
+  return 680 * std::min(icap, inner);
 }
 
 }  // namespace f12engine

@@ -19,4 +19,6 @@ int host_tickets_idle(int done, int batch, int in_flight, int event_done) {
   return f12engine::tickets_idle(t, f, [&](int) { return event_done != 0; }) ? 1 : 0;
 }
 
+int64_t host_rows_least(int64_t icap) { return f12engine::rows_least(icap); }
+
 }  // extern "C"

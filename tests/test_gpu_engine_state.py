@@ -65,3 +65,59 @@ def test_settings_are_refused_between_the_passes_of_a_batch():
         assert np.all(np.abs(out.cpu().numpy() - ref) <= tol)
     finally:
         F.f12int_destroy(ctx)
+
+
+GEMINAL = [(0.35, 0, 0, 0.4), (0.3, 0, 0, 1.3), (0.2, 0, 0, 4.5)]   # not on the grid: family by family
+
+
+def test_family_batch_under_a_tight_budget():
+    """A request that submit admits is not refused by the worker for want of
+    memory: the Hermite rows of the family path come with the engine's other
+    buffers (at least what one outer pair of a request's largest quartet takes).
+    50 MB hold the engine's 20 MB and the bounds of a few shells."""
+    basis = M.random_molecule(8, 2, 6.0, 1.8, (1, 1, 1, 1), (1, 3), (0.2, 30.0))
+    q = M.canonical_quartets(basis, 3)[::3]
+    off, tot = layout(basis, q, (3, 5))
+    ctx = make(50 << 20)
+    try:
+        F.f12int_set_factor_terms(ctx, GEMINAL)
+        F.f12int_batch_limits(ctx, 1024, 1 << 14)
+        bid = F.f12int_set_basis(ctx, basis)
+        out = torch.full((tot,), float("nan"), dtype=torch.float64, device="cuda")
+        finish(ctx, F.f12int_submit(ctx, bid, q, (3, 5), out, off))
+        got = out.cpu().numpy()
+    finally:
+        F.f12int_destroy(ctx)
+    ctx = make()
+    try:
+        F.f12int_set_factor_terms(ctx, GEMINAL)
+        bid = F.f12int_set_basis(ctx, basis)
+        for k, cls in enumerate((3, 5)):
+            ref = per_call(ctx, bid, cls, q, basis)
+            mine = got[off[k, 0]:off[k, 0] + len(ref)]
+            assert np.all(np.abs(mine - ref) <= 1e-13 * np.abs(ref) + 1e-15 * np.max(np.abs(ref)))
+    finally:
+        F.f12int_destroy(ctx)
+
+
+def test_worker_allocates_nothing():
+    """The first batch of a factor that goes family by family takes no device
+    memory of its own (64 MB leave room for the instantiated graph)."""
+    ctx = make()
+    try:
+        basis = M.random_molecule(8, 2, 6.0, 1.8, (1, 1, 1, 1), (1, 3), (0.2, 30.0))
+        q = M.canonical_quartets(basis, 3)[::3]
+        off, tot = layout(basis, q, (3,))
+        out = torch.zeros(tot, dtype=torch.float64, device="cuda")
+        F.f12int_set_factor(ctx, M.P0)
+        F.f12int_batch_limits(ctx, 4096, 1 << 18)
+        bid = F.f12int_set_basis(ctx, basis)
+        finish(ctx, F.f12int_submit(ctx, bid, q, (3,), out, off))
+        F.f12int_set_factor_terms(ctx, GEMINAL)
+        per_call(ctx, bid, 3, q, basis)
+        torch.cuda.synchronize()
+        free0 = torch.cuda.mem_get_info()[0]
+        finish(ctx, F.f12int_submit(ctx, bid, q, (3,), out, off))
+        assert free0 - torch.cuda.mem_get_info()[0] < 64 << 20
+    finally:
+        F.f12int_destroy(ctx)

@@ -37,3 +37,21 @@ def test_a_batch_is_running_until_its_last_launch(lib):
     assert idle(0, 0, 1, 0) == 0                           # in flight
     assert idle(0, 0, 1, 1) == 1                           # finished, not yet reported
     assert idle(1, -1, 0, 1) == 1                          # done
+
+
+def test_least_rows_hold_an_outer_pair_of_any_admitted_quartet(lib):
+    """Sides of a and b primitive pairs, a b <= items: the inner side is either
+    one up to 256 pairs, the smaller one past that; 680 doubles a row at the
+    highest order.  And no more than is needed for small limits (a context
+    with a tight budget)."""
+    lib.host_rows_least.restype = ctypes.c_int64
+    lib.host_rows_least.argtypes = [ctypes.c_int64]
+    for items in (1, 36, 255, 256, 257, 4096, 65536, 65537, 10 ** 6, 1 << 26):
+        least = lib.host_rows_least(items)
+        for a in sorted({1, 2, 17, 255, 256, 257, 300, int(items ** 0.5), items}):
+            b = items // a
+            if b < 1:
+                continue
+            inner = min(a, b) if max(a, b) > 256 else max(a, b)
+            assert 680 * inner <= least, (items, a, b)
+    assert lib.host_rows_least(100) == 68000
