@@ -103,6 +103,8 @@ int f12int_set_basis(f12int_ctx *ctx, int nshell, const double *centers, const i
  * Errors: F12INT_EDOMAIN when mu <= 0, c0 < 0, n < 0 or n > 20, a value is
  * not finite, or rho + 2n + 2 <= 0 (the damped long-range term must be
  * integrable at r = 0, Sec. 3.1).
+ * F12INT_ENOMEM when the tables exceed the budget; the context then has no
+ * factor (calls return F12INT_ENOTREADY) until one is set.
  * Classes: the auxiliary stage evaluates the term families x^a e^{bx - gx^2}
  * of x^2 k(x) through S(alpha, beta, gamma) (Eq. sila).  Families with a < -1
  * (a factor r^rho with rho <= -1, made integrable by its damping) are

@@ -980,6 +980,14 @@ static int set_factor_lists(f12int_ctx *ctx, const f12::TermList &T1, const f12:
     if (cls != 5) kt[cls] = f12::kernel_terms(cls, T1, T2);
   ClassTables ct;
   if (!build_class_tables(kt, ct)) return F12INT_EDOMAIN;
+  // The tables are replaced one after the other: until all of them are there the
+  // context has no factor, and a call after a failure below is refused
+  // (F12INT_ENOTREADY) instead of reading freed tables or the former grid.
+  ctx->factor_ready = false;
+  ctx->tables = Tables{};
+  ctx->grid.reset();
+  for (auto &b : ctx->bases) mark_grid(ctx, b);
+  engine_factor_changed(ctx);
   const std::vector<FamDev> &fams = ct.fams;
   const std::vector<double> &coef = ct.coef;
   Tables T{};
@@ -1050,11 +1058,9 @@ static int set_factor_lists(f12int_ctx *ctx, const f12::TermList &T1, const f12:
   {
     f12::TermList gk[7];
     for (int c = 1; c <= 6; ++c) gk[c] = kt[c];
-    ctx->grid.reset();
     ctx->grid = f12grid::acquire(ctx->device, gk, ctx->cls_ok, ctx->stream);
     for (auto &b : ctx->bases) mark_grid(ctx, b);
   }
-  engine_factor_changed(ctx);
   ctx->factor_ready = true;
   return F12INT_OK;
 }

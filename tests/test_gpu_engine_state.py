@@ -121,3 +121,38 @@ def test_worker_allocates_nothing():
         assert free0 - torch.cuda.mem_get_info()[0] < 64 << 20
     finally:
         F.f12int_destroy(ctx)
+
+
+def test_no_factor_after_a_set_factor_that_failed():
+    """set_factor replaces the tables one by one; when one of them exceeds the
+    budget the context has no factor left (neither freed tables nor the former
+    grid are read), and takes the next one."""
+    one = [(1.0, 0, 0, 0.7)]
+    xi, D = torch.tensor([0.4, 3.0], dtype=torch.float64).cuda(), torch.tensor([1.0, 0.2], dtype=torch.float64).cuda()
+    for budget in (1 << k for k in range(16, 24)):   # the least of these that holds the tables of one Gaussian
+        ctx = make(budget)
+        try:
+            F.f12int_set_factor_terms(ctx, one)
+        except F.F12IntError as e:
+            assert e.status == F.ENOMEM
+            F.f12int_destroy(ctx)
+            continue
+        break
+    try:
+        out = torch.zeros((2, 3), dtype=torch.float64, device="cuda")
+        F.f12int_aux(ctx, 3, xi, D, 2, out)
+        torch.cuda.synchronize()
+        want = out.cpu().numpy().copy()
+        with pytest.raises(F.F12IntError) as e:      # the start-value tables of its growing families alone take more
+            F.f12int_set_factor(ctx, M.P0)
+        assert e.value.status == F.ENOMEM
+        with pytest.raises(F.F12IntError) as e:
+            F.f12int_aux(ctx, 3, xi, D, 2, out)
+        assert e.value.status == F.ENOTREADY
+        F.f12int_set_factor_terms(ctx, one)
+        out.zero_()
+        F.f12int_aux(ctx, 3, xi, D, 2, out)
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), want)
+    finally:
+        F.f12int_destroy(ctx)
