@@ -43,6 +43,7 @@
 #include "kernel_common.cuh"
 #include "auxtab.h"
 #include "grid.h"
+#include "perdevice.h"
 #include "termlist.h"
 #include "tickets.h"
 
@@ -450,6 +451,7 @@ struct f12int_ctx {
   double *d_jtab = nullptr;   // start-value tables of the series families
   size_t jtab_bytes = 0;
   Tables tables{};
+  const double *boys = nullptr;   // the device's table of the Boys function
   size_t fam_bytes = 0, coef_bytes = 0;
   std::shared_ptr<const f12grid::AuxGrid> grid;   // the factor's auxiliary grids (null: none)
   // basis
@@ -571,7 +573,6 @@ PairView pair_view(const f12int_ctx *ctx, const f12int_ctx::BasisData &B, int cl
   return v;
 }
 
-const double *g_boys = nullptr;   // the Kummer table's rows of a = 1 (upload_constants)
 static_assert(BY_LSTRIDE == MT_NA * MT_NX * MT_NT && BY_NT == MT_NT && BY_XMAX <= (MT_NX - 1) * MT_DX && MT_DX == 0.5,
               "boys_eval reads the Kummer table");
 
@@ -581,7 +582,7 @@ static_assert(BY_LSTRIDE == MT_NA * MT_NX * MT_NT && BY_NT == MT_NT && BY_XMAX <
 // series.
 GridView class_view(const f12int_ctx *ctx, int cls) {
   if (ctx->series_cap < KMAX) return GridView{nullptr, nullptr, nullptr};
-  if (cls == 1) return GridView{nullptr, nullptr, g_boys};
+  if (cls == 1) return GridView{nullptr, nullptr, ctx->boys};
   const int k = cls == 5 ? 3 : cls;
   if (!ctx->grid || !ctx->grid->cells[k]) return GridView{nullptr, nullptr, nullptr};
   return GridView{ctx->grid->cells[k], ctx->grid->xt, nullptr};
@@ -595,12 +596,11 @@ void mark_grid(const f12int_ctx *ctx, f12int_ctx::BasisData &B) {
     B.grid_ok[c] = ctx->grid && ctx->cls_ok[c] && f12grid::covers(*ctx->grid, c, B.exp_lo, B.exp_hi, B.dmax);
 }
 
-bool g_const_ready = false;
-std::mutex g_const_mu;
+f12host::PerDevice<const double *> g_tables;
 
-int upload_constants() {
-  std::lock_guard<std::mutex> lk(g_const_mu);
-  if (g_const_ready) return F12INT_OK;
+// Fills the constant tables of the current device; *boys: the Kummer table's
+// rows of a = 1.
+int upload_constants(const double **boys) {
   unsigned tuv[NHMAX];
   for (int s = 0; s <= 14; ++s)
     for (int t = s; t >= 0; --t)
@@ -621,23 +621,26 @@ int upload_constants() {
   CK(cudaMemcpyToSymbol(d_cser, ac.cser, sizeof(ac.cser)));
   CK(cudaMemcpyToSymbol(d_vstep, ac.vstep, sizeof(ac.vstep)));
   CK(cudaMemcpyToSymbol(d_quarter, ac.quarter, sizeof(ac.quarter)));
+  CK(cudaMemcpyToSymbol(d_htuv, tuv, sizeof(tuv)));
+  CK(cudaMemcpyToSymbol(c_gh_x, ac.gh_x, sizeof(ac.gh_x)));
+  CK(cudaMemcpyToSymbol(c_gh_w, ac.gh_w, sizeof(ac.gh_w)));
+  CK(cudaMemcpyToSymbol(c_gl_x, ac.gl_x, sizeof(ac.gl_x)));
+  CK(cudaMemcpyToSymbol(c_gl_w, ac.gl_w, sizeof(ac.gl_w)));
   {
     // the Kummer table of the b = 0 families (13.5 MB), kept for the process
     std::vector<double> kt;
     fill_kummer_table(kt);
     double *dk = nullptr;
     CK(cudaMalloc(&dk, sizeof(double) * kt.size()));
-    CK(cudaMemcpy(dk, kt.data(), sizeof(double) * kt.size(), cudaMemcpyHostToDevice));
     const double *dkc = dk;
-    CK(cudaMemcpyToSymbol(d_mtab, &dkc, sizeof(dkc)));
-    g_boys = dk + (size_t)1 * MT_NX * MT_NT;   // a = (1 + 1)/2
+    cudaError_t e = cudaMemcpy(dk, kt.data(), sizeof(double) * kt.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(d_mtab, &dkc, sizeof(dkc));
+    if (e != cudaSuccess) {
+      cudaFree(dk);
+      return cuda_fail(e);
+    }
+    *boys = dk + (size_t)1 * MT_NX * MT_NT;   // a = (1 + 1)/2
   }
-  CK(cudaMemcpyToSymbol(d_htuv, tuv, sizeof(tuv)));
-  CK(cudaMemcpyToSymbol(c_gh_x, ac.gh_x, sizeof(ac.gh_x)));
-  CK(cudaMemcpyToSymbol(c_gh_w, ac.gh_w, sizeof(ac.gh_w)));
-  CK(cudaMemcpyToSymbol(c_gl_x, ac.gl_x, sizeof(ac.gl_x)));
-  CK(cudaMemcpyToSymbol(c_gl_w, ac.gl_w, sizeof(ac.gl_w)));
-  g_const_ready = true;
   return F12INT_OK;
 }
 
@@ -698,7 +701,7 @@ int f12int_create(f12int_ctx **out, int device, size_t hbm_budget_bytes, void *c
   ctx->device = device;
   ctx->budget = hbm_budget_bytes;
   ctx->stream = (cudaStream_t)cuda_stream;
-  int rc = upload_constants();
+  int rc = g_tables.get(device, &ctx->boys, [](const double *&boys) { return upload_constants(&boys); });
   if (rc == F12INT_OK) rc = dalloc(ctx, &ctx->d_status, sizeof(unsigned int));
   if (rc == F12INT_OK && cudaMemset(ctx->d_status, 0, sizeof(unsigned int)) != cudaSuccess) rc = F12INT_ECUDA;
   for (int i = 0; i < NSIDE && rc == F12INT_OK; ++i)

@@ -4,6 +4,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "../paper_1412_5070_gb300/csrc/perdevice.h"
 #include "../paper_1412_5070_gb300/csrc/tickets.h"
 
 extern "C" {
@@ -20,5 +21,24 @@ int host_tickets_idle(int done, int batch, int in_flight, int event_done) {
 }
 
 int64_t host_rows_least(int64_t icap) { return f12engine::rows_least(icap); }
+
+// Values of a sequence of devices (fill counts its calls and fails the first
+// time for device `bad`); returns the number of fills.
+int host_per_device(const int *device, int n, int bad, int *value, int *status) {
+  f12host::PerDevice<int> t;
+  int fills = 0;
+  bool failed = false;
+  for (int i = 0; i < n; ++i)
+    status[i] = t.get(device[i], &value[i], [&](int &v) {
+      ++fills;
+      if (device[i] == bad && !failed) {
+        failed = true;
+        return -6;
+      }
+      v = 100 + device[i];
+      return 0;
+    });
+  return fills;
+}
 
 }  // extern "C"

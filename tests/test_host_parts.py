@@ -55,3 +55,14 @@ def test_least_rows_hold_an_outer_pair_of_any_admitted_quartet(lib):
             inner = min(a, b) if max(a, b) > 256 else max(a, b)
             assert 680 * inner <= least, (items, a, b)
     assert lib.host_rows_least(100) == 68000
+
+
+def test_tables_are_filled_once_per_device(lib):
+    """The constant tables and their addresses belong to a device: a context on
+    another device of the process fills its own, and a fill that failed is
+    tried again."""
+    dev = (ctypes.c_int * 6)(0, 1, 0, 3, 3, 1)
+    val, st = (ctypes.c_int * 6)(*[-1] * 6), (ctypes.c_int * 6)()
+    assert lib.host_per_device(dev, 6, 3, val, st) == 4
+    assert list(st) == [0, 0, 0, -6, 0, 0]
+    assert list(val) == [100, 101, 100, -1, 103, 101]
