@@ -43,6 +43,7 @@
 #include "kernel_common.cuh"
 #include "auxtab.h"
 #include "grid.h"
+#include "hoststage.h"
 #include "perdevice.h"
 #include "termlist.h"
 #include "tickets.h"
@@ -399,41 +400,16 @@ struct ListLayout {
   }
 };
 
-// Host staging of a call's list: page-locked from kPinLeast to kPinMost bytes
-// (copies run at the link's rate and need no intermediate copy: with the cores
-// of plan_kinds 3.6 ms off a call of 200,000 quartets), plain memory below (the
-// driver takes a small copy from plain memory 14 us sooner per call) and past
-// that.  Grown on demand, given back with the context.
-struct HostStage {
-  static constexpr size_t kPinLeast = (size_t)256 << 10, kPinMost = (size_t)64 << 20;
-  unsigned char *p = nullptr;
-  size_t cap = 0;
-  bool pinned = false;
-  bool reserve(size_t bytes, size_t keep = 0) {   // the first `keep` bytes stay
-    if (bytes <= cap) return true;
-    const size_t want = std::max(bytes + bytes / 4, (size_t)1 << 16);
-    unsigned char *q = nullptr;
-    bool pin = want >= kPinLeast && want <= kPinMost && cudaHostAlloc((void **)&q, want, cudaHostAllocDefault) == cudaSuccess;
-    if (!pin) {
-      cudaGetLastError();
-      q = (unsigned char *)std::malloc(want);
-    }
-    if (!q) return false;
-    if (keep) std::memcpy(q, p, keep);
-    release();
-    p = q;
-    cap = want;
-    pinned = pin;
-    return true;
+// Page-locked memory of HostStage (hoststage.h).
+struct PageLocked {
+  static bool alloc(void **p, size_t bytes) {
+    if (cudaHostAlloc(p, bytes, cudaHostAllocDefault) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
   }
-  void release() {
-    if (pinned) cudaFreeHost(p);
-    else std::free(p);
-    p = nullptr;
-    cap = 0;
-    pinned = false;
-  }
+  static void free(void *p) { cudaFreeHost(p); }
 };
+using HostStage = f12host::HostStage<PageLocked>;
 
 struct f12int_ctx {
   int device = 0;
@@ -478,7 +454,8 @@ struct f12int_ctx {
   std::deque<BasisData> bases;   // deque: growing it never moves existing entries
   // scratch of compute_class (grown on demand, bounded by the budget)
   unsigned char *d_list = nullptr;   // a planned list (ListLayout)
-  HostStage stage;                   // its staging on the host
+  HostStage stage{true};             // its staging on the host
+  HostStage static_stage{false};     // that of f12int_compute_class_static
   int *d_keys = nullptr;
   unsigned *d_order = nullptr, *d_hist = nullptr;
   double *d_part = nullptr;
@@ -756,6 +733,7 @@ int f12int_destroy(f12int_ctx *ctx) {
   cudaFree(ctx->d_status);
   cudaFree(ctx->d_fma);
   ctx->stage.release();
+  ctx->static_stage.release();
   for (auto &e : ctx->ev_pool) {
     cudaEventDestroy(e.first);
     cudaEventDestroy(e.second);
@@ -2273,7 +2251,9 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
 
   const f12int_ctx::BasisData &B = ctx->bases[basis_id];
   cudaStream_t st = pick_stream(ctx, cuda_stream);
-  HostStage &hs = ctx->stage;
+  // (never page-locked: locking and unlocking pages waits for the device's other
+  // streams, which a caller of this entry point must not see)
+  HostStage &hs = ctx->static_stage;
   if (!hs.reserve(24 * (size_t)n)) return F12INT_ENOMEM;
   CK(cudaMemcpyAsync(hs.p, quartets_dev, sizeof(int32_t) * 4 * n, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(hs.p + 16 * n, offsets_dev, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, st));

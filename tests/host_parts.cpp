@@ -4,6 +4,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "../paper_1412_5070_gb300/csrc/hoststage.h"
 #include "../paper_1412_5070_gb300/csrc/perdevice.h"
 #include "../paper_1412_5070_gb300/csrc/tickets.h"
 
@@ -39,6 +40,36 @@ int host_per_device(const int *device, int n, int bad, int *value, int *status) 
       return 0;
     });
   return fills;
+}
+
+struct CountingPin {
+  static inline int locks = 0, frees = 0;
+  static bool alloc(void **p, size_t n) {
+    ++locks;
+    *p = std::malloc(n);
+    return true;
+  }
+  static void free(void *p) {
+    ++frees;
+    std::free(p);
+  }
+};
+
+// Grows a stage through n sizes, keeping its first byte; locks[0], [1]: pages
+// locked and freed.  Returns 1 if the byte survived.
+int host_stage(int may_pin, const int64_t *bytes, int n, int *locks) {
+  CountingPin::locks = CountingPin::frees = 0;
+  f12host::HostStage<CountingPin> s(may_pin != 0);
+  int ok = 1;
+  for (int i = 0; i < n; ++i) {
+    if (!s.reserve((size_t)bytes[i], i ? 1 : 0)) return 0;
+    if (i == 0) s.p[0] = 77;
+    ok = ok && s.p[0] == 77;
+  }
+  s.release();
+  locks[0] = CountingPin::locks;
+  locks[1] = CountingPin::frees;
+  return ok;
 }
 
 }  // extern "C"

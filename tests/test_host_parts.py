@@ -66,3 +66,20 @@ def test_tables_are_filled_once_per_device(lib):
     assert lib.host_per_device(dev, 6, 3, val, st) == 4
     assert list(st) == [0, 0, 0, -6, 0, 0]
     assert list(val) == [100, 101, 100, -1, 103, 101]
+
+
+def test_static_staging_never_locks_pages(lib):
+    """The staging of the static call stays in plain memory whatever the list's
+    length (locking pages waits for other streams); the allocating call's is
+    page-locked from 256 KB on, and freed as it was allocated."""
+    sizes = (ctypes.c_int64 * 5)(1000, 100_000, 400_000, 3_000_000, 200_000_000)
+    locks = (ctypes.c_int * 2)()
+    assert lib.host_stage(0, sizes, 5, locks) == 1 and list(locks) == [0, 0]
+    assert lib.host_stage(1, sizes, 5, locks) == 1 and list(locks) == [2, 2]
+
+
+def test_the_static_call_uses_that_staging():
+    src = open(os.path.join(CSRC, "f12int.cu")).read()
+    body = src[src.index('extern "C" int f12int_compute_class_static('):]
+    assert "ctx->static_stage" in body and "ctx->stage" not in body
+    assert "HostStage static_stage{false};" in src
