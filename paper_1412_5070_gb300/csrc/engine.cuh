@@ -400,7 +400,7 @@ static int engine_init(f12int_ctx *ctx, Engine &E) {
   }
   if (rc == F12INT_OK && cudaStreamCreateWithFlags(&E.stream, cudaStreamNonBlocking) != cudaSuccess)
     rc = F12INT_ECUDA;
-  if (rc == F12INT_OK && cudaMemset(E.status, 0, sizeof(unsigned)) != cudaSuccess) rc = F12INT_ECUDA;
+  if (rc == F12INT_OK && clear(E.status, sizeof(unsigned), E.stream) != cudaSuccess) rc = F12INT_ECUDA;
   if (rc != F12INT_OK) return rc;
   engine_family_rows(ctx, E);
   // persistent launch shapes: resident blocks per SM from registers and shared memory

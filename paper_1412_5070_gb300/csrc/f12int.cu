@@ -523,6 +523,18 @@ void dfree(f12int_ctx *ctx, T *&p, size_t bytes) {
   }
 }
 
+// Copy to the device, or clear there, complete when they return: a plain
+// cudaMemcpy from pageable memory (and cudaMemset) may return while its last part
+// is still to come on the legacy stream, which non-blocking streams do not wait for.
+cudaError_t upload(void *dst, const void *src, size_t bytes, cudaStream_t st) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+  return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+cudaError_t clear(void *dst, size_t bytes, cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(dst, 0, bytes, st);
+  return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
 cudaStream_t pick_stream(f12int_ctx *ctx, void *s) { return s ? (cudaStream_t)s : ctx->stream; }
 
 // NVTX range over a host scope (the stages of a call, visible in a profiler's
@@ -610,8 +622,9 @@ int upload_constants(const double **boys) {
     double *dk = nullptr;
     CK(cudaMalloc(&dk, sizeof(double) * kt.size()));
     const double *dkc = dk;
-    cudaError_t e = cudaMemcpy(dk, kt.data(), sizeof(double) * kt.size(), cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpyAsync(dk, kt.data(), sizeof(double) * kt.size(), cudaMemcpyHostToDevice, nullptr);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(d_mtab, &dkc, sizeof(dkc));
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();   // (the symbols' copies above as well)
     if (e != cudaSuccess) {
       cudaFree(dk);
       return cuda_fail(e);
@@ -680,7 +693,7 @@ int f12int_create(f12int_ctx **out, int device, size_t hbm_budget_bytes, void *c
   ctx->stream = (cudaStream_t)cuda_stream;
   int rc = g_tables.get(device, &ctx->boys, [](const double *&boys) { return upload_constants(&boys); });
   if (rc == F12INT_OK) rc = dalloc(ctx, &ctx->d_status, sizeof(unsigned int));
-  if (rc == F12INT_OK && cudaMemset(ctx->d_status, 0, sizeof(unsigned int)) != cudaSuccess) rc = F12INT_ECUDA;
+  if (rc == F12INT_OK && clear(ctx->d_status, sizeof(unsigned int), ctx->stream) != cudaSuccess) rc = F12INT_ECUDA;
   for (int i = 0; i < NSIDE && rc == F12INT_OK; ++i)
     if (cudaStreamCreateWithFlags(&ctx->side[i], cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->join[i], cudaEventDisableTiming) != cudaSuccess)
@@ -751,7 +764,7 @@ int f12int_set_timing(f12int_ctx *ctx, int on) {
   if (on && !ctx->d_fma) {
     int rc = dalloc(ctx, &ctx->d_fma, 2 * sizeof(unsigned long long));
     if (rc != F12INT_OK) return rc;
-    CK(cudaMemset(ctx->d_fma, 0, 2 * sizeof(unsigned long long)));
+    CK(clear(ctx->d_fma, 2 * sizeof(unsigned long long), ctx->stream));
   }
   ctx->timing = on != 0;
   return F12INT_OK;
@@ -774,7 +787,7 @@ int f12int_kernel_stats(f12int_ctx *ctx, int reset, double *stats) {
   if (reset) {
     ctx->aux_ms = ctx->contract_ms = 0.0;
     ctx->aux_launches = ctx->contract_launches = 0;
-    if (ctx->d_fma) CK(cudaMemset(ctx->d_fma, 0, sizeof(cnt)));
+    if (ctx->d_fma) CK(clear(ctx->d_fma, sizeof(cnt), ctx->stream));
   }
   return F12INT_OK;
 }
@@ -992,12 +1005,12 @@ static int set_factor_lists(f12int_ctx *ctx, const f12::TermList &T1, const f12:
   if (rc == F12INT_OK && ctx->grp_bytes) rc = dalloc(ctx, &ctx->d_grp, ctx->grp_bytes);
   if (rc == F12INT_OK && ctx->jtab_bytes) rc = dalloc(ctx, &ctx->d_jtab, ctx->jtab_bytes);
   if (rc != F12INT_OK) return rc;
-  CK(cudaMemcpy(ctx->d_fam, fams.data(), ctx->fam_bytes, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(ctx->d_coef, coef.data(), ctx->coef_bytes, cudaMemcpyHostToDevice));
+  CK(upload(ctx->d_fam, fams.data(), ctx->fam_bytes, ctx->stream));
+  CK(upload(ctx->d_coef, coef.data(), ctx->coef_bytes, ctx->stream));
   if (ctx->grp_bytes)
-    CK(cudaMemcpy(ctx->d_grp, ct.groups.data(), ctx->grp_bytes, cudaMemcpyHostToDevice));
+    CK(upload(ctx->d_grp, ct.groups.data(), ctx->grp_bytes, ctx->stream));
   if (ctx->jtab_bytes)
-    CK(cudaMemcpy(ctx->d_jtab, ct.jtab.data(), ctx->jtab_bytes, cudaMemcpyHostToDevice));
+    CK(upload(ctx->d_jtab, ct.jtab.data(), ctx->jtab_bytes, ctx->stream));
   T.fam = ctx->d_fam;
   T.coef = ctx->d_coef;
   T.grp = ctx->d_grp;
@@ -1034,7 +1047,7 @@ static int set_factor_lists(f12int_ctx *ctx, const f12::TermList &T1, const f12:
     ctx->kgrow_bytes = sizeof(float) * all.size();
     rc = dalloc(ctx, &ctx->d_kgrow, ctx->kgrow_bytes);
     if (rc != F12INT_OK) return rc;
-    CK(cudaMemcpy(ctx->d_kgrow, all.data(), ctx->kgrow_bytes, cudaMemcpyHostToDevice));
+    CK(upload(ctx->d_kgrow, all.data(), ctx->kgrow_bytes, ctx->stream));
   }
   {
     f12::TermList gk[7];
@@ -1921,7 +1934,7 @@ static int ensure_prim_bounds(f12int_ctx *ctx, int basis_id, int cls) {
   double *d = nullptr;
   rc = dalloc(ctx, &d, sizeof(double) * npp);
   if (rc != F12INT_OK) return rc;
-  if (cudaMemcpy(d, qpp.data(), sizeof(double) * npp, cudaMemcpyHostToDevice) != cudaSuccess) {
+  if (upload(d, qpp.data(), sizeof(double) * npp, ctx->stream) != cudaSuccess) {
     dfree(ctx, d, sizeof(double) * npp);
     return F12INT_ECUDA;
   }

@@ -149,8 +149,11 @@ __global__ void __launch_bounds__(CHECK ? ITC : GR_NC *ITB) k_rows_a(Build B, Qu
 
 // Region B: one block per cell of u.  F_m is evaluated at the Chebyshev points
 // of x/D and interpolated at the quadrature nodes; at the nodes of the check
-// point's rule it is evaluated itself.
-__global__ void __launch_bounds__(128) k_rows_b(Build B) {
+// point's rule it is evaluated itself, for the orders that are served.  A thread
+// per evaluation, and the check point in a warp of its own.
+constexpr int TRB = 288;
+static_assert(TRB >= (GR_NB + GR_NHC) * NCLS && GR_NC <= 32, "a thread each");
+__global__ void __launch_bounds__(TRB) k_rows_b(Build B) {
   extern __shared__ double sB[];   // [GR_NB][ncls][row], [GR_NHC][ncls][row], then a row of rows per node
   const int iu = blockIdx.x, cell = GR_NX * GR_NT + iu, nrow = B.ncls * GR_ROWS;
   double *sC = sB + GR_NB * nrow;
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(128) k_rows_b(Build B) {
   for (int t = threadIdx.x; t < (GR_NB + GR_NHC) * B.ncls; t += blockDim.x) {
     const int j = t / B.ncls, k = t % B.ncls;
     const double x = j < GR_NB ? D0 * (1.0 + (GR_BW + 0.02) * B.bx[j]) : cD + B.ghcx[j - GR_NB] * cis;
-    grid_radial(B.cls[k].fam, B.cls[k].nfam, B.cls[k].coef, x, GR_M, sB + j * nrow + k * GR_ROWS);
+    grid_radial(B.cls[k].fam, B.cls[k].nfam, B.cls[k].coef, x, j < GR_NB ? GR_M : GR_LMAX, sB + j * nrow + k * GR_ROWS);
   }
   __syncthreads();
   double b[NCLS];
@@ -175,10 +178,10 @@ __global__ void __launch_bounds__(128) k_rows_b(Build B) {
     for (int m = 0; m <= GR_M; ++m) sB[j * nrow + k * GR_ROWS + m] *= e;
   }
   __syncthreads();
-  const int n = threadIdx.x;
-  if (n >= NODES) return;
+  const bool check = threadIdx.x == 32;
+  const int n = check ? GR_NC : (int)threadIdx.x;
+  if (n >= GR_NC && !check) return;
   double *acc = sC + GR_NHC * nrow + n * (nrow + 1);
-  const bool check = n == GR_NC;
   const double xi = check ? cxi : 2.0 * GR_TB / (hi * (B.node[n] + 1.0)), is = 1.0 / sqrt(xi);   // (a = -1 is xi = infinity)
   const double D = check ? cD : D0;
   for (int k = 0; k < nrow; ++k) acc[k] = 0.0;
@@ -187,7 +190,11 @@ __global__ void __launch_bounds__(128) k_rows_b(Build B) {
     double jh[GR_ROWS];
     grid_jhat(B.ztab, 2.0 * xi * D * x, jh);
     if (check) {
-      for (int k = 0; k < nrow; ++k) acc[k] = fma(B.ghcw[i] * jh[k % GR_ROWS], sC[i * nrow + k], acc[k]);
+      for (int c = 0; c < B.ncls; ++c)
+        for (int m = 0; m <= GR_LMAX; ++m) {
+          const int k = c * GR_ROWS + m;
+          acc[k] = fma(B.ghcw[i] * jh[m], sC[i * nrow + k], acc[k]);
+        }
       continue;
     }
     double bw[GR_NB], den = 0.0;
@@ -260,16 +267,20 @@ bool same_terms(const f12::TermList &x, const f12::TermList &y) {
   return true;
 }
 
-// Device allocations of a build, freed on every way out.
+// Device allocations of a build, freed on every way out.  Uploads go to the
+// stream of the build's kernels, which reads them in order (the sources live to
+// the build's end).
 struct Temp {
   std::vector<void *> p;
+  cudaStream_t st;
+  explicit Temp(cudaStream_t s) : st(s) {}
   ~Temp() {
     for (void *q : p) cudaFree(q);
   }
   template <class T>
   T *up(const std::vector<T> &v, bool &good) {
     T *d = get<T>(v.size(), good);
-    if (good && !v.empty() && cudaMemcpy(d, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+    if (good && !v.empty() && cudaMemcpyAsync(d, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
       good = false;
     return d;
   }
@@ -370,7 +381,7 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
   std::shared_ptr<AuxGrid> g = std::make_shared<AuxGrid>();
   g->device = device;
   g->key = key;
-  Temp tmp;
+  Temp tmp(st);
   bool good = true;
   for (int k = 0; k < B.ncls && good; ++k) {
     B.cls[k] = ClassDev{tmp.up(gc[k].fam, good), tmp.up(gc[k].coef, good), (int)gc[k].fam.size()};
@@ -382,7 +393,7 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
     g->bytes += sizeof(double) * (size_t)GR_CELLS * GR_CELL + (size_t)GR_CELLS;
   }
   good = good && cudaMalloc((void **)&g->xt, sizeof(double) * xt.size()) == cudaSuccess &&
-         cudaMemcpy(g->xt, xt.data(), sizeof(double) * xt.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+         cudaMemcpyAsync(g->xt, xt.data(), sizeof(double) * xt.size(), cudaMemcpyHostToDevice, st) == cudaSuccess;
   const int nrow = B.ncls * GR_ROWS;
   Quad Q[2];
   for (int k = 0; k < 2; ++k) {
@@ -413,7 +424,7 @@ std::shared_ptr<const AuxGrid> acquire(int device, const f12::TermList kt[7], co
   k_rows_a<true><<<dim3(GR_NX, (GR_NT + ITC - 1) / ITC), ITC, 0, st>>>(B, Q[1]);
   const size_t smb = sizeof(double) * ((size_t)(GR_NB + GR_NHC) * nrow + (size_t)NODES * (nrow + 1));
   cudaFuncSetAttribute(k_rows_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-  k_rows_b<<<GR_NU, 128, smb, st>>>(B);
+  k_rows_b<<<GR_NU, TRB, smb, st>>>(B);
   k_fit<<<(unsigned)(((int64_t)GR_CELLS * nrow + 127) / 128), 128, 0, st>>>(B);
   k_check<<<(unsigned)(((int64_t)GR_CELLS * B.ncls + 127) / 128), 128, 0, st>>>(B);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return nullptr;

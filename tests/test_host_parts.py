@@ -3,6 +3,7 @@
 import ctypes
 import glob
 import os
+import re
 import shutil
 import subprocess
 
@@ -83,3 +84,13 @@ def test_the_static_call_uses_that_staging():
     body = src[src.index('extern "C" int f12int_compute_class_static('):]
     assert "ctx->static_stage" in body and "ctx->stage" not in body
     assert "HostStage static_stage{false};" in src
+
+
+def test_uploads_are_ordered_with_the_kernels_streams():
+    """A plain cudaMemcpy from pageable memory, or a cudaMemset, may return before
+    its last part has arrived, on a stream that non-blocking streams do not wait
+    for: every upload names its stream."""
+    for path in glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")):
+        src = re.sub(r"//[^\n]*", "", open(path).read())
+        assert not re.search(r"\bcudaMemset\(", src), path
+        assert not re.search(r"\bcudaMemcpy\([^;]*cudaMemcpyHostToDevice\)", src), path
