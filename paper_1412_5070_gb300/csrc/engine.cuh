@@ -167,9 +167,10 @@ static int engine_alloc(f12int_ctx *ctx, Engine &E, T **p, size_t n) {
 
 template <class T>
 static int stage_alloc(T **p, size_t n) {
-  return cudaHostAlloc((void **)p, sizeof(T) * std::max<size_t>(n, 1), cudaHostAllocDefault) == cudaSuccess
-             ? F12INT_OK
-             : F12INT_ENOMEM;
+  const cudaError_t e = cudaHostAlloc((void **)p, sizeof(T) * std::max<size_t>(n, 1), cudaHostAllocDefault);
+  if (e == cudaSuccess) return F12INT_OK;
+  cuda_fail(e);
+  return F12INT_ENOMEM;
 }
 
 static int lists_alloc_dev(f12int_ctx *ctx, Engine &E, ClassLists &L) {

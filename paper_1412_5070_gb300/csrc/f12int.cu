@@ -493,7 +493,11 @@ struct f12int_ctx {
 
 namespace {
 
+// The status of a CUDA call that failed.  Its error is taken off the thread's last
+// one: it is reported here, and a retry with less memory (or the next call) must
+// not find it after its own launches.
 int cuda_fail(cudaError_t e) {
+  cudaGetLastError();
   if (e == cudaErrorMemoryAllocation) return F12INT_ENOMEM;
   return F12INT_ECUDA;
 }

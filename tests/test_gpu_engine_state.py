@@ -156,3 +156,24 @@ def test_no_factor_after_a_set_factor_that_failed():
         assert np.array_equal(out.cpu().numpy(), want)
     finally:
         F.f12int_destroy(ctx)
+
+
+def test_calls_after_an_allocation_that_failed():
+    """An engine whose buffers do not fit the device (2^46 items) is refused with
+    F12INT_ENOMEM; the calls after it do not report that error again."""
+    ctx = make()
+    try:
+        F.f12int_set_factor(ctx, M.P0)
+        basis = M.two_centre_sp()
+        bid = F.f12int_set_basis(ctx, basis)
+        q = M.canonical_quartets(basis, 3)[:12]
+        want = per_call(ctx, bid, 3, q, basis)
+        F.f12int_batch_limits(ctx, 16, 1 << 46)
+        off, tot = layout(basis, q, (3,))
+        out = torch.zeros(tot, dtype=torch.float64, device="cuda")
+        with pytest.raises(F.F12IntError) as e:
+            F.f12int_submit(ctx, bid, q, (3,), out, off)
+        assert e.value.status == F.ENOMEM
+        assert np.array_equal(per_call(ctx, bid, 3, q, basis), want)
+    finally:
+        F.f12int_destroy(ctx)
