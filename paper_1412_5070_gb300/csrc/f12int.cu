@@ -45,6 +45,7 @@
 #include "grid.h"
 #include "hoststage.h"
 #include "perdevice.h"
+#include "scratchcut.h"
 #include "termlist.h"
 #include "tickets.h"
 
@@ -2264,8 +2265,6 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
   unsigned char *base = nullptr;
   int rc = static_scratch_address(ctx->device, &base);
   if (rc != F12INT_OK) return rc;
-  const size_t item_bytes = sizeof(int) + sizeof(unsigned) + sizeof(double) * kPartPitch;
-
   const f12int_ctx::BasisData &B = ctx->bases[basis_id];
   cudaStream_t st = pick_stream(ctx, cuda_stream);
   // (never page-locked: locking and unlocking pages waits for the device's other
@@ -2289,28 +2288,23 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
            align256(sizeof(int64_t) * ((size_t)n + 1)) + align256(sizeof(unsigned) * kNKeys) +
            align256(sizeof(CTask) * (size_t)P.ntask);
   };
-  // one chunk at least: the items of every quartet on its own, and the rows of
-  // one of its bra primitive pairs
   const int64_t nf = std::max(1, ctx->tables.nfam[cls == 5 ? 3 : cls]);
   const GridView G = grid_view(ctx, B, cls);
-  int64_t pitch = 4, big_cd = 1;
-  const int64_t big_pq = P.big_pq;
+  int64_t pitch = 4, big_in = 0;   // of the general quartets: row doubles, inner pairs
   for (const ListPlan::Run &r : P.runs)
     if (!r.thin) {
-      big_cd = std::max(big_cd, r.npq / r.npab);
+      big_in = std::max(big_in, r.npq / r.npab);
       pitch = std::max(pitch, r.pitch / r.npq);
     }
+  f12host::ScratchCut cut;
   auto room = [&]() -> int64_t {   // bytes of the chunk's scratch, negative when the list does not fit
     return (int64_t)F12INT_STATIC_SCRATCH_BYTES - (int64_t)fixed_bytes() - 4 * 256;
   };
-  auto enough = [&] {
-    const int64_t r = room();
-    return r >= big_pq * nf * (int64_t)item_bytes && r >= big_cd * (nf * (int64_t)item_bytes + pitch * 8 + 64);
-  };
-  if (!enough()) {   // fewer and longer tasks leave more of the array
+  auto fits = [&] { return f12host::scratch_cut(room(), G.direct(), nf, kPartPitch, P.big_pq, big_in, pitch, &cut); };
+  if (!fits()) {   // fewer and longer tasks leave more of the array
     rc = plan_kinds(B, cls, n, (const int32_t *)hs.p, fp64, P, /*fewest=*/true);
     if (rc != F12INT_OK) return rc;
-    if (!enough()) return F12INT_EINVAL;
+    if (!fits()) return F12INT_EINVAL;
   }
   const ListLayout at(n, 0, P.ntask);   // (no row offsets: every row at one pitch)
   if (!hs.reserve(24 * (size_t)n + at.bytes, 24 * (size_t)n)) return F12INT_ENOMEM;
@@ -2327,22 +2321,16 @@ extern "C" int f12int_compute_class_static(f12int_ctx *ctx, int basis_id, int cl
   D.pitch = (int)pitch;
   D.hist = d_hist;
   D.keys = (int *)scratch;
-  const int64_t r = room();
+  D.keys_cap = cut.keys_cap;
+  D.rows_cap = cut.rows_cap;
+  unsigned char *next = scratch + align256(sizeof(int) * (size_t)cut.keys_cap);
   if (G.direct()) {
-    const int64_t rows = r / (int64_t)(sizeof(int) + sizeof(double) * (size_t)pitch);   // primitive quartets
-    D.keys_cap = rows;
-    D.rows = (double *)(scratch + align256(sizeof(int) * (size_t)rows));
-    D.rows_cap = rows * pitch;
+    D.rows = (double *)next;
   } else {
-    // items over the whole of it for the thin quartets; the general ones leave
-    // its end to the rows (a quarter, or one bra pair's)
-    const int64_t items = r / (int64_t)item_bytes;
-    D.keys_cap = items;
-    D.order = (unsigned *)(scratch + align256(sizeof(int) * (size_t)items));
-    D.part = (double *)((unsigned char *)D.order + align256(sizeof(unsigned) * (size_t)items));
-    D.part_thin = items * kPartPitch;
-    D.rows_cap = std::max(items * kPartPitch / 4, big_cd * pitch) & ~(int64_t)3;
-    D.part_cap = (D.part_thin - D.rows_cap) & ~(int64_t)15;
+    D.order = (unsigned *)next;
+    D.part = (double *)(next + align256(sizeof(unsigned) * (size_t)cut.keys_cap));
+    D.part_thin = cut.part_thin;
+    D.part_cap = cut.part_cap;
     D.rows = D.part + D.part_cap;
   }
   CK(cudaMemcpyAsync(d_tk, P.tasks, sizeof(CTask) * (size_t)P.ntask, cudaMemcpyHostToDevice, st));

@@ -6,6 +6,7 @@
 
 #include "../paper_1412_5070_gb300/csrc/hoststage.h"
 #include "../paper_1412_5070_gb300/csrc/perdevice.h"
+#include "../paper_1412_5070_gb300/csrc/scratchcut.h"
 #include "../paper_1412_5070_gb300/csrc/tickets.h"
 
 extern "C" {
@@ -70,6 +71,17 @@ int host_stage(int may_pin, const int64_t *bytes, int n, int *locks) {
   locks[0] = CountingPin::locks;
   locks[1] = CountingPin::frees;
   return ok;
+}
+
+int host_scratch_cut(int64_t room, int direct, int64_t nf, int64_t big_pq, int64_t big_in, int64_t pitch,
+                     int64_t *c) {
+  f12host::ScratchCut s;
+  const bool ok = f12host::scratch_cut(room, direct != 0, nf, 16, big_pq, big_in, pitch, &s);
+  c[0] = s.keys_cap;
+  c[1] = s.part_thin;
+  c[2] = s.part_cap;
+  c[3] = s.rows_cap;
+  return ok ? 1 : 0;
 }
 
 }  // extern "C"

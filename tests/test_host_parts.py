@@ -94,3 +94,36 @@ def test_uploads_are_ordered_with_the_kernels_streams():
         src = re.sub(r"//[^\n]*", "", open(path).read())
         assert not re.search(r"\bcudaMemset\(", src), path
         assert not re.search(r"\bcudaMemcpy\([^;]*cudaMemcpyHostToDevice\)", src), path
+
+
+@pytest.mark.parametrize("direct", [0, 1])
+def test_a_static_list_that_is_accepted_runs_in_its_scratch(lib, direct):
+    """Whatever room the list leaves, an accepted one has the items and the rows of
+    one outer pair of any general quartet, the items of any thin one, and stays
+    inside the room: nothing is refused once work is queued.  Refused is what
+    lacks the items of a quartet, or the rows of one outer pair."""
+    cut = lib.host_scratch_cut
+    cut.argtypes = [ctypes.c_int64, ctypes.c_int] + [ctypes.c_int64] * 4 + [ctypes.POINTER(ctypes.c_int64)]
+    c = (ctypes.c_int64 * 4)()
+    for nf in (1, 5, 12):
+        for pq, inner in ((1, 1), (36, 6), (36, 36), (6561, 81), (4, 0), (70000, 256)):
+            for pitch in (36, 288, 680):
+                need = pq * nf * 136
+                tight = need + (inner * pitch * 8 if inner else 0)
+                for room in sorted({need - 1, need, need + 64, inner * (nf * 136 + pitch * 8 + 64), tight, tight + 136,
+                                    tight + 300, 2 * tight + 4096, 60_000_000}):
+                    ok = cut(room, direct, nf, pq, inner, pitch, c)
+                    keys, thin, part, rows = list(c)
+                    if room < need:
+                        assert not ok
+                    if room >= 2 * tight + 4096:
+                        assert ok
+                    if not ok:
+                        continue
+                    if direct:
+                        assert keys >= inner and rows >= inner * pitch and 4 * keys + 8 * rows <= room
+                        continue
+                    assert 8 * keys + 8 * thin <= room and thin >= pq * nf * 16
+                    if inner:
+                        assert part >= inner * nf * 16 and rows >= inner * pitch and part + rows <= thin
+                        assert part % 16 == 0
