@@ -22,7 +22,7 @@ SOURCES = [(os.path.join(CSRC, "f12int.cu"), ())] + \
 DEPS = sorted({src for src, _ in SOURCES}) + [os.path.join(CSRC, f) for f in (
     "aux.cuh", "auxtab.h", "engine.cuh", "termlist.h", "kernel_common.cuh", "thin.cuh", "auxgrid.cuh", "gridtab.h", "grid.h",
     "contract.cuh", "tickets.h",
-    "perdevice.h", "hoststage.h", "scratchcut.h")] + \
+    "perdevice.h", "hoststage.h", "scratchcut.h", "screen.h")] + \
     [os.path.join(os.path.dirname(HERE), "include", "f12int.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

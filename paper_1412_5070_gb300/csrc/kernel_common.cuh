@@ -8,6 +8,7 @@
 #include <cstdint>
 
 #include "auxgrid.cuh"
+#include "screen.h"
 
 namespace f12k {
 
@@ -94,8 +95,6 @@ __host__ __device__ constexpr int aux_direct_fmas(const bool boys, int L) {
   return boys ? f12dev::BY_NT - 1 + L : f12dev::grid_fmas(L);
 }
 
-// Growth of a kernel with distance, tabulated at this step (screening).
-constexpr double kGrowStep = 0.05, kGrowMax = 120.0;
 constexpr double kPrimScreen = 1e-26;
 
 
@@ -124,7 +123,7 @@ __device__ __forceinline__ bool prim_negligible(const PairView &PV, int pab, int
   float gam = 0.0f;
 #pragma unroll
   for (int k = 0; k < 7; ++k) {
-    const int i = min(PV.ngrow - 1, (int)((R + k * hw) * (float)(1.0 / kGrowStep)) + 1);
+    const int i = grow_index((R + k * hw) * (float)(1.0 / kGrowStep), PV.ngrow);
     gam = fmaxf(gam, PV.grow[i] * kOverlap[k]);
   }
   return v * (double)gam < kPrimScreen;

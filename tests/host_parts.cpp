@@ -7,6 +7,7 @@
 #include "../paper_1412_5070_gb300/csrc/hoststage.h"
 #include "../paper_1412_5070_gb300/csrc/perdevice.h"
 #include "../paper_1412_5070_gb300/csrc/scratchcut.h"
+#include "../paper_1412_5070_gb300/csrc/screen.h"
 #include "../paper_1412_5070_gb300/csrc/tickets.h"
 
 extern "C" {
@@ -83,5 +84,7 @@ int host_scratch_cut(int64_t room, int direct, int64_t nf, int64_t big_pq, int64
   c[3] = s.rows_cap;
   return ok ? 1 : 0;
 }
+
+int host_grow_index(float x, int n) { return f12k::grow_index(x, n); }
 
 }  // extern "C"

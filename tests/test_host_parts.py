@@ -127,3 +127,14 @@ def test_a_static_list_that_is_accepted_runs_in_its_scratch(lib, direct):
                     if inner:
                         assert part >= inner * nf * 16 and rows >= inner * pitch and part + rows <= thin
                         assert part % 16 == 0
+
+
+def test_growth_table_index_stays_in_the_table(lib):
+    """Distances to 1e38 bohr and past single precision's range (atoms that far
+    apart are accepted input) take the last entry."""
+    idx = lib.host_grow_index
+    idx.argtypes = [ctypes.c_float, ctypes.c_int]
+    n = 2401
+    for x in (0.0, 0.5, 1.0, 17.3, 2398.5, 2399.0, 2399.9, 2400.0, 2401.0, 1e6, 2.2e9, 4.3e9, 1e20, 3e38, float("inf"),
+              float("nan")):
+        assert idx(x, n) == (min(n - 1, int(x) + 1) if x < 1e9 else n - 1), x
