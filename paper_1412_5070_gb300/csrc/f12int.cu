@@ -481,8 +481,10 @@ struct f12int_ctx {
   // kgrow[cls][i] = G(i * kGrowStep), see screen_estimate
   std::vector<double> kgrow[7];
   // the same tables on the device for the primitive screen ([7][kgrow_n]);
-  // grows[cls]: the kernel of cls grows (G > 1 somewhere)
-  float *d_kgrow = nullptr;
+  // in both precisions; grows[cls]: the kernel of cls grows (G > 1 somewhere)
+  double *d_kgrow = nullptr;
+  float *d_kgrow32 = nullptr;
+  double grow_band[7] = {0.0};
   size_t kgrow_bytes = 0;
   int kgrow_n = 0;
   bool grows[7] = {false, false, false, false, false, false, false};
@@ -556,11 +558,14 @@ struct NvtxRange {
 // screen is set and the factors exist.
 PairView pair_view(const f12int_ctx *ctx, const f12int_ctx::BasisData &B, int cls, bool screen) {
   PairView v{B.d_pair_start, B.d_pp_p, B.d_pp_P, B.d_pp_ab, B.d_pp_eoff, B.d_epool, B.d_shell_l, B.nshell,
-             nullptr, nullptr, 0};
+             nullptr, nullptr, nullptr, 0.0, 0.0, 0};
   if (screen && B.d_qprim[cls]) {
     v.qprim = B.d_qprim[cls];
     if (ctx->grows[cls] && ctx->d_kgrow) {
       v.grow = ctx->d_kgrow + (size_t)cls * ctx->kgrow_n;
+      v.grow32 = ctx->d_kgrow32 + (size_t)cls * ctx->kgrow_n;
+      v.grow_lo = kPrimScreen / ctx->grow_band[cls];
+      v.grow_hi = kPrimScreen * ctx->grow_band[cls];
       v.ngrow = ctx->kgrow_n;
     }
   }
@@ -737,6 +742,7 @@ int f12int_destroy(f12int_ctx *ctx) {
   cudaFree(ctx->d_grp);
   cudaFree(ctx->d_jtab);
   cudaFree(ctx->d_kgrow);
+  cudaFree(ctx->d_kgrow32);
   cudaFree(ctx->d_list);
   cudaFree(ctx->d_keys);
   cudaFree(ctx->d_order);
@@ -1037,22 +1043,26 @@ static int set_factor_lists(f12int_ctx *ctx, const f12::TermList &T1, const f12:
   for (int c = 1; c <= 6; ++c) ctx->kgrow[c] = growth_table(kt[c == 5 ? 3 : c]);
   {
     dfree(ctx, ctx->d_kgrow, ctx->kgrow_bytes);
-    ctx->d_kgrow = nullptr;
+    dfree(ctx, ctx->d_kgrow32, ctx->kgrow_bytes / 2);
     ctx->kgrow_n = (int)ctx->kgrow[1].size();
-    std::vector<float> all((size_t)7 * ctx->kgrow_n, 1.0f);
+    std::vector<double> all((size_t)7 * ctx->kgrow_n, 1.0);
+    std::vector<float> single(all.size(), 1.0f);
     for (int c = 1; c <= 6; ++c) {
       ctx->grows[c] = false;
+      ctx->grow_band[c] = screen_band(ctx->kgrow[c].data(), ctx->kgrow_n);
       for (int i = 0; i < ctx->kgrow_n; ++i) {
-        // (rounded up; past single precision's range nothing is negligible)
-        const double g = ctx->kgrow[c][i] * (1.0 + 1e-6);
-        all[(size_t)c * ctx->kgrow_n + i] = g < 3e38 ? (float)g : INFINITY;
-        ctx->grows[c] = ctx->grows[c] || ctx->kgrow[c][i] > 1.0;
+        const double g = ctx->kgrow[c][i];
+        all[(size_t)c * ctx->kgrow_n + i] = g;
+        single[(size_t)c * ctx->kgrow_n + i] = g < 3e38 ? (float)g : INFINITY;
+        ctx->grows[c] = ctx->grows[c] || g > 1.0;
       }
     }
-    ctx->kgrow_bytes = sizeof(float) * all.size();
+    ctx->kgrow_bytes = sizeof(double) * all.size();
     rc = dalloc(ctx, &ctx->d_kgrow, ctx->kgrow_bytes);
+    if (rc == F12INT_OK) rc = dalloc(ctx, &ctx->d_kgrow32, ctx->kgrow_bytes / 2);
     if (rc != F12INT_OK) return rc;
     CK(upload(ctx->d_kgrow, all.data(), ctx->kgrow_bytes, ctx->stream));
+    CK(upload(ctx->d_kgrow32, single.data(), ctx->kgrow_bytes / 2, ctx->stream));
   }
   {
     f12::TermList gk[7];

@@ -27,7 +27,9 @@ struct PairView {
   const int *shell_l;
   int nshell;
   const double *qprim;       // [npp] primitive Schwarz factors of the class, or null
-  const float *grow;         // [ngrow] growth G(i kGrowStep) of the class's kernel, or null (no growth)
+  const double *grow;        // [ngrow] growth G(i kGrowStep) of the class's kernel, or null (no growth)
+  const float *grow32;       // the same in single precision, and what it settles (screen.h)
+  double grow_lo, grow_hi;
   int ngrow;
 };
 
@@ -97,7 +99,6 @@ __host__ __device__ constexpr int aux_direct_fmas(const bool boys, int L) {
 
 constexpr double kPrimScreen = 1e-26;
 
-
 // Primitive quartets whose Schwarz product is below kPrimScreen are skipped:
 // the skipped contributions stay below the absolute accuracy that elements
 // just above 1e-12 need for a relative error of 1e-10.  The diagonal
@@ -105,28 +106,20 @@ constexpr double kPrimScreen = 1e-26;
 // grows with r (Eq. rs12 with B > 0: I2, I3 like e^{Br}, k4 = f f' and
 // k6 = f_r f'_r like e^{2Br}) is larger at the separation R = |P - Q| of the
 // two charge distributions, whose overlap e^{-xi w^2} reaches out to R + w.
-// A candidate is weighed, as the shell screen weighs a shell quartet, by
-//   Gamma = max over w = 0, 0.5, .., 3 (units of 1/sqrt(xi)) of G(R + w) e^{-xi w^2}
-// (e^{-xi w^2} = e^{-k^2/4} at the k-th sample).
-// The weighing is in single precision (an index into G's table of 0.05 bohr
-// steps and its largest value): in FP64 its square roots and division, taken by
-// the whole warp whenever one lane has a candidate, were a third of the thin
+// A candidate is weighed, as the shell screen weighs a shell quartet, by the
+// growth Gamma that its overlap reaches (screen.h).  The weighing is in single
+// precision, and in double where that does not settle it (a per cent of the
+// candidates): in double precision throughout, its square roots, taken by the
+// whole warp whenever one lane has a candidate, were a third of the thin
 // contraction's FP64 instructions.
 __device__ __forceinline__ bool prim_negligible(const PairView &PV, int pab, int pcd, double u) {
   if (!PV.qprim) return false;
   const double v = PV.qprim[pab] * PV.qprim[pcd];
   if (v >= kPrimScreen) return false;
   if (!PV.grow) return true;
-  const float R = sqrtf((float)u), hw = 0.5f * sqrtf((float)(PV.pp_ab[4 * pab + 2] + PV.pp_ab[4 * pcd + 2]));
-  constexpr float kOverlap[7] = {1.0f, 0.77880078307140487f, 0.36787944117144233f, 0.10539922456186433f,
-                                 0.018315638888734179f, 0.0019304541362277093f, 0.00012340980408667956f};
-  float gam = 0.0f;
-#pragma unroll
-  for (int k = 0; k < 7; ++k) {
-    const int i = grow_index((R + k * hw) * (float)(1.0 / kGrowStep), PV.ngrow);
-    gam = fmaxf(gam, PV.grow[i] * kOverlap[k]);
-  }
-  return v * (double)gam < kPrimScreen;
+  const double iv = PV.pp_ab[4 * pab + 2] + PV.pp_ab[4 * pcd + 2];
+  const int s = screen_single(v, u, iv, PV.grow_lo, PV.grow_hi, PV.grow32, PV.ngrow);
+  return s >= 0 ? s == 1 : screen_negligible(v, u, iv, kPrimScreen, PV.grow, PV.ngrow);
 }
 
 // Thin contraction (thin_*.cu): quartets of total order L <= kThinL (I5:

@@ -87,4 +87,21 @@ int host_scratch_cut(int64_t room, int direct, int64_t nf, int64_t big_pq, int64
 
 int host_grow_index(float x, int n) { return f12k::grow_index(x, n); }
 
+// n candidates against a table: 1 negligible, 0 not, as the kernels decide
+// (got) and weighed in double precision (want); returns how many took both.
+int host_screen(const double *g, int ng, double limit, const double *v, const double *u, const double *iv, int n,
+                int *got, int *want) {
+  std::vector<float> g32;
+  for (int i = 0; i < ng; ++i) g32.push_back(g[i] < 3e38 ? (float)g[i] : INFINITY);
+  const double band = f12k::screen_band(g, ng);
+  int both = 0;
+  for (int i = 0; i < n; ++i) {
+    want[i] = f12k::screen_negligible(v[i], u[i], iv[i], limit, g, ng) ? 1 : 0;
+    const int s = f12k::screen_single(v[i], u[i], iv[i], limit / band, limit * band, g32.data(), ng);
+    got[i] = s >= 0 ? s : want[i];
+    both += s < 0;
+  }
+  return both;
+}
+
 }  // extern "C"

@@ -7,6 +7,7 @@ import re
 import shutil
 import subprocess
 
+import numpy as np
 import pytest
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -24,7 +25,7 @@ def lib():
     deps = [SRC] + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
     if not os.path.exists(LIB) or any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in deps):
         tmp = LIB + ".tmp%d" % os.getpid()
-        subprocess.run([gxx, "-O1", "-std=c++17", "-fPIC", "-shared", "-pthread", "-o", tmp, SRC], check=True)
+        subprocess.run([gxx, "-O1", "-std=c++17", "-ffp-contract=off", "-fPIC", "-shared", "-pthread", "-o", tmp, SRC], check=True)
         os.replace(tmp, LIB)
     return ctypes.CDLL(LIB)
 
@@ -138,3 +139,32 @@ def test_growth_table_index_stays_in_the_table(lib):
     for x in (0.0, 0.5, 1.0, 17.3, 2398.5, 2399.0, 2399.9, 2400.0, 2401.0, 1e6, 2.2e9, 4.3e9, 1e20, 3e38, float("inf"),
               float("nan")):
         assert idx(x, n) == (min(n - 1, int(x) + 1) if x < 1e9 else n - 1), x
+
+
+@pytest.mark.parametrize("rate", [0.02, 0.5, 1.0, 4.0, 9.0])
+def test_primitive_screen_decides_as_in_double_precision(lib, rate):
+    """Weighed in single precision first, every candidate is decided as the weighing
+    in double precision alone decides it: kernels that grow like e^{rate r}
+    (the last two past single precision's range), distances from one centre to
+    past the table, products spread around the threshold and on it."""
+    rng = np.random.default_rng(int(100 * rate))
+    r = np.arange(2401) * 0.05
+    with np.errstate(over="ignore"):
+        g = np.maximum(1.0, np.exp(rate * r) / np.exp(1.5 * rate))
+    n = 200_000
+    R = np.where(rng.random(n) < 0.1, 0.0, rng.uniform(0.0, 130.0, n))
+    R[::7] = 0.05 * np.round(R[::7] / 0.05)            # on the table's entries
+    iv = np.exp(rng.uniform(np.log(1e-3), np.log(60.0), n))
+    gam = np.interp(R, r, np.log(g))                   # about ln Gamma
+    v = 1e-26 * np.exp(-gam + rng.normal(0.0, np.where(rng.random(n) < 0.5, 1.0, 0.01) * (1 + 2 * rate)))
+    v[::11] = 0.0
+    v = np.minimum(v, 0.999e-26)
+    dp, ip = ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int)
+    u = R * R
+    got, want = np.zeros(n, np.int32), np.zeros(n, np.int32)
+    f = lib.host_screen
+    f.argtypes = [dp, ctypes.c_int, ctypes.c_double, dp, dp, dp, ctypes.c_int, ip, ip]
+    both = f(g.ctypes.data_as(dp), len(g), 1e-26, v.ctypes.data_as(dp), u.ctypes.data_as(dp), iv.ctypes.data_as(dp), n,
+             got.ctypes.data_as(ip), want.ctypes.data_as(ip))
+    assert np.array_equal(got, want)
+    assert 0 < want.sum() < n and (rate > 2.0 or both < n // 2)
