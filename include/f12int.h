@@ -68,10 +68,12 @@ typedef struct {
 } f12int_term;
 
 /* Create a context on CUDA device `device`.  hbm_budget_bytes caps the
- * device memory the context allocates (0 = no cap; the grids of auxiliary
- * functions, up to 280 MB per factor pair and shared by every context of the
- * device that uses it, are not counted).  cuda_stream is the
- * default stream for the context (NULL = the legacy default stream).
+ * device memory the context allocates (0 = no cap).  Not counted are the grids
+ * of auxiliary functions, up to 280 MB per factor pair and shared by every
+ * context of the device that uses it, and 330 MB of scratch while
+ * f12int_set_factor(_terms) builds one; where the device lacks the memory the
+ * classes are evaluated without a grid (several times slower).  cuda_stream is
+ * the default stream for the context (NULL = the legacy default stream).
  * On success *ctx receives a new context the caller must f12int_destroy. */
 int f12int_create(f12int_ctx **ctx, int device, size_t hbm_budget_bytes, void *cuda_stream);
 
