@@ -26,7 +26,7 @@ Two further workloads, each printing its own JSON line:
   --workload mixed    40 atoms, 5s4p3d2f, 1-8 primitives, exponents [0.02, 500]:
                       per class a bound-stratified sample of shell quartets (half
                       with Schwarz bound product >= 1e-4, half below), FP64 against
-                      the mixed path (FP32 recursion and contraction below 1e-4):
+                      the mixed path (contraction in FP32 below 1e-4):
                       time and the mixed path's max abs/rel difference.
   --workload perl     the 12-atom workload split by class and (la, lb, lc, ld): shell and
                       primitive quartets/s of every combination, with the FP64 rate of each

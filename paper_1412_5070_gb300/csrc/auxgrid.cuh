@@ -82,8 +82,10 @@ F12_HD constexpr int grid_terms(int L) { return L <= 8 ? 13 : 14; }
 
 // Coefficients of row L + k that a point of highest order L reads: the k-th
 // Taylor term is smaller by some 0.1^k, and so is what its last coefficients
-// add (with 15 - k the errors against the oracle stay those of all 12; 13 - k
-// costs an order at L = 8).  Takes 52 of 143 multiply-adds off the rows past L.
+// add (with 15 - k the errors against the oracle stay those of all 12 over
+// molecules' exponents and distances; 13 - k costs an order at L = 8).  Takes 52 of 143
+// multiply-adds off the rows past L.  Kernels that grow or decay too fast for it are
+// found by the cells' check, which evaluates these forms.
 F12_HD constexpr int grid_coefs(int L, int k) {
   return k <= 3 || L > 8 ? GR_NC : (k >= 11 ? 4 : 15 - k);
 }
@@ -235,6 +237,7 @@ F12_DEV inline GridPoint grid_point(const double *xt, double v, double u) {
 }
 
 // ---------------------------------------------------------- double-double --
+// (two-sum and two-product of Knuth and Dekker, the latter with a fused multiply-add)
 struct dd {
   double h, l;
 };

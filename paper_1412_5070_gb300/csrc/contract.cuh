@@ -337,8 +337,8 @@ __device__ __forceinline__ float tfma(float a, float b, float c) { return fmaf(a
 // The rows of the kept primitive quartets of a group, spread over their cubes:
 // asynchronous copies, so that the whole group's are in flight at once and the
 // products below are formed meanwhile (one load at a time, a block of one warp
-// waited about 20,000 cycles for 16 rows: 2000 mixed I4 quartets of up to 4096
-// primitive quartets 22.5 ms, so 20.1; 600,000 I5 quartets 134 and 129 ms).
+// waited about 20,000 cycles for 16 rows: 2000 mixed I4 quartets of one molecule, of up to 4096
+// primitive quartets, 22.5 ms, so 20.1; 600,000 I5 quartets 134 and 129 ms).
 __device__ __forceinline__ void stage_rows(double *cube, const double *rk, unsigned mask, int nk, int nhL, int pitch,
                                            int P3, const int *cpos, int tid, int nthr) {
   for (int i = tid; i < nhL; i += nthr) {

@@ -40,7 +40,7 @@ struct EngineReq {
   const f12int_ctx::BasisData *B = nullptr;   // stable: the deque never moves its elements
   uint32_t mask = 0;
   bool grid = false;                  // every class from the auxiliary grid
-  int precision = 0;                  // 1: FP32 recursion and contraction below the FP32 bound
+  int precision = 0;                  // 1: contraction in FP32 below the FP32 bound
   double thresh = 0.0;
   double *out = nullptr;
   std::vector<int32_t> q;
@@ -239,7 +239,7 @@ static int engine_capture(f12int_ctx *ctx, Engine &E, bool grid) {
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    k_zero_blocks<<<4 * 152, 128, 0, cs>>>(E.zero_dst, E.zero_len, E.zero_count);
+    k_zero_blocks<<<4 * kSMs, 128, 0, cs>>>(E.zero_dst, E.zero_len, E.zero_count);
     cudaEventRecord(fork, cs);
     for (int cls = 1; cls <= 6; ++cls) {
       cudaStream_t bs = E.branch[cls];
@@ -562,7 +562,7 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
       return nt;
     };
     for (Item &it : items) it.tier = it.tier ? kTiers : 0;
-    if (plan(std::min(E.task_target[cls], std::max(1e5, 2.0 * total / (152 * 12)))) > E.tcap)
+    if (plan(std::min(E.task_target[cls], std::max(1e5, 2.0 * total / (kSMs * 12)))) > E.tcap)
       plan(std::max(E.task_target[cls], kTaskFlops / 8));
     // working order: by tier, then decreasing work per task (the longest
     // tasks start first)
@@ -649,7 +649,7 @@ static int engine_launch(f12int_ctx *ctx, Engine &E, const std::vector<EngineReq
     if (large) {
       const int rc = engine_large(ctx, E, large, grid, big.swap ? big.npcd : big.npab, big.npab * big.npcd, big.rows, big.tier);
       if (rc != F12INT_OK) return rc;
-      if (first && nzero > 0) k_zero_blocks<<<4 * 152, 128, 0, st>>>(E.zero_dst, E.zero_len, E.zero_count);
+      if (first && nzero > 0) k_zero_blocks<<<4 * kSMs, 128, 0, st>>>(E.zero_dst, E.zero_len, E.zero_count);
     } else {
       CK(cudaGraphLaunch(E.exec[grid], st));
     }

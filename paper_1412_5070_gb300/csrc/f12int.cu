@@ -1497,7 +1497,7 @@ static int plan_kinds(const f12int_ctx::BasisData &B, int cls, int64_t n, const 
     if (!k.thin) total += (double)k.count * (double)(k.nab * k.ncd) * task_fmas(k.shape, k.ncd, k.shape.ncd());
   // about a dozen tasks per SM where the list has the work for it (a block's
   // result does not depend on how a quartet is cut into ranges)
-  const double target = fewest ? 1e300 : std::min(kTaskFmas, std::max(5e4, total / (152 * 12)));
+  const double target = fewest ? 1e300 : std::min(kTaskFmas, std::max(5e4, total / (kSMs * 12)));
   for (Kind &k : kinds) {
     k.pl = ContractPlan{32, 1, 0};
     if (k.thin) {
@@ -1651,12 +1651,12 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
   // (quartets of thousands of primitive quartets and few entries: a few blocks of
   // milliseconds each) go first, and every launch then to the stream with the
   // least before it: in the list's order, smallest blocks last, they had the GPU
-  // to themselves in the end (2000 mixed I4 quartets 20.4 ms, so 18.2; 3000 f-shell
+  // to themselves in the end (2000 mixed I4 quartets of one molecule 20.4 ms, so 18.2; 3000 f-shell
   // I2 quartets 3.18 and 3.04).  Lists without such launches keep their order
   // (sorting every launch by its longest block: 17.6 and 3.24 ms).
   double all_warps = 0.0;
   for (const ListPlan::Group &g : P.groups) all_warps += g.warps;
-  const double pole = 0.25 * all_warps / (152 * 16);   // cycles, at 16 warps an SM
+  const double pole = 0.25 * all_warps / (kSMs * 16);   // cycles, at 16 warps an SM
   auto is_pole = [&](const ListPlan::Group &g) { return g.longest > std::max(pole, kPoleCycles); };
   bool poles = false;
   std::vector<int> launch_order;
@@ -1676,7 +1676,7 @@ static int launch_list(f12int_ctx *ctx, const ListPlan &P, const ListBufs &D, co
   };
   auto side = [&](const ListPlan::Group &g) -> cudaStream_t {
     const int i = (int)(std::min_element(load, load + NSIDE) - load);
-    load[i] += poles ? std::max(g.longest, g.warps / (152 * 16)) : 1.0;
+    load[i] += poles ? std::max(g.longest, g.warps / (kSMs * 16)) : 1.0;
     if (!(waits >> i & 1)) cudaStreamWaitEvent(ctx->side[i], ctx->fork, 0);
     waits |= 1u << i;
     used |= 1u << i;
@@ -2004,7 +2004,7 @@ static int compute_class_impl(f12int_ctx *ctx, int basis_id, int cls, const int3
   CK(cudaMemcpyAsync(hs.p + 16 * n, offsets_dev, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   ListPlan P;
-  // mixed path: FP32 Hermite recursion and contraction below the bound
+  // mixed path: contraction in FP32 below the bound
   int rc = plan_kinds(B, cls, n, (const int32_t *)hs.p, [&](const int32_t *s) {
     return fp32_below > 0.0 && screen_estimate(ctx, B, cls, s[0], s[1], s[2], s[3]) < fp32_below ? 1 : 0;
   }, P);

@@ -9,7 +9,7 @@
 // cell at one point.  The rows of that point come from a quadrature of its own
 // (the first two kernels again, with narrower panels): against the cells' own
 // quadrature, what that does not resolve would pass.  Bound by the FP64 pipe;
-// setting a factor pair with four kernels takes 0.17 s with it.
+// setting a factor pair with four kernels takes 0.23 s with it.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

@@ -13,6 +13,7 @@
 namespace f12k {
 
 constexpr int kLaux = 14;                          // highest radial order (I5 of f shells)
+constexpr int kSMs = 152;                          // of a GB300
 constexpr int kPartPitch = 16;                     // doubles per family-partial row (128 bytes, whole sectors)
 constexpr int kSkipKey = 24 * (kLaux + 1) * 34;    // work-item key of a primitive quartet the screen drops
 

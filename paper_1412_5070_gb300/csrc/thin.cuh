@@ -19,7 +19,8 @@ namespace f12k {
 // pipe (75-90% busy): 11.3 ms for the 144,000 thin quartets of 200,000 I4 ones with
 // g_n from the grid (12.4 with the divisions and square roots of 1/xi and the
 // prefactor, which pair data now hold; 160 ms more when g_n came family by
-// family), 10% less of the call since the screen's test runs in FP32.
+// family), 10% less of the call since the screen settles most
+// candidates in single precision.
 
 __host__ __device__ constexpr int cart_i(int l, int k) {   // x exponent of component k of shell l
   int n = 0;

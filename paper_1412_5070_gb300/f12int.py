@@ -215,8 +215,8 @@ def f12int_compute_class(ctx, basis_id: int, cls: int, quartets_dev, out_dev, of
 
 def f12int_compute_class_mixed(ctx, basis_id: int, cls: int, quartets_dev, out_dev, offsets_dev, fp32_below: float,
                                stream=None) -> None:
-    """As f12int_compute_class, with the Hermite recursion and contraction in
-    FP32 for quartets whose shell-pair bound product is below fp32_below."""
+    """As f12int_compute_class, with the contraction in FP32 for quartets whose
+    screening estimate is below fp32_below."""
     n = quartets_dev.numel() // 4
     _check(load().f12int_compute_class_mixed(ctx, int(basis_id), int(cls), _ptr(quartets_dev), n, _ptr(out_dev),
                                              _ptr(offsets_dev), float(fp32_below), _stream_ptr(stream)),
