@@ -109,7 +109,7 @@ constexpr double kPrimScreen = 1e-26;
 // two charge distributions, whose overlap e^{-xi w^2} reaches out to R + w.
 // A candidate is weighed, as the shell screen weighs a shell quartet, by the
 // growth Gamma that its overlap reaches (screen.h).  The weighing is in single
-// precision, and in double where that does not settle it (a per cent of the
+// precision, and in double where that does not settle it (few of the
 // candidates): in double precision throughout, its square roots, taken by the
 // whole warp whenever one lane has a candidate, were a third of the thin
 // contraction's FP64 instructions.

@@ -21,13 +21,15 @@ F12_HD inline int grow_index(double x, int n) { return (int)fmin(x, (double)(n -
 // (e^{-xi w^2} = e^{-k^2/4} at the k-th sample), G from its table g of n entries.
 F12_HD inline bool screen_negligible(double v, double u, double iv, double limit, const double *g, int n) {
   const double R = sqrt(u), hw = 0.5 * sqrt(iv);
-  constexpr double kOverlap[7] = {1.0, 0.77880078307140487, 0.36787944117144233, 0.10539922456186433,
-                                  0.018315638888734179, 0.0019304541362277093, 0.00012340980408667956};
-  double gam = 0.0;
+  double gam = 0.0, w = 1.0, q = 0.77880078307140487;   // e^{-k^2/4} from one sample to the next
 #ifdef __CUDACC__
-#pragma unroll
+#pragma unroll 1   // (seldom taken: kept small beside the code that is)
 #endif
-  for (int k = 0; k < 7; ++k) gam = fmax(gam, g[grow_index((R + k * hw) * (1.0 / kGrowStep), n)] * kOverlap[k]);
+  for (int k = 0; k < 7; ++k) {
+    gam = fmax(gam, g[grow_index((R + k * hw) * (1.0 / kGrowStep), n)] * w);
+    w *= q;
+    q *= 0.60653065971263342;
+  }
   return v * gam < limit;
 }
 
