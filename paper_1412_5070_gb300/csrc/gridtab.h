@@ -88,7 +88,7 @@ inline bool grid_families(const f12::TermList &kernel, GridClass &gc) {
 
 constexpr int GR_NQ = 16;        // Gauss-Legendre nodes per panel
 constexpr int GR_NQ0 = 64;       // nodes of the first panel, in x = w u^8
-constexpr int GR_MAXPANEL = 400;
+constexpr int GR_MAXPANEL = 512;   // (of the check: a quarter more than the cells take)
 
 // Quadrature points of one octave of xi (all of its cells use them): panels
 // of 1.25 widths of the Gaussian -- of the narrowest family's times the

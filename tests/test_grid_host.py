@@ -164,3 +164,10 @@ def test_default_factor_stays_on_the_grid(lib):
             assert all(g.ok(xi, D) == 1 for xi in (0.02, 0.0305, 4.1, 500.0) for D in (0.0, 8.0, 20.0))
             # (high orders pass through zero here)
             assert all(g.ok(xi, np.sqrt(T / xi)) == 1 for xi in (0.133, 0.266, 0.53) for T in (0.3, 0.4, 0.9))
+
+
+def test_steep_decay_has_both_quadratures(lib):
+    """The check's narrower panels are not what a factor is refused for: a decay of
+    e^{-60 r} takes 337 panels in the lowest octave, 421 for the check."""
+    g = Grid(lib, rs12(B=-60.0), 3)
+    assert g.ok(0.0081, 0.3) != -1
