@@ -484,7 +484,7 @@ struct f12int_ctx {
   // in both precisions; grows[cls]: the kernel of cls grows (G > 1 somewhere)
   double *d_kgrow = nullptr;
   float *d_kgrow32 = nullptr;
-  double grow_band[7] = {0.0};
+  float grow_band[7] = {0.0f};
   size_t kgrow_bytes = 0;
   int kgrow_n = 0;
   bool grows[7] = {false, false, false, false, false, false, false};
@@ -558,14 +558,13 @@ struct NvtxRange {
 // screen is set and the factors exist.
 PairView pair_view(const f12int_ctx *ctx, const f12int_ctx::BasisData &B, int cls, bool screen) {
   PairView v{B.d_pair_start, B.d_pp_p, B.d_pp_P, B.d_pp_ab, B.d_pp_eoff, B.d_epool, B.d_shell_l, B.nshell,
-             nullptr, nullptr, nullptr, 0.0, 0.0, 0};
+             nullptr, nullptr, nullptr, 0.0f, 0};
   if (screen && B.d_qprim[cls]) {
     v.qprim = B.d_qprim[cls];
     if (ctx->grows[cls] && ctx->d_kgrow) {
       v.grow = ctx->d_kgrow + (size_t)cls * ctx->kgrow_n;
       v.grow32 = ctx->d_kgrow32 + (size_t)cls * ctx->kgrow_n;
-      v.grow_lo = kPrimScreen / ctx->grow_band[cls];
-      v.grow_hi = kPrimScreen * ctx->grow_band[cls];
+      v.grow_band = ctx->grow_band[cls];
       v.ngrow = ctx->kgrow_n;
     }
   }

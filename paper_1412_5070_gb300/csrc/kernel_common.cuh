@@ -29,8 +29,8 @@ struct PairView {
   int nshell;
   const double *qprim;       // [npp] primitive Schwarz factors of the class, or null
   const double *grow;        // [ngrow] growth G(i kGrowStep) of the class's kernel, or null (no growth)
-  const float *grow32;       // the same in single precision, and what it settles (screen.h)
-  double grow_lo, grow_hi;
+  const float *grow32;       // the same in single precision, and its band (screen.h)
+  float grow_band;
   int ngrow;
 };
 
@@ -99,6 +99,7 @@ __host__ __device__ constexpr int aux_direct_fmas(const bool boys, int L) {
 }
 
 constexpr double kPrimScreen = 1e-26;
+constexpr float kPrimScreenLog2 = -86.37013f;   // its binary logarithm
 
 // Primitive quartets whose Schwarz product is below kPrimScreen are skipped:
 // the skipped contributions stay below the absolute accuracy that elements
@@ -119,7 +120,7 @@ __device__ __forceinline__ bool prim_negligible(const PairView &PV, int pab, int
   if (v >= kPrimScreen) return false;
   if (!PV.grow) return true;
   const double iv = PV.pp_ab[4 * pab + 2] + PV.pp_ab[4 * pcd + 2];
-  const int s = screen_single(v, u, iv, PV.grow_lo, PV.grow_hi, PV.grow32, PV.ngrow);
+  const int s = screen_single(v, u, iv, kPrimScreenLog2, PV.grow32, PV.ngrow, PV.grow_band);
   return s >= 0 ? s == 1 : screen_negligible(v, u, iv, kPrimScreen, PV.grow, PV.ngrow);
 }
 

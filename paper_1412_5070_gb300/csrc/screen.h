@@ -33,28 +33,43 @@ F12_HD inline bool screen_negligible(double v, double u, double iv, double limit
   return v * gam < limit;
 }
 
-// The same, its outcome taken from single precision where that settles it: a
-// distance rounded there is off by at most one entry of the table, so Gamma by at
-// most the largest ratio of neighbouring entries (and a little for the
-// roundings), and lo and hi are limit over and times that.  1: negligible, 0: not,
-// -1: to be weighed in double precision.
-F12_HD inline int screen_single(double v, double u, double iv, double lo, double hi, const float *g, int n) {
+// The same, its outcome taken from single precision where that settles it,
+// without an FP64 instruction: the logarithms of v and Gamma against lim =
+// log2(limit).  Their roundings are within kScreenSlack; a distance rounded there
+// (2.5e-7 of it) is in the next entry of the table only within 2e-3 of one, and
+// Gamma then off by at most the largest ratio of neighbouring entries, 2^band.
+// 1: negligible, 0: not, -1: to be weighed in double precision.
+constexpr float kScreenSlack = 2e-4f;
+F12_HD inline int screen_single(double v, double u, double iv, float lim, const float *g, int n, float band) {
   const float R = sqrtf((float)u), hw = 0.5f * sqrtf((float)iv);
   constexpr float kOverlap[7] = {1.0f, 0.77880078307140487f, 0.36787944117144233f, 0.10539922456186433f,
                                  0.018315638888734179f, 0.0019304541362277093f, 0.00012340980408667956f};
   float gam = 0.0f;
+  bool edge = false;
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-  for (int k = 0; k < 7; ++k) gam = fmaxf(gam, g[grow_index((R + k * hw) * (float)(1.0 / kGrowStep), n)] * kOverlap[k]);
-  const double w = v * (double)gam;
-  return w < lo ? 1 : w >= hi && gam < 3e38f ? 0 : -1;
+  for (int k = 0; k < 7; ++k) {
+    const float x = (R + k * hw) * (float)(1.0 / kGrowStep);
+    edge = edge || fabsf(x - rintf(x)) < 2e-3f;
+    gam = fmaxf(gam, g[grow_index(x, n)] * kOverlap[k]);
+  }
+  const int h = f12dev::grid_hi(v), m = 0x3f800000 | (h & 0xFFFFF) << 3;   // (its mantissa as a float in [1, 2))
+#ifdef __CUDA_ARCH__
+  const float t = (float)((h >> 20) - 1023) + __log2f(__int_as_float(m)) + __log2f(gam);
+#else
+  float f;
+  std::memcpy(&f, &m, sizeof f);
+  const float t = (float)((h >> 20) - 1023) + log2f(f) + log2f(gam);
+#endif
+  const float d = kScreenSlack + (edge ? band : 0.0f);
+  return !(gam < 3e38f) ? -1 : t < lim - d ? 1 : t >= lim + d ? 0 : -1;
 }
-// that ratio of a table (one that leaves the range of numbers settles nothing)
-inline double screen_band(const double *g, int n) {
+// band of a table (one that leaves the range of numbers settles next to nothing)
+inline float screen_band(const double *g, int n) {
   double r = 1.0;
   for (int i = 0; i + 1 < n; ++i) r = fmax(r, g[i + 1] / g[i]);
-  return fmin(r * (1.0 + 1e-5), 1e300);
+  return (float)fmin(log2(r), 1e4);
 }
 
 }  // namespace f12k

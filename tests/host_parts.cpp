@@ -93,11 +93,11 @@ int host_screen(const double *g, int ng, double limit, const double *v, const do
                 int *got, int *want) {
   std::vector<float> g32;
   for (int i = 0; i < ng; ++i) g32.push_back(g[i] < 3e38 ? (float)g[i] : INFINITY);
-  const double band = f12k::screen_band(g, ng);
+  const float band = f12k::screen_band(g, ng), lim = (float)std::log2(limit);
   int both = 0;
   for (int i = 0; i < n; ++i) {
     want[i] = f12k::screen_negligible(v[i], u[i], iv[i], limit, g, ng) ? 1 : 0;
-    const int s = f12k::screen_single(v[i], u[i], iv[i], limit / band, limit * band, g32.data(), ng);
+    const int s = f12k::screen_single(v[i], u[i], iv[i], lim, g32.data(), ng, band);
     got[i] = s >= 0 ? s : want[i];
     both += s < 0;
   }

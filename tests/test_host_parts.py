@@ -164,7 +164,13 @@ def test_primitive_screen_decides_as_in_double_precision(lib, rate):
     got, want = np.zeros(n, np.int32), np.zeros(n, np.int32)
     f = lib.host_screen
     f.argtypes = [dp, ctypes.c_int, ctypes.c_double, dp, dp, dp, ctypes.c_int, ip, ip]
+    f(g.ctypes.data_as(dp), len(g), 1e-26, v.ctypes.data_as(dp), u.ctypes.data_as(dp), iv.ctypes.data_as(dp), n,
+      got.ctypes.data_as(ip), want.ctypes.data_as(ip))
+    assert np.array_equal(got, want)
+    assert 0 < want.sum() < n
+    # candidates as they come, over thirty orders of magnitude: few take both weighings
+    v = np.minimum(1e-26 * np.exp(-gam + rng.uniform(-35.0, 35.0, n)), 0.999e-26)
     both = f(g.ctypes.data_as(dp), len(g), 1e-26, v.ctypes.data_as(dp), u.ctypes.data_as(dp), iv.ctypes.data_as(dp), n,
              got.ctypes.data_as(ip), want.ctypes.data_as(ip))
     assert np.array_equal(got, want)
-    assert 0 < want.sum() < n and (rate > 2.0 or both < n // 2)
+    assert rate > 0.6 or both < n // 10   # (past that the table leaves single precision within the distances)
