@@ -118,7 +118,7 @@ __device__ __forceinline__ bool prim_negligible(const PairView &PV, int pab, int
   if (!PV.qprim) return false;
   const double v = PV.qprim[pab] * PV.qprim[pcd];
   if (v >= kPrimScreen) return false;
-  if (!PV.grow) return true;
+  if (!PV.grow32) return true;
   const double iv = PV.pp_ab[4 * pab + 2] + PV.pp_ab[4 * pcd + 2];
   const int s = screen_single(v, u, iv, kPrimScreenLog2, PV.grow32, PV.ngrow, PV.grow_band);
   return s >= 0 ? s == 1 : screen_negligible(v, u, iv, kPrimScreen, PV.grow, PV.ngrow);
